@@ -14,6 +14,7 @@ namespace lmmew {
 namespace {
 thread_local std::string g_err;
 constexpr size_t kRowBudgetFloats = size_t(1) << 30;   // 4 GiB of row block per chunk
+constexpr size_t kNodeBudgetBytes = size_t(1) << 30;   // node sums of the angles in flight
 }  // namespace
 
 int set_error(int code, const std::string& msg) {
@@ -237,8 +238,8 @@ int row_stride_of(const lm_handle* h) { return (h->mc.nq + 3) & ~3; }
 
 }  // namespace
 
-int launch_row_profiled(lm_handle* h, const RowLaunch& L, cudaStream_t st) {
-    if (!h->prof_on) return launch_row(h, L, st);
+int prof_start(lm_handle* h, cudaStream_t st) {
+    if (!h->prof_on) return LMMEW_OK;
     if (h->prof_used + 2 > h->prof_ev.size()) {
         for (int i = 0; i < 64; ++i) {
             cudaEvent_t e;
@@ -246,13 +247,25 @@ int launch_row_profiled(lm_handle* h, const RowLaunch& L, cudaStream_t st) {
             h->prof_ev.push_back(e);
         }
     }
-    cudaEvent_t e0 = h->prof_ev[h->prof_used], e1 = h->prof_ev[h->prof_used + 1];
-    LMMEW_CUDA(cudaEventRecord(e0, st));
-    const int rc = launch_row(h, L, st);
-    if (rc != LMMEW_OK) return rc;
-    LMMEW_CUDA(cudaEventRecord(e1, st));
+    LMMEW_CUDA(cudaEventRecord(h->prof_ev[h->prof_used], st));
+    return LMMEW_OK;
+}
+
+int prof_stop(lm_handle* h, double terms, cudaStream_t st) {
+    if (!h->prof_on) return LMMEW_OK;
+    LMMEW_CUDA(cudaEventRecord(h->prof_ev[h->prof_used + 1], st));
     h->prof_used += 2;
     h->prof_launches += 1;
+    h->prof_node_terms += terms;
+    return LMMEW_OK;
+}
+
+int launch_row_profiled(lm_handle* h, const RowLaunch& L, cudaStream_t st) {
+    if (!h->prof_on) return launch_row(h, L, st);
+    int rc = prof_start(h, st);
+    if (rc == LMMEW_OK) rc = launch_row(h, L, st);
+    if (rc == LMMEW_OK) rc = prof_stop(h, 0.0, st);
+    if (rc != LMMEW_OK) return rc;
     h->prof_terms_dense += (double)L.n_events * (double)h->terms_per_event;
     h->prof_elems += (double)L.n_events * (double)h->mc.nq;
     return LMMEW_OK;
@@ -325,6 +338,47 @@ int forward_async(lm_handle* h, const lm_events* ev, const float* image, float* 
     }
     if (rc == LMMEW_OK) rc = launch_invalid_out(h, se.group_start + p.G, p.n, se.perm, out_y, st);
     return rc;
+}
+
+// Forward projection through the energy nodes, the angles in blocks of
+// `block` (their node sums live in the arena); the events stay in the caller's
+// order and are not sorted.
+int forward_nodes(lm_handle* h, const lm_events* ev, const float* image, float* out_y, int block,
+                  char* arena, cudaStream_t st) {
+    const ModelConst& m = h->mc;
+    const NodeConst& N = h->nodes;
+    float* lam_v = bump<float>(arena, m.nq);
+    float* dbp = bump<float>(arena, (size_t)block * m.npc * N.nb_max * N.nl_pad);
+    float* F = bump<float>(arena, (size_t)block * m.B * N.nk_pad);
+    float* Pr = bump<float>(arena, (size_t)block * m.B * N.W);
+    int rc = launch_gather_image(h, image, lam_v, st);
+    for (int a0 = 0; a0 < m.A && rc == LMMEW_OK; a0 += block) {
+        const int cnt = std::min(block, m.A - a0);
+        rc = node_forward(h, lam_v, a0, 1, cnt, dbp, F, Pr, st);
+        if (rc == LMMEW_OK) rc = node_events_forward(h, ev, F, Pr, a0, cnt, out_y, st);
+    }
+    if (h->prof_on) h->prof_elems += (double)ev->n * (double)m.nq;
+    return rc;
+}
+
+int forward_nodes_block(const lm_handle* h, size_t bytes) {
+    const size_t fixed = bump_bytes(sizeof(float) * (size_t)h->mc.nq) + 3 * 512;
+    const size_t per = node_angle_bytes(h);
+    return (int)std::max<size_t>(1, std::min<size_t>((size_t)h->mc.A, (bytes - fixed) / per));
+}
+
+size_t forward_nodes_bytes(const lm_handle* h, int block) {
+    return bump_bytes(sizeof(float) * (size_t)h->mc.nq) + 3 * 512 +
+           (size_t)block * node_angle_bytes(h);
+}
+
+bool node_use(const lm_handle* h, int64_t n) {
+    return h->node_route && h->n_classes > 1 && h->prec == 0 &&
+           h->scatter_model == LMMEW_SCATTER_EXACT && n >= (int64_t)8 * h->mc.A;
+}
+
+bool node_use_osem(const lm_handle* h, int64_t n) {
+    return node_use(h, n) && n >= (int64_t)120 * h->mc.A;
 }
 
 }  // namespace lmmew
@@ -418,6 +472,7 @@ int lm_create(const lm_geometry* g, const lm_attenuation* at, const lm_lines* ln
     h->n_subsets_default = n_subsets;
     int rc = build_tables(h, at->rho, support);
     if (rc == LMMEW_OK) build_energy_classes(h);
+    if (rc == LMMEW_OK) rc = build_nodes(h);
     if (rc == LMMEW_OK &&
         (cudaMalloc(&h->d_term_counter, sizeof(unsigned long long)) != cudaSuccess ||
          cudaMemset(h->d_term_counter, 0, sizeof(unsigned long long)) != cudaSuccess ||
@@ -481,6 +536,9 @@ int lm_destroy(lm_handle* h) {
     cudaFree(h->d_inv);
     cudaFree(h->d_mu_line);
     cudaFree(h->d_clip);
+    cudaFree(h->d_node_g);
+    cudaFree(h->d_node_band);
+    cudaFree(h->d_chunk_bins);
     cudaFree(h->d_term_counter);
     cudaFree(h->d_work);
     cudaFree(h->d_cv);
@@ -732,6 +790,13 @@ int lm_forward(lm_handle* h, const lm_events* ev, const float* image, float* out
     if (ev->n == 0) return LMMEW_OK;
     if (surrogate_model(h)) return forward_planned(h, ev, image, out_y, stream);
     cudaStream_t st = (cudaStream_t)stream;
+    if (node_use(h, ev->n)) {
+        const int block = forward_nodes_block(h, kNodeBudgetBytes);
+        rc = ensure(h, h->scratch_sort, forward_nodes_bytes(h, block), st);
+        if (rc == LMMEW_OK)
+            return forward_nodes(h, ev, image, out_y, block, (char*)h->scratch_sort.ptr, st);
+        if (rc != LMMEW_ERR_OOM) return rc;   // no room for the node sums: the rows
+    }
     GroupArrays ga;
     rc = group_arrays(h, 1, &ga);
     if (rc != LMMEW_OK) return rc;
@@ -740,6 +805,113 @@ int lm_forward(lm_handle* h, const lm_events* ev, const float* image, float* out
     if (rc != LMMEW_OK) return rc;
     return forward_async(h, ev, image, out_y, ga, fp, (char*)h->scratch_sort.ptr, st);
 }
+
+// Scratch of the node route's sorted forms for row sets of at most `angles`
+// angles; the forward sums go `block` angles at a time.
+namespace {
+struct NodeScratch {
+    int block;
+    float *lam, *dbp, *F, *Pr, *V, *PV, *VG, *part, *part_prim;
+    double *ll, *num;
+};
+size_t node_scratch(const lm_handle* h, int angles, char* base, NodeScratch* s) {
+    const ModelConst& m = h->mc;
+    const NodeConst& N = h->nodes;
+    const size_t cells = (size_t)angles * m.B, nq_pad = (size_t)m.nqt * kQT;
+    s->block = std::min(angles, forward_nodes_block(h, kNodeBudgetBytes));
+    char* p = base;
+    s->lam = bump<float>(p, m.nq);
+    s->dbp = bump<float>(p, (size_t)s->block * m.npc * N.nb_max * N.nl_pad);
+    s->F = bump<float>(p, cells * N.nk_pad);
+    s->Pr = bump<float>(p, cells * m.W);
+    s->V = bump<float>(p, cells * N.nk_pad);
+    s->PV = bump<float>(p, cells * m.W);
+    s->VG = bump<float>(p, cells * N.nl_pad);
+    s->part = bump<float>(p, (size_t)angles * m.npc * m.W * nq_pad);
+    s->part_prim = bump<float>(p, (size_t)angles * nq_pad);
+    s->ll = bump<double>(p, cells);
+    s->num = bump<double>(p, m.nq);
+    return (size_t)(p - base) + 256;
+}
+
+int node_forward_blocks(lm_handle* h, const NodeScratch& s, int a0, int a_step, int angles,
+                        cudaStream_t st) {
+    const ModelConst& m = h->mc;
+    int rc = LMMEW_OK;
+    for (int i = 0; i < angles && rc == LMMEW_OK; i += s.block)
+        rc = node_forward(h, s.lam, a0 + i * a_step, a_step, std::min(s.block, angles - i), s.dbp,
+                          s.F + (size_t)i * m.B * h->nodes.nk_pad, s.Pr + (size_t)i * m.B * m.W, st);
+    return rc;
+}
+
+// Back projection through the energy nodes (OOM before anything is queued when
+// its scratch cannot be had).
+int backproject_nodes(lm_handle* h, const lm_events* ev, const float* weight, float* out_image,
+                      cudaStream_t st) {
+    const ModelConst& m = h->mc;
+    GroupArrays ga;
+    int rc = group_arrays(h, 1, &ga);
+    if (rc != LMMEW_OK) return rc;
+    NodeScratch s;
+    rc = ensure(h, h->scratch_sort, cell_scratch_bytes(h, ev->n), st);
+    if (rc == LMMEW_OK) rc = ensure(h, h->scratch_work, node_scratch(h, m.A, nullptr, &s), st);
+    if (rc != LMMEW_OK) return rc;
+    node_scratch(h, m.A, (char*)h->scratch_work.ptr, &s);
+    char* arena = (char*)h->scratch_sort.ptr;
+    CellEvents ce;
+    rc = sort_cells(h, ev, ga.rank_of_angle, &ce, arena, st);
+    if (rc == LMMEW_OK)
+        rc = node_cells(h, m.A, ce.cell_start, 0, ce.energy, nullptr, nullptr, weight, ce.perm, s.V,
+                        s.PV, nullptr, st);
+    if (rc == LMMEW_OK) rc = node_back(h, 0, 1, m.A, s.V, s.PV, s.VG, s.part, s.part_prim, st);
+    if (rc == LMMEW_OK) rc = node_update(h, m.A, s.part, s.part_prim, nullptr, nullptr, s.num, st);
+    if (rc != LMMEW_OK) return rc;
+    if (h->prof_on) h->prof_elems += (double)ev->n * (double)m.nq;
+    return launch_num_to_image(h, s.num, out_image, st);
+}
+
+// LM-OSEM through the energy nodes: every sub-iteration projects its subset's
+// angles forward, forms the ratios cell by cell and projects them back.
+int osem_nodes(lm_handle* h, const lm_events* ev, int n_subsets, int n_iters, int start_iter,
+               int start_subset, float* image, double* loglik, cudaStream_t st) {
+    const ModelConst& m = h->mc;
+    GroupArrays ga;
+    int rc = group_arrays(h, n_subsets, &ga);
+    if (rc != LMMEW_OK) return rc;
+    const int most = (m.A + n_subsets - 1) / n_subsets;
+    NodeScratch s;
+    rc = ensure(h, h->scratch_sort, cell_scratch_bytes(h, ev->n), st);
+    if (rc == LMMEW_OK) rc = ensure(h, h->scratch_work, node_scratch(h, most, nullptr, &s), st);
+    if (rc != LMMEW_OK) return rc;
+    node_scratch(h, most, (char*)h->scratch_work.ptr, &s);
+    char* arena = (char*)h->scratch_sort.ptr;
+    CellEvents ce;
+    rc = sort_cells(h, ev, ga.rank_of_angle, &ce, arena, st);
+    if (rc == LMMEW_OK) rc = launch_gather_image(h, image, s.lam, st);
+    for (int it = start_iter; it < n_iters && rc == LMMEW_OK; ++it) {
+        int r0 = 0;
+        for (int sub = 0; sub < n_subsets && rc == LMMEW_OK; ++sub) {
+            const int cnt = (m.A - sub + n_subsets - 1) / n_subsets, cell0 = r0 * m.B;
+            r0 += cnt;
+            if (it == start_iter && sub < start_subset) continue;
+            const double* sens = h->d_sens_sub + (size_t)sub * m.nq;
+            double* ll = loglik ? loglik + (size_t)it * n_subsets + sub : nullptr;
+            rc = node_forward_blocks(h, s, sub, n_subsets, cnt, st);
+            if (rc == LMMEW_OK)
+                rc = node_cells(h, cnt, ce.cell_start, cell0, ce.energy, s.F, s.Pr, nullptr, nullptr,
+                                s.V, s.PV, ll ? s.ll : nullptr, st);
+            if (rc == LMMEW_OK)
+                rc = node_back(h, sub, n_subsets, cnt, s.V, s.PV, s.VG, s.part, s.part_prim, st);
+            if (rc == LMMEW_OK && ll) rc = node_loglik(h, s.ll, cnt * m.B, s.lam, sens, ll, st);
+            if (rc == LMMEW_OK)
+                rc = node_update(h, cnt, s.part, s.part_prim, sens, s.lam, nullptr, st);
+        }
+        if (h->prof_on) h->prof_elems += (double)ev->n * (double)m.nq;
+    }
+    if (rc != LMMEW_OK) return rc;
+    return launch_scatter_image(h, s.lam, image, st);
+}
+}  // namespace
 
 int lm_backproject(lm_handle* h, const lm_events* ev, const float* weight, float* out_image,
                    lm_stream stream) {
@@ -754,6 +926,10 @@ int lm_backproject(lm_handle* h, const lm_events* ev, const float* weight, float
         return LMMEW_OK;
     }
     if (surrogate_model(h)) return backproject_planned(h, ev, weight, out_image, stream);
+    if (node_use(h, ev->n)) {
+        rc = backproject_nodes(h, ev, weight, out_image, st);
+        if (rc != LMMEW_ERR_OOM) return rc;   // no room for the node sums: the rows
+    }
     GroupArrays ga;
     rc = group_arrays(h, 1, &ga);
     if (rc != LMMEW_OK) return rc;
@@ -812,6 +988,10 @@ int lm_osem(lm_handle* h, const lm_events* ev, int n_subsets, int n_iters, int s
     cudaStream_t st = (cudaStream_t)stream;
     rc = subset_sensitivity(h, n_subsets, st);
     if (rc != LMMEW_OK) return rc;
+    if (node_use_osem(h, ev->n)) {
+        rc = osem_nodes(h, ev, n_subsets, n_iters, start_iter, start_subset, image, loglik, st);
+        if (rc != LMMEW_ERR_OOM) return rc;   // no room for the node sums: the rows
+    }
     GroupArrays ga;
     rc = group_arrays(h, n_subsets, &ga);
     if (rc != LMMEW_OK) return rc;
@@ -901,26 +1081,14 @@ int lm_check(lm_handle* h, lm_stream stream) {
     return take_status(h, (cudaStream_t)stream);
 }
 
-int lm_osem_batch(lm_handle* h, int n_real, const lm_events* events, int n_subsets, int n_iters,
-                  float* images, double* loglik, lm_stream stream) {
-    if (!h || !events || !images) return set_error(LMMEW_ERR_INVALID_ARG, "NULL argument");
+// The batch through shared row launches.  index: null, or the image (and
+// log-likelihood row) of each of the n_real realisations.
+static int osem_batch_rows(lm_handle* h, int n_real, const lm_events* events, const int* index,
+                           int n_subsets, int n_iters, float* images, double* loglik,
+                           lm_stream stream) {
     const ModelConst& m = h->mc;
-    if (n_real < 1 || n_real > 65535) return set_error(LMMEW_ERR_INVALID_ARG, "1..65535 realisations");
-    if (n_subsets < 1 || n_subsets > m.A)
-        return set_error(LMMEW_ERR_INVALID_ARG, "n_subsets must be in 1..n_angles");
-    if (n_iters < 0) return set_error(LMMEW_ERR_INVALID_ARG, "negative iteration count");
     int64_t n_total = 0;
-    for (int r = 0; r < n_real; ++r) {
-        int rc = check_events(h, &events[r]);
-        if (rc != LMMEW_OK) return rc;
-        n_total += events[r].n;
-    }
-    if (n_total >= (int64_t(1) << 31))
-        return set_error(LMMEW_ERR_INVALID_ARG, "at most 2^31 - 1 events per batch");
-    if (h->tab_slots && h->scatter_model == LMMEW_SCATTER_EXACT && m.np > 0)
-        return set_error(LMMEW_ERR_NOT_IMPLEMENTED,
-                         "batched reconstruction needs every angle's path tables resident "
-                         "(lm_set_table_streaming(h, 0)) or a surrogate or scatter-free model");
+    for (int r = 0; r < n_real; ++r) n_total += events[r].n;
     const int R = n_real;
     const int A_s = (m.A + n_subsets - 1) / n_subsets;
     const int64_t V = (int64_t)n_subsets * A_s;
@@ -1001,7 +1169,7 @@ int lm_osem_batch(lm_handle* h, int n_real, const lm_events* events, int n_subse
                         bump_bytes(sizeof(BpChunk) * max_chunks) +
                         bump_bytes(sizeof(int) * (size_t)n_subsets * (R + 1)) +
                         bump_bytes(sizeof(int64_t) * (size_t)(n_blk + 1)) +
-                        bump_bytes(sizeof(int) * (size_t)(G + 1));
+                        bump_bytes(sizeof(int) * (size_t)(G + 1)) + bump_bytes(sizeof(int) * (size_t)R);
     rc = ensure(h, h->scratch_work, need, st);
     if (rc != LMMEW_OK) return rc;
     char* w = (char*)h->scratch_work.ptr;
@@ -1015,6 +1183,11 @@ int lm_osem_batch(lm_handle* h, int n_real, const lm_events* events, int n_subse
     int* d_part = bump<int>(w, (size_t)n_subsets * (R + 1));
     int64_t* d_blk_start = bump<int64_t>(w, (size_t)n_blk + 1);
     int* d_grp_start = bump<int>(w, (size_t)G + 1);
+    int* d_index = bump<int>(w, (size_t)R);
+    if (index)
+        LMMEW_CUDA(cudaMemcpyAsync(d_index, index, sizeof(int) * (size_t)R, cudaMemcpyHostToDevice, st));
+    else
+        d_index = nullptr;
     std::vector<int64_t> blk_start(n_blk + 1, se.n_total);
     for (int b = 0; b < n_blk; ++b) blk_start[b] = blocks[b].e0;
     if (n_blk > 0)
@@ -1056,10 +1229,10 @@ int lm_osem_batch(lm_handle* h, int n_real, const lm_events* events, int n_subse
                                    cudaMemcpyHostToDevice, st));
     LMMEW_CUDA(cudaMemcpyAsync(d_part, part_start.data(), sizeof(int) * part_start.size(),
                                cudaMemcpyHostToDevice, st));
-    rc = launch_images_batch(h, R, images, lam_v, true, st);
+    rc = launch_images_batch(h, R, images, index, d_index, lam_v, true, st);
     if (rc != LMMEW_OK) return rc;
 
-    if (n_iters == 0) return launch_images_batch(h, R, images, lam_v, false, st);
+    if (n_iters == 0) return launch_images_batch(h, R, images, index, d_index, lam_v, false, st);
 
     // the whole reconstruction as one CUDA graph, replayed on the caller's stream
     if (!h->cap_stream) LMMEW_CUDA(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
@@ -1083,7 +1256,7 @@ int lm_osem_batch(lm_handle* h, int n_real, const lm_events* events, int n_subse
             rc = launch_reduce_update_batch(
                 h, R, bpart, d_part + (size_t)s * (R + 1), num, lam_v,
                 h->d_sens_sub + (size_t)s * m.nq, llpart,
-                loglik ? loglik + (size_t)it * n_subsets + s : nullptr, n_iters * n_subsets, cs);
+                loglik ? loglik + (size_t)it * n_subsets + s : nullptr, n_iters * n_subsets, d_index, cs);
         }
     }
     cudaGraph_t graph = nullptr;
@@ -1102,7 +1275,54 @@ int lm_osem_batch(lm_handle* h, int n_real, const lm_events* events, int n_subse
     h->graph = graph;
     h->graph_exec = exec;
     LMMEW_CUDA(cudaGraphLaunch(exec, st));
-    return launch_images_batch(h, R, images, lam_v, false, st);
+    return launch_images_batch(h, R, images, index, d_index, lam_v, false, st);
+}
+
+int lm_osem_batch(lm_handle* h, int n_real, const lm_events* events, int n_subsets, int n_iters,
+                  float* images, double* loglik, lm_stream stream) {
+    if (!h || !events || !images) return set_error(LMMEW_ERR_INVALID_ARG, "NULL argument");
+    const ModelConst& m = h->mc;
+    if (n_real < 1 || n_real > 65535) return set_error(LMMEW_ERR_INVALID_ARG, "1..65535 realisations");
+    if (n_subsets < 1 || n_subsets > m.A)
+        return set_error(LMMEW_ERR_INVALID_ARG, "n_subsets must be in 1..n_angles");
+    if (n_iters < 0) return set_error(LMMEW_ERR_INVALID_ARG, "negative iteration count");
+    int64_t n_total = 0;
+    for (int r = 0; r < n_real; ++r) {
+        int rc = check_events(h, &events[r]);
+        if (rc != LMMEW_OK) return rc;
+        n_total += events[r].n;
+    }
+    if (n_total >= (int64_t(1) << 31))
+        return set_error(LMMEW_ERR_INVALID_ARG, "at most 2^31 - 1 events per batch");
+    if (h->tab_slots && h->scatter_model == LMMEW_SCATTER_EXACT && m.np > 0)
+        return set_error(LMMEW_ERR_NOT_IMPLEMENTED,
+                         "batched reconstruction needs every angle's path tables resident "
+                         "(lm_set_table_streaming(h, 0)) or a surrogate or scatter-free model");
+    // realisations whose event lists are dense enough for the energy nodes go
+    // one after the other (each projection visits every path once whatever
+    // the number of events, so there is nothing to share); the others share
+    // row launches
+    std::vector<lm_events> rest;
+    std::vector<int> rest_of;
+    for (int r = 0; r < n_real; ++r)
+        if (!node_use_osem(h, events[r].n)) {
+            rest.push_back(events[r]);
+            rest_of.push_back(r);
+        }
+    if ((int)rest.size() == n_real)
+        return osem_batch_rows(h, n_real, events, nullptr, n_subsets, n_iters, images, loglik, stream);
+    cudaStream_t st = (cudaStream_t)stream;
+    int rc = LMMEW_OK;
+    for (int r = 0; r < n_real && rc == LMMEW_OK; ++r) rc = launch_validate(h, &events[r], st);
+    if (rc == LMMEW_OK) rc = take_status(h, st);
+    if (rc == LMMEW_OK) rc = subset_sensitivity(h, n_subsets, st);
+    for (int r = 0; r < n_real && rc == LMMEW_OK; ++r)
+        if (node_use_osem(h, events[r].n))
+            rc = lm_osem(h, &events[r], n_subsets, n_iters, 0, 0, images + (size_t)r * m.n * m.n,
+                         loglik ? loglik + (size_t)r * n_iters * n_subsets : nullptr, stream);
+    if (rc != LMMEW_OK || rest.empty()) return rc;
+    return osem_batch_rows(h, (int)rest.size(), rest.data(), rest_of.data(), n_subsets, n_iters,
+                           images, loglik, stream);
 }
 
 int lm_batch_tuning(const lm_handle* h, double* out5) {
@@ -1176,13 +1396,14 @@ int lm_profile_read(lm_handle* h, double* out5) {
     }
     out5[0] = ms;
     out5[1] = (double)h->prof_launches;
-    out5[2] = (double)evaluated;
+    out5[2] = (double)evaluated + h->prof_node_terms;
     out5[3] = h->prof_elems;
     out5[4] = (double)h->launches;
     h->launches = 0;
     h->prof_used = 0;
     h->prof_launches = 0;
     h->prof_terms_dense = 0.0;
+    h->prof_node_terms = 0.0;
     h->prof_elems = 0.0;
     return LMMEW_OK;
 }

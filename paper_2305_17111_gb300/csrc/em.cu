@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(1024) k_update_batch(float* lam, const double*
                                                        const double* sens, int nq,
                                                        const double* llpart,
                                                        const int* part_start, double* loglik,
-                                                       int ll_stride) {
+                                                       int ll_stride, const int* index) {
     __shared__ double red[1024];
     const int t = threadIdx.x, rr = blockIdx.x;
     float* l = lam + (size_t)rr * nq;
@@ -447,23 +447,26 @@ __global__ void __launch_bounds__(1024) k_update_batch(float* lam, const double*
             if (t < off) red[t] += red[t + off];
             __syncthreads();
         }
-        if (t == 0) loglik[(size_t)rr * ll_stride] = red[0];
+        if (t == 0) loglik[(size_t)(index ? index[rr] : rr) * ll_stride] = red[0];
         __syncthreads();
     }
     for (int q = t; q < nq; q += 1024)
         l[q] = sens[q] > 0.0 ? (float)((double)l[q] * nm[q] / sens[q]) : 0.f;
 }
 
-__global__ void k_gather_batch(const float* images, int npix, const int* q_pix, int nq,
-                               float* lam) {
+// (index: null, or the image of each realisation)
+__global__ void k_gather_batch(const float* images, const int* index, int npix, const int* q_pix,
+                               int nq, float* lam) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q < nq) lam[(size_t)blockIdx.y * nq + q] = images[(size_t)blockIdx.y * npix + q_pix[q]];
+    const size_t im = index ? index[blockIdx.y] : blockIdx.y;
+    if (q < nq) lam[(size_t)blockIdx.y * nq + q] = images[im * npix + q_pix[q]];
 }
 
 __global__ void k_scatter_batch(const float* lam, const int* q_pix, int nq, float* images,
-                                int npix) {
+                                const int* index, int npix) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q < nq) images[(size_t)blockIdx.y * npix + q_pix[q]] = lam[(size_t)blockIdx.y * nq + q];
+    const size_t im = index ? index[blockIdx.y] : blockIdx.y;
+    if (q < nq) images[im * npix + q_pix[q]] = lam[(size_t)blockIdx.y * nq + q];
 }
 
 }  // namespace
@@ -484,25 +487,27 @@ int launch_bp_batch(lm_handle* h, const float* rows, int row_stride, const float
 int launch_reduce_update_batch(lm_handle* h, int R, const float* bpart, const int* part_start,
                                double* num, float* lam_v, const double* sens,
                                const double* llpart, double* loglik, int ll_stride,
-                               cudaStream_t st) {
+                               const int* index, cudaStream_t st) {
     dim3 g((h->mc.nq + 255) / 256, R);
     k_voxel_reduce_batch<<<g, 256, 0, st>>>(bpart, part_start, h->mc.nq, num);
     k_update_batch<<<R, 1024, 0, st>>>(lam_v, num, sens, h->mc.nq, llpart, part_start, loglik,
-                                       ll_stride);
+                                       ll_stride, index);
     h->launches += 2;
     LMMEW_CUDA(cudaGetLastError());
     return LMMEW_OK;
 }
 
-int launch_images_batch(lm_handle* h, int R, float* images, float* lam_v, bool to_voxels,
-                        cudaStream_t st) {
+int launch_images_batch(lm_handle* h, int R, float* images, const int* h_index, const int* d_index,
+                        float* lam_v, bool to_voxels, cudaStream_t st) {
     const int npix = h->mc.n * h->mc.n;
     dim3 g((h->mc.nq + 255) / 256, R);
     if (to_voxels) {
-        k_gather_batch<<<g, 256, 0, st>>>(images, npix, h->d_q_pix, h->mc.nq, lam_v);
+        k_gather_batch<<<g, 256, 0, st>>>(images, d_index, npix, h->d_q_pix, h->mc.nq, lam_v);
     } else {
-        LMMEW_CUDA(cudaMemsetAsync(images, 0, sizeof(float) * (size_t)R * npix, st));
-        k_scatter_batch<<<g, 256, 0, st>>>(lam_v, h->d_q_pix, h->mc.nq, images, npix);
+        if (!h_index) LMMEW_CUDA(cudaMemsetAsync(images, 0, sizeof(float) * (size_t)R * npix, st));
+        for (int r = 0; h_index && r < R; ++r)
+            LMMEW_CUDA(cudaMemsetAsync(images + (size_t)h_index[r] * npix, 0, sizeof(float) * npix, st));
+        k_scatter_batch<<<g, 256, 0, st>>>(lam_v, h->d_q_pix, h->mc.nq, images, d_index, npix);
     }
     ++h->launches;
     LMMEW_CUDA(cudaGetLastError());

@@ -17,13 +17,39 @@
 
 namespace lmmew {
 
-// Reach of each line's single scatter in recorded energy, and the classes
-// its ends cut the energy axis into (see EnergyClasses).  E' runs from the
-// backscatter energy to E_w; E' -+ k sigma_E(E') is scanned in FP64 on a fine
-// grid, widened by the largest change between neighbouring samples (the
-// extremum between two samples lies within that of the nearer one), and
-// rounded outward to FP32, the precision the recorded energies are compared
-// in.  Classes are off (one class, every line) without scatter points, with
+// Reach of line w's single scatter in recorded energy (see EnergyClasses).
+// E' runs from the backscatter energy to E_w; E' -+ k sigma_E(E') is scanned
+// in FP64 on a fine grid, widened by the largest change between neighbouring
+// samples (the extremum between two samples lies within that of the nearer
+// one), and rounded outward to FP32, the precision the recorded energies are
+// compared in.
+void line_reach(const lm_handle* h, int w, float* lo, float* hi) {
+    const ModelConst& m = h->mc;
+    const double f2s = 1.0 / (2.0 * sqrt(2.0 * log(2.0)));
+    auto sigma = [&](double e) { return m.fwhm_frac * e * pow(e / m.e_ref, m.expo) * f2s; };
+    const double ew = m.line_e[w];
+    const double eb = ew / (1.0 + 2.0 * ew / 510.99895);
+    constexpr int kSteps = 4096;
+    double mn = 1e300, mx = -1e300, dl = 0.0, du = 0.0, pl = 0.0, pu = 0.0;
+    for (int k = 0; k <= kSteps; ++k) {
+        const double e = eb + (ew - eb) * k / kSteps;
+        const double s = kScatterReachSigmas * sigma(e);
+        const double l = e - s, u = e + s;
+        if (k > 0) {
+            dl = std::max(dl, fabs(l - pl));
+            du = std::max(du, fabs(u - pu));
+        }
+        pl = l;
+        pu = u;
+        mn = std::min(mn, l);
+        mx = std::max(mx, u);
+    }
+    *lo = nextafterf((float)(mn - dl), -INFINITY);
+    *hi = nextafterf((float)(mx + du), INFINITY);
+}
+
+// The classes the ends of the lines' reaches cut the energy axis into.
+// Classes are off (one class, every line) without scatter points, with
 // more than 4 lines, when pruning is switched off, or when (angle rank,
 // class, bin) keys would not fit 32 bits.
 void build_energy_classes(lm_handle* h) {
@@ -34,30 +60,10 @@ void build_energy_classes(lm_handle* h) {
     for (int c = 0; c < 2 * LMMEW_MAX_LINES + 1; ++c) h->class_lines[c] = all;
     // the row kernels instantiate a stage per staged-line count up to 4 lines
     if (!h->prune_lines || m.np == 0 || m.W > 4) return;
-    const double f2s = 1.0 / (2.0 * sqrt(2.0 * log(2.0)));
-    auto sigma = [&](double e) { return m.fwhm_frac * e * pow(e / m.e_ref, m.expo) * f2s; };
     float lo[LMMEW_MAX_LINES], hi[LMMEW_MAX_LINES];
     std::vector<float> bnd;
     for (int w = 0; w < m.W; ++w) {
-        const double ew = m.line_e[w];
-        const double eb = ew / (1.0 + 2.0 * ew / 510.99895);
-        constexpr int kSteps = 4096;
-        double mn = 1e300, mx = -1e300, dl = 0.0, du = 0.0, pl = 0.0, pu = 0.0;
-        for (int k = 0; k <= kSteps; ++k) {
-            const double e = eb + (ew - eb) * k / kSteps;
-            const double s = kScatterReachSigmas * sigma(e);
-            const double l = e - s, u = e + s;
-            if (k > 0) {
-                dl = std::max(dl, fabs(l - pl));
-                du = std::max(du, fabs(u - pu));
-            }
-            pl = l;
-            pu = u;
-            mn = std::min(mn, l);
-            mx = std::max(mx, u);
-        }
-        lo[w] = nextafterf((float)(mn - dl), -INFINITY);
-        hi[w] = nextafterf((float)(mx + du), INFINITY);
+        line_reach(h, w, &lo[w], &hi[w]);
         bnd.push_back(lo[w]);
         bnd.push_back(hi[w]);
     }
@@ -316,6 +322,24 @@ Windows windows_of(const ModelConst& m) {
                    make_float4(w[6][0], w[6][1], w[7][0], w[7][1])};
 }
 
+// Stable LSD radix sort of (keys, vals) over the ping-pong buffers; the
+// sorted pair ends in (kin, vin).
+int radix_sort_pairs(lm_handle* h, int64_t n, int bits, uint32_t*& kin, uint32_t*& kout,
+                     uint32_t*& vin, uint32_t*& vout, uint32_t* hist, cudaStream_t st) {
+    const int64_t nblk = (n + kSortChunk - 1) / kSortChunk;
+    for (int shift = 0; shift < bits; shift += 8) {
+        k_hist<<<(unsigned)nblk, kSortThreads, 0, st>>>(kin, n, shift, hist, (int)nblk);
+        k_scan<<<1, 1024, 0, st>>>(hist, 256 * nblk);
+        k_scatter<<<(unsigned)nblk, kSortThreads, 0, st>>>(kin, vin, n, shift, hist, (int)nblk, kout,
+                                                          vout);
+        LMMEW_CUDA(cudaGetLastError());
+        std::swap(kin, kout);
+        std::swap(vin, vout);
+    }
+    h->launches += 3 * ((bits + 7) / 8);
+    return LMMEW_OK;
+}
+
 // The sort shared by sort_events and sort_events_async: keys, radix passes,
 // gather, group bounds and tiles of the G = A * n_classes groups, all on
 // the caller's stream.  rank_of_angle [A], angle_of_group and lines_of_group
@@ -336,18 +360,9 @@ int sort_and_tile(lm_handle* h, const lm_events* ev, int G, const int* rank_of_a
         ++h->launches;
         LMMEW_CUDA(cudaGetLastError());
         const int bits = key_bits((uint64_t)G * (uint64_t)B);
-        const int64_t nblk = (n + kSortChunk - 1) / kSortChunk;
         uint32_t *kin = keys0, *kout = keys1, *vin = vals0, *vout = vals1;
-        for (int shift = 0; shift < bits; shift += 8) {
-            k_hist<<<(unsigned)nblk, kSortThreads, 0, st>>>(kin, n, shift, hist, (int)nblk);
-            k_scan<<<1, 1024, 0, st>>>(hist, 256 * nblk);
-            k_scatter<<<(unsigned)nblk, kSortThreads, 0, st>>>(kin, vin, n, shift, hist, (int)nblk,
-                                                              kout, vout);
-            h->launches += 3;
-            LMMEW_CUDA(cudaGetLastError());
-            std::swap(kin, kout);
-            std::swap(vin, vout);
-        }
+        const int rc = radix_sort_pairs(h, n, bits, kin, kout, vin, vout, hist, st);
+        if (rc != LMMEW_OK) return rc;
         k_gather<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(kin, vin, ev->energy_keV, n, B, perm,
                                                              bin_s, e_s);
         k_bounds<<<(G + 1 + 127) / 128, 128, 0, st>>>(kin, n, G, B, group_start);
@@ -521,6 +536,76 @@ int sort_events_async(lm_handle* h, const lm_events* ev, const GroupArrays& ga, 
     return sort_and_tile(h, ev, G, ga.rank_of_angle, ga.angle_of_group, ga.lines_of_group, keys0,
                          keys1, vals0, vals1, hist, out->perm, out->bin, out->energy,
                          out->group_start, out->tile_start, out->tile_ev, out->tiles, st);
+}
+
+namespace {
+__global__ void k_validate(const uint16_t* angle, const uint16_t* bin, const float* energy, int64_t n,
+                           int A, int B, int n_win, const NodeWindows win, int* status) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    const float e = energy[j];
+    bool in = false;
+    for (int k = 0; k < n_win; ++k) in |= e >= win.lo[k] && e < win.hi[k];
+    if (!(angle[j] < A && bin[j] < B && isfinite(e) && in)) atomicOr(status, kStatusOutOfRange);
+}
+}  // namespace
+
+int launch_validate(lm_handle* h, const lm_events* ev, cudaStream_t st) {
+    if (ev->n == 0) return LMMEW_OK;
+    const ModelConst& m = h->mc;
+    NodeWindows win{};
+    for (int k = 0; k < m.n_win; ++k) {
+        win.lo[k] = (float)m.win_lo[k];
+        win.hi[k] = (float)m.win_hi[k];
+    }
+    k_validate<<<(unsigned)((ev->n + 255) / 256), 256, 0, st>>>(ev->angle, ev->bin, ev->energy_keV,
+                                                                ev->n, m.A, m.B, m.n_win, win,
+                                                                h->d_status);
+    ++h->launches;
+    LMMEW_CUDA(cudaGetLastError());
+    return LMMEW_OK;
+}
+
+size_t cell_scratch_bytes(const lm_handle* h, int64_t n) {
+    const int64_t nblk = (n + kSortChunk - 1) / kSortChunk;
+    return 6 * bump_bytes(4 * (size_t)n) + bump_bytes(2 * (size_t)n) +
+           bump_bytes(4 * 256 * (size_t)std::max<int64_t>(nblk, 1)) +
+           bump_bytes(4 * ((size_t)h->mc.A * h->mc.B + 1));
+}
+
+int sort_cells(lm_handle* h, const lm_events* ev, const int* rank_of_angle, CellEvents* out,
+               char*& arena, cudaStream_t st) {
+    const ModelConst& m = h->mc;
+    const int64_t n = ev->n;
+    const int cells = m.A * m.B;
+    uint32_t* kin = bump<uint32_t>(arena, n);
+    uint32_t* kout = bump<uint32_t>(arena, n);
+    uint32_t* vin = bump<uint32_t>(arena, n);
+    uint32_t* vout = bump<uint32_t>(arena, n);
+    const int64_t nblk = (n + kSortChunk - 1) / kSortChunk;
+    uint32_t* hist = bump<uint32_t>(arena, 256 * std::max<int64_t>(nblk, 1));
+    out->perm = bump<uint32_t>(arena, n);
+    uint16_t* bins = bump<uint16_t>(arena, n);
+    out->energy = bump<float>(arena, n);
+    out->cell_start = bump<int>(arena, (size_t)cells + 1);
+    if (n == 0) {
+        LMMEW_CUDA(cudaMemsetAsync(out->cell_start, 0, sizeof(int) * ((size_t)cells + 1), st));
+        return LMMEW_OK;
+    }
+    const Windows wn = windows_of(m);
+    k_keys<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
+        ev->angle, ev->bin, ev->energy_keV, n, m.A, m.B, rank_of_angle, m.n_win, wn.w01, wn.w23,
+        wn.w45, wn.w67, EnergyClasses{}, kin, vin, h->d_status);
+    ++h->launches;
+    LMMEW_CUDA(cudaGetLastError());
+    const int rc = radix_sort_pairs(h, n, key_bits((uint64_t)cells), kin, kout, vin, vout, hist, st);
+    if (rc != LMMEW_OK) return rc;
+    k_gather<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(kin, vin, ev->energy_keV, n, m.B, out->perm,
+                                                         bins, out->energy);
+    k_bounds<<<(cells + 1 + 127) / 128, 128, 0, st>>>(kin, n, cells, 1, out->cell_start);
+    h->launches += 2;
+    LMMEW_CUDA(cudaGetLastError());
+    return LMMEW_OK;
 }
 
 int read_back_counts(lm_handle* h, SortedEvents* se, cudaStream_t st) {
@@ -713,23 +798,6 @@ __global__ void k_bp_keys(const uint16_t* real, int64_t n, const int64_t* blk_st
     vals[i] = (uint32_t)i;
 }
 
-// Stable LSD radix sort of (keys, vals) over the ping-pong buffers; the
-// sorted pair ends in (kin, vin).
-int radix_sort_pairs(lm_handle* h, int64_t n, int bits, uint32_t*& kin, uint32_t*& kout,
-                     uint32_t*& vin, uint32_t*& vout, uint32_t* hist, cudaStream_t st) {
-    const int64_t nblk = (n + kSortChunk - 1) / kSortChunk;
-    for (int shift = 0; shift < bits; shift += 8) {
-        k_hist<<<(unsigned)nblk, kSortThreads, 0, st>>>(kin, n, shift, hist, (int)nblk);
-        k_scan<<<1, 1024, 0, st>>>(hist, 256 * nblk);
-        k_scatter<<<(unsigned)nblk, kSortThreads, 0, st>>>(kin, vin, n, shift, hist, (int)nblk, kout,
-                                                          vout);
-        LMMEW_CUDA(cudaGetLastError());
-        std::swap(kin, kout);
-        std::swap(vin, vout);
-    }
-    h->launches += 3 * ((bits + 7) / 8);
-    return LMMEW_OK;
-}
 }  // namespace
 
 size_t sort_batch_scratch_bytes(int64_t n, int64_t G, int R) {

@@ -90,6 +90,25 @@ struct EnergyClasses {
     float bnd[2 * LMMEW_MAX_LINES];     // ascending; class = #{k : bnd[k] <= E_hat}
 };
 
+// Energy nodes of the dense-list projections (nodes.cu): t(E) = 2 sqrt(E) /
+// kappa, recorded-energy nodes k_first + k (8 per unit of t) and, per line,
+// scattered-energy nodes l_first + i (16 per unit), the lines one after the
+// other.
+struct NodeConst {
+    int W;
+    int nk, nk_pad, k_first;
+    int nl, nl_pad;
+    int l_first[4], l_count[4], l_off[4];
+    float cl, cl_lo;           // node of a scattered energy = (cl + cl_lo) / sr
+    float ck, ck_lo;           // node of a recorded energy = (ck + ck_lo) sqrt(E)
+    float reach_lo[4], reach_hi[4];   // recorded energies single scatter of the line can have
+    int nb_max;                // most bins one chunk of 32 scatter points reaches
+    int spread_warps, spread_smem, gather_smem;
+};
+struct NodeWindows {
+    float lo[LMMEW_MAX_WINDOWS], hi[LMMEW_MAX_WINDOWS];
+};
+
 struct Scratch {
     void* ptr = nullptr;
     size_t bytes = 0;
@@ -142,6 +161,12 @@ struct lm_handle {
     double* d_on_det = nullptr;    // [A][np] collimator mass of each point on the detector
     int* d_inv = nullptr;          // [A][np] point of each slot of an angle's point order
     double* d_mu_line = nullptr;   // [W] mu_water at each line energy
+    // energy nodes (dense event lists)
+    lmmew::NodeConst nodes{};
+    int node_route = 0;            // 1: the model has the node route
+    float* d_node_g = nullptr;     // Gaussian matrix [nl][nk_pad] and its transpose [nk_pad][nl_pad]
+    int2* d_chunk_bins = nullptr;  // [A][npc] bins each chunk of 32 scatter points reaches
+    int2* d_node_band = nullptr;   // its bands: [nl] nodes k of l, [W][nk_pad] nodes l of k
     lmmew::ChunkRange* d_clip = nullptr;   // a row launch's tiles clipped to one angle block
     // cached subset sensitivities for the last partition asked for
     int sens_parts = 0;
@@ -196,6 +221,7 @@ struct lm_handle {
     int64_t prof_launches = 0;
     double prof_terms_dense = 0.0;   // terms of the rows without the exact-zero skip
     double prof_elems = 0.0;
+    double prof_node_terms = 0.0;    // path weights the node route evaluated
     int64_t launches = 0;          // kernels this library launched (all kinds)
     unsigned long long* d_term_counter = nullptr;   // exponentials evaluated while timing
     int* d_work = nullptr;         // row kernel's next-unit counter, zeroed before each launch
@@ -222,8 +248,29 @@ int set_table_streaming(lm_handle* h, int max_angles);
 // setup.cu: tables larger than this are streamed by lm_create (0: no limit
 // beyond the device's free memory)
 extern int64_t g_table_budget;
-// events.cu: the energy classes of the handle's lines and energy model
+// events.cu: the energy classes of the handle's lines and energy model, and
+// the recorded energies single scatter of line w can reach (rounded outward)
 void build_energy_classes(lm_handle* h);
+void line_reach(const lm_handle* h, int w, float* lo, float* hi);
+// nodes.cu: projections of dense event lists through energy nodes
+int build_nodes(lm_handle* h);
+size_t node_angle_bytes(const lm_handle* h);   // scratch of one angle's forward sums
+int node_forward(lm_handle* h, const float* lam_v, int a0, int a_step, int angles, float* dbp,
+                 float* F, float* Pr, cudaStream_t st);
+int node_cells(lm_handle* h, int angles, const int* cell_start, int cell0, const float* energy,
+               const float* F, const float* Pr, const float* weight, const uint32_t* perm, float* V,
+               float* PV, double* ll, cudaStream_t st);
+int node_back(lm_handle* h, int a0, int a_step, int angles, const float* V, const float* PV,
+              float* VG, float* part, float* part_prim, cudaStream_t st);
+int node_update(lm_handle* h, int angles, const float* part, const float* part_prim,
+                const double* sens, float* lam, double* num, cudaStream_t st);
+int node_loglik(lm_handle* h, const double* ll, int n_ll, const float* lam, const double* sens,
+                double* out, cudaStream_t st);
+// api.cu: row-kernel timing around a launch of the node route (no-ops while off)
+int prof_start(lm_handle* h, cudaStream_t st);
+int prof_stop(lm_handle* h, double terms, cudaStream_t st);
+int node_events_forward(lm_handle* h, const lm_events* ev, const float* F, const float* Pr, int a0,
+                        int angles, float* out_y, cudaStream_t st);
 int subset_sensitivity(lm_handle* h, int n_subsets, cudaStream_t st);
 
 // events.cu: validation + stable sort by (subset rank of angle, energy class,
@@ -271,6 +318,18 @@ struct GroupArrays {
 int group_arrays(lm_handle* h, int n_subsets, GroupArrays* out);   // cached per partition
 int sort_events_async(lm_handle* h, const lm_events* ev, const GroupArrays& ga, int G,
                       SortedEvents* out, char*& arena, cudaStream_t st);
+// events.cu: validation + stable sort by (subset rank of angle, bin) alone;
+// cell_start [A B + 1]: first sorted event of each (rank, bin) cell
+struct CellEvents {
+    float* energy;       // [n]
+    uint32_t* perm;      // [n]
+    int* cell_start;
+};
+// Events outside the model set the status word (nothing else is written).
+int launch_validate(lm_handle* h, const lm_events* ev, cudaStream_t st);
+size_t cell_scratch_bytes(const lm_handle* h, int64_t n);
+int sort_cells(lm_handle* h, const lm_events* ev, const int* rank_of_angle, CellEvents* out,
+               char*& arena, cudaStream_t st);
 // Group arrays of one subset (angles in natural order) built on the device
 // into a caller-provided region (no allocation, no copy from the host).
 GroupArrays group_arrays_into(lm_handle* h, char*& arena, cudaStream_t st);
@@ -293,6 +352,15 @@ ForwardPlan forward_plan(const lm_handle* h, int64_t n, int64_t cap_max);
 size_t forward_region_bytes(const lm_handle* h, const ForwardPlan& p);
 int forward_async(lm_handle* h, const lm_events* ev, const float* image, float* out_y,
                   const GroupArrays& ga, const ForwardPlan& p, char* arena, cudaStream_t st);
+// api.cu: the same through the energy nodes, `block` angles at a time, in
+// forward_nodes_bytes(h, block) of scratch; forward_nodes_block: the angles
+// that fit `bytes`; node_use: whether an n-event projection takes that route
+int forward_nodes(lm_handle* h, const lm_events* ev, const float* image, float* out_y, int block,
+                  char* arena, cudaStream_t st);
+int forward_nodes_block(const lm_handle* h, size_t bytes);
+size_t forward_nodes_bytes(const lm_handle* h, int block);
+bool node_use(const lm_handle* h, int64_t n);
+bool node_use_osem(const lm_handle* h, int64_t n);   // the same for a whole reconstruction
 // Row blocks of n_sets consecutive rank ranges (the subsets of a partition
 // into n_subsets, or all ranks for n_subsets = 1): set s, block k covers
 // tiles [T0 + k tpc, T0 + (k + 1) tpc) of the set's tiles [T0, T1).
@@ -386,9 +454,9 @@ int launch_bp_batch(lm_handle* h, const float* rows, int row_stride, const float
 int launch_reduce_update_batch(lm_handle* h, int R, const float* bpart, const int* part_start,
                                double* num, float* lam_v, const double* sens,
                                const double* llpart, double* loglik, int ll_stride,
-                               cudaStream_t st);
-int launch_images_batch(lm_handle* h, int R, float* images, float* lam_v, bool to_voxels,
-                        cudaStream_t st);
+                               const int* index, cudaStream_t st);
+int launch_images_batch(lm_handle* h, int R, float* images, const int* h_index, const int* d_index,
+                        float* lam_v, bool to_voxels, cudaStream_t st);
 int launch_gather_image(lm_handle* h, const float* image, float* lam_v, cudaStream_t st);
 int launch_scatter_image(lm_handle* h, const float* lam_v, float* image, cudaStream_t st);
 int launch_scatter_image_d(lm_handle* h, const double* v, double* image, cudaStream_t st);

@@ -80,6 +80,8 @@ extern "C" int lm_forward_noalloc(lm_handle* h, const lm_events* ev, const float
     if (rc != LMMEW_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     char* arena = (char*)base;
+    if (node_use(h, n))
+        return forward_nodes(h, ev, image, out_y, forward_nodes_block(h, kNoAllocBytes), arena, st);
     const GroupArrays ga = group_arrays_into(h, arena, st);
     LMMEW_CUDA(cudaGetLastError());
     return forward_async(h, ev, image, out_y, ga, fp, arena, st);
