@@ -255,14 +255,24 @@ __global__ void __launch_bounds__(32 * kSpreadWarpsMax) k_node_spread(const Node
             }
             break;
         }
+        // the whole stage into registers first: the sums' stores below could
+        // alias it as far as the compiler knows, which would keep every load
+        // and all arithmetic of a path behind the stores of the one before
         const float* st = stage0 + (it & 1) * (2 * kStageRows * kPC) + lane;
-#pragma unroll 2
+        float nl[kStageRows], sr[kStageRows];
+#pragma unroll
+        for (int r = 0; r < kStageRows; ++r) {
+            nl[r] = st[r * kPC];
+            sr[r] = st[(kStageRows + r) * kPC];
+        }
+        __syncwarp();
+        if (lane == 0 && it + 2 < nt) issue(it + 2);
+#pragma unroll
         for (int r = 0; r < kStageRows; r += 2) {
             const f32x2 lam = pk(__shfl_sync(0xffffffffu, lam_l, r), __shfl_sync(0xffffffffu, lam_l, r + 1));
-            const f32x2 wt = mul2(pk(ex2f(-st[r * kPC]), ex2f(-st[(r + 1) * kPC])), lam);
+            const f32x2 wt = mul2(pk(ex2f(-nl[r]), ex2f(-nl[r + 1])), lam);
             unsigned i0, i1;
-            const f32x2 s = node_pos2(st[(kStageRows + r) * kPC], st[(kStageRows + r + 1) * kPC], c1,
-                                      c1_lo, first, last, i0, i1);
+            const f32x2 s = node_pos2(sr[r], sr[r + 1], c1, c1_lo, first, last, i0, i1);
             f32x2 c[7];
             lagrange7(s, wt, c);
             float x[7], y[7];
@@ -280,8 +290,6 @@ __global__ void __launch_bounds__(32 * kSpreadWarpsMax) k_node_spread(const Node
 #pragma unroll
             for (int k = 0; k < 7; ++k) d[k * kPC] = v[k] + y[k];
         }
-        __syncwarp();
-        if (lane == 0 && it + 2 < nt) issue(it + 2);
     }
     __syncthreads();
     const int T = blockDim.x;
