@@ -14,6 +14,7 @@ namespace lmmew {
 namespace {
 thread_local std::string g_err;
 constexpr size_t kRowBudgetFloats = size_t(1) << 30;   // 4 GiB of row block per chunk
+constexpr size_t kKeepRowBytes = size_t(16) << 30;     // rows kept over a call's iterations, at most
 constexpr size_t kNodeBudgetBytes = size_t(1) << 30;   // node sums of the angles in flight
 }  // namespace
 
@@ -235,6 +236,17 @@ int check_events(const lm_handle* h, const lm_events* ev) {
 }
 
 int row_stride_of(const lm_handle* h) { return (h->mc.nq + 3) & ~3; }
+
+// The rows do not depend on the image, so a call of several iterations forms
+// them once and keeps them when those of all n events fit kKeepRowBytes and
+// half of the free memory (what the handle's scratch holds counts as free).
+bool keep_rows_fit(const lm_handle* h, int64_t n, int iterations) {
+    if (iterations < 2) return false;
+    const size_t bytes = sizeof(float) * (size_t)n * row_stride_of(h);
+    size_t free_b = 0, total_b = 0;
+    if (bytes > kKeepRowBytes || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
+    return bytes <= (free_b + h->scratch_work.bytes) / 2;
+}
 
 }  // namespace
 
@@ -729,18 +741,26 @@ static int osem_planned(lm_handle* h, const lm_events* ev, int n_subsets, int n_
             r += cnt;
         }
     }
-    const size_t need = bump_bytes(sizeof(float) * m.nq) + bump_bytes(sizeof(float) * rs * biggest) +
-                        bump_bytes(sizeof(float) * m.nqt * biggest) +
-                        bump_bytes(sizeof(float) * std::max<int64_t>(parts_max, 1) * m.nq) +
-                        bump_bytes(sizeof(double) * std::max<int64_t>(parts_max, 1)) +
-                        bump_bytes(sizeof(double) * m.nq);
+    bool keep = keep_rows_fit(h, se.n_valid, n_iters - start_iter);
+    auto need = [&](bool all) {
+        return bump_bytes(sizeof(float) * m.nq) +
+               bump_bytes(sizeof(float) * rs * std::max<int64_t>(all ? se.n_valid : biggest, 1)) +
+               bump_bytes(sizeof(float) * m.nqt * std::max<int64_t>(biggest, 1)) +
+               bump_bytes(sizeof(float) * std::max<int64_t>(parts_max, 1) * m.nq) +
+               bump_bytes(sizeof(double) * std::max<int64_t>(parts_max, 1)) +
+               bump_bytes(sizeof(double) * m.nq);
+    };
     rc = surrogate_prepare(h, biggest, st);
     if (rc != LMMEW_OK) return rc;
-    rc = ensure(h, h->scratch_work, need, st);
+    rc = ensure(h, h->scratch_work, need(keep), st);
+    if (rc == LMMEW_ERR_OOM && keep) {
+        keep = false;
+        rc = ensure(h, h->scratch_work, need(false), st);
+    }
     if (rc != LMMEW_OK) return rc;
     char* w = (char*)h->scratch_work.ptr;
     float* lam_v = bump<float>(w, m.nq);
-    float* rows = bump<float>(w, (size_t)rs * std::max<int64_t>(biggest, 1));
+    float* rows = bump<float>(w, (size_t)rs * std::max<int64_t>(keep ? se.n_valid : biggest, 1));
     float* ypart = bump<float>(w, (size_t)m.nqt * std::max<int64_t>(biggest, 1));
     float* bpart = bump<float>(w, (size_t)std::max<int64_t>(parts_max, 1) * m.nq);
     double* llpart = bump<double>(w, std::max<int64_t>(parts_max, 1));
@@ -748,21 +768,29 @@ static int osem_planned(lm_handle* h, const lm_events* ev, int n_subsets, int n_
 
     rc = launch_gather_image(h, image, lam_v, st);
     if (rc != LMMEW_OK) return rc;
+    std::vector<char> have(n_subsets, 0);   // subsets whose rows are kept
     for (int it = start_iter; it < n_iters; ++it) {
         for (int s = (it == start_iter ? start_subset : 0); s < n_subsets; ++s) {
             int64_t row0 = 0;
             for (const Chunk& c : plan[s]) {
                 const int64_t cnt = c.e1 - c.e0;
-                RowLaunch L{se.tiles, c.t0, c.t1, se.bin, se.energy, lam_v, rows, c.e0, rs, ypart,
-                            cnt, cnt};
-                L.tile_ev = se.tile_ev;
-                rc = launch_row_profiled(h, L, st);
+                float* rows_c = rows + (keep ? (size_t)c.e0 * rs : 0);
+                if (have[s]) {
+                    rc = launch_kept_forward(h, rows_c, rs, c.e0, c.e0, cnt, nullptr, lam_v, 0, nullptr,
+                                             ypart, cnt, st);
+                } else {
+                    RowLaunch L{se.tiles, c.t0, c.t1, se.bin, se.energy, lam_v, rows_c, c.e0, rs, ypart,
+                                cnt, cnt};
+                    L.tile_ev = se.tile_ev;
+                    rc = launch_row_profiled(h, L, st);
+                }
                 if (rc != LMMEW_OK) return rc;
-                rc = launch_bp_partial(h, rows, rs, ypart, cnt, cnt, nullptr, nullptr, bpart, row0,
+                rc = launch_bp_partial(h, rows_c, rs, ypart, cnt, cnt, nullptr, nullptr, bpart, row0,
                                        loglik ? llpart : nullptr, st);
                 if (rc != LMMEW_OK) return rc;
                 row0 += bp_parts(cnt);
             }
+            have[s] = keep ? 1 : 0;
             if (row0 > 0) {
                 rc = launch_voxel_reduce(h, bpart, row0, num, st);
             } else {
@@ -1028,18 +1056,26 @@ int lm_osem(lm_handle* h, const lm_events* ev, int n_subsets, int n_iters, int s
     const int64_t cap = (int64_t)tpc * te;
     const int blocks = (int)((tiles_max + tpc - 1) / tpc);
     const int64_t ppc = bp_parts(cap);
-    rc = ensure(h, h->scratch_work,
-                bump_bytes(sizeof(float) * m.nq) + bump_bytes(sizeof(float) * (size_t)rs * cap) +
-                    bump_bytes(sizeof(float) * (size_t)m.nqt * cap) +
-                    bump_bytes(sizeof(float) * (size_t)blocks * ppc * m.nq) +
-                    bump_bytes(sizeof(double) * (size_t)blocks * ppc) +
-                    bump_bytes(sizeof(double) * m.nq) +
-                    bump_bytes(sizeof(ChunkRange) * (size_t)n_subsets * blocks),
-                st);
+    // rows of one row block, or of every event (kept after a subset's first
+    // sub-iteration)
+    bool keep = keep_rows_fit(h, n, n_iters - start_iter);
+    auto need = [&](bool all) {
+        return bump_bytes(sizeof(float) * m.nq) +
+               bump_bytes(sizeof(float) * (size_t)rs * (all ? (size_t)n : (size_t)cap)) +
+               bump_bytes(sizeof(float) * (size_t)m.nqt * cap) +
+               bump_bytes(sizeof(float) * (size_t)blocks * ppc * m.nq) +
+               bump_bytes(sizeof(double) * (size_t)blocks * ppc) + bump_bytes(sizeof(double) * m.nq) +
+               bump_bytes(sizeof(ChunkRange) * (size_t)n_subsets * blocks);
+    };
+    rc = ensure(h, h->scratch_work, need(keep), st);
+    if (rc == LMMEW_ERR_OOM && keep) {
+        keep = false;
+        rc = ensure(h, h->scratch_work, need(false), st);
+    }
     if (rc != LMMEW_OK) return rc;
     char* w = (char*)h->scratch_work.ptr;
     float* lam_v = bump<float>(w, m.nq);
-    float* rows = bump<float>(w, (size_t)rs * cap);
+    float* rows = bump<float>(w, (size_t)rs * (keep ? (size_t)n : (size_t)cap));
     float* ypart = bump<float>(w, (size_t)m.nqt * cap);
     float* bpart = bump<float>(w, (size_t)blocks * ppc * m.nq);
     double* llpart = bump<double>(w, (size_t)blocks * ppc);
@@ -1050,20 +1086,28 @@ int lm_osem(lm_handle* h, const lm_events* ev, int n_subsets, int n_iters, int s
     // the first rank of each subset (subsets ascending, angles ascending inside one)
     std::vector<int> r_first(n_subsets + 1, 0);
     for (int s = 0; s < n_subsets; ++s) r_first[s + 1] = r_first[s] + (m.A - s + n_subsets - 1) / n_subsets;
+    std::vector<char> have(n_subsets, 0);   // subsets whose rows are kept
     for (int it = start_iter; it < n_iters && rc == LMMEW_OK; ++it) {
         for (int s = (it == start_iter ? start_subset : 0); s < n_subsets && rc == LMMEW_OK; ++s) {
             const ChunkRange* rg = ranges + (size_t)s * blocks;
             for (int k = 0; k < blocks && rc == LMMEW_OK; ++k) {
-                RowLaunch L{se.tiles, 0, tpc, se.bin, se.energy, lam_v, rows, 0, rs, ypart, cap,
-                            (s == 0 && k == 0) ? n : 0};
-                L.tile_ev = te;
-                L.range = rg + k;
-                rc = launch_row_ranks(h, L, se, r_first[s], r_first[s + 1], s, n_subsets, st);
+                if (have[s]) {
+                    rc = launch_kept_forward(h, rows, rs, 0, 0, cap, rg + k, lam_v, 0, nullptr, ypart,
+                                             cap, st);
+                } else {
+                    RowLaunch L{se.tiles, 0, tpc, se.bin, se.energy, lam_v, rows, 0, rs, ypart, cap,
+                                (s == 0 && k == 0) ? n : 0};
+                    L.tile_ev = te;
+                    L.range = rg + k;
+                    L.rows_abs = keep ? 1 : 0;
+                    rc = launch_row_ranks(h, L, se, r_first[s], r_first[s + 1], s, n_subsets, st);
+                }
                 if (rc == LMMEW_OK)
                     rc = launch_bp_partial_range(h, rows, rs, ypart, cap, cap, rg + k, nullptr,
                                                  nullptr, bpart, (int64_t)k * ppc,
-                                                 loglik ? llpart : nullptr, st);
+                                                 loglik ? llpart : nullptr, st, keep ? 1 : 0);
             }
+            have[s] = keep ? 1 : 0;
             if (rc == LMMEW_OK) rc = launch_voxel_reduce_ranges(h, bpart, rg, blocks, ppc, num, st);
             if (rc == LMMEW_OK)
                 rc = launch_update_ranges(h, lam_v, num, h->d_sens_sub + (size_t)s * m.nq, llpart,
@@ -1160,21 +1204,26 @@ static int osem_batch_rows(lm_handle* h, int n_real, const lm_events* events, co
         max_chunks += c;
         parts_max = std::max(parts_max, c);
     }
-    const size_t need = bump_bytes(sizeof(float) * (size_t)R * m.nq) +
-                        bump_bytes(sizeof(float) * (size_t)rs * biggest) +
-                        bump_bytes(sizeof(float) * (size_t)m.nqt * biggest) +
-                        bump_bytes(sizeof(float) * parts_max * m.nq) +
-                        bump_bytes(sizeof(double) * parts_max) +
-                        bump_bytes(sizeof(double) * (size_t)R * m.nq) +
-                        bump_bytes(sizeof(BpChunk) * max_chunks) +
-                        bump_bytes(sizeof(int) * (size_t)n_subsets * (R + 1)) +
-                        bump_bytes(sizeof(int64_t) * (size_t)(n_blk + 1)) +
-                        bump_bytes(sizeof(int) * (size_t)(G + 1)) + bump_bytes(sizeof(int) * (size_t)R);
-    rc = ensure(h, h->scratch_work, need, st);
+    bool keep = keep_rows_fit(h, se.n_total, n_iters);
+    auto need = [&](bool all) {
+        return bump_bytes(sizeof(float) * (size_t)R * m.nq) +
+               bump_bytes(sizeof(float) * (size_t)rs * (all ? std::max<int64_t>(se.n_total, 1) : biggest)) +
+               bump_bytes(sizeof(float) * (size_t)m.nqt * biggest) +
+               bump_bytes(sizeof(float) * parts_max * m.nq) + bump_bytes(sizeof(double) * parts_max) +
+               bump_bytes(sizeof(double) * (size_t)R * m.nq) + bump_bytes(sizeof(BpChunk) * max_chunks) +
+               bump_bytes(sizeof(int) * (size_t)n_subsets * (R + 1)) +
+               bump_bytes(sizeof(int64_t) * (size_t)(n_blk + 1)) +
+               bump_bytes(sizeof(int) * (size_t)(G + 1)) + bump_bytes(sizeof(int) * (size_t)R);
+    };
+    rc = ensure(h, h->scratch_work, need(keep), st);
+    if (rc == LMMEW_ERR_OOM && keep) {
+        keep = false;
+        rc = ensure(h, h->scratch_work, need(false), st);
+    }
     if (rc != LMMEW_OK) return rc;
     char* w = (char*)h->scratch_work.ptr;
     float* lam_v = bump<float>(w, (size_t)R * m.nq);
-    float* rows = bump<float>(w, (size_t)rs * biggest);
+    float* rows = bump<float>(w, (size_t)rs * (keep ? std::max<int64_t>(se.n_total, 1) : biggest));
     float* ypart = bump<float>(w, (size_t)m.nqt * biggest);
     float* bpart = bump<float>(w, parts_max * m.nq);
     double* llpart = bump<double>(w, parts_max);
@@ -1242,13 +1291,19 @@ static int osem_batch_rows(lm_handle* h, int n_real, const lm_events* events, co
         for (int s = 0; s < n_subsets && rc == LMMEW_OK; ++s) {
             for (int b = blk_off[s]; b < blk_off[s + 1]; ++b) {
                 const RowBlock& c = blocks[b];
-                RowLaunch L{se.tiles, c.t0, c.t1, se.bin, se.energy, lam_v, rows, c.e0, rs, ypart,
-                            c.e1 - c.e0, c.e1 - c.e0, m.nq};
-                L.tile_ev = se.tile_ev;
-                L.ev_real = se.real;
-                rc = launch_row(h, L, cs);
+                float* rows_c = rows + (keep ? (size_t)c.e0 * rs : 0);
+                if (keep && it > 0) {   // the rows of the first iteration
+                    rc = launch_kept_forward(h, rows_c, rs, c.e0, c.e0, c.e1 - c.e0, nullptr, lam_v, m.nq,
+                                             se.real, ypart, c.e1 - c.e0, cs);
+                } else {
+                    RowLaunch L{se.tiles, c.t0, c.t1, se.bin, se.energy, lam_v, rows_c, c.e0, rs, ypart,
+                                c.e1 - c.e0, c.e1 - c.e0, m.nq};
+                    L.tile_ev = se.tile_ev;
+                    L.ev_real = se.real;
+                    rc = launch_row(h, L, cs);
+                }
                 if (rc != LMMEW_OK) break;
-                rc = launch_bp_batch(h, rows, rs, ypart, c.e1 - c.e0, se.bp_idx, c.e0, d_bp + c.c0,
+                rc = launch_bp_batch(h, rows_c, rs, ypart, c.e1 - c.e0, se.bp_idx, c.e0, d_bp + c.c0,
                                      c.c1 - c.c0, bpart, loglik ? llpart : nullptr, cs);
                 if (rc != LMMEW_OK) break;
             }

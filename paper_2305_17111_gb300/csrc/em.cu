@@ -3,6 +3,8 @@
 // ownership (every voxel's sum is owned by one thread, no global atomics),
 // the FP64 log-likelihood of Eq. (lll_med) and the multiplicative update.
 // All sums run in a fixed order, so an OSEM run is bit-reproducible.
+#include <algorithm>
+
 #include "lmmew_internal.cuh"
 
 namespace lmmew {
@@ -88,6 +90,7 @@ __global__ void __launch_bounds__(kBpVoxels) k_bp_partial(
     const int n_here = rem < kBpEvents ? (int)rem : kBpEvents;
     const float* rp = rows + (size_t)j0 * row_stride + q;
     float acc = 0.f;
+#pragma unroll 16
     for (int e = 0; e < n_here; ++e) acc = fmaf(r[e], rp[(size_t)e * row_stride], acc);
     bpart[(size_t)(row0 + blockIdx.x) * nq + q] = acc;
 }
@@ -98,7 +101,7 @@ __global__ void __launch_bounds__(kBpVoxels) k_bp_partial(
 __global__ void __launch_bounds__(kBpVoxels) k_bp_partial_range(
     const float* rows, int row_stride, const float* ypart, int64_t ypart_stride, int nqt,
     const ChunkRange* range, const uint32_t* perm, const float* weight, int nq, float* bpart,
-    int64_t slot0, double* llpart) {
+    int64_t slot0, double* llpart, int rows_abs) {
     __shared__ float r[kBpEvents];
     __shared__ double ll[kBpEvents];
     const ChunkRange R = *range;
@@ -139,8 +142,9 @@ __global__ void __launch_bounds__(kBpVoxels) k_bp_partial_range(
     if (q >= nq) return;
     const int64_t rem = count - j0;
     const int n_here = rem < kBpEvents ? (int)rem : kBpEvents;
-    const float* rp = rows + (size_t)j0 * row_stride + q;
+    const float* rp = rows + (size_t)(j0 + (rows_abs ? R.z : 0)) * row_stride + q;
     float acc = 0.f;
+#pragma unroll 16
     for (int e = 0; e < n_here; ++e) acc = fmaf(r[e], rp[(size_t)e * row_stride], acc);
     bpart[(size_t)(slot0 + blockIdx.x) * nq + q] = acc;
 }
@@ -168,6 +172,47 @@ __global__ void k_forward_out_range(const float* ypart, int64_t stride, int nqt,
     float y = 0.f;
     for (int t = 0; t < nqt; ++t) y += ypart[(size_t)t * stride + j];
     out_y[perm[R.z + j]] = y;
+}
+
+// Partial forward sums of kept rows.  A warp takes 32 events x 32 voxels at a
+// time: rows read coalesced (a lane per voxel), transposed through shared
+// memory, then a lane per event adds its 32 products in voxel order, exactly
+// as the row kernel does when it forms the rows, so an iteration on kept rows
+// gives the bits a recomputed one would.  Bound by reading the rows (4 bytes
+// per element, from L2 while a subset's rows fit it).
+constexpr int kKeptWarps = 8;
+__global__ void __launch_bounds__(32 * kKeptWarps) k_kept_forward(
+    const float* rows, int row_stride, int64_t row0, int64_t begin, int64_t count,
+    const ChunkRange* range, int nq, int nqt, const float* lam, int lam_stride,
+    const uint16_t* ev_real, float* ypart, int64_t ypart_stride) {
+    __shared__ float tile[kKeptWarps][32][33];
+    if (range) {
+        begin = range->z;
+        count = (int64_t)range->w - range->z;
+    }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float(*tt)[33] = tile[warp];
+    const int64_t units = (count + 31) / 32 * nqt;
+    for (int64_t u = (int64_t)blockIdx.x * kKeptWarps + warp; u < units;
+         u += (int64_t)gridDim.x * kKeptWarps) {
+        const int64_t e0 = u / nqt * 32;
+        const int q0 = (int)(u % nqt) * 32;
+        const int ne = (int)min((int64_t)32, count - e0), nv = min(32, nq - q0);
+        const float* src = rows + (size_t)(begin + e0 - row0) * row_stride + q0 + lane;
+        __syncwarp();
+#pragma unroll 16
+        for (int e = 0; e < 32; ++e)
+            tt[e][lane] = e < ne && lane < nv ? src[(size_t)e * row_stride] : 0.f;
+        __syncwarp();
+        if (lane < ne) {
+            const float* l = lam + q0;
+            if (ev_real) l += (size_t)ev_real[begin + e0 + lane] * lam_stride;
+            float s = 0.f;
+#pragma unroll 8
+            for (int k = 0; k < nv; ++k) s = fmaf(l[k], tt[lane][k], s);
+            ypart[(size_t)(q0 >> 5) * ypart_stride + e0 + lane] = s;
+        }
+    }
 }
 
 // Events that failed validation sort after the valid ones: their outputs
@@ -305,12 +350,27 @@ int launch_invalid_out(lm_handle* h, const int* n_valid, int64_t n, const uint32
 int launch_bp_partial_range(lm_handle* h, const float* rows, int row_stride, const float* ypart,
                             int64_t ypart_stride, int64_t capacity, const ChunkRange* range,
                             const uint32_t* perm, const float* weight, float* bpart,
-                            int64_t slot0, double* llpart, cudaStream_t st) {
+                            int64_t slot0, double* llpart, cudaStream_t st, int rows_abs) {
     if (capacity <= 0) return LMMEW_OK;
     const int nq = h->mc.nq;
     dim3 g((unsigned)((capacity + kBpEvents - 1) / kBpEvents), (nq + kBpVoxels - 1) / kBpVoxels);
     k_bp_partial_range<<<g, kBpVoxels, 0, st>>>(rows, row_stride, ypart, ypart_stride, h->mc.nqt,
-                                                range, perm, weight, nq, bpart, slot0, llpart);
+                                                range, perm, weight, nq, bpart, slot0, llpart, rows_abs);
+    ++h->launches;
+    LMMEW_CUDA(cudaGetLastError());
+    return LMMEW_OK;
+}
+
+int launch_kept_forward(lm_handle* h, const float* rows, int row_stride, int64_t row0, int64_t begin,
+                        int64_t count, const ChunkRange* range, const float* lam, int lam_stride,
+                        const uint16_t* ev_real, float* ypart, int64_t ypart_stride,
+                        cudaStream_t st) {
+    if (count <= 0) return LMMEW_OK;
+    const int64_t units = (count + 31) / 32 * h->mc.nqt;
+    const int grid = (int)std::min<int64_t>((units + kKeptWarps - 1) / kKeptWarps, 6 * (int64_t)h->sm_count);
+    k_kept_forward<<<grid, 32 * kKeptWarps, 0, st>>>(rows, row_stride, row0, begin, count, range,
+                                                     h->mc.nq, h->mc.nqt, lam, lam_stride, ev_real,
+                                                     ypart, ypart_stride);
     ++h->launches;
     LMMEW_CUDA(cudaGetLastError());
     return LMMEW_OK;
@@ -414,6 +474,7 @@ __global__ void __launch_bounds__(kBpVoxels) k_bp_batch(
     const int q = blockIdx.y * kBpVoxels + t;
     if (q >= nq) return;
     float acc = 0.f;
+#pragma unroll 16
     for (int e = 0; e < C.count; ++e) acc = fmaf(r[e], rows[(size_t)idx[e] * row_stride + q], acc);
     bpart[(size_t)C.slot * nq + q] = acc;
 }

@@ -398,6 +398,7 @@ struct RowLaunch {
     const uint16_t* ev_real = nullptr;   // batched: realisation of each sorted event
     int skip_scatter = 0;   // unscattered terms only (the surrogate adds the rest)
     const ChunkRange* range = nullptr;   // if set: tiles and row_base read on the device
+    int rows_abs = 0;       // rows indexed by sorted event (kept rows) instead of from row_base
 };
 int launch_row(lm_handle* h, const RowLaunch& L, cudaStream_t st);
 int set_precision(lm_handle* h, int prec);
@@ -435,7 +436,15 @@ int launch_invalid_out(lm_handle* h, const int* n_valid, int64_t n, const uint32
 int launch_bp_partial_range(lm_handle* h, const float* rows, int row_stride, const float* ypart,
                             int64_t ypart_stride, int64_t capacity, const ChunkRange* range,
                             const uint32_t* perm, const float* weight, float* bpart,
-                            int64_t slot0, double* llpart, cudaStream_t st);
+                            int64_t slot0, double* llpart, cudaStream_t st, int rows_abs = 0);
+// Partial forward sums of rows computed before (the same sums, in the same
+// order, as the row kernel forms): `count` events from sorted event `begin`
+// (or, with range, the device's range), row of sorted event j at rows +
+// (j - row0) row_stride, lam per realisation with ev_real.
+int launch_kept_forward(lm_handle* h, const float* rows, int row_stride, int64_t row0, int64_t begin,
+                        int64_t count, const ChunkRange* range, const float* lam, int lam_stride,
+                        const uint16_t* ev_real, float* ypart, int64_t ypart_stride,
+                        cudaStream_t st);
 int launch_voxel_reduce_ranges(lm_handle* h, const float* bpart, const ChunkRange* ranges,
                                int n_blocks, int64_t ppc, double* num, cudaStream_t st);
 int launch_update_ranges(lm_handle* h, float* lam_v, const double* num, const double* sens,

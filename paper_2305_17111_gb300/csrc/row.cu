@@ -54,6 +54,7 @@ static RowParams make_params(lm_handle* h, const RowLaunch& L, int prec) {
     P.unit_order = h->unit_order;
     P.rows = L.rows;
     P.row_base = L.row_base;
+    P.rows_abs = L.rows_abs;
     P.row_stride = L.row_stride;
     P.ypart = L.ypart;
     P.ypart_stride = L.ypart_stride;

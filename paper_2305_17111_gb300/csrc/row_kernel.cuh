@@ -68,6 +68,7 @@ struct RowParams {
     int skip_scatter;     // 1: unscattered terms only
     float* rows;          // or null
     int64_t row_base;
+    int rows_abs;         // 1: rows indexed by sorted event, else from row_base
     int row_stride;
     float* ypart;         // [nqt][ypart_stride] or null
     int64_t ypart_stride;
@@ -538,11 +539,12 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_row(const RowParams P) {
             for (int qi = 0; qi < VPL; ++qi) tt[(k * kLanesEv + ev_lane) * 33 + v0 + qi] = acc[k][qi];
         __syncthreads();
         if (P.rows) {
+            const int64_t rows0 = P.rows_abs ? 0 : row_base;
             for (int i = tid; i < kLanesEv * EPL * kQT; i += kRowThreads) {
                 const int e = i >> 5, ql = i & 31;
                 const int q = qt * kQT + ql;
                 if (e < T.count && q < P.nq)
-                    P.rows[(size_t)(T.begin + e - row_base) * P.row_stride + q] = tt[e * 33 + ql];
+                    P.rows[(size_t)(T.begin + e - rows0) * P.row_stride + q] = tt[e * 33 + ql];
             }
         }
         if (lam && tid < T.count) {
