@@ -179,8 +179,11 @@ __global__ void k_forward_out_range(const float* ypart, int64_t stride, int nqt,
 // memory, then a lane per event adds its 32 products in voxel order, exactly
 // as the row kernel does when it forms the rows, so an iteration on kept rows
 // gives the bits a recomputed one would.  Bound by reading the rows (4 bytes
-// per element, from L2 while a subset's rows fit it).
+// per element, from L2 while a subset's rows fit it).  The coarse-grid
+// surrogate's sums (k_interp_rows) run over a butterfly of the voxels' lanes
+// instead: kButterfly.
 constexpr int kKeptWarps = 8;
+template <bool kButterfly>
 __global__ void __launch_bounds__(32 * kKeptWarps) k_kept_forward(
     const float* rows, int row_stride, int64_t row0, int64_t begin, int64_t count,
     const ChunkRange* range, int nq, int nqt, const float* lam, int lam_stride,
@@ -191,7 +194,7 @@ __global__ void __launch_bounds__(32 * kKeptWarps) k_kept_forward(
         count = (int64_t)range->w - range->z;
     }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float(*tt)[33] = tile[warp];
+    [[maybe_unused]] float(*tt)[33] = tile[warp];
     const int64_t units = (count + 31) / 32 * nqt;
     for (int64_t u = (int64_t)blockIdx.x * kKeptWarps + warp; u < units;
          u += (int64_t)gridDim.x * kKeptWarps) {
@@ -199,6 +202,23 @@ __global__ void __launch_bounds__(32 * kKeptWarps) k_kept_forward(
         const int q0 = (int)(u % nqt) * 32;
         const int ne = (int)min((int64_t)32, count - e0), nv = min(32, nq - q0);
         const float* src = rows + (size_t)(begin + e0 - row0) * row_stride + q0 + lane;
+        if constexpr (kButterfly) {
+            float keep = 0.f;
+#pragma unroll 8
+            for (int e = 0; e < 32; ++e) {
+                float p = 0.f;
+                if (e < ne && lane < nv) {
+                    const float* l = lam + q0;
+                    if (ev_real) l += (size_t)ev_real[begin + e0 + e] * lam_stride;
+                    p = l[lane] * src[(size_t)e * row_stride];
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
+                if (lane == e) keep = p;
+            }
+            if (lane < ne) ypart[(size_t)(q0 >> 5) * ypart_stride + e0 + lane] = keep;
+            continue;
+        }
         __syncwarp();
 #pragma unroll 16
         for (int e = 0; e < 32; ++e)
@@ -368,9 +388,10 @@ int launch_kept_forward(lm_handle* h, const float* rows, int row_stride, int64_t
     if (count <= 0) return LMMEW_OK;
     const int64_t units = (count + 31) / 32 * h->mc.nqt;
     const int grid = (int)std::min<int64_t>((units + kKeptWarps - 1) / kKeptWarps, 6 * (int64_t)h->sm_count);
-    k_kept_forward<<<grid, 32 * kKeptWarps, 0, st>>>(rows, row_stride, row0, begin, count, range,
-                                                     h->mc.nq, h->mc.nqt, lam, lam_stride, ev_real,
-                                                     ypart, ypart_stride);
+    auto kernel = h->scatter_model == LMMEW_SCATTER_SURROGATE_COARSE ? k_kept_forward<true>
+                                                                     : k_kept_forward<false>;
+    kernel<<<grid, 32 * kKeptWarps, 0, st>>>(rows, row_stride, row0, begin, count, range, h->mc.nq,
+                                             h->mc.nqt, lam, lam_stride, ev_real, ypart, ypart_stride);
     ++h->launches;
     LMMEW_CUDA(cudaGetLastError());
     return LMMEW_OK;
