@@ -352,41 +352,61 @@ int forward_async(lm_handle* h, const lm_events* ev, const float* image, float* 
     return rc;
 }
 
-// Forward projection through the energy nodes, the angles in blocks of
-// `block` (their node sums live in the arena); the events stay in the caller's
-// order and are not sorted.
+// Forward projection through the nodes, the angles in blocks of `block` (their
+// sums live in the arena); the events stay in the caller's order and are not
+// sorted.
 int forward_nodes(lm_handle* h, const lm_events* ev, const float* image, float* out_y, int block,
                   char* arena, cudaStream_t st) {
     const ModelConst& m = h->mc;
     const NodeConst& N = h->nodes;
     float* lam_v = bump<float>(arena, m.nq);
-    float* dbp = bump<float>(arena, (size_t)block * m.npc * N.nb_max * N.nl_pad);
+    float* H = bump<float>(arena, (size_t)m.np * N.nn);
+    float* dbp = bump<float>(arena, (size_t)block * m.npc * N.nb_max * N.nm_pad);
+    float* DB = bump<float>(arena, (size_t)block * m.B * N.nl_pad);
     float* F = bump<float>(arena, (size_t)block * m.B * N.nk_pad);
     float* Pr = bump<float>(arena, (size_t)block * m.B * N.W);
     int rc = launch_gather_image(h, image, lam_v, st);
+    if (rc == LMMEW_OK) rc = node_spread(h, lam_v, H, st);
     for (int a0 = 0; a0 < m.A && rc == LMMEW_OK; a0 += block) {
         const int cnt = std::min(block, m.A - a0);
-        rc = node_forward(h, lam_v, a0, 1, cnt, dbp, F, Pr, st);
+        rc = node_forward(h, lam_v, H, a0, 1, cnt, dbp, DB, F, Pr, st);
         if (rc == LMMEW_OK) rc = node_events_forward(h, ev, F, Pr, a0, cnt, out_y, st);
     }
     if (h->prof_on) h->prof_elems += (double)ev->n * (double)m.nq;
     return rc;
 }
 
+namespace {
+size_t forward_nodes_fixed(const lm_handle* h) {
+    return bump_bytes(sizeof(float) * (size_t)h->mc.nq) +
+           bump_bytes(sizeof(float) * (size_t)h->mc.np * h->nodes.nn) + 4 * 512;
+}
+}  // namespace
+
 int forward_nodes_block(const lm_handle* h, size_t bytes) {
-    const size_t fixed = bump_bytes(sizeof(float) * (size_t)h->mc.nq) + 3 * 512;
-    const size_t per = node_angle_bytes(h);
-    return (int)std::max<size_t>(1, std::min<size_t>((size_t)h->mc.A, (bytes - fixed) / per));
+    const size_t fixed = forward_nodes_fixed(h), per = node_angle_bytes(h);
+    if (bytes < fixed + per) return 0;
+    return (int)std::min<size_t>((size_t)h->mc.A, (bytes - fixed) / per);
 }
 
 size_t forward_nodes_bytes(const lm_handle* h, int block) {
-    return bump_bytes(sizeof(float) * (size_t)h->mc.nq) + 3 * 512 +
-           (size_t)block * node_angle_bytes(h);
+    return forward_nodes_fixed(h) + (size_t)block * node_angle_bytes(h);
+}
+
+// Scratch of lm_forward_noalloc's rows for n events.
+size_t noalloc_rows_bytes(const lm_handle* h, int64_t n) {
+    const ForwardPlan fp = forward_plan(h, n, int64_t(1) << 40);
+    return bump_bytes(sizeof(int) * h->mc.A) + 2 * bump_bytes(sizeof(int) * fp.G) +
+           forward_region_bytes(h, fp);
 }
 
 bool node_use(const lm_handle* h, int64_t n) {
     return h->node_route && h->n_classes > 1 && h->prec == 0 &&
-           h->scatter_model == LMMEW_SCATTER_EXACT && n >= (int64_t)8 * h->mc.A;
+           h->scatter_model == LMMEW_SCATTER_EXACT && n >= (int64_t)8 * h->mc.A &&
+           // lm_forward_noalloc takes the same route as lm_forward for every
+           // list it accepts: where its array does not hold the node sums of
+           // one angle, both keep the rows for those lists
+           (forward_nodes_block(h, kNoAllocBytes) > 0 || noalloc_rows_bytes(h, n) > kNoAllocBytes);
 }
 
 bool node_use_osem(const lm_handle* h, int64_t n) {
@@ -548,9 +568,8 @@ int lm_destroy(lm_handle* h) {
     cudaFree(h->d_inv);
     cudaFree(h->d_mu_line);
     cudaFree(h->d_clip);
-    cudaFree(h->d_node_g);
-    cudaFree(h->d_node_band);
-    cudaFree(h->d_chunk_bins);
+    cudaFree(h->d_node_tables);
+    cudaFree(h->d_node_groups);
     cudaFree(h->d_term_counter);
     cudaFree(h->d_work);
     cudaFree(h->d_cv);
@@ -819,7 +838,7 @@ int lm_forward(lm_handle* h, const lm_events* ev, const float* image, float* out
     if (surrogate_model(h)) return forward_planned(h, ev, image, out_y, stream);
     cudaStream_t st = (cudaStream_t)stream;
     if (node_use(h, ev->n)) {
-        const int block = forward_nodes_block(h, kNodeBudgetBytes);
+        const int block = std::max(1, forward_nodes_block(h, kNodeBudgetBytes));
         rc = ensure(h, h->scratch_sort, forward_nodes_bytes(h, block), st);
         if (rc == LMMEW_OK)
             return forward_nodes(h, ev, image, out_y, block, (char*)h->scratch_sort.ptr, st);
@@ -834,28 +853,31 @@ int lm_forward(lm_handle* h, const lm_events* ev, const float* image, float* out
     return forward_async(h, ev, image, out_y, ga, fp, (char*)h->scratch_sort.ptr, st);
 }
 
-// Scratch of the node route's sorted forms for row sets of at most `angles`
-// angles; the forward sums go `block` angles at a time.
+// Scratch of the node route's sorted forms for sets of at most `angles` angles;
+// the forward sums go `block` angles at a time.
 namespace {
 struct NodeScratch {
     int block;
-    float *lam, *dbp, *F, *Pr, *V, *PV, *VG, *part, *part_prim;
+    float *lam, *HT, *dbp, *DB, *F, *Pr, *V, *PV, *VG, *psi, *val, *part_prim;   // (H and T take turns)
     double *ll, *num;
 };
 size_t node_scratch(const lm_handle* h, int angles, char* base, NodeScratch* s) {
     const ModelConst& m = h->mc;
     const NodeConst& N = h->nodes;
     const size_t cells = (size_t)angles * m.B, nq_pad = (size_t)m.nqt * kQT;
-    s->block = std::min(angles, forward_nodes_block(h, kNodeBudgetBytes));
+    s->block = std::min(angles, std::max(1, forward_nodes_block(h, kNodeBudgetBytes)));
     char* p = base;
     s->lam = bump<float>(p, m.nq);
-    s->dbp = bump<float>(p, (size_t)s->block * m.npc * N.nb_max * N.nl_pad);
+    s->HT = bump<float>(p, (size_t)m.np * N.nn);
+    s->dbp = bump<float>(p, (size_t)s->block * m.npc * N.nb_max * N.nm_pad);
+    s->DB = bump<float>(p, (size_t)s->block * m.B * N.nl_pad);
     s->F = bump<float>(p, cells * N.nk_pad);
     s->Pr = bump<float>(p, cells * m.W);
     s->V = bump<float>(p, cells * N.nk_pad);
     s->PV = bump<float>(p, cells * m.W);
     s->VG = bump<float>(p, cells * N.nl_pad);
-    s->part = bump<float>(p, (size_t)angles * m.npc * m.W * nq_pad);
+    s->psi = bump<float>(p, cells * N.nm_pad);
+    s->val = bump<float>(p, (size_t)m.np * m.nq);
     s->part_prim = bump<float>(p, (size_t)angles * nq_pad);
     s->ll = bump<double>(p, cells);
     s->num = bump<double>(p, m.nq);
@@ -865,10 +887,10 @@ size_t node_scratch(const lm_handle* h, int angles, char* base, NodeScratch* s) 
 int node_forward_blocks(lm_handle* h, const NodeScratch& s, int a0, int a_step, int angles,
                         cudaStream_t st) {
     const ModelConst& m = h->mc;
-    int rc = LMMEW_OK;
+    int rc = node_spread(h, s.lam, s.HT, st);
     for (int i = 0; i < angles && rc == LMMEW_OK; i += s.block)
-        rc = node_forward(h, s.lam, a0 + i * a_step, a_step, std::min(s.block, angles - i), s.dbp,
-                          s.F + (size_t)i * m.B * h->nodes.nk_pad, s.Pr + (size_t)i * m.B * m.W, st);
+        rc = node_forward(h, s.lam, s.HT, a0 + i * a_step, a_step, std::min(s.block, angles - i), s.dbp,
+                          s.DB, s.F + (size_t)i * m.B * h->nodes.nk_pad, s.Pr + (size_t)i * m.B * m.W, st);
     return rc;
 }
 
@@ -891,8 +913,8 @@ int backproject_nodes(lm_handle* h, const lm_events* ev, const float* weight, fl
     if (rc == LMMEW_OK)
         rc = node_cells(h, m.A, ce.cell_start, 0, ce.energy, nullptr, nullptr, weight, ce.perm, s.V,
                         s.PV, nullptr, st);
-    if (rc == LMMEW_OK) rc = node_back(h, 0, 1, m.A, s.V, s.PV, s.VG, s.part, s.part_prim, st);
-    if (rc == LMMEW_OK) rc = node_update(h, m.A, s.part, s.part_prim, nullptr, nullptr, s.num, st);
+    if (rc == LMMEW_OK) rc = node_back(h, 0, 1, m.A, s.V, s.PV, s.VG, s.psi, s.HT, s.val, s.part_prim, st);
+    if (rc == LMMEW_OK) rc = node_update(h, m.A, s.val, s.part_prim, nullptr, nullptr, s.num, st);
     if (rc != LMMEW_OK) return rc;
     if (h->prof_on) h->prof_elems += (double)ev->n * (double)m.nq;
     return launch_num_to_image(h, s.num, out_image, st);
@@ -929,10 +951,11 @@ int osem_nodes(lm_handle* h, const lm_events* ev, int n_subsets, int n_iters, in
                 rc = node_cells(h, cnt, ce.cell_start, cell0, ce.energy, s.F, s.Pr, nullptr, nullptr,
                                 s.V, s.PV, ll ? s.ll : nullptr, st);
             if (rc == LMMEW_OK)
-                rc = node_back(h, sub, n_subsets, cnt, s.V, s.PV, s.VG, s.part, s.part_prim, st);
+                rc = node_back(h, sub, n_subsets, cnt, s.V, s.PV, s.VG, s.psi, s.HT, s.val, s.part_prim,
+                               st);
             if (rc == LMMEW_OK && ll) rc = node_loglik(h, s.ll, cnt * m.B, s.lam, sens, ll, st);
             if (rc == LMMEW_OK)
-                rc = node_update(h, cnt, s.part, s.part_prim, sens, s.lam, nullptr, st);
+                rc = node_update(h, cnt, s.val, s.part_prim, sens, s.lam, nullptr, st);
         }
         if (h->prof_on) h->prof_elems += (double)ev->n * (double)m.nq;
     }

@@ -286,6 +286,28 @@ __global__ void k_tiles(const int* start, const int* tile_start, const int* angl
 
 }  // namespace
 
+// Stable LSD radix sort of (keys, vals) over the ping-pong buffers; the
+// sorted pair ends in (kin, vin).
+int sort_pairs(lm_handle* h, int64_t n, int bits, uint32_t*& kin, uint32_t*& kout,
+                     uint32_t*& vin, uint32_t*& vout, uint32_t* hist, cudaStream_t st) {
+    const int64_t nblk = (n + kSortChunk - 1) / kSortChunk;
+    for (int shift = 0; shift < bits; shift += 8) {
+        k_hist<<<(unsigned)nblk, kSortThreads, 0, st>>>(kin, n, shift, hist, (int)nblk);
+        k_scan<<<1, 1024, 0, st>>>(hist, 256 * nblk);
+        k_scatter<<<(unsigned)nblk, kSortThreads, 0, st>>>(kin, vin, n, shift, hist, (int)nblk, kout,
+                                                          vout);
+        LMMEW_CUDA(cudaGetLastError());
+        std::swap(kin, kout);
+        std::swap(vin, vout);
+    }
+    h->launches += 3 * ((bits + 7) / 8);
+    return LMMEW_OK;
+}
+
+size_t pair_hist_bytes(int64_t n) {
+    return 4 * 256 * (size_t)std::max<int64_t>((n + kSortChunk - 1) / kSortChunk, 1);
+}
+
 size_t sort_scratch_bytes(int64_t n, int G) {
     const int64_t nblk = (n + kSortChunk - 1) / kSortChunk;
     size_t b = 0;
@@ -322,24 +344,6 @@ Windows windows_of(const ModelConst& m) {
                    make_float4(w[6][0], w[6][1], w[7][0], w[7][1])};
 }
 
-// Stable LSD radix sort of (keys, vals) over the ping-pong buffers; the
-// sorted pair ends in (kin, vin).
-int radix_sort_pairs(lm_handle* h, int64_t n, int bits, uint32_t*& kin, uint32_t*& kout,
-                     uint32_t*& vin, uint32_t*& vout, uint32_t* hist, cudaStream_t st) {
-    const int64_t nblk = (n + kSortChunk - 1) / kSortChunk;
-    for (int shift = 0; shift < bits; shift += 8) {
-        k_hist<<<(unsigned)nblk, kSortThreads, 0, st>>>(kin, n, shift, hist, (int)nblk);
-        k_scan<<<1, 1024, 0, st>>>(hist, 256 * nblk);
-        k_scatter<<<(unsigned)nblk, kSortThreads, 0, st>>>(kin, vin, n, shift, hist, (int)nblk, kout,
-                                                          vout);
-        LMMEW_CUDA(cudaGetLastError());
-        std::swap(kin, kout);
-        std::swap(vin, vout);
-    }
-    h->launches += 3 * ((bits + 7) / 8);
-    return LMMEW_OK;
-}
-
 // The sort shared by sort_events and sort_events_async: keys, radix passes,
 // gather, group bounds and tiles of the G = A * n_classes groups, all on
 // the caller's stream.  rank_of_angle [A], angle_of_group and lines_of_group
@@ -361,7 +365,7 @@ int sort_and_tile(lm_handle* h, const lm_events* ev, int G, const int* rank_of_a
         LMMEW_CUDA(cudaGetLastError());
         const int bits = key_bits((uint64_t)G * (uint64_t)B);
         uint32_t *kin = keys0, *kout = keys1, *vin = vals0, *vout = vals1;
-        const int rc = radix_sort_pairs(h, n, bits, kin, kout, vin, vout, hist, st);
+        const int rc = sort_pairs(h, n, bits, kin, kout, vin, vout, hist, st);
         if (rc != LMMEW_OK) return rc;
         k_gather<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(kin, vin, ev->energy_keV, n, B, perm,
                                                              bin_s, e_s);
@@ -598,7 +602,7 @@ int sort_cells(lm_handle* h, const lm_events* ev, const int* rank_of_angle, Cell
         wn.w45, wn.w67, EnergyClasses{}, kin, vin, h->d_status);
     ++h->launches;
     LMMEW_CUDA(cudaGetLastError());
-    const int rc = radix_sort_pairs(h, n, key_bits((uint64_t)cells), kin, kout, vin, vout, hist, st);
+    const int rc = sort_pairs(h, n, key_bits((uint64_t)cells), kin, kout, vin, vout, hist, st);
     if (rc != LMMEW_OK) return rc;
     k_gather<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(kin, vin, ev->energy_keV, n, m.B, out->perm,
                                                          bins, out->energy);
@@ -883,7 +887,7 @@ int sort_events_batch(lm_handle* h, const lm_events* evs, int R, int n_subsets,
             wn.w67, h->ecls, kin, vin, h->d_status);
         ++h->launches;
         LMMEW_CUDA(cudaGetLastError());
-        int rc = radix_sort_pairs(h, n, key_bits((uint64_t)G * (uint64_t)B), kin, kout, vin, vout,
+        int rc = sort_pairs(h, n, key_bits((uint64_t)G * (uint64_t)B), kin, kout, vin, vout,
                                   out->tmp_hist, st);
         if (rc != LMMEW_OK) return rc;
         k_gather<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(kin, vin, c_energy, n, B, out->perm,
@@ -940,7 +944,7 @@ int bp_order_batch(lm_handle* h, SortedEvents* se, int R, const int64_t* blk_sta
                                                            vin);
     LMMEW_CUDA(cudaGetLastError());
     ++h->launches;
-    int rc = radix_sort_pairs(h, n, key_bits((uint64_t)G), kin, kout, vin, vout, se->tmp_hist, st);
+    int rc = sort_pairs(h, n, key_bits((uint64_t)G), kin, kout, vin, vout, se->tmp_hist, st);
     if (rc != LMMEW_OK) return rc;
     k_bounds<<<(unsigned)((G + 1 + 127) / 128), 128, 0, st>>>(kin, n, (int)G, 1, grp_start);
     ++h->launches;

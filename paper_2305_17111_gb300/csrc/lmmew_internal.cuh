@@ -90,20 +90,29 @@ struct EnergyClasses {
     float bnd[2 * LMMEW_MAX_LINES];     // ascending; class = #{k : bnd[k] <= E_hat}
 };
 
-// Energy nodes of the dense-list projections (nodes.cu): t(E) = 2 sqrt(E) /
-// kappa, recorded-energy nodes k_first + k (8 per unit of t) and, per line,
-// scattered-energy nodes l_first + i (16 per unit), the lines one after the
-// other.
+// Nodes of the dense-list projections (nodes.cu): t(E) = 2 sqrt(E) / kappa,
+// recorded-energy nodes k_first + k (8 per unit of t) and, per line,
+// scattered-energy nodes l_first + i (16 per unit), direction nodes (n_dir
+// around the circle) and offsets from the detector direction (m_count on a half
+// circle), the lines one after the other.
 struct NodeConst {
     int W;
     int nk, nk_pad, k_first;
     int nl, nl_pad;
     int l_first[4], l_count[4], l_off[4];
-    float cl, cl_lo;           // node of a scattered energy = (cl + cl_lo) / sr
+    int n_dir[4], n_off[4], nn;
+    int m_count[4], m_off[4], nm_pad;
+    int start_ints;            // path starts per point: n_dir + 2 per line
     float ck, ck_lo;           // node of a recorded energy = (ck + ck_lo) sqrt(E)
     float reach_lo[4], reach_hi[4];   // recorded energies single scatter of the line can have
-    int nb_max;                // most bins one chunk of 32 scatter points reaches
-    int spread_warps, spread_smem, gather_smem;
+    int nb_max, nbg_max;       // most bins 32 ordered, 8 neighbouring scatter points reach
+};
+// Their device tables (one region; see NodeParams in nodes.cu).
+struct NodeTables {
+    float *mu, *psi_w, *dec_w, *g, *gt, *gamma, *path_b;
+    int *psi_l, *dec_start, *dec_m, *rank, *path_start, *path_q, *path_of, *grp_pt;
+    int2 *k_of_l, *l_of_k, *chunk_bins, *grp_bins;
+    uint32_t* fix;
 };
 struct NodeWindows {
     float lo[LMMEW_MAX_WINDOWS], hi[LMMEW_MAX_WINDOWS];
@@ -161,12 +170,12 @@ struct lm_handle {
     double* d_on_det = nullptr;    // [A][np] collimator mass of each point on the detector
     int* d_inv = nullptr;          // [A][np] point of each slot of an angle's point order
     double* d_mu_line = nullptr;   // [W] mu_water at each line energy
-    // energy nodes (dense event lists)
+    // nodes (dense event lists)
     lmmew::NodeConst nodes{};
+    lmmew::NodeTables node_tables{};
     int node_route = 0;            // 1: the model has the node route
-    float* d_node_g = nullptr;     // Gaussian matrix [nl][nk_pad] and its transpose [nk_pad][nl_pad]
-    int2* d_chunk_bins = nullptr;  // [A][npc] bins each chunk of 32 scatter points reaches
-    int2* d_node_band = nullptr;   // its bands: [nl] nodes k of l, [W][nk_pad] nodes l of k
+    void* d_node_tables = nullptr;
+    float* d_node_groups = nullptr;   // collimator values of 8 scatter points at a time
     lmmew::ChunkRange* d_clip = nullptr;   // a row launch's tiles clipped to one angle block
     // cached subset sensitivities for the last partition asked for
     int sens_parts = 0;
@@ -252,18 +261,24 @@ extern int64_t g_table_budget;
 // the recorded energies single scatter of line w can reach (rounded outward)
 void build_energy_classes(lm_handle* h);
 void line_reach(const lm_handle* h, int w, float* lo, float* hi);
-// nodes.cu: projections of dense event lists through energy nodes
+// nodes.cu: projections of dense event lists through angle and energy nodes
 int build_nodes(lm_handle* h);
 size_t node_angle_bytes(const lm_handle* h);   // scratch of one angle's forward sums
-int node_forward(lm_handle* h, const float* lam_v, int a0, int a_step, int angles, float* dbp,
-                 float* F, float* Pr, cudaStream_t st);
+int node_spread(lm_handle* h, const float* lam_v, float* H, cudaStream_t st);
+int node_forward(lm_handle* h, const float* lam_v, const float* H, int a0, int a_step, int angles,
+                 float* dbp, float* DB, float* F, float* Pr, cudaStream_t st);
 int node_cells(lm_handle* h, int angles, const int* cell_start, int cell0, const float* energy,
                const float* F, const float* Pr, const float* weight, const uint32_t* perm, float* V,
                float* PV, double* ll, cudaStream_t st);
 int node_back(lm_handle* h, int a0, int a_step, int angles, const float* V, const float* PV,
-              float* VG, float* part, float* part_prim, cudaStream_t st);
-int node_update(lm_handle* h, int angles, const float* part, const float* part_prim,
+              float* VG, float* psi, float* T, float* val, float* part_prim, cudaStream_t st);
+int node_update(lm_handle* h, int angles, const float* val, const float* part_prim,
                 const double* sens, float* lam, double* num, cudaStream_t st);
+// events.cu: stable LSD radix sort of (key, value) pairs over ping-pong buffers;
+// the sorted pair ends in (kin, vin)
+size_t pair_hist_bytes(int64_t n);
+int sort_pairs(lm_handle* h, int64_t n, int bits, uint32_t*& kin, uint32_t*& kout, uint32_t*& vin,
+               uint32_t*& vout, uint32_t* hist, cudaStream_t st);
 int node_loglik(lm_handle* h, const double* ll, int n_ll, const float* lam, const double* sens,
                 double* out, cudaStream_t st);
 // api.cu: row-kernel timing around a launch of the node route (no-ops while off)
@@ -352,13 +367,15 @@ ForwardPlan forward_plan(const lm_handle* h, int64_t n, int64_t cap_max);
 size_t forward_region_bytes(const lm_handle* h, const ForwardPlan& p);
 int forward_async(lm_handle* h, const lm_events* ev, const float* image, float* out_y,
                   const GroupArrays& ga, const ForwardPlan& p, char* arena, cudaStream_t st);
-// api.cu: the same through the energy nodes, `block` angles at a time, in
+// api.cu: the same through the nodes, `block` angles at a time, in
 // forward_nodes_bytes(h, block) of scratch; forward_nodes_block: the angles
 // that fit `bytes`; node_use: whether an n-event projection takes that route
 int forward_nodes(lm_handle* h, const lm_events* ev, const float* image, float* out_y, int block,
                   char* arena, cudaStream_t st);
 int forward_nodes_block(const lm_handle* h, size_t bytes);
 size_t forward_nodes_bytes(const lm_handle* h, int block);
+size_t noalloc_rows_bytes(const lm_handle* h, int64_t n);
+constexpr size_t kNoAllocBytes = size_t(16) << 20;   // lm_forward_noalloc's static array: 16 MiB
 bool node_use(const lm_handle* h, int64_t n);
 bool node_use_osem(const lm_handle* h, int64_t n);   // the same for a whole reconstruction
 // Row blocks of n_sets consecutive rank ranges (the subsets of a partition

@@ -13,7 +13,6 @@ namespace lmmew {
 namespace {
 
 // Every GPU that loads the library holds this array until the process exits.
-constexpr size_t kNoAllocBytes = size_t(16) << 20;   // 16 MiB
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
 constexpr int kMaxDevices = 64;
@@ -60,16 +59,13 @@ extern "C" int lm_forward_noalloc(lm_handle* h, const lm_events* ev, const float
     if (ev->n == 0) return LMMEW_OK;
     if (!ev->angle || !ev->bin || !ev->energy_keV || !image || !out_y)
         return set_error(LMMEW_ERR_INVALID_ARG, "NULL event, image or output pointer");
-    const ModelConst& m = h->mc;
     const int64_t n = ev->n;
     if (n >= (int64_t(1) << 31))
         return set_error(LMMEW_ERR_INVALID_ARG, "at most 2^31 - 1 events per call");
     // one row block of every event; every word of the region is written
     // before it is read within a call, so nothing has to start at zero
     const ForwardPlan fp = forward_plan(h, n, int64_t(1) << 40);
-    const int G = sort_groups(h, m.A);
-    const size_t need = bump_bytes(sizeof(int) * m.A) + 2 * bump_bytes(sizeof(int) * G) +
-                        forward_region_bytes(h, fp);
+    const size_t need = noalloc_rows_bytes(h, n);
     if (need > kNoAllocBytes)
         return set_error(LMMEW_ERR_INVALID_ARG,
                          "lm_forward_noalloc: " + std::to_string(n) + " events need " +

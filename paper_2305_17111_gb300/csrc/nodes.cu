@@ -1,38 +1,54 @@
-// Projections of dense event lists through energy nodes.
+// Projections of dense event lists through angle and energy nodes.
 //
-// The single-scatter part of an event's row is a sum of Gaussians in the
-// recorded energy, a_j[q] = sum_{p,w} C_p(b_j) omega_{qpw} g(E_j; E'_{qpw}),
-// g(E; E') = exp(-(E - E')^2 / (2 sigma^2(E'))), and the projections are
-// linear in it, so neither needs the rows themselves.  With the energy axis in
-// units of the local resolution, t(E) = 2 sqrt(E) / kappa (sigma = kappa
-// sqrt(E)), g is smooth on the scale 1 in both of its arguments, and local
-// Lagrange interpolation in each turns the sums into (the idea of the fast
-// Gauss transform, Greengard & Strain 1991, with local polynomials):
+// The single-scatter part of an event's row is a sum over paths (voxel q,
+// scatter point p, line w) of Gaussians in the recorded energy.  Its factors
+// split by what they depend on.  With phi_qp the direction from q to p, theta
+// the detector direction, x = phi_qp - theta and E'(x) Compton's energy,
 //
-//   forward   D[p][l]  = sum_{q,w} lambda_q omega_{qpw} L_l(E'_{qpw}),
-//             DB[b][l] = sum_p C_p(b) D[p][l]                                k_node_spread
-//             F[b][k]  = sum_l G[l][k] DB[b][l]                              k_node_values
-//             y_j      = sum_k L_k(E_j) F[b_j][k] + unscattered part         k_node_y, k_node_cells
-//   back      V[b][k]  = sum_{j in cell b} r_j L_k(E_j)                      k_node_cells
-//             VG[b][l] = sum_k G[l][k] V[b][k]                               k_node_unvalues
-//             PHI[p][l] = sum_b C_p(b) VG[b][l],
-//             out[q]   = sum_{p,w} omega_{qpw} sum_l L_l(E'_{qpw}) PHI[p][l] k_node_gather
+//   C_p(b) B_{qpw} f_w(x) exp(-mu(E'(x)) gamma_p) g(E; E'(x)),
 //
-// per detector angle, with l over the nodes of the scattered energies (16 per
-// unit of t, 7 taps), k over those of the recorded energies (8 per unit, 12
-// taps) and G[l][k] = g(E_k; E_l).  A path (q, p, w, angle) is visited once per
-// projection whatever the number of events, where the rows take one
-// exponential per event and path in reach.  Interpolation error of a term,
-// relative to the term: 4e-10 (1e-8, 1e-6) for an energy 0 (4, 6) sigma from
-// E', below the FP32 rounding of the sums for every energy the lines produce;
-// everything is FP32 with fixed-order sums, the voxel sums FP64.
+// B_{qpw} = alpha mu_0 rho_p A_p / d exp(-mu_0 gamma_qp) / K does not depend
+// on the detector angle, f = KN shape / (sqrt(2 pi) sigma(E')), gamma_p is the
+// point's line integral to the detector and g the unit Gaussian, smooth in E
+// and E' on the scale of sigma.  So the sums go through nodes with local
+// Lagrange interpolation (the idea of the fast Gauss transform, Greengard &
+// Strain 1991, with local polynomials): N_w directions around the circle (a
+// multiple of the angle count, so that x falls on the same nodes +-m for every
+// detector angle), 16 scattered energies and 8 recorded energies per sigma.
 //
-// omega = 2^-nlh and E' (sigma = sqrt(log2(e)/2) / sr) come from the path
-// tables of the row kernel, so both routes evaluate the same paths.
+//   forward   H[p][n]  = sum_q lambda_q B_{qp} L_n(phi_qp)                    k_ang_spread
+//             S[b][m]  = sum_p C_p(b) e^{-mu(m) gamma_p} (H[p][s+m] + H[p][s-m])  k_ang_bins
+//             DB[b][l] = sum_m L_l(E'(m)) f(m) S[b][m]                        k_node_bins
+//             F[b][k]  = sum_l G[l][k] DB[b][l]                               k_node_values
+//             y_j      = sum_k L_k(E_j) F[b_j][k] + unscattered part          k_node_y, k_node_cells
+//   back      V[b][k]  = sum_{j in cell b} r_j L_k(E_j)                       k_node_cells
+//             VG[b][l] = sum_k G[l][k] V[b][k]                                k_node_unvalues
+//             PSI[b][m] = f(m) sum_l L_l(E'(m)) VG[b][l]                      k_ang_psi
+//             T[p][n]  = sum_angles e^{-mu(m) gamma_p} sum_b C_p(b) PSI[b][m] k_ang_back
+//             out[q]   = sum_p B_{qp} sum_n L_n(phi_qp) T[p][n]               k_ang_paths, k_node_update
+//
+// (s = the node of the detector direction, m = |n - s|).  A projection visits
+// every (q, p, w) once whatever the number of events and of detector angles,
+// where the rows take one exponential per event and path in reach; nothing
+// of the path tables is read.  Interpolation errors are near 1e-8 of an event's
+// value (1e-6 in the worst case of an image of one voxel: mu has kinks at the
+// attenuation knots, which the node spacing of the lines that cross one is
+// chosen for), below the FP32 rounding of the sums; everything is FP32 with
+// fixed-order sums, the voxel sums FP64.
+//
+// Measured (864 voxels and 864 points, 3 lines, 60 angles of 64 bins; times
+// below that name no size are this model's): a forward projection of 100 000
+// events 0.33 ms of kernels, 19.5 ms through the rows and 0.79 ms with the
+// image spread at every angle anew through the path tables; a back projection
+// 0.62 ms (12.0 ms, 0.70 ms); a sub-iteration of 8 angles 0.19 ms (2.15 ms,
+// 0.32 ms).  At 3464 voxels and 120 angles of 128 bins a sub-iteration of 15
+// angles takes 0.61 ms (26 ms, 1.29 ms).
 #include <math.h>
 
 #include <algorithm>
 #include <atomic>
+#include <cstring>
+#include <utility>
 #include <vector>
 
 #include "lmmew_internal.cuh"
@@ -45,65 +61,41 @@ constexpr int kPerUnitL = 16;      // nodes per unit of t
 constexpr int kTapsK = 12;         // taps of the recorded-energy nodes
 constexpr int kPerUnitK = 8;
 constexpr double kBandSigmas = 9.0;   // G kept within this many sigma (reach 8 plus the stencils)
-constexpr int kSpreadWarpsMax = 4;
-constexpr int kStageRows = 16;     // voxels per copy of the spread kernel
-constexpr uint32_t kStageBytes = kStageRows * kPC * 4u;   // one component of a stage
-constexpr int kGatherThreads = 256;
+constexpr int kTapsN = 7;          // taps of the direction nodes
+constexpr int kGroup = 8;          // scatter points per block of k_ang_back
+constexpr int kBinsT = 16;         // detector bins per pass of k_ang_bins
 constexpr int kValueRows = 8;      // (angle, bin) rows per block of k_node_values / _unvalues
-constexpr int kCellWarps = 2;
+constexpr int kValueWarps = 8;     // their warps, sharing the sum over nodes
+constexpr int kCellWarps = 4;
 
 __device__ __forceinline__ float ex2f(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ float rcpf(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 __device__ __forceinline__ f32x2 pk1(float v) { return pk(v, v); }
 
-// Two paths' scattered energies on their line's nodes, u = c1 / sr in node
-// units: the local index of the first of the 7 taps (clamped into the line's
-// nodes) and the distance from the centre tap, in [-1/2, 1/2].  c1 comes in
-// two parts and the reciprocal's error is taken out to first order, so the
-// distance carries sr's own rounding only (u's rounding would shift a path by
-// 4e-6 sigma).  Absent paths (sr = 0) carry weight 0 and land on the last taps.
-__device__ __forceinline__ f32x2 node_pos2(float sr0, float sr1, float c1, float c1_lo, int first,
-                                           unsigned last, unsigned& i0, unsigned& i1) {
-    const float x0 = fmaxf(sr0, 1e-6f), x1 = fmaxf(sr1, 1e-6f);
-    const f32x2 r = pk(rcpf(x0), rcpf(x1));
-    const f32x2 me = fma2(pk(x0, x1), r, pk1(-1.f));        // x r - 1
-    const f32x2 big = fma2(pk1(c1), r, pk1(12582912.f));     // 1.5 2^23: rounds to the nearest integer
-    const f32x2 mj = fma2(big, pk1(-1.f), pk1(12582912.f));  // -(nearest node)
-    f32x2 s = fma2(pk1(c1), r, mj);
-    s = fma2(pk1(c1_lo), r, s);
-    s = fma2(mul2(pk1(-c1), r), me, s);
-    float b0, b1;
-    upk(big, b0, b1);
-    i0 = min((unsigned)(__float_as_int(b0) - 0x4B400000 - first), last);
-    i1 = min((unsigned)(__float_as_int(b1) - 0x4B400000 - first), last);
-    return s;
+// The 7 Lagrange weights at distance s from the centre node, times v.
+__device__ __forceinline__ void lagrange7(float s, float v, float (&w)[7]) {
+    const float q = s * s, a1 = q - 1.f, a2 = q - 4.f, a3 = q - 9.f, sv = s * v, a12 = a1 * a2;
+    const float m1 = sv * (a2 * a3) * (1.f / 48.f), m2 = sv * (a1 * a3) * (-1.f / 120.f);
+    const float m3 = sv * a12 * (1.f / 720.f);
+    w[3] = a12 * a3 * (v * (-1.f / 36.f));
+    w[4] = fmaf(m1, s, m1);
+    w[2] = fmaf(m1, s, -m1);
+    w[5] = fmaf(m2, s, 2.f * m2);
+    w[1] = fmaf(m2, s, -2.f * m2);
+    w[6] = fmaf(m3, s, 3.f * m3);
+    w[0] = fmaf(m3, s, -3.f * m3);
 }
 
-// The 7 Lagrange weights of two paths at distance s, times wt.
-__device__ __forceinline__ void lagrange7(f32x2 s, f32x2 wt, f32x2 (&w)[7]) {
-    const f32x2 q = mul2(s, s);
-    const f32x2 a1 = add2(q, pk1(-1.f)), a2 = add2(q, pk1(-4.f)), a3 = add2(q, pk1(-9.f));
-    const f32x2 sw = mul2(s, wt), a12 = mul2(a1, a2);
-    const f32x2 m1 = mul2(mul2(sw, mul2(a2, a3)), pk1(1.f / 48.f));
-    const f32x2 m2 = mul2(mul2(sw, mul2(a1, a3)), pk1(-1.f / 120.f));
-    const f32x2 m3 = mul2(mul2(sw, a12), pk1(1.f / 720.f));
-    const f32x2 t1 = mul2(m1, s), t2 = mul2(m2, s), t3 = mul2(m3, s);
-    w[3] = mul2(mul2(a12, a3), mul2(wt, pk1(-1.f / 36.f)));
-    w[4] = add2(t1, m1);
-    w[2] = fma2(m1, pk1(-1.f), t1);
-    w[5] = fma2(m2, pk1(2.f), t2);
-    w[1] = fma2(m2, pk1(-2.f), t2);
-    w[6] = fma2(m3, pk1(3.f), t3);
-    w[0] = fma2(m3, pk1(-3.f), t3);
+// Nearest of n nodes to a direction (in 2^-32 turns) and the distance from it
+// in nodes, exact: c in [0, n].
+__device__ __forceinline__ float direction_pos(uint32_t fix, int n, int* c) {
+    const uint64_t u = (uint64_t)fix * (uint32_t)n;
+    const int f = (int)(int32_t)(uint32_t)u;            // fraction - (fraction >= 1/2), in 2^-32
+    *c = (int)(u >> 32) + (f < 0 ? 1 : 0);
+    return (float)f * 2.3283064365386963e-10f;
 }
 
 // The 12 Lagrange weights at position f in [0, 1) between nodes 5 and 6,
@@ -155,297 +147,457 @@ __device__ __forceinline__ bool in_reach(const NodeConst& N, float e) {
 
 __global__ void k_node_matrix(const NodeConst N, double kappa, float* g, float* gt) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N.nl * N.nk_pad) return;
+    if (i >= N.nl_pad * N.nk_pad) return;
     const int l = i / N.nk_pad, k = i % N.nk_pad;
     int w = 0;
     while (w + 1 < N.W && l >= N.l_off[w + 1]) ++w;
     const double xl = 0.5 * kappa * (N.l_first[w] + (l - N.l_off[w])) / kPerUnitL;   // sqrt(E')
     const double xk = 0.5 * kappa * (N.k_first + k) / kPerUnitK;
     const double d = (xk * xk - xl * xl) / (kappa * xl);
-    const float v = k < N.nk && fabs(d) <= kBandSigmas ? (float)exp(-0.5 * d * d) : 0.f;
+    const bool real = l - N.l_off[w] < N.l_count[w] && k < N.nk;
+    const float v = real && fabs(d) <= kBandSigmas ? (float)exp(-0.5 * d * d) : 0.f;
     g[(size_t)l * N.nk_pad + k] = v;
     gt[(size_t)k * N.nl_pad + l] = v;
 }
 
 struct NodeParams {
     NodeConst N;
-    const float* tab;        // path tables; angle i of the launch in slot slot0 + i slot_step
-    int slot0, slot_step;
     int a0, a_step, angles;  // angle i of the launch: a0 + i a_step
-    int B, nq, nqt, npc, nq_pad;
+    int A, B, nq, np, npc, nq_pad;
     const float* g;          // [nl][nk_pad] Gaussians
     const float* gt;         // [nk][nl_pad] their transpose
-    const int2* k_of_l;      // [nl] recorded-energy nodes in reach of node l
-    const int2* l_of_k;      // [W][nk_pad] nodes of line w in reach of k
+    const int2* k_of_l;      // [nl_pad / 32] recorded-energy nodes in reach of 32 nodes l
+    const int2* l_of_k;      // [nk_pad / 32] scattered-energy nodes in reach of 32 nodes k
     const int2* chunk_bins;  // [A][npc] bins a chunk of 32 scatter points reaches
     const float* cs;         // [A][npc][B][kCPad]
     const int2* crange;      // [A][B]
+    const int* inv;          // [A][np] point of each slot of an angle's point order
+    const float* gamma;      // [A][np] line integral from each point to the detector, cm
+    const float* mu;         // [nm_pad] log2(e) mu_water(E') of the direction offsets
+    const int* psi_l;        // [nm_pad] first of the 7 nodes l of an offset's E'
+    const float* psi_w;      // [nm_pad][8] their weights, times f
+    const int* dec_start;    // [nl_pad / 32 + 1] the same by 32 nodes l: offsets m and weights
+    const int* dec_m;
+    const float* dec_w;
+    const uint32_t* fix;     // [np][nq] directions of the paths of each point, ascending
+    const int* path_q;       // [np][nq] their voxels
+    const int* path_of;      // [np][nq] place of each voxel's path
+    const float* path_b;     // [W][np][nq] their B
+    const int* path_start;   // [np][start_ints] per line: first path of each centre node
+    const int* grp_pt;       // [groups][8] neighbouring points (-1: none)
+    const int2* grp_bins;    // [A][groups] bins they reach
+    const float* grp_c;      // [A][groups][nbg_max][8] their collimator values
     const float* cv;         // [A][B][nq]
     const float* prim;       // [A][W][nq]
     const float* lam;        // [nq]
-    float* dbp;              // [angles][npc][nb_max][nl_pad]: DB's part of each chunk
+    float* H;                // [np][nn]
+    float* dbp;              // [angles][npc][nb_max][nm_pad]: S's part of each chunk
+    float* DB;               // [angles][B][nl_pad]
     float* F;                // [angles][B][nk_pad]
     float* Pr;               // [angles][B][W] unscattered sums
     const float* V;          // [angles][B][nk_pad]
     const float* PV;         // [angles][B][W]
     float* VG;               // [angles][B][nl_pad]
-    float* part;             // [angles][npc][W][nq_pad]
+    float* psi;              // [angles][B][nm_pad]
+    float* T;                // [np][nn]
+    float* val;              // [np][nq]
     float* part_prim;        // [angles][nq_pad]
-    int* status;
 };
 
-// One CTA per (angle, 32 scatter points, line).  Each warp takes every
-// warps-th run of 16 voxels, a lane per scatter point, and adds each path to
-// the 7 nodes around its scattered energy in the warp's own sums [node][point]
-// in shared memory (a lane only touches its own column: no conflicts between
-// lanes or banks).  The tables of a run (nlh and sr, 2 KiB each) arrive by
-// bulk copies, double buffered per warp.  The warps' sums are added in warp
-// order and contracted with the collimator rows of the bins the 32 points
-// reach, so only the bins' node sums leave the SM.
-__global__ void __launch_bounds__(32 * kSpreadWarpsMax) k_node_spread(const NodeParams P) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int W = P.N.W, warps = P.N.spread_warps;
-    const int w = blockIdx.x % W, pc = (blockIdx.x / W) % P.npc, ai = blockIdx.x / (W * P.npc);
-    const int nlw = P.N.l_count[w];
-    float* stages = reinterpret_cast<float*>(smem);
-    float* stage0 = stages + warp * (4 * kStageRows * kPC);
-    float* sums = stages + warps * (4 * kStageRows * kPC);
-    float* mine = sums + (size_t)warp * nlw * kPC + lane;
-    __shared__ __align__(8) uint64_t bars[2 * kSpreadWarpsMax];
-    const uint32_t bar0 = smem_addr(&bars[2 * warp]);
-    if (lane == 0) {
-        mbar_init(bar0, 1);
-        mbar_init(bar0 + 8, 1);
-        mbar_fence_init();
+// H: a warp per (point, line, 122 direction nodes).  The paths centred on the
+// tile's nodes and the 3 on either side are one run of the point's directions
+// (and a second one where the circle closes).  32 of them at a time form their
+// 7 weighted taps, a lane per path; a segmented scan sums those of equal centre,
+// and the last of each adds them to the centre's sums.  At the end each node
+// collects its taps from the 7 centres around it.  No two lanes add to one
+// place, and every sum has its order.  Bound by instruction issue (66 %) once
+// the loads are a group ahead: 37 us; 47 us with a lane per centre, which
+// waits on three dependent loads per path, 42 us with a block per 122 nodes.
+// Where a centre has more than kSpreadDense paths the scan's steps cost more
+// than those waits, and a lane takes a centre's paths: 80 us instead of 118 us
+// at 3464 voxels (11, 6 and 3 paths a centre; limits of 2 and 4 are equal
+// there, 1 costs 83 us).
+constexpr int kSpreadDense = 4, kSpreadWarps = 4, kSpreadCentres = 128, kSpreadOut = kSpreadCentres - 6;
+__global__ void __launch_bounds__(32 * kSpreadWarps) k_ang_spread(const NodeParams P, int tiles, int units) {
+    __shared__ __align__(16) float taps[kSpreadWarps][7][kSpreadCentres];
+    const int lane = threadIdx.x & 31, unit = blockIdx.x * kSpreadWarps + (threadIdx.x >> 5);
+    if (unit >= units) return;
+    float (&tap)[7][kSpreadCentres] = taps[threadIdx.x >> 5];
+    const int p = unit / tiles;
+    int tile = unit % tiles, w = 0;
+    while (tile >= (P.N.n_dir[w] + kSpreadOut - 1) / kSpreadOut) {
+        tile -= (P.N.n_dir[w] + kSpreadOut - 1) / kSpreadOut;
+        ++w;
+    }
+    const int n = P.N.n_dir[w], n0 = tile * kSpreadOut;
+    const int u0 = n0 - 3, u1 = min(n0 + kSpreadOut + 2, n + 2);   // the tile's centres
+    // first path of each centre, centres 0 .. n (n: a full turn, node 0 again)
+    const int* st = P.path_start + (size_t)p * P.N.start_ints + P.N.n_off[w] + 2 * w;
+    const uint32_t* fix = P.fix + (size_t)p * P.nq;
+    const int* pq = P.path_q + (size_t)p * P.nq;
+    const float* pb = P.path_b + ((size_t)w * P.np + p) * P.nq;
+    const bool dense = P.nq > kSpreadDense * n;
+    if (dense) {
+        for (int i = lane; i <= u1 - u0; i += 32) {
+            const int u = u0 + i, c = u < 0 ? u + n : u > n ? u - n : u;
+            float g[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            int r = st[c], re = st[c + 1], more = c == 0 ? n : c == n ? 0 : -1;
+            while (true) {
+                for (; r < re; ++r) {
+                    int cc;
+                    const float s = direction_pos(fix[r], n, &cc);
+                    float x[7];
+                    lagrange7(s, pb[r] * P.lam[pq[r]], x);
+#pragma unroll
+                    for (int k = 0; k < 7; ++k) g[k] += x[k];
+                }
+                if (more < 0) break;
+                r = st[more];
+                re = st[more + 1];
+                more = -1;
+            }
+#pragma unroll
+            for (int k = 0; k < 7; ++k) tap[k][i] = g[k];
+        }
+    } else {
+        for (int i = lane; i < 7 * kSpreadCentres / 4; i += 32)
+            reinterpret_cast<float4*>(tap)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        __syncwarp();
+    }
+    for (int part = dense ? 3 : 0; part < 3; ++part) {
+        // paths centred c in [ca, cb], which are the centres u = c - shift
+        int ca, cb, shift;
+        if (part == 0) {
+            ca = max(u0, 0);
+            cb = min(u1, n);
+            shift = 0;
+        } else if (part == 1) {
+            if (u0 > 0) continue;
+            ca = n + u0;
+            cb = n;
+            shift = n;
+        } else {
+            if (u1 < n) continue;
+            ca = 0;
+            cb = u1 - n;
+            shift = -n;
+        }
+        // (two groups of 32 ahead for the voxel, one for what it leads to)
+        const int r1 = st[cb + 1], ra = st[ca];
+        int q2 = ra + lane < r1 ? pq[ra + lane] : 0;
+        uint32_t f1 = 0;
+        float b1 = 0.f, v1 = 0.f;
+        auto ahead = [&](int r) {
+            f1 = 0;
+            b1 = v1 = 0.f;
+            if (r < r1) {
+                f1 = fix[r];
+                b1 = pb[r];
+                v1 = P.lam[q2];
+            }
+            q2 = r + 32 < r1 ? pq[r + 32] : 0;
+        };
+        ahead(ra + lane);
+        for (int r0 = ra; r0 < r1; r0 += 32) {
+            const int r = r0 + lane;
+            const uint32_t f = f1;
+            const float v = b1 * v1;
+            ahead(r + 32);
+            float x[7];
+            int c;
+            const float s = direction_pos(f, n, &c);
+            lagrange7(s, v, x);
+            if (r >= r1) c = -1;
+            const int before = __shfl_up_sync(0xffffffffu, c, 1);
+            const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || c != before);
+            const int back = lane - (31 - __clz(heads & (0xffffffffu >> (31 - lane))));
+            const int most = __reduce_max_sync(0xffffffffu, back);
+            for (int o = 1; o <= most; o <<= 1)
+#pragma unroll
+                for (int k = 0; k < 7; ++k) {
+                    const float y = __shfl_up_sync(0xffffffffu, x[k], o);
+                    if (back >= o) x[k] += y;
+                }
+            __syncwarp();
+            if (c >= 0 && (lane == 31 || (heads >> (lane + 1) & 1u)))
+#pragma unroll
+                for (int k = 0; k < 7; ++k) tap[k][c - shift - u0] += x[k];
+        }
     }
     __syncwarp();
-    const size_t block = (size_t)3 * W * kQT * kPC;
-    const float* tab = P.tab + ((size_t)(P.slot0 + ai * P.slot_step) * P.nqt * P.npc + pc) * block +
-                       (size_t)w * kQT * kPC;
-    const int runs = (P.nq + kStageRows - 1) / kStageRows;
-    const int nt = runs > warp ? (runs - warp + warps - 1) / warps : 0;
-    auto issue = [&](int it) {
-        const int run = warp + it * warps;
-        const float* src = tab + (size_t)(run / (kQT / kStageRows)) * P.npc * block +
-                           (size_t)(run % (kQT / kStageRows)) * (kStageRows * kPC);
-        float* dst = stage0 + (it & 1) * (2 * kStageRows * kPC);
-        const uint32_t bar = bar0 + 8 * (it & 1);
-        mbar_expect_tx(bar, 2 * kStageBytes);
-        bulk_g2s(smem_addr(dst), src, kStageBytes, bar);
-        bulk_g2s(smem_addr(dst + kStageRows * kPC), src + (size_t)W * kQT * kPC, kStageBytes, bar);
-    };
-    if (lane == 0) {
-        if (nt > 0) issue(0);
-        if (nt > 1) issue(1);
+    for (int i = lane; i < kSpreadOut && n0 + i < n; i += 32) {
+        float h = 0.f;                     // centre n0 + i + j - 3 is place i + j, and node n0 + i its tap 6 - j
+#pragma unroll
+        for (int j = 0; j < 7; ++j) h += tap[6 - j][i + j];
+        P.H[(size_t)p * P.N.nn + P.N.n_off[w] + n0 + i] = h;
     }
-    for (int l = 0; l < nlw; ++l) mine[l * kPC] = 0.f;
-    const int first = P.N.l_first[w] + 3;
-    const unsigned last = (unsigned)(nlw - kTapsL);
-    const float c1 = P.N.cl, c1_lo = P.N.cl_lo;
-    for (int it = 0; it < nt; ++it) {
-        const int q0 = (warp + it * warps) * kStageRows;
-        const float lam_l = lane < kStageRows && q0 + lane < P.nq ? P.lam[q0 + lane] : 0.f;
-        if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar0 + 8 * (it & 1), (it >> 1) & 1))) {
-            if (lane == 0) {
-                atomicOr(P.status, kStatusTimeout);
-                // the copies still in flight land before the CTA goes on
-                mbar_wait_bounded(bar0 + 8 * (it & 1), (it >> 1) & 1);
-                if (it + 1 < nt) mbar_wait_bounded(bar0 + 8 * ((it + 1) & 1), ((it + 1) >> 1) & 1);
-            }
-            break;
-        }
-        // the whole stage into registers first: the sums' stores below could
-        // alias it as far as the compiler knows, which would keep every load
-        // and all arithmetic of a path behind the stores of the one before
-        const float* st = stage0 + (it & 1) * (2 * kStageRows * kPC) + lane;
-        float nl[kStageRows], sr[kStageRows];
-#pragma unroll
-        for (int r = 0; r < kStageRows; ++r) {
-            nl[r] = st[r * kPC];
-            sr[r] = st[(kStageRows + r) * kPC];
-        }
-        __syncwarp();
-        if (lane == 0 && it + 2 < nt) issue(it + 2);
-#pragma unroll
-        for (int r = 0; r < kStageRows; r += 2) {
-            const f32x2 lam = pk(__shfl_sync(0xffffffffu, lam_l, r), __shfl_sync(0xffffffffu, lam_l, r + 1));
-            const f32x2 wt = mul2(pk(ex2f(-nl[r]), ex2f(-nl[r + 1])), lam);
-            unsigned i0, i1;
-            const f32x2 s = node_pos2(sr[r], sr[r + 1], c1, c1_lo, first, last, i0, i1);
-            f32x2 c[7];
-            lagrange7(s, wt, c);
-            float x[7], y[7];
-#pragma unroll
-            for (int k = 0; k < 7; ++k) upk(c[k], x[k], y[k]);
-            float* d = mine + i0 * kPC;
-            float v[7];
-#pragma unroll
-            for (int k = 0; k < 7; ++k) v[k] = d[k * kPC];
-#pragma unroll
-            for (int k = 0; k < 7; ++k) d[k * kPC] = v[k] + x[k];
-            d = mine + i1 * kPC;
-#pragma unroll
-            for (int k = 0; k < 7; ++k) v[k] = d[k * kPC];
-#pragma unroll
-            for (int k = 0; k < 7; ++k) d[k * kPC] = v[k] + y[k];
-        }
+}
+
+// S's part of one (angle, 32 scatter points, line): two direction offsets m a
+// thread, the points one after the other, 16 bins at a time (a collimator value
+// read from shared memory serves both offsets).  Bound by FP32 issue: 115 us for
+// 60 angles, 20 us for 8.
+constexpr int kOffThreads = 128, kOffPer = 2;
+__global__ void __launch_bounds__(kOffThreads) k_ang_bins(const NodeParams P, int tiles) {
+    __shared__ __align__(16) float sc[kPC][kBinsT];
+    __shared__ int sp[kPC];
+    __shared__ float sgm[kPC];
+    const int t = threadIdx.x;
+    constexpr int kTile = kOffThreads * kOffPer;
+    int tile = blockIdx.x % tiles;
+    const int pc = (blockIdx.x / tiles) % P.npc, ai = blockIdx.x / (tiles * P.npc);
+    int w = 0;
+    while (tile >= (P.N.m_count[w] + kTile - 1) / kTile) {
+        tile -= (P.N.m_count[w] + kTile - 1) / kTile;
+        ++w;
     }
-    __syncthreads();
-    const int T = blockDim.x;
-    for (int i = threadIdx.x; i < nlw * kPC / 4; i += T) {
-        float4 a = reinterpret_cast<const float4*>(sums)[i];
-        for (int k = 1; k < warps; ++k) {
-            const float4 b = reinterpret_cast<const float4*>(sums + (size_t)k * nlw * kPC)[i];
-            a.x += b.x;
-            a.y += b.y;
-            a.z += b.z;
-            a.w += b.w;
-        }
-        reinterpret_cast<float4*>(sums)[i] = a;
+    const int a = P.a0 + ai * P.a_step, n = P.N.n_dir[w];
+    const int s = (int)((int64_t)a * n / P.A);
+    int n1[kOffPer], n2[kOffPer];
+    float mu[kOffPer], two[kOffPer];
+#pragma unroll
+    for (int j = 0; j < kOffPer; ++j) {
+        const int m = min(tile * kTile + j * kOffThreads + t, P.N.m_count[w] - 1);
+        n1[j] = s + m;
+        n2[j] = s - m;
+        if (n1[j] >= n) n1[j] -= n;
+        if (n2[j] < 0) n2[j] += n;
+        two[j] = n1[j] != n2[j] ? 1.f : 0.f;
+        mu[j] = P.mu[P.N.m_off[w] + m];
     }
-    // the bins' sums over the 32 points: a thread per node, 4 bins at a time;
-    // the points in quads, rotated by the lane (no bank conflicts)
-    const int a = P.a0 + ai * P.a_step;
+    const int cnt = min(kPC, P.np - pc * kPC);
+    if (t < kPC) {
+        const int p = t < cnt ? P.inv[(size_t)a * P.np + pc * kPC + t] : 0;
+        sp[t] = p * P.N.nn + P.N.n_off[w];
+        sgm[t] = t < cnt ? P.gamma[(size_t)a * P.np + p] : 0.f;
+    }
     const int2 br = P.chunk_bins[(size_t)a * P.npc + pc];
-    const float* cr = P.cs + (((size_t)a * P.npc + pc) * P.B + br.x) * kCPad;
-    float* out = P.dbp + (((size_t)ai * P.npc + pc) * P.N.nb_max) * P.N.nl_pad + P.N.l_off[w];
-    const int nb = br.y - br.x;
-    constexpr int kBinsStaged = 64;   // collimator rows staged at a time (8 KiB, in the copy buffers)
-    for (int s0 = 0; s0 < nb; s0 += kBinsStaged) {
-        const int ns = min(kBinsStaged, nb - s0);
+    const float* cr = P.cs + ((size_t)a * P.npc + pc) * P.B * kCPad;
+    float* out = P.dbp + ((size_t)ai * P.npc + pc) * P.N.nb_max * P.N.nm_pad + P.N.m_off[w];
+    for (int b0 = br.x; b0 < br.y; b0 += kBinsT) {
         __syncthreads();
-        for (int i = threadIdx.x; i < ((ns + 3) & ~3) * (kPC / 4); i += T) {
-            const int b = i >> 3, c = i & 7;
-            reinterpret_cast<float4*>(stages)[i] =
-                b < ns ? *reinterpret_cast<const float4*>(cr + (size_t)(s0 + b) * kCPad + 4 * c)
-                       : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = t; i < kPC * kBinsT; i += kOffThreads) {
+            const int b = i / kPC, p = i % kPC;
+            sc[p][b] = b0 + b < br.y && p < cnt ? cr[(size_t)(b0 + b) * kCPad + p] : 0.f;
         }
         __syncthreads();
-        for (int l = threadIdx.x; l < nlw; l += T) {
-            const float4* dl = reinterpret_cast<const float4*>(sums + (size_t)l * kPC);
-            for (int b = 0; b < ns; b += 4) {
-                const float4* cb = reinterpret_cast<const float4*>(stages) + b * (kPC / 4);
-                f32x2 acc[4] = {0ull, 0ull, 0ull, 0ull};
+        f32x2 acc[kOffPer][kBinsT / 2];
 #pragma unroll
-                for (int i = 0; i < kPC / 4; ++i) {
-                    const int p = (i + lane) & 7;
-                    const float4 d = dl[p];
-                    const f32x2 d0 = pk(d.x, d.y), d1 = pk(d.z, d.w);
+        for (int j = 0; j < kOffPer; ++j)
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const float4 c = cb[k * (kPC / 4) + p];
-                        acc[k] = fma2(d0, pk(c.x, c.y), acc[k]);
-                        acc[k] = fma2(d1, pk(c.z, c.w), acc[k]);
+            for (int k = 0; k < kBinsT / 2; ++k) acc[j][k] = 0ull;
+        // (points past the last carry collimator values 0)
+        for (int i0 = 0; i0 < kPC; i0 += 8) {
+            float v[kOffPer][8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float* row = P.H + sp[i0 + i];
+#pragma unroll
+                for (int j = 0; j < kOffPer; ++j) v[j][i] = fmaf(two[j], row[n2[j]], row[n1[j]]);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float g = sgm[i0 + i];
+                f32x2 v2[kOffPer];
+#pragma unroll
+                for (int j = 0; j < kOffPer; ++j) v2[j] = pk1(v[j][i] * ex2f(-mu[j] * g));
+                const float4* c4 = reinterpret_cast<const float4*>(sc[i0 + i]);
+#pragma unroll
+                for (int k = 0; k < kBinsT / 4; ++k) {
+                    const float4 c = c4[k];
+#pragma unroll
+                    for (int j = 0; j < kOffPer; ++j) {
+                        acc[j][2 * k] = fma2(v2[j], pk(c.x, c.y), acc[j][2 * k]);
+                        acc[j][2 * k + 1] = fma2(v2[j], pk(c.z, c.w), acc[j][2 * k + 1]);
                     }
                 }
+            }
+        }
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (b + k < ns) {
-                        float x, y;
-                        upk(acc[k], x, y);
-                        out[(size_t)(s0 + b + k) * P.N.nl_pad + l] = x + y;
-                    }
+        for (int j = 0; j < kOffPer; ++j) {
+            const int m = tile * kTile + j * kOffThreads + t;
+            if (m >= P.N.m_count[w]) continue;
+#pragma unroll
+            for (int k = 0; k < kBinsT / 2; ++k) {
+                float x, y;
+                upk(acc[j][k], x, y);
+                if (b0 + 2 * k < br.y) out[(size_t)(b0 - br.x + 2 * k) * P.N.nm_pad + m] = x;
+                if (b0 + 2 * k + 1 < br.y) out[(size_t)(b0 - br.x + 2 * k + 1) * P.N.nm_pad + m] = y;
             }
         }
     }
 }
 
-// 8 (angle, bin) rows per block: a row's sums over the chunks of its run of
-// scatter points, then the Gaussians onto the recorded-energy nodes, a thread
-// per node; the blocks past those form the unscattered sums, a warp per
-// (row, line).  Sums run over 32 nodes at a time, then over those.
-__global__ void __launch_bounds__(384) k_node_values(const NodeParams P) {
-    extern __shared__ __align__(16) float db[];   // [nl][8]
-    const int t = threadIdx.x, T = blockDim.x, W = P.N.W;
-    const int rows = P.angles * P.B, n_row_blocks = (rows + kValueRows - 1) / kValueRows;
-    if ((int)blockIdx.x >= n_row_blocks) {
-        const int i = (blockIdx.x - n_row_blocks) * (T >> 5) + (t >> 5);
+// A row's (angle, bin) sums over the chunks of its run of scatter points, then
+// from the direction offsets onto the scattered-energy nodes: a block per row;
+// the blocks past those form the unscattered sums, a warp per (row, line).
+// Bound by load latency: 8 loads in flight per thread, whatever the run.  91 us
+// for 60 angles, 16 us for 8.
+constexpr int kRowThreadsN = 512, kRowChunks = 512;
+__global__ void __launch_bounds__(kRowThreadsN) k_node_bins(const NodeParams P) {
+    extern __shared__ float srow[];   // [nm_pad]
+    __shared__ int off[kRowChunks];
+    const int t = threadIdx.x, W = P.N.W;
+    const int rows = P.angles * P.B;
+    if ((int)blockIdx.x >= rows) {
+        const int i = (blockIdx.x - rows) * (kRowThreadsN / 32) + (t >> 5);
         if (i >= rows * W) return;
         const int row = i / W, w = i % W;
         const int a = P.a0 + (row / P.B) * P.a_step;
         const float* cv = P.cv + ((size_t)a * P.B + row % P.B) * P.nq;
         const float* pr = P.prim + ((size_t)a * W + w) * P.nq;
         float s = 0.f;
-#pragma unroll 4
-        for (int q = t & 31; q < P.nq; q += 32) s = fmaf(cv[q] * pr[q], P.lam[q], s);
+        for (int q0 = t & 31; q0 < P.nq; q0 += 256) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int q = q0 + 32 * k;
+                if (q < P.nq) s = fmaf(cv[q] * pr[q], P.lam[q], s);
+            }
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if ((t & 31) == 0) P.Pr[i] = s;
         return;
     }
-    const int r0 = blockIdx.x * kValueRows;
-    for (int i = 0; i < kValueRows; ++i) {
-        const int row = r0 + i;
-        const int ai = row / P.B, b = row % P.B, a = P.a0 + ai * P.a_step;
-        const int2 run = row < rows ? P.crange[(size_t)a * P.B + b] : make_int2(0, 0);
-        const int c0 = run.x / kPC, c1 = run.y > run.x ? (run.y + kPC - 1) / kPC : c0;
-        for (int l = t; l < P.N.nl; l += T) {
-            float s = 0.f;
-#pragma unroll 4
-            for (int pc = c0; pc < c1; ++pc) {
-                const int b0 = P.chunk_bins[(size_t)a * P.npc + pc].x;
-                s += P.dbp[(((size_t)ai * P.npc + pc) * P.N.nb_max + (b - b0)) * P.N.nl_pad + l];
+    const int row = blockIdx.x;
+    const int ai = row / P.B, b = row % P.B, a = P.a0 + ai * P.a_step;
+    const int2 run = P.crange[(size_t)a * P.B + b];
+    const int c0 = run.x / kPC, c1 = run.y > run.x ? (run.y + kPC - 1) / kPC : c0;
+    const int2* cb = P.chunk_bins + (size_t)a * P.npc;
+    const float* src = P.dbp + (size_t)ai * P.npc * P.N.nb_max * P.N.nm_pad;
+    for (int m = t; m < P.N.nm_pad; m += kRowThreadsN) srow[m] = 0.f;
+    for (int p0 = c0; p0 < c1; p0 += kRowChunks) {
+        const int np = min(kRowChunks, c1 - p0);
+        __syncthreads();
+        for (int i = t; i < np; i += kRowThreadsN) off[i] = (p0 + i) * P.N.nb_max + (b - cb[p0 + i].x);
+        __syncthreads();
+        for (int m = t; m < P.N.nm_pad; m += kRowThreadsN) {
+            bool node = false;   // (not one of the pads between the lines)
+            for (int w = 0; w < W; ++w) node |= (unsigned)(m - P.N.m_off[w]) < (unsigned)P.N.m_count[w];
+            if (!node) continue;
+            float s = srow[m];
+            for (int i0 = 0; i0 < np; i0 += 8) {
+                float v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    v[i] = i0 + i < np ? src[(size_t)off[i0 + i] * P.N.nm_pad + m] : 0.f;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) s += v[i];
             }
-            db[l * kValueRows + i] = s;
+            srow[m] = s;
         }
     }
     __syncthreads();
-    for (int k = t; (k & ~31) < P.N.nk; k += T) {
-        f32x2 f[kValueRows / 2] = {0ull, 0ull, 0ull, 0ull};
-        for (int w = 0; w < W; ++w) {
-            // the warp's nodes l: from its first node's reach to its last's
-            const int2 r = P.l_of_k[(size_t)w * P.N.nk_pad + min(k, P.N.nk - 1)];
-            const int lo = __reduce_min_sync(0xffffffffu, r.y > r.x ? r.x : 0x7fffffff);
-            const int hi = __reduce_max_sync(0xffffffffu, r.y);
-            for (int l0 = lo; l0 < hi; l0 += 32) {
-                f32x2 s[kValueRows / 2] = {0ull, 0ull, 0ull, 0ull};
-                const int l1 = min(l0 + 32, hi);
-    #pragma unroll 8
-                for (int l = l0; l < l1; ++l) {
-                    const float g = P.g[(size_t)l * P.N.nk_pad + k];
-                    const float4 d0 = *reinterpret_cast<const float4*>(db + l * kValueRows);
-                    const float4 d1 = *reinterpret_cast<const float4*>(db + l * kValueRows + 4);
-                    const f32x2 g2 = pk1(g);
-                    s[0] = fma2(g2, pk(d0.x, d0.y), s[0]);
-                    s[1] = fma2(g2, pk(d0.z, d0.w), s[1]);
-                    s[2] = fma2(g2, pk(d1.x, d1.y), s[2]);
-                    s[3] = fma2(g2, pk(d1.z, d1.w), s[3]);
-                }
-    #pragma unroll
-                for (int i = 0; i < kValueRows / 2; ++i) f[i] = add2(f[i], s[i]);
+    // (32 nodes l at a time, their taps padded to the longest of the 32)
+    for (int l = t; l < P.N.nl_pad; l += kRowThreadsN) {
+        float s = 0.f;
+        const int d1 = P.dec_start[(l >> 5) + 1];
+        for (int d0 = P.dec_start[l >> 5] + (l & 31); d0 < d1; d0 += 256) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int d = d0 + 32 * k;
+                if (d < d1) s = fmaf(P.dec_w[d], srow[P.dec_m[d]], s);
             }
         }
-    #pragma unroll
-        for (int i = 0; i < kValueRows / 2; ++i) {
-            float x, y;
-            upk(f[i], x, y);
-            if (r0 + 2 * i < rows) P.F[(size_t)(r0 + 2 * i) * P.N.nk_pad + k] = x;
-            if (r0 + 2 * i + 1 < rows) P.F[(size_t)(r0 + 2 * i + 1) * P.N.nk_pad + k] = y;
-        }
+        P.DB[(size_t)row * P.N.nl_pad + l] = s;
     }
 }
 
-// Transposed: the Gaussians from the recorded-energy nodes onto the scattered-
-// energy nodes, 8 (angle, bin) rows per block, a thread per node; the blocks
-// past those form the unscattered part of the back projection, a thread per
-// voxel.
-__global__ void __launch_bounds__(256) k_node_unvalues(const NodeParams P) {
-    extern __shared__ __align__(16) float vb[];   // [nk][8]
-    const int t = threadIdx.x, W = P.N.W;
-    const int rows = P.angles * P.B;
-    const int lt = (P.N.nl + 255) / 256;
+// out[row][x] = sum_y m[y][x] in[row][y] over the band of y each x reaches,
+// for 8 rows and 32 x per block: the warps share the band's y (a run each, the
+// loads of a run in flight together), their sums are added in warp order.  63 us
+// forward and 78 us back for 60 angles, 13 and 14 us for 8.
+__device__ __forceinline__ void band_product(const float* in, int in_stride, const float* m,
+                                             int m_stride, float* out, int out_stride, int rows,
+                                             int r0, int x0, int lo, int hi, float* sh) {
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    float* red = sh;                                   // [warps][8][32]
+    float* st = sh + kValueWarps * kValueRows * 32;    // [y][8]
+    const int per = (hi - lo + kValueWarps - 1) / kValueWarps;
+    const int y0 = min(lo + warp * per, hi), y1 = min(y0 + per, hi);
+    const float* mp = m + x0 + lane;
+    // 16 y at a time, the next 16 matrix entries in flight (the first ones
+    // while the rows are staged, a warp per row)
+    float g[16];
+    auto load = [&](int yb) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) g[k] = yb + k < y1 ? mp[(size_t)(yb + k) * m_stride] : 0.f;
+    };
+    load(y0);
+    const float* src = in + (size_t)(r0 + warp) * in_stride + lo;
+    const int len = r0 + warp < rows ? hi - lo : 0;
+    for (int yb = lane; yb < hi - lo; yb += 256) {
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = yb + 32 * k < len ? src[yb + 32 * k] : 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (yb + 32 * k < hi - lo) st[(yb + 32 * k) * kValueRows + warp] = v[k];
+    }
+    __syncthreads();
+    f32x2 s[kValueRows / 2] = {0ull, 0ull, 0ull, 0ull};
+    for (int yb = y0; yb < y1; yb += 16) {
+        float c[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) c[k] = g[k];
+        if (yb + 16 < y1) load(yb + 16);
+        f32x2 u[kValueRows / 2] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const int y = min(yb + k, y1 - 1);
+            const f32x2 g2 = pk1(c[k]);
+            const float4 d0 = *reinterpret_cast<const float4*>(st + (y - lo) * kValueRows);
+            const float4 d1 = *reinterpret_cast<const float4*>(st + (y - lo) * kValueRows + 4);
+            u[0] = fma2(g2, pk(d0.x, d0.y), u[0]);
+            u[1] = fma2(g2, pk(d0.z, d0.w), u[1]);
+            u[2] = fma2(g2, pk(d1.x, d1.y), u[2]);
+            u[3] = fma2(g2, pk(d1.z, d1.w), u[3]);
+        }
+#pragma unroll
+        for (int i = 0; i < kValueRows / 2; ++i) s[i] = add2(s[i], u[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < kValueRows / 2; ++i) {
+        float x, y;
+        upk(s[i], x, y);
+        red[(warp * kValueRows + 2 * i) * 32 + lane] = x;
+        red[(warp * kValueRows + 2 * i + 1) * 32 + lane] = y;
+    }
+    __syncthreads();
+    static_assert(kValueWarps == kValueRows, "a warp per row in the last step");
+    float v = 0.f;
+#pragma unroll
+    for (int k = 0; k < kValueWarps; ++k) v += red[(k * kValueRows + warp) * 32 + lane];
+    if (r0 + warp < rows) out[(size_t)(r0 + warp) * out_stride + x0 + lane] = v;
+}
+
+// The Gaussians from the scattered-energy nodes onto the recorded-energy nodes.
+__global__ void __launch_bounds__(32 * kValueWarps) k_node_values(const NodeParams P) {
+    extern __shared__ __align__(16) float sh[];
+    const int kt = P.N.nk_pad / 32;
+    const int r0 = blockIdx.x / kt * kValueRows, tile = blockIdx.x % kt;
+    const int2 r = P.l_of_k[tile];
+    band_product(P.DB, P.N.nl_pad, P.g, P.N.nk_pad, P.F, P.N.nk_pad, P.angles * P.B, r0, tile * 32, r.x,
+                 r.y, sh);
+}
+
+// Transposed, for the back projection; the blocks past those form its
+// unscattered part, a thread per voxel.
+__global__ void __launch_bounds__(32 * kValueWarps) k_node_unvalues(const NodeParams P) {
+    extern __shared__ __align__(16) float sh[];
+    const int rows = P.angles * P.B, W = P.N.W;
+    const int lt = P.N.nl_pad / 32;
     const int n_row_blocks = (rows + kValueRows - 1) / kValueRows * lt;
     if ((int)blockIdx.x >= n_row_blocks) {
         const int qb = (P.nq + 255) / 256;
         const int ai = (blockIdx.x - n_row_blocks) / qb;
-        const int q = ((blockIdx.x - n_row_blocks) % qb) * 256 + t;
+        const int q = ((blockIdx.x - n_row_blocks) % qb) * 256 + threadIdx.x;
         if (q >= P.nq) return;
         const int a = P.a0 + ai * P.a_step;
         float s[4] = {0.f, 0.f, 0.f, 0.f};
         const float* cv = P.cv + (size_t)a * P.B * P.nq + q;
         const float* pv = P.PV + (size_t)ai * P.B * W;
-#pragma unroll 8
+#pragma unroll 16
         for (int b = 0; b < P.B; ++b) {
             const float c = cv[(size_t)b * P.nq];
 #pragma unroll
@@ -459,128 +611,163 @@ __global__ void __launch_bounds__(256) k_node_unvalues(const NodeParams P) {
         P.part_prim[(size_t)ai * P.nq_pad + q] = o;
         return;
     }
-    const int r0 = (blockIdx.x / lt) * kValueRows;
-    for (int i = 0; i < kValueRows; ++i)
-        for (int k = t; k < P.N.nk; k += 256)
-            vb[k * kValueRows + i] = r0 + i < rows ? P.V[(size_t)(r0 + i) * P.N.nk_pad + k] : 0.f;
+    const int r0 = blockIdx.x / lt * kValueRows, tile = blockIdx.x % lt;
+    const int2 r = P.k_of_l[tile];
+    band_product(P.V, P.N.nk_pad, P.gt, P.N.nl_pad, P.VG, P.N.nl_pad, rows, r0, tile * 32, r.x, r.y, sh);
+}
+
+// PSI: the rows' values at the direction offsets, a block per row.
+__global__ void __launch_bounds__(256) k_ang_psi(const NodeParams P) {
+    extern __shared__ float srow[];   // [nl_pad]
+    const size_t row = blockIdx.x;
+    for (int l = threadIdx.x; l < P.N.nl_pad; l += 256) srow[l] = P.VG[row * P.N.nl_pad + l];
     __syncthreads();
-    const int l = (blockIdx.x % lt) * 256 + t;
-    if ((l & ~31) >= P.N.nl) return;
-    const int2 r = P.k_of_l[min(l, P.N.nl - 1)];
-    const int lo = __reduce_min_sync(0xffffffffu, r.y > r.x ? r.x : 0x7fffffff);
-    const int hi = __reduce_max_sync(0xffffffffu, r.y);
-    f32x2 f[kValueRows / 2] = {0ull, 0ull, 0ull, 0ull};
-    for (int k0 = lo; k0 < hi; k0 += 32) {
-        f32x2 s[kValueRows / 2] = {0ull, 0ull, 0ull, 0ull};
-        const int k1 = min(k0 + 32, hi);
-#pragma unroll 8
-        for (int k = k0; k < k1; ++k) {
-            const float g = P.gt[(size_t)k * P.N.nl_pad + l];
-            const float4 d0 = *reinterpret_cast<const float4*>(vb + k * kValueRows);
-            const float4 d1 = *reinterpret_cast<const float4*>(vb + k * kValueRows + 4);
-            const f32x2 g2 = pk1(g);
-            s[0] = fma2(g2, pk(d0.x, d0.y), s[0]);
-            s[1] = fma2(g2, pk(d0.z, d0.w), s[1]);
-            s[2] = fma2(g2, pk(d1.x, d1.y), s[2]);
-            s[3] = fma2(g2, pk(d1.z, d1.w), s[3]);
-        }
-#pragma unroll
-        for (int i = 0; i < kValueRows / 2; ++i) f[i] = add2(f[i], s[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < kValueRows / 2; ++i) {
-        float x, y;
-        upk(f[i], x, y);
-        if (r0 + 2 * i < rows) P.VG[(size_t)(r0 + 2 * i) * P.N.nl_pad + l] = x;
-        if (r0 + 2 * i + 1 < rows) P.VG[(size_t)(r0 + 2 * i + 1) * P.N.nl_pad + l] = y;
+    for (int m = threadIdx.x; m < P.N.nm_pad; m += 256) {
+        const float4* w = reinterpret_cast<const float4*>(P.psi_w + (size_t)m * 8);
+        const float4 w0 = w[0], w1 = w[1];
+        const float* v = srow + P.psi_l[m];
+        float s = w0.x * v[0];
+        s = fmaf(w0.y, v[1], s);
+        s = fmaf(w0.z, v[2], s);
+        s = fmaf(w0.w, v[3], s);
+        s = fmaf(w1.x, v[4], s);
+        s = fmaf(w1.y, v[5], s);
+        s = fmaf(w1.z, v[6], s);
+        P.psi[row * P.N.nm_pad + m] = s;
     }
 }
 
-// One CTA per (angle, 32 scatter points, line): PHI of the 32 points [node]
-// [point] in shared memory, then every voxel's sum over the 32 points, a lane
-// per point, each warp every 8th tile of 32 voxels (8 at a time: loads in
-// flight together, the lanes' values added by a butterfly that leaves voxel r
-// in lanes 4 r .. 4 r + 3).
-__global__ void __launch_bounds__(kGatherThreads) k_node_gather(const NodeParams P) {
-    extern __shared__ __align__(16) float phi[];   // [node][32]
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int kWarps = kGatherThreads / 32;
-    const int W = P.N.W;
-    const int w = blockIdx.x % W, pc = (blockIdx.x / W) % P.npc, ai = blockIdx.x / (W * P.npc);
-    const int a = P.a0 + ai * P.a_step;
-    const int nlw = P.N.l_count[w];
-    const int2 br = P.chunk_bins[(size_t)a * P.npc + pc];
-    {
-        const float* cr = P.cs + (((size_t)a * P.npc + pc) * P.B) * kCPad + lane;
-        const float* vg = P.VG + (size_t)ai * P.B * P.N.nl_pad + P.N.l_off[w];
-        for (int l0 = warp * 8; l0 < nlw; l0 += kWarps * 8) {
-            float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll 2
-            for (int b = br.x; b < br.y; ++b) {
-                const float c = cr[(size_t)b * kCPad];
-                const float* v = vg + (size_t)b * P.N.nl_pad + l0;
+// T: a warp per (64 direction nodes, 8 neighbouring scatter points), two nodes a
+// lane; the four warps of a block take neighbouring groups of points on the same
+// nodes, so that one reads PSI from L2 and the others find it in L1.  The
+// launch's angles one after the other, each over the bins the 8 points reach;
+// the points' collimator values, bins and line integrals of a batch of angles
+// are staged in shared memory together, which leaves one load latency (PSI's, 8
+// bins in flight) per angle.  Bound by issue (54 %) and that latency; eight
+// blocks an SM put every warp of the grid on the chip at once: 412 us for 60
+// angles and 54 us for 8 (503 and 66 us with the collimator values read bin by
+// bin; 16 or 4 bins in flight: 426, 468 us; one warp a block: 410 us, but 264
+// instead of 210 us for 15 angles at 3464 voxels).
+constexpr int kBackWarps = 4, kBackTile = 64, kBackAngles = 4;
+constexpr size_t kBackStage = 16 * 1024;
+__global__ void __launch_bounds__(32 * kBackWarps, 8) k_ang_back(const NodeParams P, int tiles, int groups,
+                                                              int batch) {
+    extern __shared__ __align__(16) float sc[];   // [batch][kBackWarps][nbg_max][8]
+    __shared__ float sg[kBackAngles][kBackWarps][kGroup];
+    __shared__ int2 sb[kBackAngles][kBackWarps];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    int tile = blockIdx.x % tiles;
+    const int grp0 = blockIdx.x / tiles * kBackWarps, grp = grp0 + warp;
+    int w = 0;
+    while (tile >= (P.N.n_dir[w] + kBackTile - 1) / kBackTile) {
+        tile -= (P.N.n_dir[w] + kBackTile - 1) / kBackTile;
+        ++w;
+    }
+    const int n = P.N.n_dir[w], nmp = P.N.nm_pad, per = P.N.nbg_max * kGroup;
+    const int nd0 = min(tile * kBackTile + lane, n - 1), nd1 = min(tile * kBackTile + 32 + lane, n - 1);
+    f32x2 acc0[kGroup / 2] = {0ull, 0ull, 0ull, 0ull}, acc1[kGroup / 2] = {0ull, 0ull, 0ull, 0ull};
+    for (int a1 = 0; a1 < P.angles; a1 += batch) {
+        const int na = min(batch, P.angles - a1);
+        __syncthreads();
+        for (int i = t; i < na * kBackWarps * per / 4; i += 32 * kBackWarps) {
+            const int x = i % (per / 4), g = i / (per / 4) % kBackWarps, k = i / (per / 4) / kBackWarps;
+            const int a = P.a0 + (a1 + k) * P.a_step;
+            if (grp0 + g < groups)
+                reinterpret_cast<float4*>(sc)[i] =
+                    reinterpret_cast<const float4*>(P.grp_c)[((size_t)a * groups + grp0 + g) * (per / 4) + x];
+        }
+        for (int i = t; i < na * kBackWarps * kGroup; i += 32 * kBackWarps) {
+            const int j = i % kGroup, g = i / kGroup % kBackWarps, k = i / kGroup / kBackWarps;
+            const int a = P.a0 + (a1 + k) * P.a_step;
+            if (grp0 + g >= groups) continue;
+            sg[k][g][j] = P.gamma[(size_t)a * P.np + max(P.grp_pt[(grp0 + g) * kGroup + j], 0)];
+            if (j == 0) sb[k][g] = P.grp_bins[(size_t)a * groups + grp0 + g];
+        }
+        __syncthreads();
+        if (grp >= groups) continue;
+        for (int k = 0; k < na; ++k) {
+            const int a = P.a0 + (a1 + k) * P.a_step;
+            const int sh = (int)((int64_t)a * n / P.A);
+            const int2 br = sb[k][warp];
+            const float4* c = reinterpret_cast<const float4*>(sc + (size_t)(k * kBackWarps + warp) * per);
+            int d0 = nd0 - sh, d1 = nd1 - sh;
+            if (d0 < 0) d0 += n;
+            if (d1 < 0) d1 += n;
+            const int m0 = P.N.m_off[w] + min(d0, n - d0), m1 = P.N.m_off[w] + min(d1, n - d1);
+            const float mu0 = P.mu[m0], mu1 = P.mu[m1];
+            const float* psi = P.psi + ((size_t)(a1 + k) * P.B + br.x) * nmp;
+            f32x2 s0[kGroup / 2] = {0ull, 0ull, 0ull, 0ull}, s1[kGroup / 2] = {0ull, 0ull, 0ull, 0ull};
+            const int nb = br.y - br.x;
+            for (int b = 0; b < nb; b += 8) {
+                float v0[8], v1[8];
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    if (l0 + i < nlw) acc[i] = fmaf(c, v[i], acc[i]);
+                for (int i = 0; i < 8; ++i) {
+                    const bool on = b + i < nb;
+                    v0[i] = on ? psi[(b + i) * nmp + m0] : 0.f;
+                    v1[i] = on ? psi[(b + i) * nmp + m1] : 0.f;
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    if (b + i >= nb) break;
+                    const float4 ca = c[2 * (b + i)], cb = c[2 * (b + i) + 1];
+                    const f32x2 x0 = pk1(v0[i]), x1 = pk1(v1[i]);
+                    s0[0] = fma2(x0, pk(ca.x, ca.y), s0[0]);
+                    s0[1] = fma2(x0, pk(ca.z, ca.w), s0[1]);
+                    s0[2] = fma2(x0, pk(cb.x, cb.y), s0[2]);
+                    s0[3] = fma2(x0, pk(cb.z, cb.w), s0[3]);
+                    s1[0] = fma2(x1, pk(ca.x, ca.y), s1[0]);
+                    s1[1] = fma2(x1, pk(ca.z, ca.w), s1[1]);
+                    s1[2] = fma2(x1, pk(cb.x, cb.y), s1[2]);
+                    s1[3] = fma2(x1, pk(cb.z, cb.w), s1[3]);
+                }
             }
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if (l0 + i < nlw) phi[(l0 + i) * kPC + lane] = acc[i];
+            for (int i = 0; i < kGroup / 2; ++i) {
+                const float ga = sg[k][warp][2 * i], gb = sg[k][warp][2 * i + 1];
+                acc0[i] = fma2(pk(ex2f(-mu0 * ga), ex2f(-mu0 * gb)), s0[i], acc0[i]);
+                acc1[i] = fma2(pk(ex2f(-mu1 * ga), ex2f(-mu1 * gb)), s1[i], acc1[i]);
+            }
         }
     }
-    __syncthreads();
-    const size_t block = (size_t)3 * W * kQT * kPC;
-    const float* tab = P.tab + ((size_t)(P.slot0 + ai * P.slot_step) * P.nqt * P.npc + pc) * block +
-                       (size_t)w * kQT * kPC + lane;
-    const float* col = phi + lane;
-    float* out = P.part + (size_t)blockIdx.x * P.nq_pad;
-    const int first = P.N.l_first[w] + 3;
-    const unsigned last = (unsigned)(nlw - kTapsL);
-    const float c1 = P.N.cl, c1_lo = P.N.cl_lo;
-    for (int qt = warp; qt < P.nqt; qt += kWarps) {
-        const float* src = tab + (size_t)qt * P.npc * block;
-#pragma unroll 1
-        for (int r0 = 0; r0 < kQT; r0 += 8) {
-            float nl[8], sr[8], v[8];
+    if (grp >= groups) return;
+    float* out = P.T + P.N.n_off[w] + tile * kBackTile + lane;
+    const bool on0 = tile * kBackTile + lane < n, on1 = tile * kBackTile + 32 + lane < n;
 #pragma unroll
-            for (int r = 0; r < 8; ++r) {
-                nl[r] = src[(r0 + r) * kPC];
-                sr[r] = src[(size_t)W * kQT * kPC + (r0 + r) * kPC];
-            }
+    for (int i = 0; i < kGroup; ++i) {
+        const int p = P.grp_pt[grp * kGroup + i];
+        if (p < 0) continue;
+        float x[2], y[2];
+        upk(acc0[i / 2], x[0], x[1]);
+        upk(acc1[i / 2], y[0], y[1]);
+        float* o = out + (size_t)p * P.N.nn;
+        if (on0) o[0] = x[i & 1];
+        if (on1) o[32] = y[i & 1];
+    }
+}
+
+// The paths' values in direction order, a thread per (point, path): the taps
+// of consecutive paths are consecutive nodes.  15 us.
+__global__ void __launch_bounds__(256) k_ang_paths(const NodeParams P) {
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= (int64_t)P.np * P.nq) return;
+    const int p = (int)(i / P.nq);
+    const uint32_t fix = P.fix[i];
+    float v = 0.f;
+    for (int w = 0; w < P.N.W; ++w) {
+        const int n = P.N.n_dir[w];
+        int c;
+        const float s = direction_pos(fix, n, &c);
+        float x[7];
+        lagrange7(s, P.path_b[(size_t)w * P.np * P.nq + i], x);
+        const float* T = P.T + (size_t)p * P.N.nn + P.N.n_off[w];
 #pragma unroll
-            for (int r = 0; r < 8; r += 2) {
-                unsigned i0, i1;
-                const f32x2 s = node_pos2(sr[r], sr[r + 1], c1, c1_lo, first, last, i0, i1);
-                f32x2 c[7];
-                lagrange7(s, pk(ex2f(-nl[r]), ex2f(-nl[r + 1])), c);
-                const float *d0 = col + i0 * kPC, *d1 = col + i1 * kPC;
-                f32x2 acc = mul2(c[0], pk(d0[0], d1[0]));
-#pragma unroll
-                for (int k = 1; k < 7; ++k) acc = fma2(c[k], pk(d0[k * kPC], d1[k * kPC]), acc);
-                upk(acc, v[r], v[r + 1]);
-            }
-            // lanes' sums: after the three exchanges lane keeps voxel (lane >> 2)
-            const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
-            float u[4], x[2], z;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float give = h16 ? v[i] : v[i + 4], keep = h16 ? v[i + 4] : v[i];
-                u[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
-            }
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const float give = h8 ? u[i] : u[i + 2], keep = h8 ? u[i + 2] : u[i];
-                x[i] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
-            }
-            {
-                const float give = h4 ? x[0] : x[1], keep = h4 ? x[1] : x[0];
-                z = keep + __shfl_xor_sync(0xffffffffu, give, 4);
-            }
-            z += __shfl_xor_sync(0xffffffffu, z, 2);
-            z += __shfl_xor_sync(0xffffffffu, z, 1);
-            if ((lane & 3) == 0) out[qt * kQT + r0 + (lane >> 2)] = z;
+        for (int k = 0; k < 7; ++k) {
+            int j = c + k - 3;
+            j = j < 0 ? j + n : j >= n ? j - n : j;
+            v = fmaf(x[k], T[j], v);
         }
     }
+    P.val[i] = v;
 }
 
 struct EventParams {
@@ -645,7 +832,8 @@ __global__ void __launch_bounds__(256) k_node_y(const EventParams P, const uint1
 // the cell's node weights V = sum_j r_j L(E_j) and unscattered weights PV.  A
 // lane forms the values of one event; the events' 12 taps are then added one
 // event per half-warp at a time into the half-warp's own row, 12 lanes one tap
-// each.  The rows are emptied into second sums every 256 events of a warp.
+// each.  In cells of more than 1024 events the rows are emptied into second
+// sums every 256 events of a warp.
 __global__ void __launch_bounds__(32 * kCellWarps) k_node_cells(
     const EventParams P, const int* cell_start, int cell0, const float* energy, const float* weight,
     const uint32_t* perm, float* V, float* PV, double* ll) {
@@ -663,6 +851,7 @@ __global__ void __launch_bounds__(32 * kCellWarps) k_node_cells(
     const size_t cell = blockIdx.x;
     const int e0 = cell_start[cell0 + blockIdx.x], e1 = cell_start[cell0 + blockIdx.x + 1];
     float* out = V + cell * nkp;
+    const bool large = e1 - e0 > 1024;
     if (e0 == e1) {
         for (int k = t; k < nkp; k += 32 * kCellWarps) out[k] = 0.f;
         if (t < W) PV[cell * W + t] = 0.f;
@@ -671,7 +860,9 @@ __global__ void __launch_bounds__(32 * kCellWarps) k_node_cells(
     }
     for (int k = t; k < nkp; k += 32 * kCellWarps) {
         if (P.F) Fs[k] = P.F[cell * nkp + k];
-        for (int i = 0; i < kRows; ++i) acc[i * nkp + k] = tot[i * nkp + k] = 0.f;
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) acc[i * nkp + k] = 0.f;
+        for (int i = 0; large && i < kRows; ++i) tot[i * nkp + k] = 0.f;
     }
     __syncthreads();
     float pv[4] = {0.f, 0.f, 0.f, 0.f};
@@ -728,7 +919,7 @@ __global__ void __launch_bounds__(32 * kCellWarps) k_node_cells(
             if (ev < n_here && tap < kTapsK) mine[kpos[warp][ev] + tap] += wts[warp][ev][tap];
             __syncwarp();
         }
-        if ((++batches & 7) == 0) {
+        if (large && (++batches & 7) == 0) {
             for (int k2 = tap; k2 < nkp; k2 += 16) {
                 tot[mine - acc + k2] += mine[k2];
                 mine[k2] = 0.f;
@@ -749,7 +940,8 @@ __global__ void __launch_bounds__(32 * kCellWarps) k_node_cells(
     __syncthreads();
     for (int k = t; k < nkp; k += 32 * kCellWarps) {
         float s = 0.f;
-        for (int i = 0; i < kRows; ++i) s += tot[i * nkp + k] + acc[i * nkp + k];
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) s += large ? tot[i * nkp + k] + acc[i * nkp + k] : acc[i * nkp + k];
         out[k] = s;
     }
     if (t < W) {
@@ -764,31 +956,49 @@ __global__ void __launch_bounds__(32 * kCellWarps) k_node_cells(
     }
 }
 
-// Voxel sums over the parts (FP64, 32 strands in fixed order) and, with sens,
-// the multiplicative update of lam; else the sums go to num.  One block per
-// 32 voxels.
-__global__ void __launch_bounds__(1024) k_node_update(const float* part, int64_t n_part,
-                                                      const float* part_prim, int n_prim,
-                                                      int nq, int nq_pad, const double* sens,
-                                                      float* lam, double* num) {
-    __shared__ double red[32][33];
-    const int lane = threadIdx.x & 31, strand = threadIdx.x >> 5;
-    const int q = blockIdx.x * 32 + lane;
+// Voxel sums over the scatter points' paths and the angles' unscattered parts
+// (FP64, 128 strands in fixed order) and, with sens, the multiplicative update
+// of lam; else the sums go to num.  One block per 8 voxels: the sums are short
+// (a few points a strand) and bound by load latency, so they want many strands
+// (11 us; 33 us at 3464 voxels, half of the measured copy bandwidth).
+constexpr int kUpdVox = 8, kUpdStrands = 128;
+__global__ void __launch_bounds__(kUpdVox * kUpdStrands) k_node_update(
+    const float* val, const int* path_of, int np, const float* part_prim, int n_prim, int nq,
+    int nq_pad, const double* sens, float* lam, double* num) {
+    __shared__ double red[kUpdStrands][kUpdVox + 1];
+    const int v = threadIdx.x % kUpdVox, strand = threadIdx.x / kUpdVox;
+    const int q = blockIdx.x * kUpdVox + v;
     double s = 0.0;
     if (q < nq) {
-#pragma unroll 4
-        for (int64_t i = strand; i < n_part; i += 32) s += (double)part[(size_t)i * nq_pad + q];
-        for (int i = strand; i < n_prim; i += 32) s += (double)part_prim[(size_t)i * nq_pad + q];
+        for (int p0 = strand; p0 < np; p0 += 8 * kUpdStrands) {
+            int r[8];
+            float x[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int p = p0 + k * kUpdStrands;
+                r[k] = p < np ? path_of[(size_t)p * nq + q] : 0;
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int p = p0 + k * kUpdStrands;
+                x[k] = p < np ? val[(size_t)p * nq + r[k]] : 0.f;
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) s += (double)x[k];
+        }
+        for (int i = strand; i < n_prim; i += kUpdStrands) s += (double)part_prim[(size_t)i * nq_pad + q];
     }
-    red[strand][lane] = s;
-    __syncthreads();
+    red[strand][v] = s;
+    for (int o = kUpdStrands / 2; o > 0; o >>= 1) {
+        __syncthreads();
+        if (strand < o) red[strand][v] += red[strand + o][v];
+    }
     if (strand == 0 && q < nq) {
-        double v = 0.0;
-        for (int i = 0; i < 32; ++i) v += red[i][lane];
+        const double t = red[0][v];
         if (sens)
-            lam[q] = sens[q] > 0.0 ? (float)((double)lam[q] * v / sens[q]) : 0.f;
+            lam[q] = sens[q] > 0.0 ? (float)((double)lam[q] * t / sens[q]) : 0.f;
         else
-            num[q] = v;
+            num[q] = t;
     }
 }
 
@@ -809,6 +1019,8 @@ __global__ void __launch_bounds__(1024) k_node_loglik(const double* ll, int n_ll
     if (t == 0) *out = red[0];
 }
 
+// ------------------------------------------------------------------ set-up
+
 // Bins a chunk of 32 scatter points reaches: those whose run overlaps it.
 __global__ void k_chunk_bins(const int2* crange, int B, int npc, int2* chunk_bins, int* most) {
     const int a = blockIdx.y, pc = blockIdx.x * blockDim.x + threadIdx.x;
@@ -825,6 +1037,123 @@ __global__ void k_chunk_bins(const int2* crange, int B, int npc, int2* chunk_bin
     atomicMax(most, max(hi - lo, 0));
 }
 
+// Place of each point in an angle's order, and its line integral to the
+// detector in FP32.
+__global__ void k_point_tables(const int* inv, const double* g_p, int np, int* rank, float* gamma) {
+    const int a = blockIdx.y, i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= np) return;
+    rank[(size_t)a * np + inv[(size_t)a * np + i]] = i;
+    gamma[(size_t)a * np + i] = (float)g_p[(size_t)a * np + i];
+}
+
+// Bins the 8 points of a group reach.
+__global__ void k_group_bins(const int2* crange, const int* rank, const int* grp_pt, int B, int np,
+                             int groups, int2* grp_bins, int* most) {
+    const int a = blockIdx.y, g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= groups) return;
+    int lo = B, hi = 0;
+    for (int b = 0; b < B; ++b) {
+        const int2 r = crange[(size_t)a * B + b];
+        bool any = false;
+        for (int i = 0; i < kGroup; ++i) {
+            const int p = grp_pt[g * kGroup + i];
+            if (p < 0) continue;
+            const int k = rank[(size_t)a * np + p];
+            any |= k >= r.x && k < r.y;
+        }
+        if (any) {
+            lo = min(lo, b);
+            hi = b + 1;
+        }
+    }
+    grp_bins[(size_t)a * groups + g] = lo < hi ? make_int2(lo, hi) : make_int2(0, 0);
+    atomicMax(most, max(hi - lo, 0));
+}
+
+__global__ void k_group_values(const float* cs, const int* rank, const int* grp_pt,
+                               const int2* grp_bins, int B, int np, int npc, int groups, int nbg_max,
+                               float* grp_c) {
+    const int a = blockIdx.y;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)groups * nbg_max * kGroup) return;
+    const int k = (int)(i % kGroup), b = (int)(i / kGroup % nbg_max), g = (int)(i / kGroup / nbg_max);
+    const int2 br = grp_bins[(size_t)a * groups + g];
+    const int p = grp_pt[g * kGroup + k];
+    float v = 0.f;
+    if (p >= 0 && br.x + b < br.y) {
+        const int r = rank[(size_t)a * np + p];
+        v = cs[(((size_t)a * npc + r / kPC) * B + br.x + b) * kCPad + r % kPC];
+    }
+    grp_c[(size_t)a * groups * nbg_max * kGroup + i] = v;
+}
+
+// Direction from voxel q to point p in 2^-32 turns; pair p nq + q.
+__global__ void k_pair_direction(ModelConst m, const int* q_pix, const int* p_cell, uint32_t* fix,
+                                 uint32_t* idx) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)m.np * m.nq) return;
+    const int p = (int)(i / m.nq), q = (int)(i % m.nq);
+    const int pix = q_pix[q], c = p_cell[p];
+    const double dx = ((c % m.S) + 0.5) * m.f - ((pix % m.n) + 0.5);
+    const double dy = ((c / m.S) + 0.5) * m.f - ((pix / m.n) + 0.5);
+    double t = (dx == 0.0 && dy == 0.0) ? 0.0 : atan2(dy, dx) * 0.15915494309189533577;   // / 2 pi
+    t -= floor(t);
+    fix[i] = (uint32_t)(uint64_t)(t * 4294967296.0);
+    idx[i] = (uint32_t)i;
+}
+
+__global__ void k_pair_points(const uint32_t* idx, int64_t n, int nq, uint32_t* key) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) key[i] = idx[i] / (uint32_t)nq;
+}
+
+// The sorted paths of every point: direction, voxel, place and, per line, the
+// weight B = alpha mu_0 rho_p A_p / d exp(-mu_0 gamma_qp) / K (0 for voxels in
+// the point's own cell).
+__global__ void k_pair_fill(ModelConst m, const uint32_t* order, const uint32_t* fix0,
+                            const int* q_pix, const int* p_cell, const double* p_rho,
+                            const double* g_qp, const double* d_qp, const double* mu_line,
+                            uint32_t* fix, int* path_q, int* path_of, float* path_b) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t n = (int64_t)m.np * m.nq;
+    if (i >= n) return;
+    const uint32_t src = order[i];
+    const int p = (int)(src / (uint32_t)m.nq), q = (int)(src % (uint32_t)m.nq);
+    fix[i] = fix0[src];
+    path_q[i] = q;
+    path_of[(size_t)p * m.nq + q] = (int)(i - (int64_t)p * m.nq);
+    const int pix = q_pix[q];
+    const bool own = ((pix / m.n) / m.f) * m.S + (pix % m.n) / m.f == p_cell[p];
+    const size_t k = (size_t)q * m.np + p;
+    for (int w = 0; w < m.W; ++w)
+        path_b[(size_t)w * n + i] =
+            own ? 0.f
+                : (float)(m.alpha[w] * mu_line[w] * p_rho[p] * m.cell_area / d_qp[k] *
+                          exp(-mu_line[w] * g_qp[k]) / m.kn_norm[w]);
+}
+
+// First path of each point at every line's centre nodes 0 .. n, and the count.
+__global__ void k_path_starts(const NodeConst N, const uint32_t* fix, int np, int nq, int* start) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)np * N.start_ints) return;
+    const int p = (int)(i / N.start_ints);
+    int node = (int)(i % N.start_ints), w = 0;
+    while (node >= N.n_dir[w] + 2) {
+        node -= N.n_dir[w] + 2;
+        ++w;
+    }
+    const int n = N.n_dir[w];
+    const uint32_t* f = fix + (size_t)p * nq;
+    int lo = 0, hi = nq;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        int c;
+        direction_pos(f[mid], n, &c);
+        if (c < node) lo = mid + 1; else hi = mid;
+    }
+    start[i] = lo;
+}
+
 // Shared-memory opt-in of the node kernels, once per device.
 int node_kernel_attrs() {
     static std::atomic<unsigned long long> done{0};
@@ -833,42 +1162,90 @@ int node_kernel_attrs() {
     const unsigned long long bit = 1ull << (dev & 63);
     if (done.load() & bit) return LMMEW_OK;
     LMMEW_CUDA(cudaDeviceGetAttribute(&cap, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    cudaFuncAttributes fa;
-    LMMEW_CUDA(cudaFuncGetAttributes(&fa, k_node_spread));
-    LMMEW_CUDA(cudaFuncSetAttribute(k_node_spread, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    cap - (int)fa.sharedSizeBytes));
-    LMMEW_CUDA(cudaFuncSetAttribute(k_node_gather, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    cap - 1024));
-    LMMEW_CUDA(cudaFuncSetAttribute(k_node_values, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    cap - 1024));
+    for (auto k : {k_node_values, k_node_bins, k_ang_psi})
+        LMMEW_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, cap - 4096));
     LMMEW_CUDA(cudaFuncSetAttribute(k_node_unvalues, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    cap - 1024));
+                                    cap - 4096));
+    LMMEW_CUDA(cudaFuncSetAttribute(k_ang_back, cudaFuncAttributeMaxDynamicSharedMemorySize, cap - 4096));
     LMMEW_CUDA(cudaFuncSetAttribute(k_node_cells, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    64 * 1024));
+                                    80 * 1024));
     done.fetch_or(bit);
     return LMMEW_OK;
 }
 
+NodeParams node_params(const lm_handle* h, int a0, int a_step, int angles) {
+    const ModelConst& m = h->mc;
+    NodeParams P{};
+    P.N = h->nodes;
+    P.a0 = a0;
+    P.a_step = a_step;
+    P.angles = angles;
+    P.A = m.A;
+    P.B = m.B;
+    P.nq = m.nq;
+    P.np = m.np;
+    P.npc = m.npc;
+    P.nq_pad = m.nqt * kQT;
+    const NodeTables& t = h->node_tables;
+    P.g = t.g;
+    P.gt = t.gt;
+    P.k_of_l = t.k_of_l;
+    P.l_of_k = t.l_of_k;
+    P.chunk_bins = t.chunk_bins;
+    P.cs = h->d_cs;
+    P.crange = h->d_crange;
+    P.inv = h->d_inv;
+    P.gamma = t.gamma;
+    P.mu = t.mu;
+    P.psi_l = t.psi_l;
+    P.psi_w = t.psi_w;
+    P.dec_start = t.dec_start;
+    P.dec_m = t.dec_m;
+    P.dec_w = t.dec_w;
+    P.fix = t.fix;
+    P.path_q = t.path_q;
+    P.path_of = t.path_of;
+    P.path_b = t.path_b;
+    P.path_start = t.path_start;
+    P.grp_pt = t.grp_pt;
+    P.grp_bins = t.grp_bins;
+    P.grp_c = h->d_node_groups;
+    P.cv = h->d_cv;
+    P.prim = h->d_prim;
+    return P;
+}
+
+// Shared memory of band_product for at most `band` nodes.
+size_t band_smem(int band) {
+    return sizeof(float) * ((size_t)kValueWarps * kValueRows * 32 + (size_t)kValueRows * band);
+}
+
 }  // namespace
 
-// Nodes of the model's energies and the Gaussians between them.  The route
-// exists for the square-root energy resolution, with energy classes on, when
-// the node sums of 32 scatter points fit shared memory and one angle's sums
-// the static scratch of lm_forward_noalloc (so that call takes the same route).
+// The nodes of the model and everything the route reads.  It exists for the
+// square-root energy resolution, up to 4 lines and node counts and pair tables
+// (12 + 4 W bytes per voxel and scatter point) of sane sizes; other models keep
+// the rows.
 int build_nodes(lm_handle* h) {
     const ModelConst& m = h->mc;
     NodeConst& N = h->nodes;
+    NodeTables& T = h->node_tables;
     h->node_route = 0;
     N = NodeConst{};
-    if (m.np == 0 || m.W > 4 || m.expo != -0.5) return LMMEW_OK;
-    const double f2s = 1.0 / (2.0 * sqrt(2.0 * log(2.0)));
-    const double kappa = m.fwhm_frac * sqrt(m.e_ref) * f2s;   // sigma = kappa sqrt(E)
+    const int64_t pairs = (int64_t)m.np * m.nq;
+    if (m.np == 0 || m.W > 4 || m.expo != -0.5 || pairs >= (int64_t(1) << 31)) return LMMEW_OK;
+    const double pi = 3.14159265358979323846, log2e = 1.4426950408889634, me = 510.99895;
+    const double kappa = m.fwhm_frac * sqrt(m.e_ref) / (2.0 * sqrt(2.0 * log(2.0)));   // sigma = kappa sqrt(E)
     auto t_of = [&](double e) { return 2.0 * sqrt(e) / kappa; };
+    auto mu_of = [&](double e) {
+        if (m.n_knots == 1) return m.knot_mu[0];
+        int s = 0;
+        while (s < m.n_knots - 2 && e >= m.knot_e[s + 1]) ++s;
+        return m.knot_mu[s] + (e - m.knot_e[s]) * m.knot_slope[s];
+    };
     N.W = m.W;
-    const double cl = kPerUnitL * 2.0 * sqrt(0.5 * 1.4426950408889634) / (kappa * kappa);
+    // recorded energies
     const double ck = kPerUnitK * 2.0 / kappa;
-    N.cl = (float)cl;
-    N.cl_lo = (float)(cl - (double)N.cl);
     N.ck = (float)ck;
     N.ck_lo = (float)(ck - (double)N.ck);
     double e_lo = 1e300, e_hi = 0.0;
@@ -881,162 +1258,284 @@ int build_nodes(lm_handle* h) {
     N.k_first = (int)floor(t_of(e_lo) * kPerUnitK) - 6;
     N.nk = (int)floor(t_hi) + 7 - N.k_first + 1;
     N.nk_pad = (N.nk + 31) & ~31;
-    int most = 0;
+    // scattered energies and directions of each line
     for (int w = 0; w < m.W; ++w) {
-        const double eb = m.line_e[w] / (1.0 + 2.0 * m.line_e[w] / 510.99895);
-        const double u0 = t_of(eb) * kPerUnitL, u1 = t_of(m.line_e[w]) * kPerUnitL;
+        const double e0 = m.line_e[w], k0 = e0 / me, eb = e0 / (1.0 + 2.0 * k0);
+        const double u0 = t_of(eb) * kPerUnitL, u1 = t_of(e0) * kPerUnitL;
         if (!(u1 < 1.0e6)) return LMMEW_OK;
         N.l_first[w] = (int)floor(u0) - 4;
         N.l_count[w] = (int)ceil(u1) + 4 - N.l_first[w] + 1;
         if (N.l_first[w] < 1) return LMMEW_OK;
-        N.l_off[w] = N.nl;
-        N.nl += N.l_count[w];
-        most = std::max(most, N.l_count[w]);
+        N.l_off[w] = N.nl;               // (lines start at multiples of 8 nodes)
+        N.nl += (N.l_count[w] + 7) & ~7;
+        // 18 nodes per sigma where E'(x) is steepest (7 taps: 1e-8 of a term),
+        // 29 for a line whose E' crosses an attenuation knot, and there enough
+        // that exp(-mu gamma) over 10 cm bends by 4e-4 per node at most
+        auto slope = [&](double x) {     // |dE'/dx|
+            const double e = e0 / (1.0 + k0 * (1.0 - cos(x)));
+            return e * e / e0 * k0 * sin(x);
+        };
+        double steep = 0.0, want = 0.0;
+        for (int i = 1; i < 512; ++i) {
+            const double x = pi * i / 512, e = e0 / (1.0 + k0 * (1.0 - cos(x)));
+            steep = std::max(steep, slope(x) / (kappa * sqrt(e)));
+        }
+        want = 2.0 * pi * steep * 18.0;
+        for (int k = 1; k + 1 < m.n_knots; ++k) {
+            const double e = m.knot_e[k], bend = fabs(m.knot_slope[k] - m.knot_slope[k - 1]);
+            if (!(e > eb && e < e0) || bend == 0.0) continue;
+            const double x = acos(1.0 - (e0 / e - 1.0) / k0);
+            want = std::max(want, std::max(2.0 * pi * steep * 29.0, 2.0 * pi * 10.0 * bend * slope(x) / 4e-4));
+        }
+        want = std::max(want, 32.0);
+        if (!(want < 16384.0) || m.A > 16384) return LMMEW_OK;
+        N.n_dir[w] = ((int)ceil(want) + m.A - 1) / m.A * m.A;
+        N.n_off[w] = N.nn;
+        N.nn += N.n_dir[w];
+        N.m_count[w] = N.n_dir[w] / 2 + 1;
+        N.m_off[w] = N.nm_pad;
+        N.nm_pad += (N.m_count[w] + 31) & ~31;
+        N.start_ints += N.n_dir[w] + 2;
+        line_reach(h, w, &N.reach_lo[w], &N.reach_hi[w]);
     }
     N.nl_pad = (N.nl + 31) & ~31;
-    int dev = 0, max_smem = 0;
-    LMMEW_CUDA(cudaGetDevice(&dev));
-    LMMEW_CUDA(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    const size_t per_warp = 4 * kStageBytes + (size_t)most * kPC * 4;
-    N.spread_warps = (int)std::min<size_t>(kSpreadWarpsMax, (size_t)(max_smem - 1024) / per_warp);
-    N.spread_smem = (int)(N.spread_warps * per_warp);
-    N.gather_smem = most * kPC * 4;
-    if (N.spread_warps < 1 || N.gather_smem > 200 * 1024 || N.nl > 6000 || N.nk > 1024) return LMMEW_OK;
-    LMMEW_CUDA(cudaMalloc(&h->d_chunk_bins, sizeof(int2) * ((size_t)m.A * m.npc + 1)));
-    int* d_most = reinterpret_cast<int*>(h->d_chunk_bins + (size_t)m.A * m.npc);
-    LMMEW_CUDA(cudaMemset(d_most, 0, sizeof(int)));
-    k_chunk_bins<<<dim3((m.npc + 31) / 32, m.A), 32>>>(h->d_crange, m.B, m.npc, h->d_chunk_bins, d_most);
-    ++h->launches;
-    LMMEW_CUDA(cudaGetLastError());
-    LMMEW_CUDA(cudaMemcpy(&N.nb_max, d_most, sizeof(int), cudaMemcpyDeviceToHost));
-    if (N.nb_max < 1) return LMMEW_OK;
-    // one angle (with the voxel values) fits lm_forward_noalloc's array
-    if (node_angle_bytes(h) + sizeof(float) * (size_t)m.nq + 4096 > (size_t(16) << 20)) return LMMEW_OK;
-    for (int w = 0; w < m.W; ++w) line_reach(h, w, &N.reach_lo[w], &N.reach_hi[w]);
-    // bands of the Gaussian matrix
-    auto e_l = [&](int w, int i) { const double x = 0.5 * kappa * (N.l_first[w] + i) / kPerUnitL; return x * x; };
-    auto e_k = [&](int k) { const double x = 0.5 * kappa * (N.k_first + k) / kPerUnitK; return x * x; };
-    std::vector<int2> bands((size_t)N.nl + (size_t)m.W * N.nk_pad, make_int2(0, 0));
+    if (N.nl > 6000 || N.nk > 1024 || N.nn > 32768 || (int64_t)m.np * N.nn >= (int64_t(1) << 31))
+        return LMMEW_OK;
+    const size_t pair_bytes = (12 + 4 * (size_t)m.W) * (size_t)pairs;
+    size_t free_b = 0, total_b = 0;
+    LMMEW_CUDA(cudaMemGetInfo(&free_b, &total_b));
+    if (2 * pair_bytes > free_b / 4) return LMMEW_OK;
+
+    // host tables: offsets' attenuation and taps (also by node l), bands
+    std::vector<float> mu(N.nm_pad, 0.f), psi_w((size_t)8 * N.nm_pad, 0.f), dec_w;
+    std::vector<int> psi_l(N.nm_pad, 0), dec_start(N.nl_pad / 32 + 1, 0), dec_m, taps(N.nl_pad, 0);
+    for (int w = 0; w < m.W; ++w) {
+        const double e0 = m.line_e[w], k0 = e0 / me;
+        for (int i = 0; i < N.m_count[w]; ++i) {
+            const double c = cos(2.0 * pi * i / N.n_dir[w]), r = 1.0 / (1.0 + k0 * (1.0 - c)), e = e0 * r;
+            const double kn = r * r * (r + 1.0 / r - (1.0 - c * c));
+            const double f = kn / (sqrt(2.0 * pi) * kappa * sqrt(e));
+            const double u = t_of(e) * kPerUnitL - N.l_first[w];
+            const int c0 = (int)floor(u + 0.5);
+            const double s = u - c0;
+            const int o = N.m_off[w] + i;
+            mu[o] = (float)(mu_of(e) * log2e);
+            psi_l[o] = N.l_off[w] + c0 - 3;
+            for (int k = 0; k < 7; ++k) {
+                double v = f;
+                for (int j = 0; j < 7; ++j)
+                    if (j != k) v *= (s - (j - 3)) / (double)(k - j);
+                psi_w[(size_t)8 * o + k] = (float)v;
+                ++taps[psi_l[o] + k];
+            }
+        }
+    }
+    for (int t = 0; t < N.nl_pad / 32; ++t)
+        dec_start[t + 1] =
+            dec_start[t] + 32 * *std::max_element(taps.begin() + 32 * t, taps.begin() + 32 * (t + 1));
+    dec_m.assign(dec_start[N.nl_pad / 32], 0);
+    dec_w.assign(dec_m.size(), 0.f);
+    std::fill(taps.begin(), taps.end(), 0);
+    for (int w = 0; w < m.W; ++w)
+        for (int i = 0; i < N.m_count[w]; ++i)
+            for (int k = 0; k < 7; ++k) {
+                const int o = N.m_off[w] + i, l = psi_l[o] + k;
+                const int d = dec_start[l >> 5] + 32 * taps[l]++ + (l & 31);
+                dec_m[d] = o;
+                dec_w[d] = psi_w[(size_t)8 * o + k];
+            }
+    const int lt = N.nl_pad / 32, kt = N.nk_pad / 32;
+    std::vector<int2> bands((size_t)lt + kt, make_int2(1 << 30, 0));
     int2* k_of_l = bands.data();
-    int2* l_of_k = k_of_l + N.nl;
+    int2* l_of_k = k_of_l + lt;
     for (int w = 0; w < m.W; ++w)
         for (int i = 0; i < N.l_count[w]; ++i) {
-            const double e = e_l(w, i), s = kBandSigmas * kappa * sqrt(e);
-            int2 r = make_int2(N.nk, 0);
-            for (int k = 0; k < N.nk; ++k)
-                if (fabs(e_k(k) - e) <= s) {
-                    r.x = std::min(r.x, k);
-                    r.y = k + 1;
-                    int2& q = l_of_k[(size_t)w * N.nk_pad + k];
-                    if (q.y == 0) q.x = N.l_off[w] + i;
-                    q.y = N.l_off[w] + i + 1;
-                }
-            if (r.y == 0) r.x = 0;
-            k_of_l[N.l_off[w] + i] = r;
+            // |E_k - E_l| <= 9 sigma_l between the nodes just outside the band
+            const int l = N.l_off[w] + i;
+            const double x = 0.5 * kappa * (N.l_first[w] + i) / kPerUnitL, e = x * x;
+            const double s = kBandSigmas * kappa * x;
+            const double v0 = e > s ? t_of(e - s) * kPerUnitK : -1e9;
+            const int k0 = std::max(0, (int)floor(v0) - N.k_first);
+            const int k1 = std::min(N.nk, (int)ceil(t_of(e + s) * kPerUnitK) - N.k_first + 1);
+            if (k0 >= k1) continue;
+            k_of_l[l / 32].x = std::min(k_of_l[l / 32].x, k0);
+            k_of_l[l / 32].y = std::max(k_of_l[l / 32].y, k1);
+            for (int k = k0 / 32; k <= (k1 - 1) / 32; ++k) {
+                l_of_k[k].x = std::min(l_of_k[k].x, l);
+                l_of_k[k].y = std::max(l_of_k[k].y, l + 1);
+            }
         }
-    const size_t gm = (size_t)N.nl_pad * N.nk_pad;
-    if (cudaMalloc(&h->d_node_g, 2 * gm * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&h->d_node_band, bands.size() * sizeof(int2)) != cudaSuccess) {
-        cudaGetLastError();
-        return set_error(LMMEW_ERR_OOM, "cannot allocate the energy nodes");
+    for (int2& r : bands)
+        if (r.y == 0) r.x = 0;
+
+    // one device region; the host tables lie together at its start
+    // 8 neighbouring points at a time (cells of 4 x 2), which reach fewer bins
+    // together than 8 in a row
+    std::vector<int> grp_pt;
+    {
+        std::vector<int> cell(m.np);
+        LMMEW_CUDA(cudaMemcpy(cell.data(), h->d_p_cell, sizeof(int) * m.np, cudaMemcpyDeviceToHost));
+        std::vector<std::pair<int64_t, int>> key(m.np);
+        for (int p = 0; p < m.np; ++p) {
+            const int x = cell[p] % m.S, y = cell[p] / m.S;
+            key[p] = {((int64_t)(y / 2) * (m.S / 4 + 1) + x / 4) * 8 + (y % 2) * 4 + x % 4, p};
+        }
+        std::sort(key.begin(), key.end());
+        for (const auto& k : key) grp_pt.push_back(k.second);
+        while (grp_pt.size() % kGroup) grp_pt.push_back(-1);
     }
-    LMMEW_CUDA(cudaMemset(h->d_node_g, 0, 2 * gm * sizeof(float)));
-    LMMEW_CUDA(cudaMemcpy(h->d_node_band, bands.data(), bands.size() * sizeof(int2),
-                          cudaMemcpyHostToDevice));
-    const int total = N.nl * N.nk_pad;
-    k_node_matrix<<<(total + 255) / 256, 256>>>(N, kappa, h->d_node_g, h->d_node_g + gm);
-    ++h->launches;
+    const int groups = (int)grp_pt.size() / kGroup;
+    const size_t gm = (size_t)N.nl_pad * N.nk_pad;
+    size_t host_bytes = 0;
+    int* d_most = nullptr;
+    auto layout = [&](char* p) {
+        char* base = p;
+        T.mu = bump<float>(p, mu.size());
+        T.psi_w = bump<float>(p, psi_w.size());
+        T.dec_w = bump<float>(p, dec_w.size());
+        T.psi_l = bump<int>(p, psi_l.size());
+        T.dec_start = bump<int>(p, dec_start.size());
+        T.dec_m = bump<int>(p, dec_m.size());
+        T.grp_pt = bump<int>(p, grp_pt.size());
+        T.k_of_l = bump<int2>(p, bands.size());
+        T.l_of_k = T.k_of_l + lt;
+        d_most = bump<int>(p, 2);
+        host_bytes = (size_t)(p - base);
+        T.g = bump<float>(p, gm);
+        T.gt = bump<float>(p, gm);
+        T.chunk_bins = bump<int2>(p, (size_t)m.A * m.npc);
+        T.grp_bins = bump<int2>(p, (size_t)m.A * groups);
+        T.gamma = bump<float>(p, (size_t)m.A * m.np);
+        T.rank = bump<int>(p, (size_t)m.A * m.np);
+        T.path_start = bump<int>(p, (size_t)m.np * N.start_ints);
+        T.fix = bump<uint32_t>(p, pairs);
+        T.path_q = bump<int>(p, pairs);
+        T.path_of = bump<int>(p, pairs);
+        T.path_b = bump<float>(p, (size_t)m.W * pairs);
+        return (size_t)(p - base) + 256;
+    };
+    const size_t bytes = layout(nullptr);
+    const size_t sort_bytes = 4 * bump_bytes(4 * (size_t)pairs) + bump_bytes(pair_hist_bytes(pairs));
+    struct Temp {
+        void* p = nullptr;
+        ~Temp() { cudaFree(p); }
+    } temp;
+    if (cudaMalloc(&h->d_node_tables, bytes) != cudaSuccess || cudaMalloc(&temp.p, sort_bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return LMMEW_OK;                 // no room: the rows
+    }
+    layout((char*)h->d_node_tables);
+    std::vector<char> blob(host_bytes, 0);
+    auto put = [&](const void* dst, const void* src, size_t n) {
+        std::memcpy(blob.data() + ((const char*)dst - (const char*)h->d_node_tables), src, n);
+    };
+    put(T.mu, mu.data(), 4 * mu.size());
+    put(T.psi_w, psi_w.data(), 4 * psi_w.size());
+    put(T.dec_w, dec_w.data(), 4 * dec_w.size());
+    put(T.psi_l, psi_l.data(), 4 * psi_l.size());
+    put(T.dec_start, dec_start.data(), 4 * dec_start.size());
+    put(T.dec_m, dec_m.data(), 4 * dec_m.size());
+    put(T.grp_pt, grp_pt.data(), 4 * grp_pt.size());
+    put(T.k_of_l, bands.data(), 8 * bands.size());
+    LMMEW_CUDA(cudaMemcpy(h->d_node_tables, blob.data(), host_bytes, cudaMemcpyHostToDevice));
+
+    k_node_matrix<<<(unsigned)((gm + 255) / 256), 256>>>(N, kappa, T.g, T.gt);
+    k_chunk_bins<<<dim3((m.npc + 31) / 32, m.A), 32>>>(h->d_crange, m.B, m.npc, T.chunk_bins, d_most);
+    k_point_tables<<<dim3((m.np + 127) / 128, m.A), 128>>>(h->d_inv, h->d_gp, m.np, T.rank, T.gamma);
+    k_group_bins<<<dim3((groups + 31) / 32, m.A), 32>>>(h->d_crange, T.rank, T.grp_pt, m.B, m.np, groups,
+                                                        T.grp_bins, d_most + 1);
+    // the paths of each point by direction: stable sorts by direction, then point
+    char* tp = (char*)temp.p;
+    uint32_t* kin = bump<uint32_t>(tp, pairs);
+    uint32_t* kout = bump<uint32_t>(tp, pairs);
+    uint32_t* vin = bump<uint32_t>(tp, pairs);
+    uint32_t* vout = bump<uint32_t>(tp, pairs);
+    uint32_t* hist = bump<uint32_t>(tp, pair_hist_bytes(pairs) / 4);
+    const unsigned pb = (unsigned)((pairs + 255) / 256);
+    uint32_t* fix0 = reinterpret_cast<uint32_t*>(T.path_b);   // (free until the fill) unsorted directions
+    k_pair_direction<<<pb, 256>>>(m, h->d_q_pix, h->d_p_cell, fix0, vin);
+    LMMEW_CUDA(cudaMemcpyAsync(kin, fix0, 4 * (size_t)pairs, cudaMemcpyDeviceToDevice, 0));
+    int rc = sort_pairs(h, pairs, 32, kin, kout, vin, vout, hist, 0);
+    if (rc != LMMEW_OK) return rc;
+    k_pair_points<<<pb, 256>>>(vin, pairs, m.nq, kin);
+    int bits = 1;
+    while (bits < 32 && ((uint32_t)(m.np - 1) >> bits) != 0) ++bits;
+    rc = sort_pairs(h, pairs, bits, kin, kout, vin, vout, hist, 0);
+    if (rc != LMMEW_OK) return rc;
+    LMMEW_CUDA(cudaMemcpyAsync(kin, fix0, 4 * (size_t)pairs, cudaMemcpyDeviceToDevice, 0));
+    k_pair_fill<<<pb, 256>>>(m, vin, kin, h->d_q_pix, h->d_p_cell, h->d_p_rho, h->d_gqp, h->d_dqp,
+                             h->d_mu_line, T.fix, T.path_q, T.path_of, T.path_b);
+    k_path_starts<<<(unsigned)(((int64_t)m.np * N.start_ints + 127) / 128), 128>>>(N, T.fix, m.np, m.nq,
+                                                                                  T.path_start);
     LMMEW_CUDA(cudaGetLastError());
-    LMMEW_CUDA(cudaDeviceSynchronize());
-    h->node_route = 1;
-    return node_kernel_attrs();
+    int most[2] = {0, 0};
+    LMMEW_CUDA(cudaMemcpy(most, d_most, sizeof(most), cudaMemcpyDeviceToHost));
+    N.nb_max = std::max(most[0], 1);
+    N.nbg_max = std::max(most[1], 1);
+    if (N.nbg_max > 1024) return LMMEW_OK;   // (its staging would not fit shared memory)
+    const size_t per_angle = (size_t)groups * N.nbg_max * kGroup;
+    if (cudaMalloc(&h->d_node_groups, sizeof(float) * per_angle * m.A) != cudaSuccess) {
+        cudaGetLastError();
+        return LMMEW_OK;
+    }
+    k_group_values<<<dim3((unsigned)((per_angle + 255) / 256), m.A), 256>>>(
+        h->d_cs, T.rank, T.grp_pt, T.grp_bins, m.B, m.np, m.npc, groups, N.nbg_max, h->d_node_groups);
+    h->launches += 9;
+    LMMEW_CUDA(cudaGetLastError());
+    LMMEW_CUDA(cudaDeviceSynchronize());   // (the sort's scratch goes)
+    rc = node_kernel_attrs();
+    if (rc == LMMEW_OK) h->node_route = 1;
+    return rc;
 }
 
 size_t node_angle_bytes(const lm_handle* h) {
     const NodeConst& N = h->nodes;
-    return bump_bytes(sizeof(float) * (size_t)h->mc.npc * N.nb_max * N.nl_pad) +
+    return bump_bytes(sizeof(float) * (size_t)h->mc.npc * N.nb_max * N.nm_pad) +
+           bump_bytes(sizeof(float) * (size_t)h->mc.B * N.nl_pad) +
            bump_bytes(sizeof(float) * (size_t)h->mc.B * N.nk_pad) +
            bump_bytes(sizeof(float) * (size_t)h->mc.B * N.W);
 }
 
-namespace {
-
-NodeParams node_params(const lm_handle* h, int a0, int a_step, int angles) {
-    const ModelConst& m = h->mc;
-    const NodeConst& N = h->nodes;
-    NodeParams P{};
-    P.N = N;
-    P.tab = h->d_tab;
-    P.a0 = a0;
-    P.a_step = a_step;
-    P.angles = angles;
-    P.B = m.B;
-    P.nq = m.nq;
-    P.nqt = m.nqt;
-    P.npc = m.npc;
-    P.nq_pad = m.nqt * kQT;
-    P.g = h->d_node_g;
-    P.gt = h->d_node_g + (size_t)N.nl_pad * N.nk_pad;
-    P.k_of_l = h->d_node_band;
-    P.l_of_k = h->d_node_band + N.nl;
-    P.chunk_bins = h->d_chunk_bins;
-    P.cs = h->d_cs;
-    P.crange = h->d_crange;
-    P.cv = h->d_cv;
-    P.prim = h->d_prim;
-    P.status = h->d_status;
-    return P;
-}
-
-// The slot of the block's first angle in the table buffer and the step
-// between slots (streamed tables: the block is built first).
-int table_slots(lm_handle* h, int a0, int a_step, int angles, int* slot0, int* step,
-                cudaStream_t st) {
-    *slot0 = a0;
-    *step = a_step;
-    if (!h->tab_slots) return LMMEW_OK;
-    const int rc = stream_tables(h, a0, a_step, angles, st);
+// The image on the direction nodes of every scatter point.
+int node_spread(lm_handle* h, const float* lam_v, float* H, cudaStream_t st) {
+    NodeParams P = node_params(h, 0, 1, 0);
+    P.lam = lam_v;
+    P.H = H;
+    int tiles = 0;
+    for (int w = 0; w < P.N.W; ++w) tiles += (P.N.n_dir[w] + kSpreadOut - 1) / kSpreadOut;
+    int rc = prof_start(h, st);
     if (rc != LMMEW_OK) return rc;
-    *slot0 = (a0 - h->tab_a0) / h->tab_astep;
-    *step = angles > 1 ? a_step / h->tab_astep : 0;
-    return LMMEW_OK;
+    const int units = h->mc.np * tiles;
+    k_ang_spread<<<(unsigned)((units + kSpreadWarps - 1) / kSpreadWarps), 32 * kSpreadWarps, 0, st>>>(
+        P, tiles, units);
+    ++h->launches;
+    LMMEW_CUDA(cudaGetLastError());
+    return prof_stop(h, (double)h->mc.W * h->mc.nq * h->mc.np, st);
 }
 
-}  // namespace
-
-// DB, F and the unscattered sums of angles a0 + i a_step, i < angles.
-int node_forward(lm_handle* h, const float* lam_v, int a0, int a_step, int angles, float* dbp,
-                 float* F, float* Pr, cudaStream_t st) {
+// F and the unscattered sums of angles a0 + i a_step, i < angles.
+int node_forward(lm_handle* h, const float* lam_v, const float* H, int a0, int a_step, int angles,
+                 float* dbp, float* DB, float* F, float* Pr, cudaStream_t st) {
     if (angles <= 0) return LMMEW_OK;
     const ModelConst& m = h->mc;
     const NodeConst& N = h->nodes;
-    // angles in blocks of the streamed table buffer (all of them if resident)
-    const int per = h->tab_slots ? h->tab_slots : angles;
-    for (int i = 0; i < angles; i += per) {
-        const int cnt = std::min(per, angles - i);
-        NodeParams P = node_params(h, a0 + i * a_step, a_step, cnt);
-        int rc = table_slots(h, P.a0, a_step, cnt, &P.slot0, &P.slot_step, st);
-        if (rc != LMMEW_OK) return rc;
-        P.tab = h->d_tab;
-        P.lam = lam_v;
-        P.dbp = dbp + (size_t)i * m.npc * N.nb_max * N.nl_pad;
-        rc = prof_start(h, st);
-        if (rc != LMMEW_OK) return rc;
-        k_node_spread<<<(unsigned)(cnt * m.npc * m.W), 32 * N.spread_warps, N.spread_smem, st>>>(P);
-        ++h->launches;
-        LMMEW_CUDA(cudaGetLastError());
-        rc = prof_stop(h, (double)cnt * m.W * m.nq * m.np, st);
-        if (rc != LMMEW_OK) return rc;
-    }
     NodeParams P = node_params(h, a0, a_step, angles);
     P.lam = lam_v;
+    P.H = const_cast<float*>(H);
     P.dbp = dbp;
+    P.DB = DB;
     P.F = F;
     P.Pr = Pr;
+    constexpr int kTile = kOffThreads * kOffPer;
+    int tiles = 0;
+    for (int w = 0; w < N.W; ++w) tiles += (N.m_count[w] + kTile - 1) / kTile;
+    k_ang_bins<<<(unsigned)(tiles * m.npc * angles), kOffThreads, 0, st>>>(P, tiles);
     const int rows = angles * m.B;
-    const int blocks = (rows + kValueRows - 1) / kValueRows + (rows * m.W + 11) / 12;
-    k_node_values<<<(unsigned)blocks, 384, sizeof(float) * kValueRows * N.nl, st>>>(P);
-    ++h->launches;
+    k_node_bins<<<(unsigned)(rows + (rows * m.W + kRowThreadsN / 32 - 1) / (kRowThreadsN / 32)), kRowThreadsN,
+                  sizeof(float) * N.nm_pad, st>>>(P);
+    k_node_values<<<(unsigned)((rows + kValueRows - 1) / kValueRows * (N.nk_pad / 32)),
+                    32 * kValueWarps, band_smem(N.nl_pad), st>>>(P);
+    h->launches += 3;
     LMMEW_CUDA(cudaGetLastError());
     return LMMEW_OK;
 }
@@ -1056,53 +1555,48 @@ int node_cells(lm_handle* h, int angles, const int* cell_start, int cell0, const
     return LMMEW_OK;
 }
 
-// Back projection of the node weights of angles a0 + i a_step: parts of the
-// voxel sums per (angle, 32 points, line) and, unscattered, per angle.
+// Back projection of the node weights of angles a0 + i a_step: the paths' values
+// and the unscattered part of every angle.
 int node_back(lm_handle* h, int a0, int a_step, int angles, const float* V, const float* PV,
-              float* VG, float* part, float* part_prim, cudaStream_t st) {
-    if (angles <= 0) return LMMEW_OK;
+              float* VG, float* psi, float* T, float* val, float* part_prim, cudaStream_t st) {
     const ModelConst& m = h->mc;
     const NodeConst& N = h->nodes;
-    {
-        NodeParams P = node_params(h, a0, a_step, angles);
-        P.V = V;
-        P.PV = PV;
-        P.VG = VG;
-        P.part_prim = part_prim;
-        const int rows = angles * m.B;
-        const int blocks = (rows + kValueRows - 1) / kValueRows * ((N.nl + 255) / 256) +
-                           angles * ((m.nq + 255) / 256);
-        k_node_unvalues<<<(unsigned)blocks, 256, sizeof(float) * kValueRows * N.nk, st>>>(P);
-        ++h->launches;
-        LMMEW_CUDA(cudaGetLastError());
+    NodeParams P = node_params(h, a0, a_step, angles);
+    P.V = V;
+    P.PV = PV;
+    P.VG = VG;
+    P.psi = psi;
+    P.T = T;
+    P.val = val;
+    P.part_prim = part_prim;
+    const int rows = angles * m.B;
+    const int blocks = (rows + kValueRows - 1) / kValueRows * (N.nl_pad / 32) +
+                       angles * ((m.nq + 255) / 256);
+    if (rows > 0) {
+        k_node_unvalues<<<(unsigned)blocks, 32 * kValueWarps, band_smem(N.nk_pad), st>>>(P);
+        k_ang_psi<<<(unsigned)rows, 256, sizeof(float) * N.nl_pad, st>>>(P);
     }
-    const int per = h->tab_slots ? h->tab_slots : angles;
-    for (int i = 0; i < angles; i += per) {
-        const int cnt = std::min(per, angles - i);
-        NodeParams P = node_params(h, a0 + i * a_step, a_step, cnt);
-        int rc = table_slots(h, P.a0, a_step, cnt, &P.slot0, &P.slot_step, st);
-        if (rc != LMMEW_OK) return rc;
-        P.tab = h->d_tab;
-        P.VG = VG + (size_t)i * m.B * N.nl_pad;
-        P.part = part + (size_t)i * m.npc * m.W * P.nq_pad;
-        rc = prof_start(h, st);
-        if (rc != LMMEW_OK) return rc;
-        k_node_gather<<<(unsigned)(cnt * m.npc * m.W), kGatherThreads, N.gather_smem, st>>>(P);
-        ++h->launches;
-        LMMEW_CUDA(cudaGetLastError());
-        rc = prof_stop(h, (double)cnt * m.W * m.nq * m.np, st);
-        if (rc != LMMEW_OK) return rc;
-    }
-    return LMMEW_OK;
+    int tiles = 0;
+    for (int w = 0; w < N.W; ++w) tiles += (N.n_dir[w] + kBackTile - 1) / kBackTile;
+    const int groups = (m.np + kGroup - 1) / kGroup;
+    const size_t one = sizeof(float) * kBackWarps * (size_t)N.nbg_max * kGroup;   // staged per angle
+    const int batch = (int)std::max<size_t>(1, std::min<size_t>(kBackAngles, kBackStage / one));
+    k_ang_back<<<(unsigned)(tiles * ((groups + kBackWarps - 1) / kBackWarps)), 32 * kBackWarps,
+                 batch * one, st>>>(P, tiles, groups, batch);
+    int rc = prof_start(h, st);
+    if (rc != LMMEW_OK) return rc;
+    k_ang_paths<<<(unsigned)(((int64_t)m.np * m.nq + 255) / 256), 256, 0, st>>>(P);
+    h->launches += 4;
+    LMMEW_CUDA(cudaGetLastError());
+    return prof_stop(h, (double)m.W * m.nq * m.np, st);
 }
 
-// The voxel sums of `angles` angles' parts: with sens the update of lam, else
-// into num.
-int node_update(lm_handle* h, int angles, const float* part, const float* part_prim,
+// The voxel sums: with sens the update of lam, else into num.
+int node_update(lm_handle* h, int angles, const float* val, const float* part_prim,
                 const double* sens, float* lam, double* num, cudaStream_t st) {
     const ModelConst& m = h->mc;
-    k_node_update<<<(m.nq + 31) / 32, 1024, 0, st>>>(part, (int64_t)angles * m.npc * m.W, part_prim,
-                                                     angles, m.nq, m.nqt * kQT, sens, lam, num);
+    k_node_update<<<(m.nq + kUpdVox - 1) / kUpdVox, kUpdVox * kUpdStrands, 0, st>>>(
+        val, h->node_tables.path_of, m.np, part_prim, angles, m.nq, m.nqt * kQT, sens, lam, num);
     ++h->launches;
     LMMEW_CUDA(cudaGetLastError());
     return LMMEW_OK;

@@ -1,4 +1,4 @@
-"""Projections of dense event lists through energy nodes (csrc/nodes.cu).
+"""Projections of dense event lists through angle and energy nodes (csrc/nodes.cu).
 
 Against the FP64 oracle at the parity tolerances, and against the row kernel's
 route (every line evaluated: energy classes off), whose FP32 sums it must
@@ -55,8 +55,8 @@ def _case(name, over, n_events, seed=3):
 
 
 def _paths(gpu):
-    """Path weights one projection of the node route evaluates."""
-    return gpu.n_angles * gpu.n_lines * gpu.nq * gpu.np_scatter
+    """Path weights one projection of the node route visits."""
+    return gpu.n_lines * gpu.nq * gpu.np_scatter
 
 
 @pytest.mark.parametrize("name,over,n", CASES)
