@@ -651,10 +651,35 @@ __device__ bool tc_network(const TcShared& S, const TcGroup& G, uint32_t& phase,
     return true;
 }
 
-// Network outputs for n BF16 input rows; with kTrain also the pre-activations
-// of the three hidden layers, BF16 [3][n][128] at z (the training forward).
-template <bool kTrain>
-__global__ void __launch_bounds__(kTcThreads, 1) k_tc_forward(Weights w, const bf16* x, int64_t n,
+// 8 consecutive inputs of a row as BF16; FP32 rows that do not start on 16
+// bytes (vec false) are read one by one.
+__device__ __forceinline__ uint4 load_inputs8(const bf16* x, bool) {
+    return *reinterpret_cast<const uint4*>(x);
+}
+__device__ __forceinline__ uint4 load_inputs8(const float* x, bool vec) {
+    float v[8];
+    if (vec) {
+        const float4 a = reinterpret_cast<const float4*>(x)[0], b = reinterpret_cast<const float4*>(x)[1];
+        v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+        v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = x[i];
+    }
+    uint4 r;
+    __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&r);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) h[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+    return r;
+}
+
+// Network outputs for n input rows, BF16 or FP32 (rounded to BF16 on the way to
+// shared memory: a pass of their own over 500 000 rows cost 19 of 120 us); with
+// kTrain also the pre-activations of the three hidden layers, BF16 [3][n][128]
+// at z (the training forward).  Bound by issue of the GELU epilogue; a row is
+// one cache line, which each thread asks into L2 a tile ahead.
+template <bool kTrain, typename X>
+__global__ void __launch_bounds__(kTcThreads, 1) k_tc_forward(Weights w, const X* x, int64_t n,
                                                               float* out, int* status,
                                                               bf16* z = nullptr) {
     extern __shared__ unsigned char smem_raw[];
@@ -662,18 +687,21 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_forward(Weights w, const b
     const uint32_t tmem_base = tc_setup(S, w);
     const TcGroup G = tc_group(S, tmem_base);
     const float b4 = w.p[kOffB4];
+    const bool vec = (reinterpret_cast<uintptr_t>(x) & 15) == 0;
     uint32_t phase = 0;
     const int64_t n_tiles = (n + 127) / 128;
     // tiles group-major across the CTAs, so that few tiles still use many SMs
-    for (int64_t t = (int64_t)G.g * gridDim.x + blockIdx.x; t < n_tiles;
-         t += (int64_t)gridDim.x * kTcGroups) {
+    const int64_t step = (int64_t)gridDim.x * kTcGroups;
+    for (int64_t t = (int64_t)G.g * gridDim.x + blockIdx.x; t < n_tiles; t += step) {
         const int64_t base = t * 128;
         for (int k = G.gt; k < 128 * 4; k += kGrpThreads) {   // 128 rows x 4 chunks of 8 inputs
             const int r = k & 127, j = k >> 7;
             uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (base + r < n) v = *reinterpret_cast<const uint4*>(x + (size_t)(base + r) * kIn + j * 8);
+            if (base + r < n) v = load_inputs8(x + (size_t)(base + r) * kIn + j * 8, vec);
             *reinterpret_cast<uint4*>(S.base + G.h + sw_chunk(r, 0, j)) = v;
         }
+        if (sizeof(X) == 4 && base + step * 128 + G.gt < n)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(x + (size_t)(base + step * 128 + G.gt) * kIn));
         tc_input_constants(S, G);
         fence_async_smem();
         group_sync(G.g);
@@ -1168,9 +1196,9 @@ int surrogate_kernel_attrs() {
     LMMEW_CUDA(cudaGetDevice(&dev));
     const unsigned long long bit = 1ull << (dev & 63);
     if (done.load() & bit) return LMMEW_OK;
-    LMMEW_CUDA(cudaFuncSetAttribute(mlp::k_tc_forward<false>,
+    LMMEW_CUDA(cudaFuncSetAttribute(mlp::k_tc_forward<false, float>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp::kTcSmem));
-    LMMEW_CUDA(cudaFuncSetAttribute(mlp::k_tc_forward<true>,
+    LMMEW_CUDA(cudaFuncSetAttribute(mlp::k_tc_forward<true, bf16>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp::kTcSmem));
     LMMEW_CUDA(cudaFuncSetAttribute(mlp::k_surrogate_rows,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp::kTcSmem));
@@ -1384,10 +1412,20 @@ int sm_count() {
     return count > 0 ? count : 1;
 }
 
-// Full-batch gradient of mean squared error over n samples of BF16 inputs
-// xb; grad (device) receives dL/dp.  Optionally the loss (host).
-int gradient(lm_surrogate* s, const bf16* xb, const float* t, const float* v, int64_t n,
-             double* loss, cudaStream_t st) {
+int to_bf16_inputs(const float* x, int64_t n, bf16* xb, cudaStream_t st) {
+    M::k_to_bf16<<<(unsigned)((n * M::kIn + 255) / 256), 256, 0, st>>>(x, n * M::kIn, xb);
+    LMMEW_CUDA(cudaGetLastError());
+    return LMMEW_OK;
+}
+
+// Full-batch gradient of mean squared error over n samples of BF16 inputs xb
+// (or, with xb NULL, of FP32 inputs x, rounded into the scratch); grad (device)
+// receives dL/dp.  Optionally the loss (host).  The rounded inputs lie in the
+// object's scratch with the rest: an allocation of their own, freed after a
+// synchronisation, and a copy of the gradient took 230 of the 344 us of a call
+// with 16 384 samples.
+int gradient(lm_surrogate* s, const float* x, const bf16* xb, const float* t, const float* v, int64_t n,
+             float* grad, double* loss, cudaStream_t st) {
     const int64_t n_cta = (n + M::kTile - 1) / M::kTile;
     const int64_t npad = n_cta * M::kTile;
     size_t off = 0;
@@ -1405,11 +1443,17 @@ int gradient(lm_surrogate* s, const bf16* xb, const float* t, const float* v, in
     const size_t o_pb3 = take(sizeof(float) * n_cta * M::kHid);
     const size_t o_po = take(sizeof(float) * n_cta * (M::kHid + 1));
     const size_t o_mse = take(sizeof(double) * 256);
+    const size_t o_x = take(xb ? 0 : sizeof(bf16) * (size_t)n * M::kIn);
     int rc = ensure_scratch(s, off);
     if (rc != LMMEW_OK) return rc;
     rc = set_attrs();
     if (rc != LMMEW_OK) return rc;
     char* base = (char*)s->scratch;
+    if (!xb) {
+        rc = to_bf16_inputs(x, n, (bf16*)(base + o_x), st);
+        if (rc != LMMEW_OK) return rc;
+        xb = (const bf16*)(base + o_x);
+    }
     float* out = (float*)(base + o_out);
     bf16* z = (bf16*)(base + o_z);
     bf16* d3 = (bf16*)(base + o_d3);
@@ -1419,7 +1463,7 @@ int gradient(lm_surrogate* s, const bf16* xb, const float* t, const float* v, in
     // forward on the tensor cores, keeping the hidden pre-activations
     // one 128-sample tile per group; as many CTAs as SMs allow
     const int fwd_grid = (int)std::min<int64_t>(n_cta, sm_count());
-    M::k_tc_forward<true><<<fwd_grid, M::kTcThreads, M::kTcSmem, st>>>(w, xb, n, out, s->status, z);
+    M::k_tc_forward<true, bf16><<<fwd_grid, M::kTcThreads, M::kTcSmem, st>>>(w, xb, n, out, s->status, z);
     M::k_back_out<<<(unsigned)n_cta, M::kThreads, 0, st>>>(s->p, out, t, v, z + 2 * n * M::kHid, n,
                                                           1.f / (float)n, d3, (float*)(base + o_po));
     // hidden layers 3, 2, 1 on the tensor cores
@@ -1431,13 +1475,13 @@ int gradient(lm_surrogate* s, const bf16* xb, const float* t, const float* v, in
     M::k_tc_back_layer<M::kIn><<<(unsigned)n_cta, 128, M::BackTc<M::kIn>::kSmem, st>>>(
         d1, nullptr, xb, s->W1, n, (float*)(base + o_pw1), (float*)(base + o_pb1), nullptr,
         s->status);
+    double* mse = (double*)(base + o_mse);
+    if (loss) M::k_mse<<<64, 256, 0, st>>>(out, t, v, n, mse);   // (before grad is written)
     M::k_reduce_grad<<<(M::kParams + 255) / 256, 256, 0, st>>>(
         (float*)(base + o_pw1), (float*)(base + o_pb1), (float*)(base + o_pw2), (float*)(base + o_pb2),
-        (float*)(base + o_pw3), (float*)(base + o_pb3), (float*)(base + o_po), (int)n_cta, s->grad);
+        (float*)(base + o_pw3), (float*)(base + o_pb3), (float*)(base + o_po), (int)n_cta, grad);
     LMMEW_CUDA(cudaGetLastError());
     if (loss) {
-        double* mse = (double*)(base + o_mse);
-        M::k_mse<<<64, 256, 0, st>>>(out, t, v, n, mse);
         double host[64];
         LMMEW_CUDA(cudaMemcpyAsync(host, mse, sizeof(host), cudaMemcpyDeviceToHost, st));
         LMMEW_CUDA(cudaStreamSynchronize(st));
@@ -1445,15 +1489,6 @@ int gradient(lm_surrogate* s, const bf16* xb, const float* t, const float* v, in
         for (int i = 0; i < 64; ++i) sum += host[i];
         *loss = sum / (double)n;
     }
-    return LMMEW_OK;
-}
-
-int to_bf16_inputs(lm_surrogate* s, const float* x, int64_t n, bf16** xb, size_t extra_off,
-                   cudaStream_t st) {
-    (void)s;
-    M::k_to_bf16<<<(unsigned)((n * M::kIn + 255) / 256), 256, 0, st>>>(x, n * M::kIn, *xb);
-    LMMEW_CUDA(cudaGetLastError());
-    (void)extra_off;
     return LMMEW_OK;
 }
 
@@ -1558,17 +1593,20 @@ int lm_surrogate_forward(lm_surrogate* s, const float* x, int64_t n, float* out,
     if (!s || (n > 0 && (!x || !out))) return set_error(LMMEW_ERR_INVALID_ARG, "NULL argument");
     if (n <= 0) return LMMEW_OK;
     cudaStream_t st = (cudaStream_t)stream;
-    int rc = ensure_scratch(s, sizeof(bf16) * (size_t)n * M::kIn + 256);
+    int rc = set_attrs();
     if (rc != LMMEW_OK) return rc;
-    rc = set_attrs();
-    if (rc != LMMEW_OK) return rc;
-    bf16* xb = (bf16*)s->scratch;
-    rc = to_bf16_inputs(s, x, n, &xb, 0, st);
-    if (rc != LMMEW_OK) return rc;
+    const size_t in_bytes = sizeof(float) * (size_t)n * M::kIn;
+    const uintptr_t xa = (uintptr_t)x, oa = (uintptr_t)out;
+    if (xa < oa + sizeof(float) * (size_t)n && oa < xa + in_bytes) {   // outputs over the inputs
+        rc = ensure_scratch(s, in_bytes);
+        if (rc != LMMEW_OK) return rc;
+        LMMEW_CUDA(cudaMemcpyAsync(s->scratch, x, in_bytes, cudaMemcpyDeviceToDevice, st));
+        x = (const float*)s->scratch;
+    }
     M::Weights w{s->W1, s->W2, s->W3, s->p};
     const int64_t tiles = (n + 127) / 128;
     const unsigned grid = (unsigned)std::min<int64_t>((tiles + M::kTcGroups - 1) / M::kTcGroups, sm_count());
-    M::k_tc_forward<false><<<grid, M::kTcThreads, M::kTcSmem, st>>>(w, xb, n, out, s->status);
+    M::k_tc_forward<false, float><<<grid, M::kTcThreads, M::kTcSmem, st>>>(w, x, n, out, s->status);
     LMMEW_CUDA(cudaGetLastError());
     return LMMEW_OK;
 }
@@ -1579,19 +1617,8 @@ int lm_surrogate_gradient(lm_surrogate* s, const float* x, const float* target,
     if (!s || !x || !target || !grad_out || n <= 0)
         return set_error(LMMEW_ERR_INVALID_ARG, "bad argument");
     cudaStream_t st = (cudaStream_t)stream;
-    bf16* xb = nullptr;
-    if (cudaMalloc(&xb, sizeof(bf16) * (size_t)n * M::kIn) != cudaSuccess) {
-        cudaGetLastError();
-        return set_error(LMMEW_ERR_OOM, "cannot allocate the BF16 inputs");
-    }
-    int rc = to_bf16_inputs(s, x, n, &xb, 0, st);
-    if (rc == LMMEW_OK) rc = gradient(s, xb, target, weight, n, loss_out, st);
-    if (rc == LMMEW_OK &&
-        cudaMemcpyAsync(grad_out, s->grad, sizeof(float) * M::kParams, cudaMemcpyDeviceToDevice,
-                        st) != cudaSuccess)
-        rc = set_error(LMMEW_ERR_CUDA, "gradient copy");
+    const int rc = gradient(s, x, nullptr, target, weight, n, grad_out, loss_out, st);
     cudaStreamSynchronize(st);
-    cudaFree(xb);
     return rc;
 }
 
@@ -1620,7 +1647,7 @@ int lm_surrogate_train(lm_surrogate* s, const float* x, const float* target, int
         cudaFree(xall); cudaFree(xb); cudaFree(tb); cudaFree(idx); cudaFree(vall); cudaFree(vb);
         return set_error(LMMEW_ERR_OOM, "cannot allocate training buffers");
     }
-    int rc = to_bf16_inputs(s, x, n, &xall, 0, st);
+    int rc = to_bf16_inputs(x, n, xall, st);
     if (weighted) M::k_train_weights<<<1, 1024, 0, st>>>(target, n, weight_power, vall);
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     for (int k = 0; k < steps && rc == LMMEW_OK; ++k) {
@@ -1629,7 +1656,7 @@ int lm_surrogate_train(lm_surrogate* s, const float* x, const float* target, int
         M::k_gather_batch_rows<<<(batch * (M::kIn / 8) + 255) / 256, 256, 0, st>>>(
             xall, target, vall, idx, batch, xb, tb, vb);
         double loss = 0.0;
-        rc = gradient(s, xb, tb, vb, batch, loss_history ? &loss : nullptr, st);
+        rc = gradient(s, nullptr, xb, tb, vb, batch, s->grad, loss_history ? &loss : nullptr, st);
         if (rc != LMMEW_OK) break;
         if (loss_history) loss_history[k] = loss;
         s->step += 1;
