@@ -47,14 +47,18 @@
  *     lm_osem_batch and the surrogate scatter models read the event counts
  *     back once per call;
  *   - a handle serves one stream at a time;
- *   - dense event lists are projected through energy nodes: the exact model's
- *     forward and back projections and LM-OSEM take, instead of one row per
- *     event, sums on energy nodes whose cost does not grow with the events
- *     (the same model to FP32 rounding; lm_forward and lm_backproject from 8
+ *   - dense event lists are projected through nodes: the exact model's forward
+ *     and back projections and LM-OSEM take, instead of one row per event, sums
+ *     on direction and energy nodes whose cost hardly grows with the events
+ *     (the same model to FP32 rounding; lm_forward and lm_backproject from 2
  *     events per angle, lm_osem and lm_osem_batch from 120 per angle and
  *     realisation).  The route needs up to 4 lines, the square-root energy
  *     resolution (exponent -1/2), the FP32 form and energy pruning on;
  *     everything else goes through the rows;
+ *   - reconstructions of two iterations or more that go through the rows keep
+ *     their scatter rows from the first iteration for the later ones, in the
+ *     handle's scratch, when the rows of the whole call take at most 16 GiB
+ *     and half of the free memory (the results are the same bits);
  *   - there is no CPU fallback: every step runs in this library's kernels.
  *
  * Images are n*n arrays in raster order [iy*n + ix]; pixel (ix, iy) has its
@@ -235,7 +239,7 @@ int lm_backproject(lm_handle* h, const lm_events* events, const float* weight,
  * (Eq. lll_med without J log T - log J!).  Resuming with the image returned
  * by an earlier call and the next (start_iter, start_subset) reproduces an
  * uninterrupted run bit for bit.  The row kernel's launch shape (event lists
- * below the energy nodes' density) is chosen by the autotuner described at
+ * below the nodes' density) is chosen by the autotuner described at
  * lm_batch_tuning before the first sub-iteration.
  * Errors: as lm_forward. */
 int lm_osem(lm_handle* h, const lm_events* events, int n_subsets, int n_iters,
@@ -276,7 +280,7 @@ int lm_set_scatter_precision(lm_handle* h, int precision);
  * events: HOST array of n_real lm_events (device pointers inside); images:
  * DEVICE float[n_real][n*n], lambda^0 in, lambda out; loglik: NULL or DEVICE
  * double[n_real][n_iters*n_subsets].  Realisations dense enough for the
- * energy nodes run through them one after the other, as lm_osem would.  Every
+ * nodes run through them one after the other, as lm_osem would.  Every
  * realisation's result equals lm_osem's on its own events bit for bit while each subset's events (all
  * realisations together) fit one row block; beyond that the back
  * projection's event chunks break at row-block edges and results agree to
@@ -468,12 +472,13 @@ const char* lm_last_error(void);
  * library, not part of the paper's method).  While enabled, CUDA events are
  * recorded on the caller's stream around every launch of the fused
  * system-matrix row kernel or, for dense event lists, of the two kernels that
- * visit the paths of the energy nodes.  lm_profile_read synchronises those events and
+ * visit the paths (forward, back).  lm_profile_read synchronises those events and
  * writes out5[0] = total row-kernel time in ms, out5[1] = row-kernel
  * launches, out5[2] = exponentials those launches evaluated for real
  * (event, voxel) pairs -- one per path term whose collimator factor is not
- * an exact zero -- counted on the device, or path weights the energy nodes
- * evaluated (one per angle, line, voxel and scatter point), out5[3] = system-matrix elements
+ * an exact zero -- counted on the device, or path weights of the node
+ * route (one per line, voxel and scatter point and launch, whatever the
+ * number of angles and events), out5[3] = system-matrix elements
  * (events x support voxels),
  * out5[4] = kernels of every kind this handle launched (counted whether or
  * not timing is enabled); then it resets the counters.

@@ -86,6 +86,29 @@ def test_projections_match_rows_and_oracle(name, over, n):
     gpu.close()
 
 
+@pytest.mark.parametrize("name", ["tiny_8", "small_24"])
+@pytest.mark.parametrize("less", [0, 1])
+def test_either_side_of_two_events_per_angle(name, less):
+    n = 2 * preset(name).n_angles - less
+    sc, ph, ev, lam, wt, gpu, dev = _case(name, {}, n)
+    x, wv = torch.from_numpy(lam).cuda(), torch.from_numpy(wt).cuda()
+    gpu.profile_enable(True)
+    y = gpu.forward(dev, x)
+    assert (gpu.profile_read()["terms"] == _paths(gpu)) == (less == 0)
+    gpu.profile_enable(False)
+    bp = gpu.backproject(dev, wv).double()
+    out = torch.empty_like(y)
+    gpu.forward_noalloc(dev, x, out)
+    assert torch.equal(out, y)
+    gpu.set_energy_pruning(False)
+    y_rows, bp_rows = gpu.forward(dev, x).double(), gpu.backproject(dev, wv).double()
+    assert float(((y.double() - y_rows) / y_rows).abs().max()) < ROUTE_RTOL
+    on = bp_rows != 0
+    assert bool((bp[~on] == 0).all())
+    assert float(((bp - bp_rows)[on] / bp_rows[on]).abs().max()) < ROUTE_RTOL
+    gpu.close()
+
+
 @pytest.mark.parametrize("name,over,n", CASES)
 def test_reconstruction_matches_the_row_route_and_resumes(name, over, n):
     sc, ph, ev, lam, wt, gpu, dev = _case(name, over, n, seed=5)
