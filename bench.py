@@ -1,13 +1,14 @@
 #!/usr/bin/env python
 """Benchmark of the LM-MEW OSEM hot path on GB300.
 
-One step = one full LM-OSEM iteration (every subset: system-matrix rows
-computed on the fly, forward projection, ratio, back projection, update) over
-the 64x64 study-scale workload (300k events, 60 angles, 64 bins, 64x64
-scatter grid, 3 emission lines, 8 subsets), through the C ABI.  The K timed
-steps are K iterations of one lm_osem call (the events are sorted once per
-call); the end-to-end measure makes one call per step, with that step's host
-copies.
+One step = one full LM-OSEM iteration (every subset: forward projection through
+the on-the-fly system model, ratio, back projection, update) over the 64x64
+study-scale workload (300k events, 60 angles, 64 bins, 64x64 scatter grid, 3
+emission lines, 8 subsets), through the C ABI.  Each timed step is an lm_osem
+call of one iteration (its event sort included), after a write larger than L2
+that is not timed; the end-to-end measure adds that step's host copies.  This
+event density goes through the direction and energy nodes, which form the
+projections of the same system-matrix elements without forming each element.
 
 Metric: system-matrix elements per second (events x support voxels per
 step / step time), plus seconds per OSEM iteration.  With --gpus N under
@@ -137,18 +138,11 @@ def measured_peaks():
         return None
 
 
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the
-# current k_row revision on this workload.  Measured on the small case
-# `--case row_rows` (60 000 events of subset 0's 8 angles, rows stored as
-# lm_osem does, 64-event tiles): 217 606 144 B read (the 8 angles' path
-# tables) + 175 658 496 B written (the row block), in a one-launch capture;
-# scaled to one OSEM launch of this workload by angles for the reads (7.5 of
-# 8) and by events for the writes (37 500 of 60 000).  Emptied whenever
-# k_row or the tables it streams change until the counters are taken again.
-ROW_TRAFFIC_BYTES_PER_LAUNCH = {"lmmew_64": 204_005_760 + 109_786_560}
+# Written before each timed step: four times L2 (129 MB).
+L2_FLUSH_BYTES = 512 << 20
 
 # Exponential (MUFU ex2) issue rate of one GB300 SM per clock.  The roofline
-# of the exact path is the SFU rate: every path term needs one ex2.
+# of the rows is the SFU rate: every path term needs one ex2.
 EX2_PER_SM_PER_CLK = 32
 
 
@@ -293,20 +287,22 @@ def run_e2e(model, ev, img, sc, n_sub, it, steps, stream, barrier, dist):
     img2 = img.clone()
     barrier()
     torch.cuda.synchronize()
-    f0 = torch.cuda.Event(enable_timing=True)
-    f1 = torch.cuda.Event(enable_timing=True)
-    f0.record(stream)
-    for _ in range(steps):
+    spans = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True))
+             for _ in range(steps)]
+    flush = torch.empty(L2_FLUSH_BYTES, dtype=torch.uint8, device="cuda")
+    for f0, f1 in spans:
+        flush.zero_()                          # not timed
+        f0.record(stream)
         d_ang.copy_(h_ang, non_blocking=True)
         d_bin.copy_(h_bin, non_blocking=True)
         d_en.copy_(h_en, non_blocking=True)
         model.osem(dev2, img2, n_sub, it + 1, start_iter=it)
         h_img.copy_(img2, non_blocking=True)
+        f1.record(stream)
         it += 1
-    f1.record(stream)
     torch.cuda.synchronize()
     barrier()
-    ms_e2e = max_over_ranks(f0.elapsed_time(f1), dist, "cuda")
+    ms_e2e = max_over_ranks(sum(f0.elapsed_time(f1) for f0, f1 in spans), dist, "cuda")
     h2d = h_ang.numel() * 2 + h_bin.numel() * 2 + h_en.numel() * 4
     d2h = h_img.numel() * 4
 
@@ -855,18 +851,21 @@ def run_gpu(args, rank, local_rank, world):
     torch.cuda.synchronize()
     clocks.start()
     stream = torch.cuda.current_stream()
-    e0 = torch.cuda.Event(enable_timing=True)
-    e1 = torch.cuda.Event(enable_timing=True)
-    e0.record(stream)
-    # the K timed steps are K LM-OSEM iterations of one lm_osem call, as a
-    # reconstruction runs them (the events are sorted once per call)
-    model.osem(dev, img, n_sub, it + args.steps, start_iter=it)
-    it += args.steps
-    e1.record(stream)
+    spans = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True))
+             for _ in range(args.steps)]
+    flush = torch.empty(L2_FLUSH_BYTES, dtype=torch.uint8, device="cuda")
+    for e0, e1 in spans:
+        flush.zero_()                          # not timed
+        e0.record(stream)
+        model.osem(dev, img, n_sub, it + 1, start_iter=it, check=False)
+        e1.record(stream)
+        it += 1
     torch.cuda.synchronize()
     barrier()
     clk = clocks.stop()
-    ms = e0.elapsed_time(e1)
+    model.check()
+    ms = sum(e0.elapsed_time(e1) for e0, e1 in spans)
+    del flush
     prof = model.profile_read()
     model.profile_enable(False)
     row_tuning = model.batch_tuning()           # the launch shape the timed steps ran
@@ -891,17 +890,41 @@ def run_gpu(args, rank, local_rank, world):
     peak = ex2_peak(sm_count, sm_max)
     achieved = prof["terms"] / (prof["ms"] / 1e3) if prof["ms"] > 0 else 0.0
     probe = lm.probe_ex2_rate()          # measured exponential rate of this GPU
+    # the rows are launched (and their shape tuned) only below the nodes' density
+    on_nodes = not row_tuning["tuned"]
+    if on_nodes:
+        # each sub-iteration reads a path's direction, voxel and W factors in
+        # either projection and writes and reads its back-projected value
+        step_bytes = n_sub * nq * model.np_scatter * (2 * (8 + 4 * model.n_lines) + 8)
+        hbm = float(peaks.get("hbm_gbs") or 6800.0)
+        gbs = step_bytes * args.steps / (ms / 1e3) / 1e9
+        roofline = {"bound": "instruction issue and load latency", "kernel":
+                    "node route (k_ang_back, k_ang_spread, k_ang_bins and 9 more per subset)",
+                    "achieved": gbs, "peak": hbm, "unit": "GB/s of path data", "frac": gbs / hbm,
+                    "traffic": None,
+                    "peak_basis": "measured copy bandwidth" if peaks.get("hbm_gbs") else "fallback",
+                    "path_kernels_share": prof["ms"] / ms if ms > 0 else None}
+    else:
+        roofline = {
+            "bound": "alu", "kernel": "k_row (fused row + forward)",
+            "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "Tex2/s",
+            "frac": achieved / peak if peak else None, "traffic": None,
+            "peak_basis": f"{sm_count} SMs x {EX2_PER_SM_PER_CLK} ex2/clk x {sm_max:.0f} MHz",
+            "peak_probe": probe["f32"] * sm_count * probe["sm_mhz"] * 1e6 / 1e12,
+            "probe_ex2_per_clk_per_sm": {k: probe[k] for k in ("f32", "f16x2", "bf16x2")},
+            "row_kernel_share": prof["ms"] / ms if ms > 0 else None,
+            "row_tuning": row_tuning}
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": dict(workload_config(sc, nq, model.np_scatter),
-                       l2="inputs larger than L2: %.2f GB of path tables stream every step"
-                          % (model.table_bytes / 1e9),
+                       l2="flushed by a %d MiB write before every timed step"
+                          % (L2_FLUSH_BYTES >> 20),
                        parallelism=f"replicas x{world}" if world > 1 else "single GPU",
-                       timed="the K steps as K iterations of one lm_osem call (events sorted "
-                             "once per call); e2e: one call per step with the step's host "
-                             "copies"),
+                       route="nodes" if on_nodes else "rows",
+                       timed="one lm_osem call of one iteration per step, the event sort "
+                             "included; e2e: with the step's host copies"),
         "s_per_osem_iter": ms_per_step / 1e3,
         "terms_per_s": prof["terms"] / (ms / 1e3) if ms > 0 else None,
         "terms_evaluated_per_step": prof["terms"] / args.steps,
@@ -911,17 +934,7 @@ def run_gpu(args, rank, local_rank, world):
         "e2e": ({"value": whole_job_throughput(elems_step, args.steps, world, ms_e2e), "unit": UNIT,
                  "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h} if ms_e2e else None),
         "gpu_launches": int(prof["kernels"]),
-        "roofline": {"bound": "alu", "kernel": "k_row (fused row + forward)",
-                     "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "Tex2/s",
-                     "frac": achieved / peak if peak else None,
-                     "traffic": (ROW_TRAFFIC_BYTES_PER_LAUNCH.get(sc.name)
-                                 if not args.events else None),
-                     "peak_basis": f"{sm_count} SMs x {EX2_PER_SM_PER_CLK} ex2/clk x "
-                                   f"{sm_max:.0f} MHz",
-                     "peak_probe": probe["f32"] * sm_count * probe["sm_mhz"] * 1e6 / 1e12,
-                     "probe_ex2_per_clk_per_sm": {k: probe[k] for k in ("f32", "f16x2", "bf16x2")},
-                     "row_kernel_share": prof["ms"] / ms if ms > 0 else None,
-                     "row_tuning": row_tuning},
+        "roofline": roofline,
     }
     if world == 1 and not args.no_forms and not args.events:
         model.close()
@@ -1019,13 +1032,11 @@ def run_surrogate_rows_case(n_events=20_000, repeats=3):
     return 0
 
 
-def run_row_case(n_events=60_000, tile_events=64, repeats=3, store_rows=False):
-    """Small case for profiling the exact row kernel in the launch shape the
-    benchmark's workload uses: the 64 x 64 object (its 1.6 GB of path
-    tables), n_events MC events of the subset-0 angles (8 angles, about one
-    lm_osem sub-iteration's work), tiles of tile_events; lm_forward (forward
-    sums only) or, with store_rows, lm_backproject (the row block written, as
-    lm_osem's launches do).  One row-kernel launch per call.  Prints one
+def run_row_case(n_events=7_000, tile_events=64, repeats=3):
+    """Small case for profiling the row kernel: the 64 x 64 object (1.6 GB of
+    path tables), n_events MC events of the subset-0 angles (8 angles; fewer
+    events than the node route takes), tiles of tile_events, one lm_osem
+    iteration per call: one row launch with events, its rows kept.  Prints one
     JSON line."""
     import numpy as np
     import torch
@@ -1040,13 +1051,9 @@ def run_row_case(n_events=60_000, tile_events=64, repeats=3, store_rows=False):
     model.set_tile_events(tile_events)
     dev = lm.DeviceEvents.from_list(ev)
     lam = torch.from_numpy(ph.activity.reshape(-1).astype(np.float32)).cuda()
-    wt = torch.ones(len(ev), dtype=torch.float32, device="cuda")
 
     def call():
-        if store_rows:
-            model.backproject(dev, wt)
-        else:
-            model.forward(dev, lam)
+        model.osem(dev, lam.clone(), sc.n_subsets, 1)
     model.profile_enable(True)
     call()
     model.profile_read()
@@ -1054,7 +1061,7 @@ def run_row_case(n_events=60_000, tile_events=64, repeats=3, store_rows=False):
         call()
     prof = model.profile_read()
     model.profile_enable(False)
-    print(json.dumps({"case": "row_rows" if store_rows else "row", "events": len(ev),
+    print(json.dumps({"case": "row_rows", "events": len(ev),
                       "tile_events": tile_events,
                       "row_ms": prof["ms"] / repeats, "terms": prof["terms"] / repeats,
                       "Tterms_per_s": prof["terms"] / (prof["ms"] / 1e3) / 1e12}), flush=True)
@@ -1149,7 +1156,7 @@ def main():
     args = parse_args()
     rank, local_rank, world = dist_env()
     if args.case in ("row", "row_rows"):
-        return run_row_case(n_events=args.events or 60_000, store_rows=args.case == "row_rows")
+        return run_row_case(n_events=args.events or 7_000)
     if args.case == "surrogate_rows":
         return run_surrogate_rows_case()
     if args.case == "surrogate_train":
