@@ -413,12 +413,24 @@ bool node_use(const lm_handle* h, int64_t n) {
            (forward_nodes_block(h, kNoAllocBytes) > 0 || noalloc_rows_bytes(h, n) > kNoAllocBytes);
 }
 
-// Reconstructions keep the rows up to 120 events per angle: their rows are kept
-// from the second iteration on, and a sub-iteration on kept rows costs less
-// (83 events per angle, 4 subsets, 16 iterations: 91 us each, the first ones
-// included; the nodes take 190 us whatever the list).
-bool node_use_osem(const lm_handle* h, int64_t n) {
-    return node_use(h, n) && n >= (int64_t)120 * h->mc.A;
+// Reconstructions: the estimated time of a sub-iteration's rows has to be twice
+// that of its nodes.  Both are fits in us to single iterations at 52 to 1470
+// points, 30 to 88 angles and 120 to 800 events per angle, and hold within 30 %:
+// rows 70 + 2e-8 voxels points lines (events + 700 per angle), the 700 for tiles
+// that are not full; nodes a chain of 12 kernels, 75, and their work per angle
+// and path.  Twice, because rows are kept from the second iteration on and cost
+// little then, and the route may not depend on the iterations (a reconstruction
+// resumed in parts gives the same bits).  52 points, 30 angles, 800 events per
+// angle, 10 subsets: rows 67 us, 37 kept, nodes 84; 864 points, 60 angles, 5000
+// events, 8 subsets: rows 2150, nodes 190.  Below 120 events per angle the rows
+// cost less than the nodes once kept at any size.
+bool node_use_osem(const lm_handle* h, int64_t n, int n_subsets) {
+    if (!node_use(h, n) || n < (int64_t)120 * h->mc.A) return false;
+    const double angles = (double)h->mc.A / std::max(1, n_subsets);
+    const double paths = (double)h->mc.nq * h->mc.np;
+    const double rows = 70.0 + 2e-8 * paths * h->mc.W * ((double)n / std::max(1, n_subsets) + 700.0 * angles);
+    const double nodes = 75.0 + angles * (3.5 + 0.012 * h->mc.np) * h->mc.B / 64.0 + 6e-5 * paths;
+    return rows > 2.0 * nodes;
 }
 
 }  // namespace lmmew
@@ -876,7 +888,7 @@ size_t node_scratch(const lm_handle* h, int angles, char* base, NodeScratch* s) 
     s->block = std::min(angles, std::max(1, forward_nodes_block(h, kNodeBudgetBytes)));
     char* p = base;
     s->lam = bump<float>(p, m.nq);
-    s->HT = bump<float>(p, (size_t)m.np * N.nn);
+    s->HT = bump<float>(p, (size_t)node_back_parts(h, angles) * m.np * N.nn);
     s->dbp = bump<float>(p, (size_t)s->block * m.npc * N.nb_max * N.nm_pad);
     s->DB = bump<float>(p, (size_t)s->block * m.B * N.nl_pad);
     s->F = bump<float>(p, cells * N.nk_pad);
@@ -1047,7 +1059,7 @@ int lm_osem(lm_handle* h, const lm_events* ev, int n_subsets, int n_iters, int s
     cudaStream_t st = (cudaStream_t)stream;
     rc = subset_sensitivity(h, n_subsets, st);
     if (rc != LMMEW_OK) return rc;
-    if (node_use_osem(h, ev->n)) {
+    if (node_use_osem(h, ev->n, n_subsets)) {
         rc = osem_nodes(h, ev, n_subsets, n_iters, start_iter, start_subset, image, loglik, st);
         if (rc != LMMEW_ERR_OOM) return rc;   // no room for the node sums: the rows
     }
@@ -1391,7 +1403,7 @@ int lm_osem_batch(lm_handle* h, int n_real, const lm_events* events, int n_subse
     std::vector<lm_events> rest;
     std::vector<int> rest_of;
     for (int r = 0; r < n_real; ++r)
-        if (!node_use_osem(h, events[r].n)) {
+        if (!node_use_osem(h, events[r].n, n_subsets)) {
             rest.push_back(events[r]);
             rest_of.push_back(r);
         }
@@ -1403,7 +1415,7 @@ int lm_osem_batch(lm_handle* h, int n_real, const lm_events* events, int n_subse
     if (rc == LMMEW_OK) rc = take_status(h, st);
     if (rc == LMMEW_OK) rc = subset_sensitivity(h, n_subsets, st);
     for (int r = 0; r < n_real && rc == LMMEW_OK; ++r)
-        if (node_use_osem(h, events[r].n))
+        if (node_use_osem(h, events[r].n, n_subsets))
             rc = lm_osem(h, &events[r], n_subsets, n_iters, 0, 0, images + (size_t)r * m.n * m.n,
                          loglik ? loglik + (size_t)r * n_iters * n_subsets : nullptr, stream);
     if (rc != LMMEW_OK || rest.empty()) return rc;

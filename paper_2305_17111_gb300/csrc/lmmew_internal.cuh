@@ -270,6 +270,7 @@ int node_forward(lm_handle* h, const float* lam_v, const float* H, int a0, int a
 int node_cells(lm_handle* h, int angles, const int* cell_start, int cell0, const float* energy,
                const float* F, const float* Pr, const float* weight, const uint32_t* perm, float* V,
                float* PV, double* ll, cudaStream_t st);
+int node_back_parts(const lm_handle* h, int angles);   // sums T[np][nn] it writes
 int node_back(lm_handle* h, int a0, int a_step, int angles, const float* V, const float* PV,
               float* VG, float* psi, float* T, float* val, float* part_prim, cudaStream_t st);
 int node_update(lm_handle* h, int angles, const float* val, const float* part_prim,
@@ -377,7 +378,7 @@ size_t forward_nodes_bytes(const lm_handle* h, int block);
 size_t noalloc_rows_bytes(const lm_handle* h, int64_t n);
 constexpr size_t kNoAllocBytes = size_t(16) << 20;   // lm_forward_noalloc's static array: 16 MiB
 bool node_use(const lm_handle* h, int64_t n);
-bool node_use_osem(const lm_handle* h, int64_t n);   // the same for a whole reconstruction
+bool node_use_osem(const lm_handle* h, int64_t n, int n_subsets);   // the same for a whole reconstruction
 // Row blocks of n_sets consecutive rank ranges (the subsets of a partition
 // into n_subsets, or all ranks for n_subsets = 1): set s, block k covers
 // tiles [T0 + k tpc, T0 + (k + 1) tpc) of the set's tiles [T0, T1).

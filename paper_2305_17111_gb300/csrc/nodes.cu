@@ -164,6 +164,7 @@ struct NodeParams {
     NodeConst N;
     int a0, a_step, angles;  // angle i of the launch: a0 + i a_step
     int A, B, nq, np, npc, nq_pad;
+    int parts;               // sums T[part] the angles of a back projection are split over
     const float* g;          // [nl][nk_pad] Gaussians
     const float* gt;         // [nk][nl_pad] their transpose
     const int2* k_of_l;      // [nl_pad / 32] recorded-energy nodes in reach of 32 nodes l
@@ -647,7 +648,9 @@ __global__ void __launch_bounds__(256) k_ang_psi(const NodeParams P) {
 // blocks an SM put every warp of the grid on the chip at once: 412 us for 60
 // angles and 54 us for 8 (503 and 66 us with the collimator values read bin by
 // bin; 16 or 4 bins in flight: 426, 468 us; one warp a block: 410 us, but 264
-// instead of 210 us for 15 angles at 3464 voxels).
+// instead of 210 us for 15 angles at 3464 voxels).  A grid that leaves most of
+// the chip idle is split over the angles, up to 8 parts that k_ang_paths adds
+// in order: a back projection of 52 points and 88 angles took 355 us with one.
 constexpr int kBackWarps = 4, kBackTile = 64, kBackAngles = 4;
 constexpr size_t kBackStage = 16 * 1024;
 __global__ void __launch_bounds__(32 * kBackWarps, 8) k_ang_back(const NodeParams P, int tiles, int groups,
@@ -666,8 +669,9 @@ __global__ void __launch_bounds__(32 * kBackWarps, 8) k_ang_back(const NodeParam
     const int n = P.N.n_dir[w], nmp = P.N.nm_pad, per = P.N.nbg_max * kGroup;
     const int nd0 = min(tile * kBackTile + lane, n - 1), nd1 = min(tile * kBackTile + 32 + lane, n - 1);
     f32x2 acc0[kGroup / 2] = {0ull, 0ull, 0ull, 0ull}, acc1[kGroup / 2] = {0ull, 0ull, 0ull, 0ull};
-    for (int a1 = 0; a1 < P.angles; a1 += batch) {
-        const int na = min(batch, P.angles - a1);
+    const int a_end = P.angles * ((int)blockIdx.y + 1) / P.parts;   // (at most 8 x 16384)
+    for (int a1 = P.angles * (int)blockIdx.y / P.parts; a1 < a_end; a1 += batch) {
+        const int na = min(batch, a_end - a1);
         __syncthreads();
         for (int i = t; i < na * kBackWarps * per / 4; i += 32 * kBackWarps) {
             const int x = i % (per / 4), g = i / (per / 4) % kBackWarps, k = i / (per / 4) / kBackWarps;
@@ -730,7 +734,7 @@ __global__ void __launch_bounds__(32 * kBackWarps, 8) k_ang_back(const NodeParam
         }
     }
     if (grp >= groups) return;
-    float* out = P.T + P.N.n_off[w] + tile * kBackTile + lane;
+    float* out = P.T + (size_t)blockIdx.y * P.np * P.N.nn + P.N.n_off[w] + tile * kBackTile + lane;
     const bool on0 = tile * kBackTile + lane < n, on1 = tile * kBackTile + 32 + lane < n;
 #pragma unroll
     for (int i = 0; i < kGroup; ++i) {
@@ -764,7 +768,9 @@ __global__ void __launch_bounds__(256) k_ang_paths(const NodeParams P) {
         for (int k = 0; k < 7; ++k) {
             int j = c + k - 3;
             j = j < 0 ? j + n : j >= n ? j - n : j;
-            v = fmaf(x[k], T[j], v);
+            float t = T[j];
+            for (int o = 1; o < P.parts; ++o) t += T[(size_t)o * P.np * P.N.nn + j];
+            v = fmaf(x[k], t, v);
         }
     }
     P.val[i] = v;
@@ -1555,6 +1561,20 @@ int node_cells(lm_handle* h, int angles, const int* cell_start, int cell0, const
     return LMMEW_OK;
 }
 
+static int back_tiles(const NodeConst& N) {
+    int tiles = 0;
+    for (int w = 0; w < N.W; ++w) tiles += (N.n_dir[w] + kBackTile - 1) / kBackTile;
+    return tiles;
+}
+
+// Sums a back projection of so many angles is split over: as many as the chip
+// holds grids of k_ang_back (8 blocks an SM), with 2 angles or more in each.
+int node_back_parts(const lm_handle* h, int angles) {
+    const int groups = (h->mc.np + kGroup - 1) / kGroup;
+    const int blocks = back_tiles(h->nodes) * ((groups + kBackWarps - 1) / kBackWarps);
+    return std::max(1, std::min({8, angles / 2, 8 * h->sm_count / blocks}));
+}
+
 // Back projection of the node weights of angles a0 + i a_step: the paths' values
 // and the unscattered part of every angle.
 int node_back(lm_handle* h, int a0, int a_step, int angles, const float* V, const float* PV,
@@ -1576,13 +1596,12 @@ int node_back(lm_handle* h, int a0, int a_step, int angles, const float* V, cons
         k_node_unvalues<<<(unsigned)blocks, 32 * kValueWarps, band_smem(N.nk_pad), st>>>(P);
         k_ang_psi<<<(unsigned)rows, 256, sizeof(float) * N.nl_pad, st>>>(P);
     }
-    int tiles = 0;
-    for (int w = 0; w < N.W; ++w) tiles += (N.n_dir[w] + kBackTile - 1) / kBackTile;
-    const int groups = (m.np + kGroup - 1) / kGroup;
+    const int tiles = back_tiles(N), groups = (m.np + kGroup - 1) / kGroup;
+    P.parts = node_back_parts(h, angles);
     const size_t one = sizeof(float) * kBackWarps * (size_t)N.nbg_max * kGroup;   // staged per angle
     const int batch = (int)std::max<size_t>(1, std::min<size_t>(kBackAngles, kBackStage / one));
-    k_ang_back<<<(unsigned)(tiles * ((groups + kBackWarps - 1) / kBackWarps)), 32 * kBackWarps,
-                 batch * one, st>>>(P, tiles, groups, batch);
+    k_ang_back<<<dim3((unsigned)(tiles * ((groups + kBackWarps - 1) / kBackWarps)), P.parts),
+                 32 * kBackWarps, batch * one, st>>>(P, tiles, groups, batch);
     int rc = prof_start(h, st);
     if (rc != LMMEW_OK) return rc;
     k_ang_paths<<<(unsigned)(((int64_t)m.np * m.nq + 255) / 256), 256, 0, st>>>(P);

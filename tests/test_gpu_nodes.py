@@ -36,6 +36,19 @@ CASES = [
 ]
 
 
+# the same models, and lists long enough for a reconstruction through the nodes
+OSEM_CASES = [
+    ("small_16", {}, 1_500_000),
+    ("small_16", {"line_keV": (140.0,), "yields": (1.0,), "windows": ((90.0, 160.0),),
+                  "n_subsets": 1}, 1_500_000),
+    ("small_24", {"line_keV": (82.0, 154.0), "yields": (0.7, 0.3)}, 150_000),
+    ("small_24", {"line_keV": (82.0, 154.0, 270.0, 300.0), "yields": (0.4, 0.2, 0.2, 0.2),
+                  "n_bins": 29, "n_angles": 7, "n_subsets": 7}, 200_000),
+    ("small_32_4w", {}, 250_000),
+    ("lmmew_32", {"n_bins": 37, "n_angles": 9, "n_subsets": 2, "scatter_n": 32}, 60_000),
+]
+
+
 @pytest.fixture(scope="module", autouse=True)
 def _cuda():
     if not torch.cuda.is_available():
@@ -52,6 +65,11 @@ def _case(name, over, n_events, seed=3):
     wt = rng.uniform(0.1, 1.0, len(ev)).astype(np.float32)
     gpu = lm.Model.from_scenario(sc, ph.rho)
     return sc, ph, ev, lam, wt, gpu, lm.DeviceEvents.from_list(ev)
+
+
+def _repeat(ev, n, seed=9):
+    """n events drawn from a list with replacement."""
+    return ev.subset(np.random.default_rng(seed).integers(0, len(ev), size=n))
 
 
 def _paths(gpu):
@@ -109,9 +127,10 @@ def test_either_side_of_two_events_per_angle(name, less):
     gpu.close()
 
 
-@pytest.mark.parametrize("name,over,n", CASES)
+@pytest.mark.parametrize("name,over,n", OSEM_CASES)
 def test_reconstruction_matches_the_row_route_and_resumes(name, over, n):
-    sc, ph, ev, lam, wt, gpu, dev = _case(name, over, n, seed=5)
+    sc, ph, ev, lam, wt, gpu, dev = _case(name, over, 4000, seed=5)
+    dev = lm.DeviceEvents.from_list(_repeat(ev, n))
     n_sub = sc.n_subsets
     lam0 = torch.from_numpy((ph.rho.reshape(-1) > 0).astype(np.float32)).cuda()
     a, la = lam0.clone(), torch.zeros(2 * n_sub, dtype=torch.float64, device="cuda")
@@ -133,18 +152,20 @@ def test_reconstruction_matches_the_row_route_and_resumes(name, over, n):
 
 
 def test_streamed_tables_give_the_same_bits():
-    sc, ph, ev, lam, wt, gpu, dev = _case("lmmew_32", {"n_angles": 10}, 5000)
+    sc, ph, ev, lam, wt, gpu, dev = _case("lmmew_32", {"n_angles": 10, "scatter_n": 32}, 5000)
+    dense = lm.DeviceEvents.from_list(_repeat(ev, 120_000))
     x, wv = torch.from_numpy(lam).cuda(), torch.from_numpy(wt).cuda()
     lam0 = torch.from_numpy((ph.rho.reshape(-1) > 0).astype(np.float32)).cuda()
     img = lam0.clone()
     y, bp = gpu.forward(dev, x), gpu.backproject(dev, wv)
-    gpu.osem(dev, img, 4, 2)
+    gpu.osem(dense, img, 4, 2)
+    assert not gpu.batch_tuning()["tuned"]
     for slots in (1, 3):
         gpu.set_table_streaming(slots)
         assert torch.equal(gpu.forward(dev, x), y)
         assert torch.equal(gpu.backproject(dev, wv), bp)
         img2 = lam0.clone()
-        gpu.osem(dev, img2, 4, 2)
+        gpu.osem(dense, img2, 4, 2)
         assert torch.equal(img2, img)
     gpu.close()
 
@@ -198,7 +219,7 @@ def test_energies_far_from_every_line():
     x = torch.from_numpy(lam).cuda()
     y = gpu.forward(evs, x).double().cpu().numpy()
     gpu.set_tile_events(64)
-    small = 7 * sc.n_angles          # the row route, with energy classes
+    small = 2 * sc.n_angles - 1      # the row route, with energy classes
     rows = np.concatenate([gpu.forward(lm.DeviceEvents(evs.angle[i:i + small], evs.bin[i:i + small],
                                                        evs.energy[i:i + small]), x).double().cpu().numpy()
                            for i in range(0, n, small)])
@@ -216,9 +237,9 @@ def test_energies_far_from_every_line():
 def test_batch_of_dense_and_sparse_realisations():
     """Dense realisations run through the nodes, sparse ones share row launches;
     each equals its own lm_osem bit for bit, and a bad event is refused."""
-    sc, ph, ev, lam, wt, gpu, dev = _case("small_24", {}, 10)
-    sizes = [1500, 300, 0, 2000, 451]
-    evs = [simulate(sc, n_events=max(n, 1), seed=60 + i).subset(np.arange(n)) for i, n in enumerate(sizes)]
+    sc, ph, ev, lam, wt, gpu, dev = _case("small_24", {}, 4000)
+    sizes = [150_000, 300, 0, 200_000, 1500]
+    evs = [_repeat(ev, n, seed=60 + i) for i, n in enumerate(sizes)]
     devs = [lm.DeviceEvents.from_list(e) for e in evs]
     rng = np.random.default_rng(0)
     lam0 = torch.from_numpy(np.stack([rng.uniform(0.5, 2.0, ph.rho.size) * (ph.rho.reshape(-1) > 0)
