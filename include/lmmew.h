@@ -51,7 +51,7 @@
  *     and back projections and LM-OSEM take, instead of one row per event, sums
  *     on direction and energy nodes whose cost hardly grows with the events
  *     (the same model to FP32 rounding; lm_forward and lm_backproject from 2
- *     events per angle, lm_osem and lm_osem_batch, per realisation, from 120
+ *     events per angle (8 for back projections of small models), lm_osem and lm_osem_batch, per realisation, from 120
  *     per angle where a sub-iteration's rows are estimated to take twice the
  *     nodes' time).  The route needs up to 4 lines, the square-root energy
  *     resolution (exponent -1/2), the FP32 form and energy pruning on;

@@ -413,6 +413,14 @@ bool node_use(const lm_handle* h, int64_t n) {
            (forward_nodes_block(h, kNoAllocBytes) > 0 || noalloc_rows_bytes(h, n) > kNoAllocBytes);
 }
 
+// Back projections of small models (fewer than 100 000 voxel-point pairs) from 8
+// events per angle: 24 x 24 voxels, 52 points, 88 angles: rows 188, 215 and 250 us
+// for 2, 4 and 8 events per angle, nodes 220 to 247.  From 827 voxels x 207 points
+// on the nodes are ahead at 2 (347 for 376 us).
+bool node_use_back(const lm_handle* h, int64_t n) {
+    return node_use(h, n) && ((int64_t)h->mc.nq * h->mc.np >= 100000 || n >= (int64_t)8 * h->mc.A);
+}
+
 // Reconstructions: the estimated time of a sub-iteration's rows has to be twice
 // that of its nodes.  Both are fits in us to single iterations at 52 to 1470
 // points, 30 to 88 angles and 120 to 800 events per angle, and hold within 30 %:
@@ -997,7 +1005,7 @@ int lm_backproject(lm_handle* h, const lm_events* ev, const float* weight, float
         return LMMEW_OK;
     }
     if (surrogate_model(h)) return backproject_planned(h, ev, weight, out_image, stream);
-    if (node_use(h, ev->n)) {
+    if (node_use_back(h, ev->n)) {
         rc = backproject_nodes(h, ev, weight, out_image, st);
         if (rc != LMMEW_ERR_OOM) return rc;   // no room for the node sums: the rows
     }

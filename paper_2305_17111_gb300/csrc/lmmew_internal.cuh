@@ -378,6 +378,7 @@ size_t forward_nodes_bytes(const lm_handle* h, int block);
 size_t noalloc_rows_bytes(const lm_handle* h, int64_t n);
 constexpr size_t kNoAllocBytes = size_t(16) << 20;   // lm_forward_noalloc's static array: 16 MiB
 bool node_use(const lm_handle* h, int64_t n);
+bool node_use_back(const lm_handle* h, int64_t n);   // the same for lm_backproject
 bool node_use_osem(const lm_handle* h, int64_t n, int n_subsets);   // the same for a whole reconstruction
 // Row blocks of n_sets consecutive rank ranges (the subsets of a partition
 // into n_subsets, or all ranks for n_subsets = 1): set s, block k covers
