@@ -531,8 +531,11 @@ int lm_create(const lm_geometry* g, const lm_attenuation* at, const lm_lines* ln
                               : 0.0;
     h->n_subsets_default = n_subsets;
     int rc = build_tables(h, at->rho, support);
-    if (rc == LMMEW_OK) build_energy_classes(h);
-    if (rc == LMMEW_OK) rc = build_nodes(h);
+    if (rc == LMMEW_OK) {
+        line_reaches(h);
+        build_energy_classes(h);
+        rc = build_nodes(h);
+    }
     if (rc == LMMEW_OK &&
         (cudaMalloc(&h->d_term_counter, sizeof(unsigned long long)) != cudaSuccess ||
          cudaMemset(h->d_term_counter, 0, sizeof(unsigned long long)) != cudaSuccess ||

@@ -148,6 +148,7 @@ struct lm_handle {
     lmmew::EnergyClasses ecls{};
     int n_classes = 1;
     int class_lines[2 * LMMEW_MAX_LINES + 1] = {};
+    float reach_lo[LMMEW_MAX_LINES] = {}, reach_hi[LMMEW_MAX_LINES] = {};   // of each line's single scatter
     int prune_lines = 1;           // 0: every tile evaluates every line (lm_set_energy_pruning)
     // device copies of the sort's group arrays, one set per subset partition
     // (rank of each angle [A], angle and line mask of each group [G]) for the
@@ -162,6 +163,7 @@ struct lm_handle {
     int tab_a0 = 0, tab_astep = 1, tab_count = 0;
     // what k_scatter needs to rebuild tables, kept from the set-up
     double* d_cs_a = nullptr;      // [A][2] cos, sin of each detector direction
+    std::vector<int> p_cell;       // scatter cell of each point
     int* d_p_cell = nullptr;       // [np] cell of each scatter point
     double* d_p_rho = nullptr;     // [np] its mean density
     double* d_gqp = nullptr;       // [nq][np] voxel-to-point line integrals of rho
@@ -257,10 +259,10 @@ int set_table_streaming(lm_handle* h, int max_angles);
 // setup.cu: tables larger than this are streamed by lm_create (0: no limit
 // beyond the device's free memory)
 extern int64_t g_table_budget;
-// events.cu: the energy classes of the handle's lines and energy model, and
-// the recorded energies single scatter of line w can reach (rounded outward)
+// events.cu: the recorded energies single scatter of each line can reach
+// (rounded outward) and the energy classes their ends form
+void line_reaches(lm_handle* h);
 void build_energy_classes(lm_handle* h);
-void line_reach(const lm_handle* h, int w, float* lo, float* hi);
 // nodes.cu: projections of dense event lists through angle and energy nodes
 int build_nodes(lm_handle* h);
 size_t node_angle_bytes(const lm_handle* h);   // scratch of one angle's forward sums

@@ -57,6 +57,7 @@ namespace lmmew {
 namespace {
 
 constexpr int kTapsL = 7;          // taps of the scattered-energy nodes
+constexpr int kPsiStride = 8;      // a direction offset's weights for them, padded
 constexpr int kPerUnitL = 16;      // nodes per unit of t
 constexpr int kTapsK = 12;         // taps of the recorded-energy nodes
 constexpr int kPerUnitK = 8;
@@ -176,7 +177,7 @@ struct NodeParams {
     const float* gamma;      // [A][np] line integral from each point to the detector, cm
     const float* mu;         // [nm_pad] log2(e) mu_water(E') of the direction offsets
     const int* psi_l;        // [nm_pad] first of the 7 nodes l of an offset's E'
-    const float* psi_w;      // [nm_pad][8] their weights, times f
+    const float* psi_w;      // [nm_pad][kPsiStride] their weights, times f
     const int* dec_start;    // [nl_pad / 32 + 1] the same by 32 nodes l: offsets m and weights
     const int* dec_m;
     const float* dec_w;
@@ -624,7 +625,7 @@ __global__ void __launch_bounds__(256) k_ang_psi(const NodeParams P) {
     for (int l = threadIdx.x; l < P.N.nl_pad; l += 256) srow[l] = P.VG[row * P.N.nl_pad + l];
     __syncthreads();
     for (int m = threadIdx.x; m < P.N.nm_pad; m += 256) {
-        const float4* w = reinterpret_cast<const float4*>(P.psi_w + (size_t)m * 8);
+        const float4* w = reinterpret_cast<const float4*>(P.psi_w + (size_t)m * kPsiStride);
         const float4 w0 = w[0], w1 = w[1];
         const float* v = srow + P.psi_l[m];
         float s = w0.x * v[0];
@@ -1031,20 +1032,34 @@ __global__ void __launch_bounds__(1024) k_node_loglik(const double* ll, int n_ll
 
 // ------------------------------------------------------------------ set-up
 
-// Bins a chunk of 32 scatter points reaches: those whose run overlaps it.
+// First and last + 1 of the bins the lanes found, over the warp.
+__device__ __forceinline__ int2 warp_bins(int lo, int hi) {
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    return lo < hi ? make_int2(lo, hi) : make_int2(0, 0);
+}
+
+// Bins a chunk of 32 scatter points reaches: those whose run overlaps it.  A
+// warp per chunk, a lane per bin (one thread a chunk waits for the bins one by
+// one).
+constexpr int kBinsWarps = 4;
 __global__ void k_chunk_bins(const int2* crange, int B, int npc, int2* chunk_bins, int* most) {
-    const int a = blockIdx.y, pc = blockIdx.x * blockDim.x + threadIdx.x;
+    const int a = blockIdx.y, lane = threadIdx.x & 31;
+    const int pc = blockIdx.x * kBinsWarps + (threadIdx.x >> 5);
     if (pc >= npc) return;
     int lo = B, hi = 0;
-    for (int b = 0; b < B; ++b) {
+    for (int b = lane; b < B; b += 32) {
         const int2 r = crange[(size_t)a * B + b];
         if (r.y > r.x && r.x < (pc + 1) * kPC && r.y > pc * kPC) {
             lo = min(lo, b);
             hi = b + 1;
         }
     }
-    chunk_bins[(size_t)a * npc + pc] = lo < hi ? make_int2(lo, hi) : make_int2(0, 0);
-    atomicMax(most, max(hi - lo, 0));
+    const int2 br = warp_bins(lo, hi);
+    if (lane == 0) {
+        chunk_bins[(size_t)a * npc + pc] = br;
+        atomicMax(most, br.y - br.x);
+    }
 }
 
 // Place of each point in an angle's order, and its line integral to the
@@ -1056,28 +1071,34 @@ __global__ void k_point_tables(const int* inv, const double* g_p, int np, int* r
     gamma[(size_t)a * np + i] = (float)g_p[(size_t)a * np + i];
 }
 
-// Bins the 8 points of a group reach.
+// Bins the 8 points of a group reach (a warp per group, a lane per bin).
 __global__ void k_group_bins(const int2* crange, const int* rank, const int* grp_pt, int B, int np,
                              int groups, int2* grp_bins, int* most) {
-    const int a = blockIdx.y, g = blockIdx.x * blockDim.x + threadIdx.x;
+    const int a = blockIdx.y, lane = threadIdx.x & 31;
+    const int g = blockIdx.x * kBinsWarps + (threadIdx.x >> 5);
     if (g >= groups) return;
+    int at[kGroup];
+#pragma unroll
+    for (int i = 0; i < kGroup; ++i) {
+        const int p = grp_pt[g * kGroup + i];
+        at[i] = p < 0 ? -1 : rank[(size_t)a * np + p];
+    }
     int lo = B, hi = 0;
-    for (int b = 0; b < B; ++b) {
+    for (int b = lane; b < B; b += 32) {
         const int2 r = crange[(size_t)a * B + b];
         bool any = false;
-        for (int i = 0; i < kGroup; ++i) {
-            const int p = grp_pt[g * kGroup + i];
-            if (p < 0) continue;
-            const int k = rank[(size_t)a * np + p];
-            any |= k >= r.x && k < r.y;
-        }
+#pragma unroll
+        for (int i = 0; i < kGroup; ++i) any |= at[i] >= r.x && at[i] < r.y;
         if (any) {
             lo = min(lo, b);
             hi = b + 1;
         }
     }
-    grp_bins[(size_t)a * groups + g] = lo < hi ? make_int2(lo, hi) : make_int2(0, 0);
-    atomicMax(most, max(hi - lo, 0));
+    const int2 br = warp_bins(lo, hi);
+    if (lane == 0) {
+        grp_bins[(size_t)a * groups + g] = br;
+        atomicMax(most, br.y - br.x);
+    }
 }
 
 __global__ void k_group_values(const float* cs, const int* rank, const int* grp_pt,
@@ -1097,18 +1118,76 @@ __global__ void k_group_values(const float* cs, const int* rank, const int* grp_
     grp_c[(size_t)a * groups * nbg_max * kGroup + i] = v;
 }
 
-// Direction from voxel q to point p in 2^-32 turns; pair p nq + q.
-__global__ void k_pair_direction(ModelConst m, const int* q_pix, const int* p_cell, uint32_t* fix,
-                                 uint32_t* idx) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)m.np * m.nq) return;
-    const int p = (int)(i / m.nq), q = (int)(i % m.nq);
-    const int pix = q_pix[q], c = p_cell[p];
+// Direction from voxel q to point p in 2^-32 turns.
+__device__ __forceinline__ uint32_t pair_direction(const ModelConst& m, int pix, int c) {
     const double dx = ((c % m.S) + 0.5) * m.f - ((pix % m.n) + 0.5);
     const double dy = ((c / m.S) + 0.5) * m.f - ((pix / m.n) + 0.5);
     double t = (dx == 0.0 && dy == 0.0) ? 0.0 : atan2(dy, dx) * 0.15915494309189533577;   // / 2 pi
     t -= floor(t);
-    fix[i] = (uint32_t)(uint64_t)(t * 4294967296.0);
+    return (uint32_t)(uint64_t)(t * 4294967296.0);
+}
+
+// What a path's weights are formed from and where the sorted paths go.
+struct PathTables {
+    const int *q_pix, *p_cell;
+    const double *p_rho, *g_qp, *d_qp, *mu_line;
+    uint32_t* fix;
+    int *path_q, *path_of;
+    float* path_b;
+};
+
+// Path i of point p leads from voxel q: its voxel, the voxel's place and, per
+// line, the weight B = alpha mu_0 rho_p A_p / d exp(-mu_0 gamma_qp) / K (0 for
+// voxels in the point's own cell).
+__device__ __forceinline__ void put_path(const ModelConst& m, const PathTables& T, int p, int q, int i,
+                                         uint32_t fix) {
+    const int64_t at = (int64_t)p * m.nq + i, n = (int64_t)m.np * m.nq;
+    T.fix[at] = fix;
+    T.path_q[at] = q;
+    T.path_of[(size_t)p * m.nq + q] = i;
+    const int pix = T.q_pix[q];
+    const bool own = ((pix / m.n) / m.f) * m.S + (pix % m.n) / m.f == T.p_cell[p];
+    const size_t k = (size_t)q * m.np + p;
+    for (int w = 0; w < m.W; ++w)
+        T.path_b[(size_t)w * n + at] =
+            own ? 0.f
+                : (float)(m.alpha[w] * T.mu_line[w] * T.p_rho[p] * m.cell_area / T.d_qp[k] *
+                          exp(-T.mu_line[w] * T.g_qp[k]) / m.kn_norm[w]);
+}
+
+// The paths of each point by direction (then voxel): a block per point sorts
+// them in shared memory, `size` (a power of two) keys of direction and voxel.
+// 24 x 24 pixels and 52 points took 16 launches through the global sort.
+constexpr int kSortPoint = 16384;        // most voxels of a point sorted this way: 128 KB
+__global__ void __launch_bounds__(512) k_point_paths(ModelConst m, const PathTables T, int size) {
+    extern __shared__ unsigned long long key[];
+    const int p = blockIdx.x, c = T.p_cell[p];
+    for (int q = threadIdx.x; q < size; q += blockDim.x)
+        key[q] = q < m.nq ? (unsigned long long)pair_direction(m, T.q_pix[q], c) << 32 | (unsigned)q : ~0ull;
+    for (int run = 2; run <= size; run <<= 1)
+        for (int d = run >> 1; d > 0; d >>= 1) {
+            __syncthreads();
+            for (int i = threadIdx.x; i < size / 2; i += blockDim.x) {
+                const int x = (i & ~(d - 1)) * 2 + (i & (d - 1)), y = x + d;
+                const unsigned long long u = key[x], v = key[y];
+                if ((u > v) == ((x & run) == 0)) {
+                    key[x] = v;
+                    key[y] = u;
+                }
+            }
+        }
+    __syncthreads();
+    for (int i = threadIdx.x; i < m.nq; i += blockDim.x)
+        put_path(m, T, p, (int)(key[i] & 0xffffffffu), i, (uint32_t)(key[i] >> 32));
+}
+
+// The same where a point has more voxels: keys of the global sorts (pair
+// p nq + q), then the sorted paths.
+__global__ void k_pair_direction(ModelConst m, const int* q_pix, const int* p_cell, uint32_t* fix,
+                                 uint32_t* idx) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)m.np * m.nq) return;
+    fix[i] = pair_direction(m, q_pix[i % m.nq], p_cell[i / m.nq]);
     idx[i] = (uint32_t)i;
 }
 
@@ -1117,29 +1196,12 @@ __global__ void k_pair_points(const uint32_t* idx, int64_t n, int nq, uint32_t* 
     if (i < n) key[i] = idx[i] / (uint32_t)nq;
 }
 
-// The sorted paths of every point: direction, voxel, place and, per line, the
-// weight B = alpha mu_0 rho_p A_p / d exp(-mu_0 gamma_qp) / K (0 for voxels in
-// the point's own cell).
-__global__ void k_pair_fill(ModelConst m, const uint32_t* order, const uint32_t* fix0,
-                            const int* q_pix, const int* p_cell, const double* p_rho,
-                            const double* g_qp, const double* d_qp, const double* mu_line,
-                            uint32_t* fix, int* path_q, int* path_of, float* path_b) {
+__global__ void k_pair_fill(ModelConst m, const PathTables T, const uint32_t* order, const uint32_t* fix0) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t n = (int64_t)m.np * m.nq;
-    if (i >= n) return;
+    if (i >= (int64_t)m.np * m.nq) return;
     const uint32_t src = order[i];
-    const int p = (int)(src / (uint32_t)m.nq), q = (int)(src % (uint32_t)m.nq);
-    fix[i] = fix0[src];
-    path_q[i] = q;
-    path_of[(size_t)p * m.nq + q] = (int)(i - (int64_t)p * m.nq);
-    const int pix = q_pix[q];
-    const bool own = ((pix / m.n) / m.f) * m.S + (pix % m.n) / m.f == p_cell[p];
-    const size_t k = (size_t)q * m.np + p;
-    for (int w = 0; w < m.W; ++w)
-        path_b[(size_t)w * n + i] =
-            own ? 0.f
-                : (float)(m.alpha[w] * mu_line[w] * p_rho[p] * m.cell_area / d_qp[k] *
-                          exp(-mu_line[w] * g_qp[k]) / m.kn_norm[w]);
+    const int p = (int)(src / (uint32_t)m.nq);
+    put_path(m, T, p, (int)(src % (uint32_t)m.nq), (int)(i - (int64_t)p * m.nq), fix0[src]);
 }
 
 // First path of each point at every line's centre nodes 0 .. n, and the count.
@@ -1164,6 +1226,60 @@ __global__ void k_path_starts(const NodeConst N, const uint32_t* fix, int np, in
     start[i] = lo;
 }
 
+// The direction offsets' attenuation (log2(e) mu_water(E')) and the weights, times
+// f, of the kTapsL scattered-energy nodes from psi_l on that E' lies between.
+__global__ void k_offset_tables(ModelConst m, const NodeConst N, double kappa, const int* psi_l, float* mu,
+                                float* psi_w) {
+    const int o = blockIdx.x * blockDim.x + threadIdx.x;
+    if (o >= N.nm_pad) return;
+    int w = 0;
+    while (w + 1 < N.W && o >= N.m_off[w + 1]) ++w;
+    const int i = o - N.m_off[w];
+    if (i >= N.m_count[w]) {             // pads between the lines
+        mu[o] = 0.f;
+        for (int k = 0; k < kPsiStride; ++k) psi_w[(size_t)kPsiStride * o + k] = 0.f;
+        return;
+    }
+    const double e0 = m.line_e[w], k0 = e0 / 510.99895;
+    const double c = cospi(2.0 * i / N.n_dir[w]), r = 1.0 / (1.0 + k0 * (1.0 - c)), e = e0 * r;
+    const double kn = r * r * (r + 1.0 / r - (1.0 - c * c));
+    const double f = kn / (2.506628274631000502 * kappa * sqrt(e));   // / (sqrt(2 pi) sigma)
+    const double u = 2.0 * sqrt(e) / kappa * kPerUnitL - N.l_first[w];
+    const double s = u - (psi_l[o] - N.l_off[w] + kTapsL / 2);
+    double mu_e = m.knot_mu[0];
+    if (m.n_knots > 1) {
+        int k = 0;
+        while (k < m.n_knots - 2 && e >= m.knot_e[k + 1]) ++k;
+        mu_e = m.knot_mu[k] + (e - m.knot_e[k]) * m.knot_slope[k];
+    }
+    mu[o] = (float)(mu_e * 1.4426950408889634);
+    for (int k = 0; k < kPsiStride; ++k) {
+        double v = k < kTapsL ? f : 0.0, d = 1.0;
+        for (int j = 0; j < kTapsL; ++j)
+            if (j != k) {
+                v *= s - (j - kTapsL / 2);
+                d *= k - j;
+            }
+        psi_w[(size_t)kPsiStride * o + k] = (float)(v / d);
+    }
+}
+
+// The same weights by node l, 32 nodes at a time: entries dec_start[l / 32] + 32 i
+// + l % 32 are the offsets (dec_m) and weights of node l, i < the most any of the
+// 32 nodes has.  The offsets of a node are consecutive (E' falls with the offset).
+__global__ void k_offset_lists(const NodeConst N, const int* psi_l, const float* psi_w, const int2* run,
+                               const int* dec_start, int* dec_m, float* dec_w) {
+    const int l = blockIdx.x * blockDim.x + threadIdx.x;
+    if (l >= N.nl_pad) return;
+    const int2 r = run[l];
+    const int d1 = dec_start[(l >> 5) + 1];
+    int o = r.x;
+    for (int d = dec_start[l >> 5] + (l & 31); d < d1; d += 32, ++o) {
+        dec_m[d] = o < r.y ? o : 0;
+        dec_w[d] = o < r.y ? psi_w[(size_t)kPsiStride * o + l - psi_l[o]] : 0.f;
+    }
+}
+
 // Shared-memory opt-in of the node kernels, once per device.
 int node_kernel_attrs() {
     static std::atomic<unsigned long long> done{0};
@@ -1179,6 +1295,8 @@ int node_kernel_attrs() {
     LMMEW_CUDA(cudaFuncSetAttribute(k_ang_back, cudaFuncAttributeMaxDynamicSharedMemorySize, cap - 4096));
     LMMEW_CUDA(cudaFuncSetAttribute(k_node_cells, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     80 * 1024));
+    LMMEW_CUDA(cudaFuncSetAttribute(k_point_paths, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    8 * kSortPoint));
     done.fetch_or(bit);
     return LMMEW_OK;
 }
@@ -1235,7 +1353,10 @@ size_t band_smem(int band) {
 // The nodes of the model and everything the route reads.  It exists for the
 // square-root energy resolution, up to 4 lines and node counts and pair tables
 // (12 + 4 W bytes per voxel and scatter point) of sane sizes; other models keep
-// the rows.
+// the rows.  Built with every model, so it may not cost a small one much: nine
+// launches, one allocation more for the grouped collimator values, a copy up and
+// one down; a model of 24 x 24 voxels, 12 x 12 cells and 24 angles takes 1.5 ms
+// with them (2.2 ms with host tables and global sorts, 1.75 ms without any).
 int build_nodes(lm_handle* h) {
     const ModelConst& m = h->mc;
     NodeConst& N = h->nodes;
@@ -1306,54 +1427,47 @@ int build_nodes(lm_handle* h) {
         N.m_off[w] = N.nm_pad;
         N.nm_pad += (N.m_count[w] + 31) & ~31;
         N.start_ints += N.n_dir[w] + 2;
-        line_reach(h, w, &N.reach_lo[w], &N.reach_hi[w]);
+        N.reach_lo[w] = h->reach_lo[w];
+        N.reach_hi[w] = h->reach_hi[w];
     }
     N.nl_pad = (N.nl + 31) & ~31;
     if (N.nl > 6000 || N.nk > 1024 || N.nn > 32768 || (int64_t)m.np * N.nn >= (int64_t(1) << 31))
         return LMMEW_OK;
     const size_t pair_bytes = (12 + 4 * (size_t)m.W) * (size_t)pairs;
-    size_t free_b = 0, total_b = 0;
-    LMMEW_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    if (2 * pair_bytes > free_b / 4) return LMMEW_OK;
+    if (pair_bytes > (size_t(64) << 20)) {
+        size_t free_b = 0, total_b = 0;
+        LMMEW_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        if (2 * pair_bytes > free_b / 4) return LMMEW_OK;
+    }
 
-    // host tables: offsets' attenuation and taps (also by node l), bands
-    std::vector<float> mu(N.nm_pad, 0.f), psi_w((size_t)8 * N.nm_pad, 0.f), dec_w;
-    std::vector<int> psi_l(N.nm_pad, 0), dec_start(N.nl_pad / 32 + 1, 0), dec_m, taps(N.nl_pad, 0);
+    // host tables: first of the scattered-energy nodes each offset's E' lies
+    // between (its cosine by the three-term recurrence: it only has to name the
+    // nearest node), the offsets of each node and the bands
+    std::vector<int> psi_l(N.nm_pad, 0), dec_start(N.nl_pad / 32 + 1, 0);
+    std::vector<int2> run(N.nl_pad, make_int2(0, 0));
     for (int w = 0; w < m.W; ++w) {
-        const double e0 = m.line_e[w], k0 = e0 / me;
+        const double e0 = m.line_e[w], k0 = e0 / me, step = cos(2.0 * pi / N.n_dir[w]);
+        double c = 1.0, before = step;
         for (int i = 0; i < N.m_count[w]; ++i) {
-            const double c = cos(2.0 * pi * i / N.n_dir[w]), r = 1.0 / (1.0 + k0 * (1.0 - c)), e = e0 * r;
-            const double kn = r * r * (r + 1.0 / r - (1.0 - c * c));
-            const double f = kn / (sqrt(2.0 * pi) * kappa * sqrt(e));
-            const double u = t_of(e) * kPerUnitL - N.l_first[w];
-            const int c0 = (int)floor(u + 0.5);
-            const double s = u - c0;
-            const int o = N.m_off[w] + i;
-            mu[o] = (float)(mu_of(e) * log2e);
-            psi_l[o] = N.l_off[w] + c0 - 3;
-            for (int k = 0; k < 7; ++k) {
-                double v = f;
-                for (int j = 0; j < 7; ++j)
-                    if (j != k) v *= (s - (j - 3)) / (double)(k - j);
-                psi_w[(size_t)8 * o + k] = (float)v;
-                ++taps[psi_l[o] + k];
+            const double u = t_of(e0 / (1.0 + k0 * (1.0 - c))) * kPerUnitL - N.l_first[w];
+            const int o = N.m_off[w] + i, first = N.l_off[w] + (int)floor(u + 0.5) - kTapsL / 2;
+            psi_l[o] = first;
+            for (int l = first; l < first + kTapsL; ++l) {
+                if (run[l].y == 0) run[l].x = o;
+                run[l].y = o + 1;
             }
+            const double next = 2.0 * step * c - before;
+            before = c;
+            c = next;
         }
     }
-    for (int t = 0; t < N.nl_pad / 32; ++t)
-        dec_start[t + 1] =
-            dec_start[t] + 32 * *std::max_element(taps.begin() + 32 * t, taps.begin() + 32 * (t + 1));
-    dec_m.assign(dec_start[N.nl_pad / 32], 0);
-    dec_w.assign(dec_m.size(), 0.f);
-    std::fill(taps.begin(), taps.end(), 0);
-    for (int w = 0; w < m.W; ++w)
-        for (int i = 0; i < N.m_count[w]; ++i)
-            for (int k = 0; k < 7; ++k) {
-                const int o = N.m_off[w] + i, l = psi_l[o] + k;
-                const int d = dec_start[l >> 5] + 32 * taps[l]++ + (l & 31);
-                dec_m[d] = o;
-                dec_w[d] = psi_w[(size_t)8 * o + k];
-            }
+    size_t dec_n = 0;
+    for (int t = 0; t < N.nl_pad / 32; ++t) {
+        int most = 0;
+        for (int l = 32 * t; l < 32 * t + 32; ++l) most = std::max(most, run[l].y - run[l].x);
+        dec_n += 32 * (size_t)most;
+        dec_start[t + 1] = (int)dec_n;
+    }
     const int lt = N.nl_pad / 32, kt = N.nk_pad / 32;
     std::vector<int2> bands((size_t)lt + kt, make_int2(1 << 30, 0));
     int2* k_of_l = bands.data();
@@ -1383,8 +1497,7 @@ int build_nodes(lm_handle* h) {
     // together than 8 in a row
     std::vector<int> grp_pt;
     {
-        std::vector<int> cell(m.np);
-        LMMEW_CUDA(cudaMemcpy(cell.data(), h->d_p_cell, sizeof(int) * m.np, cudaMemcpyDeviceToHost));
+        const std::vector<int>& cell = h->p_cell;
         std::vector<std::pair<int64_t, int>> key(m.np);
         for (int p = 0; p < m.np; ++p) {
             const int x = cell[p] % m.S, y = cell[p] / m.S;
@@ -1398,19 +1511,21 @@ int build_nodes(lm_handle* h) {
     const size_t gm = (size_t)N.nl_pad * N.nk_pad;
     size_t host_bytes = 0;
     int* d_most = nullptr;
+    int2* d_run = nullptr;
     auto layout = [&](char* p) {
         char* base = p;
-        T.mu = bump<float>(p, mu.size());
-        T.psi_w = bump<float>(p, psi_w.size());
-        T.dec_w = bump<float>(p, dec_w.size());
         T.psi_l = bump<int>(p, psi_l.size());
         T.dec_start = bump<int>(p, dec_start.size());
-        T.dec_m = bump<int>(p, dec_m.size());
         T.grp_pt = bump<int>(p, grp_pt.size());
         T.k_of_l = bump<int2>(p, bands.size());
         T.l_of_k = T.k_of_l + lt;
+        d_run = bump<int2>(p, run.size());
         d_most = bump<int>(p, 2);
         host_bytes = (size_t)(p - base);
+        T.mu = bump<float>(p, N.nm_pad);
+        T.psi_w = bump<float>(p, (size_t)kPsiStride * N.nm_pad);
+        T.dec_m = bump<int>(p, dec_n);
+        T.dec_w = bump<float>(p, dec_n);
         T.g = bump<float>(p, gm);
         T.gt = bump<float>(p, gm);
         T.chunk_bins = bump<int2>(p, (size_t)m.A * m.npc);
@@ -1425,12 +1540,15 @@ int build_nodes(lm_handle* h) {
         return (size_t)(p - base) + 256;
     };
     const size_t bytes = layout(nullptr);
+    // (points of up to kSortPoint voxels sort their paths in shared memory)
+    const bool sort_global = m.nq > kSortPoint;
     const size_t sort_bytes = 4 * bump_bytes(4 * (size_t)pairs) + bump_bytes(pair_hist_bytes(pairs));
     struct Temp {
         void* p = nullptr;
         ~Temp() { cudaFree(p); }
     } temp;
-    if (cudaMalloc(&h->d_node_tables, bytes) != cudaSuccess || cudaMalloc(&temp.p, sort_bytes) != cudaSuccess) {
+    if (cudaMalloc(&h->d_node_tables, bytes) != cudaSuccess ||
+        (sort_global && cudaMalloc(&temp.p, sort_bytes) != cudaSuccess)) {
         cudaGetLastError();
         return LMMEW_OK;                 // no room: the rows
     }
@@ -1439,42 +1557,53 @@ int build_nodes(lm_handle* h) {
     auto put = [&](const void* dst, const void* src, size_t n) {
         std::memcpy(blob.data() + ((const char*)dst - (const char*)h->d_node_tables), src, n);
     };
-    put(T.mu, mu.data(), 4 * mu.size());
-    put(T.psi_w, psi_w.data(), 4 * psi_w.size());
-    put(T.dec_w, dec_w.data(), 4 * dec_w.size());
     put(T.psi_l, psi_l.data(), 4 * psi_l.size());
     put(T.dec_start, dec_start.data(), 4 * dec_start.size());
-    put(T.dec_m, dec_m.data(), 4 * dec_m.size());
     put(T.grp_pt, grp_pt.data(), 4 * grp_pt.size());
     put(T.k_of_l, bands.data(), 8 * bands.size());
+    put(d_run, run.data(), 8 * run.size());
     LMMEW_CUDA(cudaMemcpy(h->d_node_tables, blob.data(), host_bytes, cudaMemcpyHostToDevice));
+    int rc = node_kernel_attrs();
+    if (rc != LMMEW_OK) return rc;
 
+    k_offset_tables<<<(N.nm_pad + 63) / 64, 64>>>(m, N, kappa, T.psi_l, T.mu, T.psi_w);
+    k_offset_lists<<<(N.nl_pad + 63) / 64, 64>>>(N, T.psi_l, T.psi_w, d_run, T.dec_start, T.dec_m, T.dec_w);
     k_node_matrix<<<(unsigned)((gm + 255) / 256), 256>>>(N, kappa, T.g, T.gt);
-    k_chunk_bins<<<dim3((m.npc + 31) / 32, m.A), 32>>>(h->d_crange, m.B, m.npc, T.chunk_bins, d_most);
+    k_chunk_bins<<<dim3((m.npc + kBinsWarps - 1) / kBinsWarps, m.A), 32 * kBinsWarps>>>(
+        h->d_crange, m.B, m.npc, T.chunk_bins, d_most);
     k_point_tables<<<dim3((m.np + 127) / 128, m.A), 128>>>(h->d_inv, h->d_gp, m.np, T.rank, T.gamma);
-    k_group_bins<<<dim3((groups + 31) / 32, m.A), 32>>>(h->d_crange, T.rank, T.grp_pt, m.B, m.np, groups,
-                                                        T.grp_bins, d_most + 1);
-    // the paths of each point by direction: stable sorts by direction, then point
-    char* tp = (char*)temp.p;
-    uint32_t* kin = bump<uint32_t>(tp, pairs);
-    uint32_t* kout = bump<uint32_t>(tp, pairs);
-    uint32_t* vin = bump<uint32_t>(tp, pairs);
-    uint32_t* vout = bump<uint32_t>(tp, pairs);
-    uint32_t* hist = bump<uint32_t>(tp, pair_hist_bytes(pairs) / 4);
-    const unsigned pb = (unsigned)((pairs + 255) / 256);
-    uint32_t* fix0 = reinterpret_cast<uint32_t*>(T.path_b);   // (free until the fill) unsorted directions
-    k_pair_direction<<<pb, 256>>>(m, h->d_q_pix, h->d_p_cell, fix0, vin);
-    LMMEW_CUDA(cudaMemcpyAsync(kin, fix0, 4 * (size_t)pairs, cudaMemcpyDeviceToDevice, 0));
-    int rc = sort_pairs(h, pairs, 32, kin, kout, vin, vout, hist, 0);
-    if (rc != LMMEW_OK) return rc;
-    k_pair_points<<<pb, 256>>>(vin, pairs, m.nq, kin);
-    int bits = 1;
-    while (bits < 32 && ((uint32_t)(m.np - 1) >> bits) != 0) ++bits;
-    rc = sort_pairs(h, pairs, bits, kin, kout, vin, vout, hist, 0);
-    if (rc != LMMEW_OK) return rc;
-    LMMEW_CUDA(cudaMemcpyAsync(kin, fix0, 4 * (size_t)pairs, cudaMemcpyDeviceToDevice, 0));
-    k_pair_fill<<<pb, 256>>>(m, vin, kin, h->d_q_pix, h->d_p_cell, h->d_p_rho, h->d_gqp, h->d_dqp,
-                             h->d_mu_line, T.fix, T.path_q, T.path_of, T.path_b);
+    k_group_bins<<<dim3((groups + kBinsWarps - 1) / kBinsWarps, m.A), 32 * kBinsWarps>>>(
+        h->d_crange, T.rank, T.grp_pt, m.B, m.np, groups, T.grp_bins, d_most + 1);
+    const PathTables paths{h->d_q_pix, h->d_p_cell, h->d_p_rho, h->d_gqp, h->d_dqp, h->d_mu_line,
+                           T.fix, T.path_q, T.path_of, T.path_b};
+    if (!sort_global) {
+        int size = 64;
+        while (size < m.nq) size *= 2;
+        k_point_paths<<<m.np, std::min(512, size / 2), 8 * (size_t)size>>>(m, paths, size);
+        ++h->launches;
+    } else {
+        // stable sorts by direction, then point
+        char* tp = (char*)temp.p;
+        uint32_t* kin = bump<uint32_t>(tp, pairs);
+        uint32_t* kout = bump<uint32_t>(tp, pairs);
+        uint32_t* vin = bump<uint32_t>(tp, pairs);
+        uint32_t* vout = bump<uint32_t>(tp, pairs);
+        uint32_t* hist = bump<uint32_t>(tp, pair_hist_bytes(pairs) / 4);
+        const unsigned pb = (unsigned)((pairs + 255) / 256);
+        uint32_t* fix0 = reinterpret_cast<uint32_t*>(T.path_b);   // (free until the fill) unsorted directions
+        k_pair_direction<<<pb, 256>>>(m, h->d_q_pix, h->d_p_cell, fix0, vin);
+        LMMEW_CUDA(cudaMemcpyAsync(kin, fix0, 4 * (size_t)pairs, cudaMemcpyDeviceToDevice, 0));
+        rc = sort_pairs(h, pairs, 32, kin, kout, vin, vout, hist, 0);
+        if (rc != LMMEW_OK) return rc;
+        k_pair_points<<<pb, 256>>>(vin, pairs, m.nq, kin);
+        int bits = 1;
+        while (bits < 32 && ((uint32_t)(m.np - 1) >> bits) != 0) ++bits;
+        rc = sort_pairs(h, pairs, bits, kin, kout, vin, vout, hist, 0);
+        if (rc != LMMEW_OK) return rc;
+        LMMEW_CUDA(cudaMemcpyAsync(kin, fix0, 4 * (size_t)pairs, cudaMemcpyDeviceToDevice, 0));
+        k_pair_fill<<<pb, 256>>>(m, paths, vin, kin);
+        h->launches += 3;
+    }
     k_path_starts<<<(unsigned)(((int64_t)m.np * N.start_ints + 127) / 128), 128>>>(N, T.fix, m.np, m.nq,
                                                                                   T.path_start);
     LMMEW_CUDA(cudaGetLastError());
@@ -1490,12 +1619,11 @@ int build_nodes(lm_handle* h) {
     }
     k_group_values<<<dim3((unsigned)((per_angle + 255) / 256), m.A), 256>>>(
         h->d_cs, T.rank, T.grp_pt, T.grp_bins, m.B, m.np, m.npc, groups, N.nbg_max, h->d_node_groups);
-    h->launches += 9;
+    h->launches += 8;
     LMMEW_CUDA(cudaGetLastError());
-    LMMEW_CUDA(cudaDeviceSynchronize());   // (the sort's scratch goes)
-    rc = node_kernel_attrs();
-    if (rc == LMMEW_OK) h->node_route = 1;
-    return rc;
+    LMMEW_CUDA(cudaDeviceSynchronize());   // (the tables are used on any stream)
+    h->node_route = 1;
+    return LMMEW_OK;
 }
 
 size_t node_angle_bytes(const lm_handle* h) {

@@ -615,6 +615,7 @@ int build_tables(lm_handle* h, const float* rho_host, const uint8_t* support_hos
             if (mean[c] > 0.0) { p_cell.push_back(c); p_rho.push_back(mean[c]); }
     }
     m.np = (int)p_cell.size();
+    h->p_cell = p_cell;
     m.npc = (m.np + kPC - 1) / kPC;
 
     // The single-scatter path tables hold 3 floats per (angle, line, voxel,

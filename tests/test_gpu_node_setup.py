@@ -1,0 +1,73 @@
+"""Set-up of the node route's tables (csrc/nodes.cu): the paths of a scatter
+point are sorted in shared memory up to 16 384 voxels and by the global sort
+above, so projections through the nodes are compared with the rows' (the same
+model, FP32 sums in another order) at voxel counts on either side of that and
+of the sort's powers of two; and what the tables add to the creation of a
+small model."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_2305_17111_gb300 as lm  # noqa: E402
+from synthetic import preset  # noqa: E402
+
+ROUTE_RTOL = 2e-6   # node route vs row route: FP32 sums in another order
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+
+
+def _events(sc, per_cell, seed):
+    """per_cell events in every (angle, bin) cell, energies over the lines' scatter."""
+    rng = np.random.default_rng(seed)
+    a, b = np.meshgrid(np.arange(sc.n_angles), np.arange(sc.n_bins), indexing="ij")
+    a, b = np.repeat(a.reshape(-1), per_cell), np.repeat(b.reshape(-1), per_cell)
+    return lm.DeviceEvents(a, b, rng.uniform(62.0, 280.0, a.size).astype(np.float32))
+
+
+# pixels, scatter cells, voxels of the support (the first ones): 64 and 65 (the
+# smallest sort and past it), a power of two, the largest sort in shared memory
+@pytest.mark.parametrize("n,scatter_n,voxels", [(8, 4, 64), (9, 3, 65), (32, 8, 1024), (128, 4, 16384)])
+def test_projections_for_every_sort_size(n, scatter_n, voxels):
+    sc = preset("tiny_8").with_(n=n, pixel_cm=25.6 / n, n_bins=9, scatter_n=scatter_n)
+    rho = np.ones((n, n), np.float32)
+    support = (np.arange(n * n) < voxels).astype(np.uint8)
+    gpu = lm.Model.from_scenario(sc, rho, support=support)
+    assert gpu.nq == voxels
+    dev = _events(sc, 5, n)
+    rng = np.random.default_rng(voxels)
+    x = torch.from_numpy((rng.uniform(0.2, 3.0, n * n) * support).astype(np.float32)).cuda()
+    wv = torch.from_numpy(rng.uniform(0.1, 1.0, len(dev)).astype(np.float32)).cuda()
+    gpu.profile_enable(True)
+    y = gpu.forward(dev, x).double()
+    assert gpu.profile_read()["terms"] == gpu.n_lines * gpu.nq * gpu.np_scatter    # the node route
+    gpu.profile_enable(False)
+    bp = gpu.backproject(dev, wv).double()
+    gpu.set_energy_pruning(False)
+    y_rows, bp_rows = gpu.forward(dev, x).double(), gpu.backproject(dev, wv).double()
+    assert float(((y - y_rows) / y_rows).abs().max()) < ROUTE_RTOL
+    on = bp_rows != 0
+    assert bool((bp[~on] == 0).all())
+    assert float(((bp - bp_rows)[on] / bp_rows[on]).abs().max()) < ROUTE_RTOL
+    gpu.close()
+
+
+def test_tables_of_a_small_model_take_few_launches():
+    """Nine kernels; the same model at a resolution whose energy nodes are too
+    many for the route has none of them."""
+    sc = preset("small_24").with_(n_angles=24, scatter_n=12)
+    rho = sc.make_phantom().rho
+    count = {}
+    for frac in (0.10, 0.02):
+        gpu = lm.Model.from_scenario(sc.with_(fwhm_frac=frac), rho)
+        count[frac] = gpu.profile_read()["kernels"]
+        gpu.close()
+    assert 1 <= count[0.10] - count[0.02] <= 9
