@@ -365,11 +365,12 @@ int forward_nodes(lm_handle* h, const lm_events* ev, const float* image, float* 
     float* DB = bump<float>(arena, (size_t)block * m.B * N.nl_pad);
     float* F = bump<float>(arena, (size_t)block * m.B * N.nk_pad);
     float* Pr = bump<float>(arena, (size_t)block * m.B * N.W);
+    float* side = bump<float>(arena, (size_t)block * m.np * N.slots);
     int rc = launch_gather_image(h, image, lam_v, st);
-    if (rc == LMMEW_OK) rc = node_spread(h, lam_v, H, st);
     for (int a0 = 0; a0 < m.A && rc == LMMEW_OK; a0 += block) {
         const int cnt = std::min(block, m.A - a0);
-        rc = node_forward(h, lam_v, H, a0, 1, cnt, dbp, DB, F, Pr, st);
+        rc = node_spread(h, lam_v, a0 == 0 ? H : nullptr, a0, 1, cnt, side, st);
+        if (rc == LMMEW_OK) rc = node_forward(h, lam_v, H, side, a0, 1, cnt, dbp, DB, F, Pr, st);
         if (rc == LMMEW_OK) rc = node_events_forward(h, ev, F, Pr, a0, cnt, out_y, st);
     }
     if (h->prof_on) h->prof_elems += (double)ev->n * (double)m.nq;
@@ -493,6 +494,7 @@ int lm_create(const lm_geometry* g, const lm_attenuation* at, const lm_lines* ln
             return set_error(LMMEW_ERR_INVALID_ARG, "rho must be finite and >= 0");
 
     lm_handle* h = new lm_handle();
+    for (int i = 0; i < n * n; ++i) h->rho_max = std::max(h->rho_max, (double)at->rho[i]);
     ModelConst& m = h->mc;
     std::memset(&m, 0, sizeof(m));
     m.n = n;
@@ -889,7 +891,7 @@ int lm_forward(lm_handle* h, const lm_events* ev, const float* image, float* out
 namespace {
 struct NodeScratch {
     int block;
-    float *lam, *HT, *dbp, *DB, *F, *Pr, *V, *PV, *VG, *psi, *val, *part_prim;   // (H and T take turns)
+    float *lam, *HT, *dbp, *DB, *F, *Pr, *V, *PV, *VG, *psi, *side, *val, *part_prim;   // (H and T take turns)
     double *ll, *num;
 };
 size_t node_scratch(const lm_handle* h, int angles, char* base, NodeScratch* s) {
@@ -908,6 +910,7 @@ size_t node_scratch(const lm_handle* h, int angles, char* base, NodeScratch* s) 
     s->PV = bump<float>(p, cells * m.W);
     s->VG = bump<float>(p, cells * N.nl_pad);
     s->psi = bump<float>(p, cells * N.nm_pad);
+    s->side = bump<float>(p, (size_t)angles * m.np * N.slots);
     s->val = bump<float>(p, (size_t)m.np * m.nq);
     s->part_prim = bump<float>(p, (size_t)angles * nq_pad);
     s->ll = bump<double>(p, cells);
@@ -918,10 +921,12 @@ size_t node_scratch(const lm_handle* h, int angles, char* base, NodeScratch* s) 
 int node_forward_blocks(lm_handle* h, const NodeScratch& s, int a0, int a_step, int angles,
                         cudaStream_t st) {
     const ModelConst& m = h->mc;
-    int rc = node_spread(h, s.lam, s.HT, st);
+    const size_t per_side = (size_t)m.np * h->nodes.slots;
+    int rc = node_spread(h, s.lam, s.HT, a0, a_step, angles, s.side, st);
     for (int i = 0; i < angles && rc == LMMEW_OK; i += s.block)
-        rc = node_forward(h, s.lam, s.HT, a0 + i * a_step, a_step, std::min(s.block, angles - i), s.dbp,
-                          s.DB, s.F + (size_t)i * m.B * h->nodes.nk_pad, s.Pr + (size_t)i * m.B * m.W, st);
+        rc = node_forward(h, s.lam, s.HT, s.side + i * per_side, a0 + i * a_step, a_step,
+                          std::min(s.block, angles - i), s.dbp, s.DB, s.F + (size_t)i * m.B * h->nodes.nk_pad,
+                          s.Pr + (size_t)i * m.B * m.W, st);
     return rc;
 }
 
@@ -944,7 +949,8 @@ int backproject_nodes(lm_handle* h, const lm_events* ev, const float* weight, fl
     if (rc == LMMEW_OK)
         rc = node_cells(h, m.A, ce.cell_start, 0, ce.energy, nullptr, nullptr, weight, ce.perm, s.V,
                         s.PV, nullptr, st);
-    if (rc == LMMEW_OK) rc = node_back(h, 0, 1, m.A, s.V, s.PV, s.VG, s.psi, s.HT, s.val, s.part_prim, st);
+    if (rc == LMMEW_OK)
+        rc = node_back(h, 0, 1, m.A, s.V, s.PV, s.VG, s.psi, s.HT, s.side, s.val, s.part_prim, st);
     if (rc == LMMEW_OK) rc = node_update(h, m.A, s.val, s.part_prim, nullptr, nullptr, s.num, st);
     if (rc != LMMEW_OK) return rc;
     if (h->prof_on) h->prof_elems += (double)ev->n * (double)m.nq;
@@ -982,8 +988,8 @@ int osem_nodes(lm_handle* h, const lm_events* ev, int n_subsets, int n_iters, in
                 rc = node_cells(h, cnt, ce.cell_start, cell0, ce.energy, s.F, s.Pr, nullptr, nullptr,
                                 s.V, s.PV, ll ? s.ll : nullptr, st);
             if (rc == LMMEW_OK)
-                rc = node_back(h, sub, n_subsets, cnt, s.V, s.PV, s.VG, s.psi, s.HT, s.val, s.part_prim,
-                               st);
+                rc = node_back(h, sub, n_subsets, cnt, s.V, s.PV, s.VG, s.psi, s.HT, s.side, s.val,
+                               s.part_prim, st);
             if (rc == LMMEW_OK && ll) rc = node_loglik(h, s.ll, cnt * m.B, s.lam, sens, ll, st);
             if (rc == LMMEW_OK)
                 rc = node_update(h, cnt, s.val, s.part_prim, sens, s.lam, nullptr, st);

@@ -106,12 +106,27 @@ struct NodeConst {
     float ck, ck_lo;           // node of a recorded energy = (ck + ck_lo) sqrt(E)
     float reach_lo[4], reach_hi[4];   // recorded energies single scatter of the line can have
     int nb_max, nbg_max;       // most bins 32 ordered, 8 neighbouring scatter points reach
+    // attenuation knots inside each line's E': offsets (in direction nodes,
+    // ascending), the slots of the nodes beside them (see nodes.cu)
+    int kinks[4], slots, tile_slots;
+    float kink[4][LMMEW_MAX_KNOTS];
+    int win_off[5];            // windows of each line's offsets near a knot
+};
+// A direction offset seen from the other side of a knot.
+struct NodeSlot {
+    int offset;                // of all lines' (m_off + m)
+    int branch;                // the paths' side: number of knots below their offset
+    int d0, d1;                // centres such paths can have, from the offset's node on
+    float lo, hi;              // their offsets: lo < u <= hi
+    float mu;                  // log2(e) mu_water(E') continued from that side
 };
 // Their device tables (one region; see NodeParams in nodes.cu).
 struct NodeTables {
     float *mu, *psi_w, *dec_w, *g, *gt, *gamma, *path_b;
     int *psi_l, *dec_start, *dec_m, *rank, *path_start, *path_q, *path_of, *grp_pt;
-    int2 *k_of_l, *l_of_k, *chunk_bins, *grp_bins;
+    int2 *k_of_l, *l_of_k, *chunk_bins, *grp_bins, *win;
+    int* slot_start;
+    NodeSlot* slot;
     uint32_t* fix;
 };
 struct NodeWindows {
@@ -133,6 +148,7 @@ typedef int4 ChunkRange;
 struct lm_handle {
     lmmew::ModelConst mc;
     lmmew::LineConst lc;
+    double rho_max = 0.0;          // largest density of the map
     int n_subsets_default;
     // geometry on the device
     int* d_q_pix = nullptr;        // [nq] pixel index of each support voxel
@@ -266,15 +282,16 @@ void build_energy_classes(lm_handle* h);
 // nodes.cu: projections of dense event lists through angle and energy nodes
 int build_nodes(lm_handle* h);
 size_t node_angle_bytes(const lm_handle* h);   // scratch of one angle's forward sums
-int node_spread(lm_handle* h, const float* lam_v, float* H, cudaStream_t st);
-int node_forward(lm_handle* h, const float* lam_v, const float* H, int a0, int a_step, int angles,
-                 float* dbp, float* DB, float* F, float* Pr, cudaStream_t st);
+int node_spread(lm_handle* h, const float* lam_v, float* H, int a0, int a_step, int angles, float* side,
+                cudaStream_t st);
+int node_forward(lm_handle* h, const float* lam_v, const float* H, const float* side, int a0, int a_step,
+                 int angles, float* dbp, float* DB, float* F, float* Pr, cudaStream_t st);
 int node_cells(lm_handle* h, int angles, const int* cell_start, int cell0, const float* energy,
                const float* F, const float* Pr, const float* weight, const uint32_t* perm, float* V,
                float* PV, double* ll, cudaStream_t st);
 int node_back_parts(const lm_handle* h, int angles);   // sums T[np][nn] it writes
 int node_back(lm_handle* h, int a0, int a_step, int angles, const float* V, const float* PV,
-              float* VG, float* psi, float* T, float* val, float* part_prim, cudaStream_t st);
+              float* VG, float* psi, float* T, float* side, float* val, float* part_prim, cudaStream_t st);
 int node_update(lm_handle* h, int angles, const float* val, const float* part_prim,
                 const double* sens, float* lam, double* num, cudaStream_t st);
 // events.cu: stable LSD radix sort of (key, value) pairs over ping-pong buffers;

@@ -30,11 +30,24 @@
 // (s = the node of the detector direction, m = |n - s|).  A projection visits
 // every (q, p, w) once whatever the number of events and of detector angles,
 // where the rows take one exponential per event and path in reach; nothing
-// of the path tables is read.  Interpolation errors are near 1e-8 of an event's
-// value (1e-6 in the worst case of an image of one voxel: mu has kinks at the
-// attenuation knots, which the node spacing of the lines that cross one is
-// chosen for), below the FP32 rounding of the sums; everything is FP32 with
-// fixed-order sums, the voxel sums FP64.
+// of the path tables is read.
+//
+// mu(E'(x)) has a kink where E' meets an attenuation knot, which a polynomial
+// through nodes on both sides would miss by the first power of their spacing
+// (1.5e-5 of an event's value with a node every 1/29 sigma).  So each path sees
+// mu continued smoothly from its own side: a node on the knot's other side is a
+// slot with that mu, and the paths' taps on it (a few paths in a hundred) are
+// summed apart, for every detector angle, and get the difference of the two
+// attenuations:
+//
+//   forward   W[a][p][z] = sum_{q beyond the knot} lambda_q B_{qp} L_n(phi_qp)   k_ang_spread
+//             S[b][m]   += sum_p C_p(b) (e^{-mu_z gamma_p} - e^{-mu(m) gamma_p}) W   k_ang_bins
+//   back      Y[a][p][z] = (e^{-mu_z gamma_p} - e^{-mu(m) gamma_p}) sum_b C_p(b) PSI[b][m]   k_ang_back
+//             out[q]    += sum_p B_{qp} sum_{n beyond the knot} L_n(phi_qp) Y         k_ang_paths
+//
+// Interpolation errors are near 1e-8 of an event's value, below the FP32
+// rounding of the sums; everything is FP32 with fixed-order sums, the voxel sums
+// FP64.
 //
 // Measured (864 voxels and 864 points, 3 lines, 60 angles of 64 bins; times
 // below that name no size are this model's): a forward projection of 100 000
@@ -186,6 +199,9 @@ struct NodeParams {
     const int* path_of;      // [np][nq] place of each voxel's path
     const float* path_b;     // [W][np][nq] their B
     const int* path_start;   // [np][start_ints] per line: first path of each centre node
+    const NodeSlot* slot;    // nodes beside a knot, seen from its other side
+    const int* slot_start;   // [nm_pad + 1] the slots of each offset
+    const int2* win;         // per line, windows of centres whose taps can cross a knot
     const int* grp_pt;       // [groups][8] neighbouring points (-1: none)
     const int2* grp_bins;    // [A][groups] bins they reach
     const float* grp_c;      // [A][groups][nbg_max][8] their collimator values
@@ -202,9 +218,61 @@ struct NodeParams {
     float* VG;               // [angles][B][nl_pad]
     float* psi;              // [angles][B][nm_pad]
     float* T;                // [np][nn]
+    float* side;             // [angles][np][slots] what a slot adds to its node, from the bins
     float* val;              // [np][nq]
     float* part_prim;        // [angles][nq_pad]
 };
+
+// The weighted taps on a slot's node of those paths of point p that lie on the
+// slot's side of the knot, for the detector direction of angle a.
+__device__ __forceinline__ float slot_taps(const NodeParams& P, const NodeSlot& z, int p, int a) {
+    constexpr int kHalf = kTapsN / 2;
+    int w = 0;
+    while (w + 1 < P.N.W && z.offset >= P.N.m_off[w + 1]) ++w;
+    const int n = P.N.n_dir[w], m = z.offset - P.N.m_off[w], s = (int)((int64_t)a * n / P.A);
+    const int* st = P.path_start + (size_t)p * P.N.start_ints + P.N.n_off[w] + 2 * w;
+    const uint32_t* fix = P.fix + (size_t)p * P.nq;
+    const int* pq = P.path_q + (size_t)p * P.nq;
+    const float* pb = P.path_b + ((size_t)w * P.np + p) * P.nq;
+    float sum = 0.f;
+    for (int sign = 1; sign >= -1; sign -= 2) {
+        int j = s + sign * m;                       // the node, in [0, n)
+        if (j >= n) j -= n;
+        if (j < 0) j += n;
+        if (sign < 0 && (2 * m == n || m == 0)) break;
+        // centres lo .. hi: one run of the point's directions, two where the circle
+        // closes (centres 0 and n are the same node)
+        int lo = j + (sign > 0 ? z.d0 : -z.d1), hi = j + (sign > 0 ? z.d1 : -z.d0);
+        if (hi < 0) {
+            lo += n;
+            hi += n;
+        } else if (lo >= n) {
+            lo -= n;
+            hi -= n;
+        }
+        const bool closes = lo <= 0 || hi >= n;
+        for (int part = 0; part < (closes ? 2 : 1); ++part) {
+            const int ca = !closes ? lo : part == 0 ? (lo <= 0 ? lo + n : lo) : 0;
+            const int cb = !closes ? hi : part == 0 ? n : (hi >= n ? hi - n : hi);
+            for (int r = st[ca]; r < st[cb + 1]; ++r) {
+                int c;
+                const float f = direction_pos(fix[r], n, &c);
+                int d = c - j;                      // centre past the node
+                if (2 * d > n) d -= n;
+                if (2 * d < -n) d += n;
+                float u = fabsf((float)(sign * m + d) + f);
+                if (2.f * u > (float)n) u = (float)n - u;
+                if (!(u > z.lo && u <= z.hi)) continue;
+                float x[kTapsN];
+                lagrange7(f, pb[r] * P.lam[pq[r]], x);
+#pragma unroll
+                for (int k = 0; k < kTapsN; ++k)
+                    if (k == kHalf - d) sum += x[k];
+            }
+        }
+    }
+    return sum;
+}
 
 // H: a warp per (point, line, 122 direction nodes).  The paths centred on the
 // tile's nodes and the 3 on either side are one run of the point's directions
@@ -218,10 +286,19 @@ struct NodeParams {
 // Where a centre has more than kSpreadDense paths the scan's steps cost more
 // than those waits, and a lane takes a centre's paths: 80 us instead of 118 us
 // at 3464 voxels (11, 6 and 3 paths a centre; limits of 2 and 4 are equal
-// there, 1 costs 83 us).
+// there, 1 costs 83 us).  The blocks past those form the slots' taps, a thread
+// per (angle, point, slot).
 constexpr int kSpreadDense = 4, kSpreadWarps = 4, kSpreadCentres = 128, kSpreadOut = kSpreadCentres - 6;
 __global__ void __launch_bounds__(32 * kSpreadWarps) k_ang_spread(const NodeParams P, int tiles, int units) {
     __shared__ __align__(16) float taps[kSpreadWarps][7][kSpreadCentres];
+    const int unit_blocks = (units + kSpreadWarps - 1) / kSpreadWarps;
+    if ((int)blockIdx.x >= unit_blocks) {
+        const int64_t i = (int64_t)(blockIdx.x - unit_blocks) * (32 * kSpreadWarps) + threadIdx.x;
+        if (i >= (int64_t)P.angles * P.np * P.N.slots) return;
+        const int64_t ap = i / P.N.slots;
+        P.side[i] = slot_taps(P, P.slot[i - ap * P.N.slots], (int)(ap % P.np), P.a0 + (int)(ap / P.np) * P.a_step);
+        return;
+    }
     const int lane = threadIdx.x & 31, unit = blockIdx.x * kSpreadWarps + (threadIdx.x >> 5);
     if (unit >= units) return;
     float (&tap)[7][kSpreadCentres] = taps[threadIdx.x >> 5];
@@ -340,7 +417,9 @@ __global__ void __launch_bounds__(32 * kSpreadWarps) k_ang_spread(const NodePara
 // read from shared memory serves both offsets).  Bound by FP32 issue: 115 us for
 // 60 angles, 20 us for 8.
 constexpr int kOffThreads = 128, kOffPer = 2;
-__global__ void __launch_bounds__(kOffThreads) k_ang_bins(const NodeParams P, int tiles) {
+
+__global__ void __launch_bounds__(kOffThreads, 6) k_ang_bins(const NodeParams P, int tiles) {
+    extern __shared__ float sside[];   // [tile's slots][kPC] what they add to their nodes
     __shared__ __align__(16) float sc[kPC][kBinsT];
     __shared__ int sp[kPC];
     __shared__ float sgm[kPC];
@@ -357,6 +436,9 @@ __global__ void __launch_bounds__(kOffThreads) k_ang_bins(const NodeParams P, in
     const int s = (int)((int64_t)a * n / P.A);
     int n1[kOffPer], n2[kOffPer];
     float mu[kOffPer], two[kOffPer];
+    // slots of the tile
+    const int z0 = P.slot_start[P.N.m_off[w] + tile * kTile];
+    const int z1 = P.slot_start[P.N.m_off[w] + min((tile + 1) * kTile, P.N.m_count[w])];
 #pragma unroll
     for (int j = 0; j < kOffPer; ++j) {
         const int m = min(tile * kTile + j * kOffThreads + t, P.N.m_count[w] - 1);
@@ -372,6 +454,14 @@ __global__ void __launch_bounds__(kOffThreads) k_ang_bins(const NodeParams P, in
         const int p = t < cnt ? P.inv[(size_t)a * P.np + pc * kPC + t] : 0;
         sp[t] = p * P.N.nn + P.N.n_off[w];
         sgm[t] = t < cnt ? P.gamma[(size_t)a * P.np + p] : 0.f;
+    }
+    if (z1 > z0) {
+        __syncthreads();
+        for (int i = t; i < (z1 - z0) * kPC; i += kOffThreads) {
+            const int z = z0 + i / kPC, k = i % kPC, p = sp[k] / P.N.nn;
+            const float own = ex2f(-P.mu[P.slot[z].offset] * sgm[k]), other = ex2f(-P.slot[z].mu * sgm[k]);
+            sside[i] = k < cnt ? P.side[((size_t)ai * P.np + p) * P.N.slots + z] * (other - own) : 0.f;
+        }
     }
     const int2 br = P.chunk_bins[(size_t)a * P.npc + pc];
     const float* cr = P.cs + ((size_t)a * P.npc + pc) * P.B * kCPad;
@@ -412,6 +502,24 @@ __global__ void __launch_bounds__(kOffThreads) k_ang_bins(const NodeParams P, in
                         acc[j][2 * k] = fma2(v2[j], pk(c.x, c.y), acc[j][2 * k]);
                         acc[j][2 * k + 1] = fma2(v2[j], pk(c.z, c.w), acc[j][2 * k + 1]);
                     }
+                }
+            }
+        }
+        // nodes beside a knot: paths beyond it have its other side's attenuation
+#pragma unroll
+        for (int j = 0; j < kOffPer; ++j) {
+            if (z1 == z0) break;
+            const int* zs = P.slot_start + P.N.m_off[w] + min(tile * kTile + j * kOffThreads + t, P.N.m_count[w] - 1);
+            const int i1 = (zs[1] - z0) * kPC;
+#pragma unroll 1
+            for (int i = (zs[0] - z0) * kPC; i < i1; ++i) {
+                const f32x2 y = pk1(sside[i]);
+                const float4* c4 = reinterpret_cast<const float4*>(sc[i % kPC]);
+#pragma unroll
+                for (int k = 0; k < kBinsT / 4; ++k) {
+                    const float4 c = c4[k];
+                    acc[j][2 * k] = fma2(y, pk(c.x, c.y), acc[j][2 * k]);
+                    acc[j][2 * k + 1] = fma2(y, pk(c.z, c.w), acc[j][2 * k + 1]);
                 }
             }
         }
@@ -660,6 +768,29 @@ __global__ void __launch_bounds__(32 * kBackWarps, 8) k_ang_back(const NodeParam
     __shared__ float sg[kBackAngles][kBackWarps][kGroup];
     __shared__ int2 sb[kBackAngles][kBackWarps];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int main_blocks = tiles * ((groups + kBackWarps - 1) / kBackWarps);
+    if ((int)blockIdx.x >= main_blocks) {
+        // the blocks past the grid: a thread per (slot, angle, point), what the
+        // bins add to the node for paths beyond the knot
+        const int64_t i = (int64_t)(blockIdx.x - main_blocks) * (32 * kBackWarps) + t;
+        const int z = (int)(i % P.N.slots), ai = (int)(i / P.N.slots % P.angles);
+        const int gp = (int)(i / ((int64_t)P.N.slots * P.angles));
+        if (blockIdx.y > 0 || gp >= groups * kGroup) return;
+        const int p = P.grp_pt[gp];
+        if (p < 0) return;
+        const NodeSlot zs = P.slot[z];
+        const int a = P.a0 + ai * P.a_step;
+        const size_t ag = (size_t)a * groups + gp / kGroup;
+        const int2 br = P.grp_bins[ag];
+        const float* c = P.grp_c + ag * P.N.nbg_max * kGroup + gp % kGroup;
+        const float* psi = P.psi + ((size_t)ai * P.B + br.x) * P.N.nm_pad + zs.offset;
+        float sum = 0.f;
+#pragma unroll 8
+        for (int b = 0; b < br.y - br.x; ++b) sum = fmaf(c[b * kGroup], psi[(size_t)b * P.N.nm_pad], sum);
+        const float g = P.gamma[(size_t)a * P.np + p];
+        P.side[((size_t)ai * P.np + p) * P.N.slots + z] = sum * (ex2f(-zs.mu * g) - ex2f(-P.mu[zs.offset] * g));
+        return;
+    }
     int tile = blockIdx.x % tiles;
     const int grp0 = blockIdx.x / tiles * kBackWarps, grp = grp0 + warp;
     int w = 0;
@@ -750,6 +881,41 @@ __global__ void __launch_bounds__(32 * kBackWarps, 8) k_ang_back(const NodeParam
     }
 }
 
+// v plus what the slots add to a path with its centre at node c and taps x: for
+// every detector angle that has a knot within reach of its taps, the nodes on
+// the knot's other side.  The windows of a line are disjoint, so that no angle
+// comes twice.
+__device__ __forceinline__ float beyond_knots(const NodeParams& P, int w, int p, int c, float s,
+                                              const float (&x)[kTapsN], float v) {
+    const int n = P.N.n_dir[w], g = n / P.A;      // nodes between two detector angles
+    for (int k = P.N.win_off[w]; k < P.N.win_off[w + 1]; ++k) {
+        const int2 win = P.win[k];
+        // angles j (of the unrolled circle) with c - j g inside the window
+        const int lo = c - win.y, hi = c - win.x;
+        for (int j = lo > 0 ? (lo + g - 1) / g : -(-lo / g); j * g <= hi; ++j) {
+            const int a = (j % P.A + P.A) % P.A, ai = (a - P.a0) / P.a_step;
+            if (a < P.a0 || ai >= P.angles || P.a0 + ai * P.a_step != a) continue;
+            int r = c - j * g;
+            if (2 * r > n) r -= n;
+            if (2 * r < -n) r += n;
+            float u = fabsf((float)r + s);
+            if (2.f * u > (float)n) u = (float)n - u;
+            int branch = 0;
+            while (branch < P.N.kinks[w] && u > P.N.kink[w][branch]) ++branch;
+            const float* side = P.side + ((size_t)ai * P.np + p) * P.N.slots;
+#pragma unroll
+            for (int t = 0; t < kTapsN; ++t) {
+                int m = abs(r + t - kTapsN / 2);
+                if (2 * m > n) m = n - m;
+                const int o = P.N.m_off[w] + m;
+                for (int z = P.slot_start[o]; z < P.slot_start[o + 1]; ++z)
+                    if (P.slot[z].branch == branch) v = fmaf(x[t], side[z], v);
+            }
+        }
+    }
+    return v;
+}
+
 // The paths' values in direction order, a thread per (point, path): the taps
 // of consecutive paths are consecutive nodes.  15 us; kSplit adds the parts of
 // a split k_ang_back (a loop over one part cost 17 us, and 79 instead of 52 us
@@ -777,6 +943,7 @@ __global__ void __launch_bounds__(256) k_ang_paths(const NodeParams P) {
                 for (int o = 1; o < P.parts; ++o) t += T[(size_t)o * P.np * P.N.nn + j];
             v = fmaf(x[k], t, v);
         }
+        if (P.N.kinks[w] > 0) v = beyond_knots(P, w, p, c, s, x, v);
     }
     P.val[i] = v;
 }
@@ -1335,6 +1502,9 @@ NodeParams node_params(const lm_handle* h, int a0, int a_step, int angles) {
     P.path_of = t.path_of;
     P.path_b = t.path_b;
     P.path_start = t.path_start;
+    P.slot = t.slot;
+    P.slot_start = t.slot_start;
+    P.win = t.win;
     P.grp_pt = t.grp_pt;
     P.grp_bins = t.grp_bins;
     P.grp_c = h->d_node_groups;
@@ -1375,6 +1545,9 @@ int build_nodes(lm_handle* h) {
         return m.knot_mu[s] + (e - m.knot_e[s]) * m.knot_slope[s];
     };
     N.W = m.W;
+    std::vector<NodeSlot> slots;
+    std::vector<int> slot_start;
+    std::vector<int2> wins;
     // recorded energies
     const double ck = kPerUnitK * 2.0 / kappa;
     N.ck = (float)ck;
@@ -1399,26 +1572,40 @@ int build_nodes(lm_handle* h) {
         if (N.l_first[w] < 1) return LMMEW_OK;
         N.l_off[w] = N.nl;               // (lines start at multiples of 8 nodes)
         N.nl += (N.l_count[w] + 7) & ~7;
-        // 18 nodes per sigma where E'(x) is steepest (7 taps: 1e-8 of a term),
-        // 29 for a line whose E' crosses an attenuation knot, and there enough
-        // that exp(-mu gamma) over 10 cm bends by 4e-4 per node at most
-        auto slope = [&](double x) {     // |dE'/dx|
-            const double e = e0 / (1.0 + k0 * (1.0 - cos(x)));
-            return e * e / e0 * k0 * sin(x);
+        // 18 nodes per sigma where E'(x) is steepest (7 taps: 1e-8 of a term), and
+        // enough that the attenuation changes by 4 % per node at most over the
+        // longest way through the map
+        auto slope = [&](double e) {     // |dE'/dx|
+            const double c = std::min(std::max(1.0 - (e0 / e - 1.0) / k0, -1.0), 1.0);
+            return e * e / e0 * k0 * sqrt(1.0 - c * c);
         };
-        double steep = 0.0, want = 0.0;
-        for (int i = 1; i < 512; ++i) {
-            const double x = pi * i / 512, e = e0 / (1.0 + k0 * (1.0 - cos(x)));
-            steep = std::max(steep, slope(x) / (kappa * sqrt(e)));
+        const double way = h->rho_max * m.n * m.h * sqrt(2.0);
+        auto mu_slope = [&](double e) {
+            int s = 0;
+            while (s < m.n_knots - 2 && e >= m.knot_e[s + 1]) ++s;
+            return m.n_knots > 1 ? fabs(m.knot_slope[s]) : 0.0;
+        };
+        double want = 32.0;
+        auto sample = [&](double e) {
+            want = std::max(want, 2.0 * pi * slope(e) * std::max(18.0 / (kappa * sqrt(e)), mu_slope(e) * way / 0.04));
+        };
+        for (int i = 1; i < 512; ++i) sample(e0 / (1.0 + k0 * (1.0 - cos(pi * i / 512))));
+        // knots inside E', by offset; the segment of mu on either side
+        std::vector<double> at;
+        int seg = 0;
+        while (seg < m.n_knots - 2 && e0 > m.knot_e[seg + 1]) ++seg;
+        std::vector<int> segs(1, seg);
+        for (; seg > 0 && m.knot_e[seg] > eb; --seg) {
+            const double e = m.knot_e[seg];
+            sample(e);
+            sample(std::nextafter(e, 0.0));
+            if (m.knot_slope[seg] == m.knot_slope[seg - 1]) {
+                segs.back() = seg - 1;   // (the same line)
+                continue;
+            }
+            at.push_back(acos(1.0 - (e0 / e - 1.0) / k0));
+            segs.push_back(seg - 1);
         }
-        want = 2.0 * pi * steep * 18.0;
-        for (int k = 1; k + 1 < m.n_knots; ++k) {
-            const double e = m.knot_e[k], bend = fabs(m.knot_slope[k] - m.knot_slope[k - 1]);
-            if (!(e > eb && e < e0) || bend == 0.0) continue;
-            const double x = acos(1.0 - (e0 / e - 1.0) / k0);
-            want = std::max(want, std::max(2.0 * pi * steep * 29.0, 2.0 * pi * 10.0 * bend * slope(x) / 4e-4));
-        }
-        want = std::max(want, 32.0);
         if (!(want < 16384.0) || m.A > 16384) return LMMEW_OK;
         N.n_dir[w] = ((int)ceil(want) + m.A - 1) / m.A * m.A;
         N.n_off[w] = N.nn;
@@ -1427,10 +1614,77 @@ int build_nodes(lm_handle* h) {
         N.m_off[w] = N.nm_pad;
         N.nm_pad += (N.m_count[w] + 31) & ~31;
         N.start_ints += N.n_dir[w] + 2;
+        // the nodes whose taps a knot lies between, once per other side
+        const int count = N.m_count[w], n = N.n_dir[w], half = kTapsN / 2;
+        N.kinks[w] = (int)at.size();
+        for (size_t k = 0; k < at.size(); ++k) N.kink[w][k] = (float)(at[k] * n / (2.0 * pi));
+        auto branch_of = [&](double u) {
+            int b = 0;
+            while (b < N.kinks[w] && u > N.kink[w][b]) ++b;
+            return b;
+        };
+        auto fold = [&](double u) { return fabs(u) > 0.5 * n ? n - fabs(u) : fabs(u); };
+        slot_start.resize(N.m_off[w] + count + 1, (int)slots.size());
+        for (int i = 0; i < count; ++i) {
+            slot_start[N.m_off[w] + i] = (int)slots.size();
+            const int own = branch_of(i);
+            for (int b = 0; b <= N.kinks[w]; ++b) {
+                if (b == own) continue;
+                const float lo = b == 0 ? -1.f : N.kink[w][b - 1], hi = b == N.kinks[w] ? 1e9f : N.kink[w][b];
+                int d0 = half + 1, d1 = -half - 1;
+                for (int d = -half; d <= half; ++d) {
+                    // paths centred there: i + d - 1/2 .. i + d + 1/2, folded
+                    const double u0 = fold(i + d - 0.5), u1 = fold(i + d + 0.5);
+                    const double a = std::min({u0, u1, fold(i + d)}), z = std::max({u0, u1, fold(i + d)});
+                    if (z < lo || a > hi) continue;
+                    d0 = std::min(d0, d);
+                    d1 = std::max(d1, d);
+                }
+                if (d0 > d1) continue;
+                const double e = e0 / (1.0 + k0 * (1.0 - cos(2.0 * pi * i / n)));
+                const double mu_b = m.knot_mu[segs[b]] + (e - m.knot_e[segs[b]]) * m.knot_slope[segs[b]];
+                slots.push_back({N.m_off[w] + i, b, d0, d1, lo, hi, (float)(mu_b * log2e)});
+            }
+        }
+        slot_start.back() = (int)slots.size();
+        slot_start.resize(N.nm_pad + 1, (int)slots.size());
+        constexpr int kTile = kOffThreads * kOffPer;
+        for (int i = 0; i < count; i += kTile)
+            N.tile_slots = std::max(N.tile_slots, slot_start[N.m_off[w] + std::min(i + kTile, count)] -
+                                                      slot_start[N.m_off[w] + i]);
+        // windows of centres (from the detector direction) with a knot among their taps
+        N.win_off[w] = (int)wins.size();
+        std::vector<int2> around;
+        for (double x : at) {
+            const double u = x * n / (2.0 * pi);
+            const int lo = (int)floor(u) - half - 1, hi = (int)ceil(u) + half + 1;
+            around.push_back(make_int2(lo, hi));
+            around.push_back(make_int2(-hi, -lo));
+        }
+        // a window past half a turn goes on at the other end: unrolled, merged
+        std::sort(around.begin(), around.end(), [](int2 a, int2 b) { return a.x < b.x; });
+        for (const int2& r : around) {
+            if ((int)wins.size() > N.win_off[w] && r.x <= wins.back().y + 1)
+                wins.back().y = std::max(wins.back().y, r.y);
+            else
+                wins.push_back(r);
+        }
+        if ((int)wins.size() > N.win_off[w]) {
+            int2& first = wins[N.win_off[w]];
+            if ((int)wins.size() > N.win_off[w] + 1 && wins.back().y >= first.x + n) {   // they meet
+                first.x = wins.back().x - n;
+                wins.pop_back();
+            }
+            if (first.y - first.x >= n) first.y = first.x + n - 1;
+        }
         N.reach_lo[w] = h->reach_lo[w];
         N.reach_hi[w] = h->reach_hi[w];
     }
+    N.win_off[m.W] = (int)wins.size();
+    for (int w = m.W; w < 4; ++w) N.win_off[w + 1] = N.win_off[w];
+    N.slots = (int)slots.size();
     N.nl_pad = (N.nl + 31) & ~31;
+    if (N.tile_slots > 256) return LMMEW_OK;   // (k_ang_bins stages them)
     if (N.nl > 6000 || N.nk > 1024 || N.nn > 32768 || (int64_t)m.np * N.nn >= (int64_t(1) << 31))
         return LMMEW_OK;
     const size_t pair_bytes = (12 + 4 * (size_t)m.W) * (size_t)pairs;
@@ -1519,6 +1773,9 @@ int build_nodes(lm_handle* h) {
         T.grp_pt = bump<int>(p, grp_pt.size());
         T.k_of_l = bump<int2>(p, bands.size());
         T.l_of_k = T.k_of_l + lt;
+        T.slot = bump<NodeSlot>(p, slots.size());
+        T.slot_start = bump<int>(p, slot_start.size());
+        T.win = bump<int2>(p, wins.size());
         d_run = bump<int2>(p, run.size());
         d_most = bump<int>(p, 2);
         host_bytes = (size_t)(p - base);
@@ -1561,6 +1818,9 @@ int build_nodes(lm_handle* h) {
     put(T.dec_start, dec_start.data(), 4 * dec_start.size());
     put(T.grp_pt, grp_pt.data(), 4 * grp_pt.size());
     put(T.k_of_l, bands.data(), 8 * bands.size());
+    put(T.slot, slots.data(), sizeof(NodeSlot) * slots.size());
+    put(T.slot_start, slot_start.data(), 4 * slot_start.size());
+    put(T.win, wins.data(), 8 * wins.size());
     put(d_run, run.data(), 8 * run.size());
     LMMEW_CUDA(cudaMemcpy(h->d_node_tables, blob.data(), host_bytes, cudaMemcpyHostToDevice));
     int rc = node_kernel_attrs();
@@ -1628,38 +1888,46 @@ int build_nodes(lm_handle* h) {
 
 size_t node_angle_bytes(const lm_handle* h) {
     const NodeConst& N = h->nodes;
-    return bump_bytes(sizeof(float) * (size_t)h->mc.npc * N.nb_max * N.nm_pad) +
+    return bump_bytes(sizeof(float) * (size_t)h->mc.np * N.slots) +
+           bump_bytes(sizeof(float) * (size_t)h->mc.npc * N.nb_max * N.nm_pad) +
            bump_bytes(sizeof(float) * (size_t)h->mc.B * N.nl_pad) +
            bump_bytes(sizeof(float) * (size_t)h->mc.B * N.nk_pad) +
            bump_bytes(sizeof(float) * (size_t)h->mc.B * N.W);
 }
 
-// The image on the direction nodes of every scatter point.
-int node_spread(lm_handle* h, const float* lam_v, float* H, cudaStream_t st) {
-    NodeParams P = node_params(h, 0, 1, 0);
+// The image on the direction nodes of every scatter point (H null: not again),
+// and on the slots of angles a0 + i a_step.
+int node_spread(lm_handle* h, const float* lam_v, float* H, int a0, int a_step, int angles, float* side,
+                cudaStream_t st) {
+    NodeParams P = node_params(h, a0, a_step, angles);
     P.lam = lam_v;
     P.H = H;
+    P.side = side;
     int tiles = 0;
     for (int w = 0; w < P.N.W; ++w) tiles += (P.N.n_dir[w] + kSpreadOut - 1) / kSpreadOut;
     int rc = prof_start(h, st);
     if (rc != LMMEW_OK) return rc;
-    const int units = h->mc.np * tiles;
-    k_ang_spread<<<(unsigned)((units + kSpreadWarps - 1) / kSpreadWarps), 32 * kSpreadWarps, 0, st>>>(
-        P, tiles, units);
+    const int units = H ? h->mc.np * tiles : 0;
+    const int64_t sides = (int64_t)angles * h->mc.np * P.N.slots;
+    const int64_t blocks = (units + kSpreadWarps - 1) / kSpreadWarps +
+                           (sides + 32 * kSpreadWarps - 1) / (32 * kSpreadWarps);
+    if (blocks == 0) return LMMEW_OK;
+    k_ang_spread<<<(unsigned)blocks, 32 * kSpreadWarps, 0, st>>>(P, tiles, units);
     ++h->launches;
     LMMEW_CUDA(cudaGetLastError());
-    return prof_stop(h, (double)h->mc.W * h->mc.nq * h->mc.np, st);
+    return prof_stop(h, H ? (double)h->mc.W * h->mc.nq * h->mc.np : 0.0, st);
 }
 
 // F and the unscattered sums of angles a0 + i a_step, i < angles.
-int node_forward(lm_handle* h, const float* lam_v, const float* H, int a0, int a_step, int angles,
-                 float* dbp, float* DB, float* F, float* Pr, cudaStream_t st) {
+int node_forward(lm_handle* h, const float* lam_v, const float* H, const float* side, int a0, int a_step,
+                 int angles, float* dbp, float* DB, float* F, float* Pr, cudaStream_t st) {
     if (angles <= 0) return LMMEW_OK;
     const ModelConst& m = h->mc;
     const NodeConst& N = h->nodes;
     NodeParams P = node_params(h, a0, a_step, angles);
     P.lam = lam_v;
     P.H = const_cast<float*>(H);
+    P.side = const_cast<float*>(side);
     P.dbp = dbp;
     P.DB = DB;
     P.F = F;
@@ -1667,7 +1935,8 @@ int node_forward(lm_handle* h, const float* lam_v, const float* H, int a0, int a
     constexpr int kTile = kOffThreads * kOffPer;
     int tiles = 0;
     for (int w = 0; w < N.W; ++w) tiles += (N.m_count[w] + kTile - 1) / kTile;
-    k_ang_bins<<<(unsigned)(tiles * m.npc * angles), kOffThreads, 0, st>>>(P, tiles);
+    k_ang_bins<<<(unsigned)(tiles * m.npc * angles), kOffThreads, sizeof(float) * kPC * N.tile_slots, st>>>(
+        P, tiles);
     const int rows = angles * m.B;
     k_node_bins<<<(unsigned)(rows + (rows * m.W + kRowThreadsN / 32 - 1) / (kRowThreadsN / 32)), kRowThreadsN,
                   sizeof(float) * N.nm_pad, st>>>(P);
@@ -1710,7 +1979,7 @@ int node_back_parts(const lm_handle* h, int angles) {
 // Back projection of the node weights of angles a0 + i a_step: the paths' values
 // and the unscattered part of every angle.
 int node_back(lm_handle* h, int a0, int a_step, int angles, const float* V, const float* PV,
-              float* VG, float* psi, float* T, float* val, float* part_prim, cudaStream_t st) {
+              float* VG, float* psi, float* T, float* side, float* val, float* part_prim, cudaStream_t st) {
     const ModelConst& m = h->mc;
     const NodeConst& N = h->nodes;
     NodeParams P = node_params(h, a0, a_step, angles);
@@ -1719,6 +1988,7 @@ int node_back(lm_handle* h, int a0, int a_step, int angles, const float* V, cons
     P.VG = VG;
     P.psi = psi;
     P.T = T;
+    P.side = side;
     P.val = val;
     P.part_prim = part_prim;
     const int rows = angles * m.B;
@@ -1732,7 +2002,9 @@ int node_back(lm_handle* h, int a0, int a_step, int angles, const float* V, cons
     P.parts = node_back_parts(h, angles);
     const size_t one = sizeof(float) * kBackWarps * (size_t)N.nbg_max * kGroup;   // staged per angle
     const int batch = (int)std::max<size_t>(1, std::min<size_t>(kBackAngles, kBackStage / one));
-    k_ang_back<<<dim3((unsigned)(tiles * ((groups + kBackWarps - 1) / kBackWarps)), P.parts),
+    const int64_t side_threads = (int64_t)N.slots * angles * groups * kGroup;
+    const unsigned side_blocks = (unsigned)((side_threads + 32 * kBackWarps - 1) / (32 * kBackWarps));
+    k_ang_back<<<dim3((unsigned)(tiles * ((groups + kBackWarps - 1) / kBackWarps)) + side_blocks, P.parts),
                  32 * kBackWarps, batch * one, st>>>(P, tiles, groups, batch);
     int rc = prof_start(h, st);
     if (rc != LMMEW_OK) return rc;
