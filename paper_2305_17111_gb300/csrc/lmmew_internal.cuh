@@ -91,34 +91,35 @@ struct EnergyClasses {
 };
 
 // Nodes of the dense-list projections (nodes.cu): t(E) = 2 sqrt(E) / kappa,
-// recorded-energy nodes k_first + k (8 per unit of t) and, per line,
-// scattered-energy nodes l_first + i (16 per unit), direction nodes (n_dir
+// recorded-energy nodes k_first + k (9 per unit of t or more) and, per line,
+// scattered-energy nodes l_first + i (14 per unit or more), direction nodes (n_dir
 // around the circle) and offsets from the detector direction (m_count on a half
 // circle), the lines one after the other.
 struct NodeConst {
     int W;
+    int per_l, per_k;          // nodes per unit of t
     int nk, nk_pad, k_first;
     int nl, nl_pad;
     int l_first[4], l_count[4], l_off[4];
     int n_dir[4], n_off[4], nn;
+    int angle_step[4];         // direction nodes from one detector angle to the next
     int m_count[4], m_off[4], nm_pad;
     int start_ints;            // path starts per point: n_dir + 2 per line
     float ck, ck_lo;           // node of a recorded energy = (ck + ck_lo) sqrt(E)
     float reach_lo[4], reach_hi[4];   // recorded energies single scatter of the line can have
     int nb_max, nbg_max;       // most bins 32 ordered, 8 neighbouring scatter points reach
     // attenuation knots inside each line's E': offsets (in direction nodes,
-    // ascending), the slots of the nodes beside them (see nodes.cu)
+    // ascending), the slots of the nodes beside them and the windows of centres
+    // (from the detector direction) whose taps can cross one (see nodes.cu)
     int kinks[4], slots, tile_slots;
     float kink[4][LMMEW_MAX_KNOTS];
-    int win_off[5];            // windows of each line's offsets near a knot
+    int win_off[5], slot_off[5];
 };
-// A direction offset seen from the other side of a knot.
+// A direction offset (m_off + m) with log2(e) mu_water(E') continued from the
+// other side of a knot.
 struct NodeSlot {
-    int offset;                // of all lines' (m_off + m)
-    int branch;                // the paths' side: number of knots below their offset
-    int d0, d1;                // centres such paths can have, from the offset's node on
-    float lo, hi;              // their offsets: lo < u <= hi
-    float mu;                  // log2(e) mu_water(E') continued from that side
+    int offset, side;          // side: number of knots below the offsets it is for
+    float mu;
 };
 // Their device tables (one region; see NodeParams in nodes.cu).
 struct NodeTables {
@@ -126,6 +127,7 @@ struct NodeTables {
     int *psi_l, *dec_start, *dec_m, *rank, *path_start, *path_q, *path_of, *grp_pt;
     int2 *k_of_l, *l_of_k, *chunk_bins, *grp_bins, *win;
     int* slot_start;
+    short* slot_at;
     NodeSlot* slot;
     uint32_t* fix;
 };

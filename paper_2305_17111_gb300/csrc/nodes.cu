@@ -45,9 +45,12 @@
 //   back      Y[a][p][z] = (e^{-mu_z gamma_p} - e^{-mu(m) gamma_p}) sum_b C_p(b) PSI[b][m]   k_ang_back
 //             out[q]    += sum_p B_{qp} sum_{n beyond the knot} L_n(phi_qp) Y         k_ang_paths
 //
-// Interpolation errors are near 1e-8 of an event's value, below the FP32
-// rounding of the sums; everything is FP32 with fixed-order sums, the voxel sums
-// FP64.
+// Interpolation errors are below the FP32 rounding of the sums up to 6 sigma from
+// every reachable energy (1e-7 of a path's value there) and 3e-6 at the 8 sigma
+// where the reach ends, as far as the rows' exponents are good there; everything
+// is FP32 with fixed-order sums, the voxel sums FP64.  (7, 7 and 12 taps at 18
+// direction nodes per sigma, 16 scattered- and 8 recorded-energy nodes were
+// 2.4e-4 off at 8 sigma, at a higher cost: more nodes cost more than more taps.)
 //
 // Measured (864 voxels and 864 points, 3 lines, 60 angles of 64 bins; times
 // below that name no size are this model's): a forward projection of 100 000
@@ -69,13 +72,15 @@
 namespace lmmew {
 namespace {
 
-constexpr int kTapsL = 7;          // taps of the scattered-energy nodes
-constexpr int kPsiStride = 8;      // a direction offset's weights for them, padded
-constexpr int kPerUnitL = 16;      // nodes per unit of t
-constexpr int kTapsK = 12;         // taps of the recorded-energy nodes
-constexpr int kPerUnitK = 8;
-constexpr double kBandSigmas = 9.0;   // G kept within this many sigma (reach 8 plus the stencils)
-constexpr int kTapsN = 7;          // taps of the direction nodes
+constexpr int kTapsL = 11;         // taps of the scattered-energy nodes
+constexpr int kPsiStride = 12;     // a direction offset's weights for them, padded
+constexpr int kPerUnitL = 14;      // nodes per unit of t, at least
+constexpr int kTapsK = 16;         // taps of the recorded-energy nodes
+constexpr int kPerUnitK = 9;
+constexpr double kBandSigmas = 10.2;  // G kept within this many sigma: at 8 sigma from the nearest path the
+                                      // dropped ones are 6e-10 of it each
+constexpr int kTapsN = 9;          // taps of the direction nodes
+constexpr double kPerSigmaN = 17.0;   // direction nodes per sigma, at least
 constexpr int kGroup = 8;          // scatter points per block of k_ang_back
 constexpr int kBinsT = 16;         // detector bins per pass of k_ang_bins
 constexpr int kValueRows = 8;      // (angle, bin) rows per block of k_node_values / _unvalues
@@ -89,18 +94,21 @@ __device__ __forceinline__ float ex2f(float x) {
 }
 __device__ __forceinline__ f32x2 pk1(float v) { return pk(v, v); }
 
-// The 7 Lagrange weights at distance s from the centre node, times v.
-__device__ __forceinline__ void lagrange7(float s, float v, float (&w)[7]) {
-    const float q = s * s, a1 = q - 1.f, a2 = q - 4.f, a3 = q - 9.f, sv = s * v, a12 = a1 * a2;
-    const float m1 = sv * (a2 * a3) * (1.f / 48.f), m2 = sv * (a1 * a3) * (-1.f / 120.f);
-    const float m3 = sv * a12 * (1.f / 720.f);
-    w[3] = a12 * a3 * (v * (-1.f / 36.f));
-    w[4] = fmaf(m1, s, m1);
-    w[2] = fmaf(m1, s, -m1);
-    w[5] = fmaf(m2, s, 2.f * m2);
-    w[1] = fmaf(m2, s, -2.f * m2);
-    w[6] = fmaf(m3, s, 3.f * m3);
-    w[0] = fmaf(m3, s, -3.f * m3);
+// The 9 Lagrange weights at distance s from the centre node, times v.
+__device__ __forceinline__ void lagrange9(float s, float v, float (&w)[9]) {
+    const float q = s * s, a1 = q - 1.f, a2 = q - 4.f, a3 = q - 9.f, a4 = q - 16.f, sv = s * v;
+    const float a12 = a1 * a2, a34 = a3 * a4;
+    const float m1 = sv * (a2 * a34) * (-1.f / 720.f), m2 = sv * (a1 * a34) * (1.f / 1440.f);
+    const float m3 = sv * (a12 * a4) * (-1.f / 5040.f), m4 = sv * (a12 * a3) * (1.f / 40320.f);
+    w[4] = a12 * a34 * (v * (1.f / 576.f));
+    w[5] = fmaf(m1, s, m1);
+    w[3] = fmaf(m1, s, -m1);
+    w[6] = fmaf(m2, s, 2.f * m2);
+    w[2] = fmaf(m2, s, -2.f * m2);
+    w[7] = fmaf(m3, s, 3.f * m3);
+    w[1] = fmaf(m3, s, -3.f * m3);
+    w[8] = fmaf(m4, s, 4.f * m4);
+    w[0] = fmaf(m4, s, -4.f * m4);
 }
 
 // Nearest of n nodes to a direction (in 2^-32 turns) and the distance from it
@@ -112,37 +120,38 @@ __device__ __forceinline__ float direction_pos(uint32_t fix, int n, int* c) {
     return (float)f * 2.3283064365386963e-10f;
 }
 
-// The 12 Lagrange weights at position f in [0, 1) between nodes 5 and 6,
+// The 16 Lagrange weights at position f in [0, 1) between nodes 7 and 8,
 // normalised to sum 1 (their common rounding cancels).
-__device__ __forceinline__ void lagrange12(float f, float (&w)[12]) {
-    // nodes at +-1/2, +-3/2, .. +-11/2 from the middle, x = f - 1/2;
+__device__ __forceinline__ void lagrange16(float f, float (&w)[16]) {
+    // nodes at +-1/2, +-3/2, .. +-15/2 from the middle, x = f - 1/2;
     // 1 / prod_{j != i} (x_i - x_j) for the pair at +-(i + 1/2)
-    constexpr float c[6] = {-1.f / 86400.f, 1.f / 120960.f,   -1.f / 241920.f,
-                            1.f / 725760.f, -1.f / 3628800.f, 1.f / 39916800.f};
+    constexpr float c[8] = {-1.f / 203212800.f,  1.f / 261273600.f,   -1.f / 435456000.f,
+                            1.f / 958003200.f,   -1.f / 2874009600.f, 1.f / 12454041600.f,
+                            -1.f / 87178291200.f, 1.f / 1307674368000.f};
     const float x = f - 0.5f, q = x * x;
-    float a[6], pre[6], suf[6];
+    float a[8], pre[8], suf[8];
 #pragma unroll
-    for (int i = 0; i < 6; ++i) a[i] = q - (i + 0.5f) * (i + 0.5f);
+    for (int i = 0; i < 8; ++i) a[i] = q - (i + 0.5f) * (i + 0.5f);
     pre[0] = 1.f;
-    suf[5] = 1.f;
+    suf[7] = 1.f;
 #pragma unroll
-    for (int i = 1; i < 6; ++i) pre[i] = pre[i - 1] * a[i - 1];
+    for (int i = 1; i < 8; ++i) pre[i] = pre[i - 1] * a[i - 1];
 #pragma unroll
-    for (int i = 4; i >= 0; --i) suf[i] = suf[i + 1] * a[i + 1];
+    for (int i = 6; i >= 0; --i) suf[i] = suf[i + 1] * a[i + 1];
     float sum = 0.f;
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
+    for (int i = 0; i < 8; ++i) {
         const float m = pre[i] * suf[i] * c[i], n = m * (i + 0.5f);
-        w[6 + i] = fmaf(m, x, n);        // node at +(i + 1/2): factor (x + (i + 1/2))
-        w[5 - i] = -fmaf(m, x, -n);
-        sum += w[6 + i] + w[5 - i];
+        w[8 + i] = fmaf(m, x, n);        // node at +(i + 1/2): factor (x + (i + 1/2))
+        w[7 - i] = -fmaf(m, x, -n);
+        sum += w[8 + i] + w[7 - i];
     }
     const float inv = 1.f / sum;
 #pragma unroll
-    for (int i = 0; i < 12; ++i) w[i] *= inv;
+    for (int i = 0; i < 16; ++i) w[i] *= inv;
 }
 
-// Position of a recorded energy on its nodes, u = ck sqrt(E): first of its 12
+// Position of a recorded energy on its nodes, u = ck sqrt(E): first of its 16
 // taps (local index) and the fraction.  ck comes in two parts and the square
 // root's rounding is taken out to first order: the fraction is good to its
 // own FP32 rounding, where u's would shift the event by 4e-6 sigma.
@@ -150,7 +159,7 @@ __device__ __forceinline__ float energy_pos(const NodeConst& N, float e, int* k)
     const float r = sqrtf(e);
     const float j = floorf(N.ck * r);
     const float lo = e > 0.f ? 0.5f * fmaf(-r, r, e) / r : 0.f;
-    *k = min(max((int)j - 5 - N.k_first, 0), N.nk - kTapsK);
+    *k = min(max((int)j - (kTapsK / 2 - 1) - N.k_first, 0), N.nk - kTapsK);
     return fmaf(N.ck, r, -j) + fmaf(N.ck_lo, r, N.ck * lo);
 }
 __device__ __forceinline__ bool in_reach(const NodeConst& N, float e) {
@@ -165,8 +174,8 @@ __global__ void k_node_matrix(const NodeConst N, double kappa, float* g, float* 
     const int l = i / N.nk_pad, k = i % N.nk_pad;
     int w = 0;
     while (w + 1 < N.W && l >= N.l_off[w + 1]) ++w;
-    const double xl = 0.5 * kappa * (N.l_first[w] + (l - N.l_off[w])) / kPerUnitL;   // sqrt(E')
-    const double xk = 0.5 * kappa * (N.k_first + k) / kPerUnitK;
+    const double xl = 0.5 * kappa * (N.l_first[w] + (l - N.l_off[w])) / N.per_l;   // sqrt(E')
+    const double xk = 0.5 * kappa * (N.k_first + k) / N.per_k;
     const double d = (xk * xk - xl * xl) / (kappa * xl);
     const bool real = l - N.l_off[w] < N.l_count[w] && k < N.nk;
     const float v = real && fabs(d) <= kBandSigmas ? (float)exp(-0.5 * d * d) : 0.f;
@@ -189,7 +198,7 @@ struct NodeParams {
     const int* inv;          // [A][np] point of each slot of an angle's point order
     const float* gamma;      // [A][np] line integral from each point to the detector, cm
     const float* mu;         // [nm_pad] log2(e) mu_water(E') of the direction offsets
-    const int* psi_l;        // [nm_pad] first of the 7 nodes l of an offset's E'
+    const int* psi_l;        // [nm_pad] first of the 11 nodes l of an offset's E'
     const float* psi_w;      // [nm_pad][kPsiStride] their weights, times f
     const int* dec_start;    // [nl_pad / 32 + 1] the same by 32 nodes l: offsets m and weights
     const int* dec_m;
@@ -201,7 +210,10 @@ struct NodeParams {
     const int* path_start;   // [np][start_ints] per line: first path of each centre node
     const NodeSlot* slot;    // nodes beside a knot, seen from its other side
     const int* slot_start;   // [nm_pad + 1] the slots of each offset
-    const int2* win;         // per line, windows of centres whose taps can cross a knot
+    const short* slot_at;    // [kinks + 1][nm_pad] slot of an offset for paths of a side (-1: none)
+    const int2* win;         // per line, disjoint windows of c - s (centre, detector direction; both
+                             // ends of the circle apart) whose taps can cross a knot
+    float inv_step[4];       // 1 / direction nodes from one angle of the launch to the next
     const int* grp_pt;       // [groups][8] neighbouring points (-1: none)
     const int2* grp_bins;    // [A][groups] bins they reach
     const float* grp_c;      // [A][groups][nbg_max][8] their collimator values
@@ -223,85 +235,143 @@ struct NodeParams {
     float* part_prim;        // [angles][nq_pad]
 };
 
-// The weighted taps on a slot's node of those paths of point p that lie on the
-// slot's side of the knot, for the detector direction of angle a.
-__device__ __forceinline__ float slot_taps(const NodeParams& P, const NodeSlot& z, int p, int a) {
+// Side of the knots a path lies on, r + f nodes from the detector direction: the
+// number of knots below its offset.
+__device__ __forceinline__ int side_of_knots(const NodeConst& N, int w, int r, float f) {
+    const int n = N.n_dir[w];
+    if (2 * r > n) r -= n;
+    if (2 * r < -n) r += n;
+    float u = fabsf((float)r + f);
+    if (2.f * u > (float)n) u = (float)n - u;
+    int b = 0;
+    while (b < N.kinks[w] && u > N.kink[w][b]) ++b;
+    return b;
+}
+// Offset (of all lines) of the node r nodes from the detector direction.
+__device__ __forceinline__ int offset_of(const NodeConst& N, int w, int r) {
+    const int n = N.n_dir[w];
+    int m = abs(r);
+    if (m >= n) m -= n;
+    if (2 * m > n) m = n - m;
+    return N.m_off[w] + m;
+}
+
+// The slots' weighted taps of one (angle, point, line), by a warp: 32 paths of the
+// line's windows at a time, a lane per path, leave their taps in shared memory;
+// then a lane per slot (the 32 paths shared between as many lanes as fit) adds
+// those on its node from paths on its side, in path order.  (A thread per slot
+// that walks its paths takes 28 us more for 60 angles, a thread for all slots
+// 290 us instead of 10 at 3464 voxels: both wait for one path after the other.)
+constexpr int kMostWindows = 64;   // of a line: 4 per knot
+constexpr int kSlotWords = (kTapsN + 2) * 32 + 2 * kMostWindows;   // a warp's: taps, positions, sides, runs
+__device__ __forceinline__ void slot_taps(const NodeParams& P, int ai, int p, int w, float* sh) {
     constexpr int kHalf = kTapsN / 2;
-    int w = 0;
-    while (w + 1 < P.N.W && z.offset >= P.N.m_off[w + 1]) ++w;
-    const int n = P.N.n_dir[w], m = z.offset - P.N.m_off[w], s = (int)((int64_t)a * n / P.A);
+    const int lane = threadIdx.x & 31;
+    const int n = P.N.n_dir[w], s = (P.a0 + ai * P.a_step) * P.N.angle_step[w];
     const int* st = P.path_start + (size_t)p * P.N.start_ints + P.N.n_off[w] + 2 * w;
     const uint32_t* fix = P.fix + (size_t)p * P.nq;
     const int* pq = P.path_q + (size_t)p * P.nq;
     const float* pb = P.path_b + ((size_t)w * P.np + p) * P.nq;
-    float sum = 0.f;
-    for (int sign = 1; sign >= -1; sign -= 2) {
-        int j = s + sign * m;                       // the node, in [0, n)
-        if (j >= n) j -= n;
-        if (j < 0) j += n;
-        if (sign < 0 && (2 * m == n || m == 0)) break;
-        // centres lo .. hi: one run of the point's directions, two where the circle
-        // closes (centres 0 and n are the same node)
-        int lo = j + (sign > 0 ? z.d0 : -z.d1), hi = j + (sign > 0 ? z.d1 : -z.d0);
-        if (hi < 0) {
-            lo += n;
-            hi += n;
-        } else if (lo >= n) {
-            lo -= n;
-            hi -= n;
-        }
-        const bool closes = lo <= 0 || hi >= n;
-        for (int part = 0; part < (closes ? 2 : 1); ++part) {
-            const int ca = !closes ? lo : part == 0 ? (lo <= 0 ? lo + n : lo) : 0;
-            const int cb = !closes ? hi : part == 0 ? n : (hi >= n ? hi - n : hi);
-            for (int r = st[ca]; r < st[cb + 1]; ++r) {
-                int c;
-                const float f = direction_pos(fix[r], n, &c);
-                int d = c - j;                      // centre past the node
-                if (2 * d > n) d -= n;
-                if (2 * d < -n) d += n;
-                float u = fabsf((float)(sign * m + d) + f);
-                if (2.f * u > (float)n) u = (float)n - u;
-                if (!(u > z.lo && u <= z.hi)) continue;
-                float x[kTapsN];
-                lagrange7(f, pb[r] * P.lam[pq[r]], x);
-#pragma unroll
-                for (int k = 0; k < kTapsN; ++k)
-                    if (k == kHalf - d) sum += x[k];
-            }
-        }
+    int* pos = reinterpret_cast<int*>(sh + kTapsN * 32);
+    int* on = pos + 32;
+    // the windows' runs of directions, a lane each
+    const int windows = P.N.win_off[w + 1] - P.N.win_off[w];
+    int2* run = reinterpret_cast<int2*>(on + 32);
+    for (int k = lane; k < windows; k += 32) {
+        const int2 win = P.win[P.N.win_off[w] + k];
+        const int c0 = max(s + win.x, 0), c1 = min(s + win.y, n);
+        run[k] = c0 <= c1 ? make_int2(st[c0], st[c1 + 1]) : make_int2(0, 0);
     }
-    return sum;
+    __syncwarp();
+    for (int z0 = P.N.slot_off[w]; z0 < P.N.slot_off[w + 1]; z0 += 32) {
+        const int count = min(32, P.N.slot_off[w + 1] - z0), shares = 32 / count;
+        const int z = z0 + lane % count, share = lane / count;
+        const int m = P.slot[z].offset - P.N.m_off[w], side = P.slot[z].side;
+        float sum = 0.f;
+        int k = 0, r = 0, r1 = 0;
+        while (true) {
+            int fill = 0, mine = -1;
+            while (fill < 32) {
+                if (r >= r1) {          // the next window's run of directions
+                    if (k == windows) break;
+                    r = run[k].x;
+                    r1 = run[k].y;
+                    ++k;
+                    continue;
+                }
+                const int take = min(32 - fill, r1 - r);
+                if (lane >= fill && lane < fill + take) mine = r + lane - fill;
+                r += take;
+                fill += take;
+            }
+            if (fill == 0) break;
+            __syncwarp();
+            if (mine >= 0) {
+                int c;
+                const float f = direction_pos(fix[mine], n, &c);
+                float x[kTapsN];
+                lagrange9(f, pb[mine] * P.lam[pq[mine]], x);
+#pragma unroll
+                for (int t = 0; t < kTapsN; ++t) sh[t * 32 + lane] = x[t];
+                int d = c - s;          // in (-n / 2, n / 2]
+                if (2 * d > n) d -= n;
+                if (2 * d <= -n) d += n;
+                pos[lane] = d;
+                on[lane] = side_of_knots(P.N, w, d, f);
+            }
+            __syncwarp();
+            if (share < shares)
+                for (int i = share; i < fill; i += shares) {
+                    if (on[i] != side) continue;
+                    // the path's tap on node s + m, and on s - m where that is another
+                    int t = m - pos[i] + kHalf;
+                    if (t >= n) t -= n;
+                    if ((unsigned)t < kTapsN) sum += sh[t * 32 + i];
+                    t = -m - pos[i] + kHalf;
+                    if (t < 0) t += n;
+                    if ((unsigned)t < kTapsN && m > 0 && 2 * m != n) sum += sh[t * 32 + i];
+                }
+        }
+        float all = sum;
+        for (int j = 1; j < shares; ++j) all += __shfl_down_sync(0xffffffffu, sum, j * count);
+        if (lane < count) P.side[((size_t)ai * P.np + p) * P.N.slots + z] = all;
+    }
 }
 
-// H: a warp per (point, line, 122 direction nodes).  The paths centred on the
-// tile's nodes and the 3 on either side are one run of the point's directions
+// H: a warp per (point, line, 120 direction nodes).  The paths centred on the
+// tile's nodes and the 4 on either side are one run of the point's directions
 // (and a second one where the circle closes).  32 of them at a time form their
-// 7 weighted taps, a lane per path; a segmented scan sums those of equal centre,
+// 9 weighted taps, a lane per path; a segmented scan sums those of equal centre,
 // and the last of each adds them to the centre's sums.  At the end each node
-// collects its taps from the 7 centres around it.  No two lanes add to one
+// collects its taps from the 9 centres around it.  No two lanes add to one
 // place, and every sum has its order.  Bound by instruction issue (66 %) once
 // the loads are a group ahead: 37 us; 47 us with a lane per centre, which
 // waits on three dependent loads per path, 42 us with a block per 122 nodes.
 // Where a centre has more than kSpreadDense paths the scan's steps cost more
 // than those waits, and a lane takes a centre's paths: 80 us instead of 118 us
 // at 3464 voxels (11, 6 and 3 paths a centre; limits of 2 and 4 are equal
-// there, 1 costs 83 us).  The blocks past those form the slots' taps, a thread
-// per (angle, point, slot).
-constexpr int kSpreadDense = 4, kSpreadWarps = 4, kSpreadCentres = 128, kSpreadOut = kSpreadCentres - 6;
-__global__ void __launch_bounds__(32 * kSpreadWarps) k_ang_spread(const NodeParams P, int tiles, int units) {
-    __shared__ __align__(16) float taps[kSpreadWarps][7][kSpreadCentres];
-    const int unit_blocks = (units + kSpreadWarps - 1) / kSpreadWarps;
-    if ((int)blockIdx.x >= unit_blocks) {
-        const int64_t i = (int64_t)(blockIdx.x - unit_blocks) * (32 * kSpreadWarps) + threadIdx.x;
-        if (i >= (int64_t)P.angles * P.np * P.N.slots) return;
-        const int64_t ap = i / P.N.slots;
-        P.side[i] = slot_taps(P, P.slot[i - ap * P.N.slots], (int)(ap % P.np), P.a0 + (int)(ap / P.np) * P.a_step);
+// there, 1 costs 83 us).  The first blocks form the slots' taps, a warp per
+// (angle, point, line with a knot).
+constexpr int kSpreadDense = 4, kSpreadWarps = 4, kSpreadCentres = 128, kSpreadOut = kSpreadCentres - (kTapsN - 1);
+__global__ void __launch_bounds__(32 * kSpreadWarps) k_ang_spread(const NodeParams P, int tiles, int units,
+                                                                 int side_blocks) {
+    __shared__ __align__(16) float taps[kSpreadWarps][kTapsN][kSpreadCentres];
+    if ((int)blockIdx.x < side_blocks) {
+        static_assert(kSlotWords <= kTapsN * kSpreadCentres, "the slots' taps lie in the taps' place");
+        int i = blockIdx.x * kSpreadWarps + (threadIdx.x >> 5);
+        for (int w = 0; w < P.N.W; ++w) {
+            if (P.N.kinks[w] == 0) continue;
+            if (i < P.angles * P.np) {
+                slot_taps(P, i / P.np, i % P.np, w, &taps[threadIdx.x >> 5][0][0]);
+                return;
+            }
+            i -= P.angles * P.np;
+        }
         return;
     }
-    const int lane = threadIdx.x & 31, unit = blockIdx.x * kSpreadWarps + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31, unit = (blockIdx.x - side_blocks) * kSpreadWarps + (threadIdx.x >> 5);
     if (unit >= units) return;
-    float (&tap)[7][kSpreadCentres] = taps[threadIdx.x >> 5];
+    float (&tap)[kTapsN][kSpreadCentres] = taps[threadIdx.x >> 5];
     const int p = unit / tiles;
     int tile = unit % tiles, w = 0;
     while (tile >= (P.N.n_dir[w] + kSpreadOut - 1) / kSpreadOut) {
@@ -309,7 +379,7 @@ __global__ void __launch_bounds__(32 * kSpreadWarps) k_ang_spread(const NodePara
         ++w;
     }
     const int n = P.N.n_dir[w], n0 = tile * kSpreadOut;
-    const int u0 = n0 - 3, u1 = min(n0 + kSpreadOut + 2, n + 2);   // the tile's centres
+    const int u0 = n0 - kTapsN / 2, u1 = min(n0 + kSpreadOut, n) + kTapsN / 2 - 1;   // the tile's centres
     // first path of each centre, centres 0 .. n (n: a full turn, node 0 again)
     const int* st = P.path_start + (size_t)p * P.N.start_ints + P.N.n_off[w] + 2 * w;
     const uint32_t* fix = P.fix + (size_t)p * P.nq;
@@ -319,16 +389,16 @@ __global__ void __launch_bounds__(32 * kSpreadWarps) k_ang_spread(const NodePara
     if (dense) {
         for (int i = lane; i <= u1 - u0; i += 32) {
             const int u = u0 + i, c = u < 0 ? u + n : u > n ? u - n : u;
-            float g[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            float g[kTapsN] = {};
             int r = st[c], re = st[c + 1], more = c == 0 ? n : c == n ? 0 : -1;
             while (true) {
                 for (; r < re; ++r) {
                     int cc;
                     const float s = direction_pos(fix[r], n, &cc);
-                    float x[7];
-                    lagrange7(s, pb[r] * P.lam[pq[r]], x);
+                    float x[kTapsN];
+                    lagrange9(s, pb[r] * P.lam[pq[r]], x);
 #pragma unroll
-                    for (int k = 0; k < 7; ++k) g[k] += x[k];
+                    for (int k = 0; k < kTapsN; ++k) g[k] += x[k];
                 }
                 if (more < 0) break;
                 r = st[more];
@@ -336,10 +406,10 @@ __global__ void __launch_bounds__(32 * kSpreadWarps) k_ang_spread(const NodePara
                 more = -1;
             }
 #pragma unroll
-            for (int k = 0; k < 7; ++k) tap[k][i] = g[k];
+            for (int k = 0; k < kTapsN; ++k) tap[k][i] = g[k];
         }
     } else {
-        for (int i = lane; i < 7 * kSpreadCentres / 4; i += 32)
+        for (int i = lane; i < kTapsN * kSpreadCentres / 4; i += 32)
             reinterpret_cast<float4*>(tap)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         __syncwarp();
     }
@@ -382,10 +452,10 @@ __global__ void __launch_bounds__(32 * kSpreadWarps) k_ang_spread(const NodePara
             const uint32_t f = f1;
             const float v = b1 * v1;
             ahead(r + 32);
-            float x[7];
+            float x[kTapsN];
             int c;
             const float s = direction_pos(f, n, &c);
-            lagrange7(s, v, x);
+            lagrange9(s, v, x);
             if (r >= r1) c = -1;
             const int before = __shfl_up_sync(0xffffffffu, c, 1);
             const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || c != before);
@@ -393,21 +463,21 @@ __global__ void __launch_bounds__(32 * kSpreadWarps) k_ang_spread(const NodePara
             const int most = __reduce_max_sync(0xffffffffu, back);
             for (int o = 1; o <= most; o <<= 1)
 #pragma unroll
-                for (int k = 0; k < 7; ++k) {
+                for (int k = 0; k < kTapsN; ++k) {
                     const float y = __shfl_up_sync(0xffffffffu, x[k], o);
                     if (back >= o) x[k] += y;
                 }
             __syncwarp();
             if (c >= 0 && (lane == 31 || (heads >> (lane + 1) & 1u)))
 #pragma unroll
-                for (int k = 0; k < 7; ++k) tap[k][c - shift - u0] += x[k];
+                for (int k = 0; k < kTapsN; ++k) tap[k][c - shift - u0] += x[k];
         }
     }
     __syncwarp();
     for (int i = lane; i < kSpreadOut && n0 + i < n; i += 32) {
-        float h = 0.f;                     // centre n0 + i + j - 3 is place i + j, and node n0 + i its tap 6 - j
+        float h = 0.f;                     // centre n0 + i + j - 4 is place i + j, and node n0 + i its tap 8 - j
 #pragma unroll
-        for (int j = 0; j < 7; ++j) h += tap[6 - j][i + j];
+        for (int j = 0; j < kTapsN; ++j) h += tap[kTapsN - 1 - j][i + j];
         P.H[(size_t)p * P.N.nn + P.N.n_off[w] + n0 + i] = h;
     }
 }
@@ -433,7 +503,7 @@ __global__ void __launch_bounds__(kOffThreads, 6) k_ang_bins(const NodeParams P,
         ++w;
     }
     const int a = P.a0 + ai * P.a_step, n = P.N.n_dir[w];
-    const int s = (int)((int64_t)a * n / P.A);
+    const int s = a * P.N.angle_step[w];
     int n1[kOffPer], n2[kOffPer];
     float mu[kOffPer], two[kOffPer];
     // slots of the tile
@@ -734,7 +804,7 @@ __global__ void __launch_bounds__(256) k_ang_psi(const NodeParams P) {
     __syncthreads();
     for (int m = threadIdx.x; m < P.N.nm_pad; m += 256) {
         const float4* w = reinterpret_cast<const float4*>(P.psi_w + (size_t)m * kPsiStride);
-        const float4 w0 = w[0], w1 = w[1];
+        const float4 w0 = w[0], w1 = w[1], w2 = w[2];
         const float* v = srow + P.psi_l[m];
         float s = w0.x * v[0];
         s = fmaf(w0.y, v[1], s);
@@ -743,6 +813,10 @@ __global__ void __launch_bounds__(256) k_ang_psi(const NodeParams P) {
         s = fmaf(w1.x, v[4], s);
         s = fmaf(w1.y, v[5], s);
         s = fmaf(w1.z, v[6], s);
+        s = fmaf(w1.w, v[7], s);
+        s = fmaf(w2.x, v[8], s);
+        s = fmaf(w2.y, v[9], s);
+        s = fmaf(w2.z, v[10], s);
         P.psi[row * P.N.nm_pad + m] = s;
     }
 }
@@ -823,7 +897,7 @@ __global__ void __launch_bounds__(32 * kBackWarps, 8) k_ang_back(const NodeParam
         if (grp >= groups) continue;
         for (int k = 0; k < na; ++k) {
             const int a = P.a0 + (a1 + k) * P.a_step;
-            const int sh = (int)((int64_t)a * n / P.A);
+            const int sh = a * P.N.angle_step[w];
             const int2 br = sb[k][warp];
             const float4* c = reinterpret_cast<const float4*>(sc + (size_t)(k * kBackWarps + warp) * per);
             int d0 = nd0 - sh, d1 = nd1 - sh;
@@ -882,35 +956,33 @@ __global__ void __launch_bounds__(32 * kBackWarps, 8) k_ang_back(const NodeParam
 }
 
 // v plus what the slots add to a path with its centre at node c and taps x: for
-// every detector angle that has a knot within reach of its taps, the nodes on
-// the knot's other side.  The windows of a line are disjoint, so that no angle
-// comes twice.
+// every detector angle of the launch that has a knot within reach of its taps,
+// the nodes on the knot's other side.  The windows are disjoint, so that no angle
+// comes twice; angle i is in one of them for i between two quotients, which FP32
+// gives exactly (half a node from the next whole number).
 __device__ __forceinline__ float beyond_knots(const NodeParams& P, int w, int p, int c, float s,
                                               const float (&x)[kTapsN], float v) {
-    const int n = P.N.n_dir[w], g = n / P.A;      // nodes between two detector angles
+    const int step = P.N.angle_step[w] * P.a_step, r0 = c - P.a0 * P.N.angle_step[w], n = P.N.n_dir[w];
     for (int k = P.N.win_off[w]; k < P.N.win_off[w + 1]; ++k) {
         const int2 win = P.win[k];
-        // angles j (of the unrolled circle) with c - j g inside the window
-        const int lo = c - win.y, hi = c - win.x;
-        for (int j = lo > 0 ? (lo + g - 1) / g : -(-lo / g); j * g <= hi; ++j) {
-            const int a = (j % P.A + P.A) % P.A, ai = (a - P.a0) / P.a_step;
-            if (a < P.a0 || ai >= P.angles || P.a0 + ai * P.a_step != a) continue;
-            int r = c - j * g;
-            if (2 * r > n) r -= n;
-            if (2 * r < -n) r += n;
-            float u = fabsf((float)r + s);
-            if (2.f * u > (float)n) u = (float)n - u;
-            int branch = 0;
-            while (branch < P.N.kinks[w] && u > P.N.kink[w][branch]) ++branch;
-            const float* side = P.side + ((size_t)ai * P.np + p) * P.N.slots;
+        const int i0 = max((int)floorf(((float)(r0 - win.y) - 0.5f) * P.inv_step[w]) + 1, 0);
+        const int i1 = min((int)floorf(((float)(r0 - win.x) + 0.5f) * P.inv_step[w]), P.angles - 1);
+        for (int i = i0; i <= i1; ++i) {
+            const int r = r0 - i * step;
+            const short* at = P.slot_at + side_of_knots(P.N, w, r, s) * P.N.nm_pad;
+            const float* side = P.side + ((size_t)i * P.np + p) * P.N.slots;
+            int z[kTapsN];
+            const int m = abs(r), turn = r > 0 ? 1 : -1;
+            if (m >= kTapsN / 2 && 2 * (m + kTapsN / 2) <= n) {   // the offsets in a row
 #pragma unroll
-            for (int t = 0; t < kTapsN; ++t) {
-                int m = abs(r + t - kTapsN / 2);
-                if (2 * m > n) m = n - m;
-                const int o = P.N.m_off[w] + m;
-                for (int z = P.slot_start[o]; z < P.slot_start[o + 1]; ++z)
-                    if (P.slot[z].branch == branch) v = fmaf(x[t], side[z], v);
+                for (int t = 0; t < kTapsN; ++t) z[t] = at[P.N.m_off[w] + m + turn * (t - kTapsN / 2)];
+            } else {
+#pragma unroll
+                for (int t = 0; t < kTapsN; ++t) z[t] = at[offset_of(P.N, w, r + t - kTapsN / 2)];
             }
+#pragma unroll
+            for (int t = 0; t < kTapsN; ++t)
+                if (z[t] >= 0) v = fmaf(x[t], side[z[t]], v);
         }
     }
     return v;
@@ -931,12 +1003,12 @@ __global__ void __launch_bounds__(256) k_ang_paths(const NodeParams P) {
         const int n = P.N.n_dir[w];
         int c;
         const float s = direction_pos(fix, n, &c);
-        float x[7];
-        lagrange7(s, P.path_b[(size_t)w * P.np * P.nq + i], x);
+        float x[kTapsN];
+        lagrange9(s, P.path_b[(size_t)w * P.np * P.nq + i], x);
         const float* T = P.T + (size_t)p * P.N.nn + P.N.n_off[w];
 #pragma unroll
-        for (int k = 0; k < 7; ++k) {
-            int j = c + k - 3;
+        for (int k = 0; k < kTapsN; ++k) {
+            int j = c + k - kTapsN / 2;
             j = j < 0 ? j + n : j >= n ? j - n : j;
             float t = T[j];
             if (kSplit)
@@ -991,11 +1063,11 @@ __global__ void __launch_bounds__(256) k_node_y(const EventParams P, const uint1
     if (in_reach(P.N, e)) {
         const float* F = P.F + cell * P.N.nk_pad;
         int k;
-        float wt[12];
-        lagrange12(energy_pos(P.N, e, &k), wt);
+        float wt[kTapsK];
+        lagrange16(energy_pos(P.N, e, &k), wt);
         float s0 = 0.f, s1 = 0.f;
 #pragma unroll
-        for (int i = 0; i < 12; i += 2) {
+        for (int i = 0; i < kTapsK; i += 2) {
             s0 = fmaf(wt[i], F[k + i], s0);
             s1 = fmaf(wt[i + 1], F[k + i + 1], s1);
         }
@@ -1008,9 +1080,8 @@ __global__ void __launch_bounds__(256) k_node_y(const EventParams P, const uint1
 // forward values, the ratios r_j = 1 / y_j (0 where y_j <= 0) and, when ll is
 // set, the cell's FP64 sum of log y_j; else r_j = the caller's weights.  Then
 // the cell's node weights V = sum_j r_j L(E_j) and unscattered weights PV.  A
-// lane forms the values of one event; the events' 12 taps are then added one
-// event per half-warp at a time into the half-warp's own row, 12 lanes one tap
-// each.  In cells of more than 1024 events the rows are emptied into second
+// lane forms the values of one event; the events' 16 taps are then added one
+// event per half-warp at a time into the half-warp's own row, a tap a lane.  In cells of more than 1024 events the rows are emptied into second
 // sums every 256 events of a warp.
 __global__ void __launch_bounds__(32 * kCellWarps) k_node_cells(
     const EventParams P, const int* cell_start, int cell0, const float* energy, const float* weight,
@@ -1021,7 +1092,7 @@ __global__ void __launch_bounds__(32 * kCellWarps) k_node_cells(
     float* Fs = sh;                          // [nk_pad]
     float* acc = Fs + nkp;                   // [kRows][nk_pad]
     float* tot = acc + kRows * nkp;          // [kRows][nk_pad]
-    __shared__ float wts[kCellWarps][32][13];
+    __shared__ float wts[kCellWarps][32][kTapsK + 1];
     __shared__ int kpos[kCellWarps][32];
     __shared__ float pv_s[kCellWarps][4];
     __shared__ double ll_s[kCellWarps];
@@ -1046,11 +1117,12 @@ __global__ void __launch_bounds__(32 * kCellWarps) k_node_cells(
     float pv[4] = {0.f, 0.f, 0.f, 0.f};
     double lsum = 0.0;
     float* mine = acc + (2 * warp + (lane >> 4)) * nkp;
+    static_assert(kTapsK == 16, "a tap a lane of the half-warp");
     const int tap = lane & 15;
     int batches = 0;
     for (int b0 = e0 + 32 * warp; b0 < e1; b0 += 32 * kCellWarps) {
         const int j = b0 + lane;
-        float r = 0.f, wt[12];
+        float r = 0.f, wt[kTapsK];
         int k = 0;
         bool reach = false;
         if (j < e1) {
@@ -1064,12 +1136,12 @@ __global__ void __launch_bounds__(32 * kCellWarps) k_node_cells(
                     if (P.F) y = fmaf(P.Pr[cell * W + w], g[w], y);
                 }
             reach = in_reach(P.N, e);
-            if (reach) lagrange12(energy_pos(P.N, e, &k), wt);
+            if (reach) lagrange16(energy_pos(P.N, e, &k), wt);
             if (P.F) {
                 if (reach) {
                     float s0 = 0.f, s1 = 0.f;
 #pragma unroll
-                    for (int i = 0; i < 12; i += 2) {
+                    for (int i = 0; i < kTapsK; i += 2) {
                         s0 = fmaf(wt[i], Fs[k + i], s0);
                         s1 = fmaf(wt[i + 1], Fs[k + i + 1], s1);
                     }
@@ -1088,13 +1160,13 @@ __global__ void __launch_bounds__(32 * kCellWarps) k_node_cells(
         }
         kpos[warp][lane] = k;
 #pragma unroll
-        for (int i = 0; i < 12; ++i) wts[warp][lane][i] = reach ? r * wt[i] : 0.f;
+        for (int i = 0; i < kTapsK; ++i) wts[warp][lane][i] = reach ? r * wt[i] : 0.f;
         __syncwarp();
         const int n_here = min(32, e1 - b0);
         const int h0 = (lane >> 4) * 16;
         for (int i = 0; i < 16; ++i) {
             const int ev = h0 + i;
-            if (ev < n_here && tap < kTapsK) mine[kpos[warp][ev] + tap] += wts[warp][ev][tap];
+            if (ev < n_here) mine[kpos[warp][ev] + tap] += wts[warp][ev][tap];
             __syncwarp();
         }
         if (large && (++batches & 7) == 0) {
@@ -1173,8 +1245,8 @@ __global__ void __launch_bounds__(kUpdVox * kUpdStrands) k_node_update(
     }
     if (strand == 0 && q < nq) {
         const double t = red[0][v];
-        if (sens)
-            lam[q] = sens[q] > 0.0 ? (float)((double)lam[q] * t / sens[q]) : 0.f;
+        if (sens)   // (the ratios and the rows are not negative: nor is their sum, but for rounding)
+            lam[q] = sens[q] > 0.0 ? (float)((double)lam[q] * (t < 0.0 ? 0.0 : t) / sens[q]) : 0.f;
         else
             num[q] = t;
     }
@@ -1411,7 +1483,7 @@ __global__ void k_offset_tables(ModelConst m, const NodeConst N, double kappa, c
     const double c = cospi(2.0 * i / N.n_dir[w]), r = 1.0 / (1.0 + k0 * (1.0 - c)), e = e0 * r;
     const double kn = r * r * (r + 1.0 / r - (1.0 - c * c));
     const double f = kn / (2.506628274631000502 * kappa * sqrt(e));   // / (sqrt(2 pi) sigma)
-    const double u = 2.0 * sqrt(e) / kappa * kPerUnitL - N.l_first[w];
+    const double u = 2.0 * sqrt(e) / kappa * N.per_l - N.l_first[w];
     const double s = u - (psi_l[o] - N.l_off[w] + kTapsL / 2);
     double mu_e = m.knot_mu[0];
     if (m.n_knots > 1) {
@@ -1504,7 +1576,9 @@ NodeParams node_params(const lm_handle* h, int a0, int a_step, int angles) {
     P.path_start = t.path_start;
     P.slot = t.slot;
     P.slot_start = t.slot_start;
+    P.slot_at = t.slot_at;
     P.win = t.win;
+    for (int w = 0; w < m.W; ++w) P.inv_step[w] = (float)m.A / ((float)P.N.n_dir[w] * (float)a_step);
     P.grp_pt = t.grp_pt;
     P.grp_bins = t.grp_bins;
     P.grp_c = h->d_node_groups;
@@ -1549,7 +1623,16 @@ int build_nodes(lm_handle* h) {
     std::vector<int> slot_start;
     std::vector<int2> wins;
     // recorded energies
-    const double ck = kPerUnitK * 2.0 / kappa;
+    // the Gaussian's exponent changes by up to 1 + 4 kappa / sqrt(E') per unit of
+    // t at 8 sigma, 1.25 for 62 keV and 10 % at 140 keV: denser nodes where more
+    auto denser = [&](double e) { return std::max(1.0, (1.0 + 4.0 * kappa / sqrt(e)) / 1.26); };
+    double dense = 1.0;
+    for (int w = 0; w < m.W; ++w)
+        dense = std::max(dense, denser(m.line_e[w] / (1.0 + 2.0 * m.line_e[w] / me)));
+    if (!(dense < 16.0)) return LMMEW_OK;
+    N.per_l = (int)ceil(kPerUnitL * dense);
+    N.per_k = (int)ceil(kPerUnitK * dense);
+    const double ck = N.per_k * 2.0 / kappa;
     N.ck = (float)ck;
     N.ck_lo = (float)(ck - (double)N.ck);
     double e_lo = 1e300, e_hi = 0.0;
@@ -1557,22 +1640,23 @@ int build_nodes(lm_handle* h) {
         e_lo = std::min(e_lo, std::max(m.win_lo[k], 0.0));
         e_hi = std::max(e_hi, m.win_hi[k]);
     }
-    const double t_hi = t_of(e_hi) * kPerUnitK;
+    const double t_hi = t_of(e_hi) * N.per_k;
     if (!(t_hi < 8192.0)) return LMMEW_OK;
-    N.k_first = (int)floor(t_of(e_lo) * kPerUnitK) - 6;
-    N.nk = (int)floor(t_hi) + 7 - N.k_first + 1;
+    N.k_first = (int)floor(t_of(e_lo) * N.per_k) - kTapsK / 2;
+    N.nk = (int)floor(t_hi) + kTapsK / 2 + 1 - N.k_first + 1;
     N.nk_pad = (N.nk + 31) & ~31;
     // scattered energies and directions of each line
     for (int w = 0; w < m.W; ++w) {
         const double e0 = m.line_e[w], k0 = e0 / me, eb = e0 / (1.0 + 2.0 * k0);
-        const double u0 = t_of(eb) * kPerUnitL, u1 = t_of(e0) * kPerUnitL;
+        const double u0 = t_of(eb) * N.per_l, u1 = t_of(e0) * N.per_l;
         if (!(u1 < 1.0e6)) return LMMEW_OK;
-        N.l_first[w] = (int)floor(u0) - 4;
-        N.l_count[w] = (int)ceil(u1) + 4 - N.l_first[w] + 1;
+        N.l_first[w] = (int)floor(u0) - kTapsL / 2 - 1;
+        N.l_count[w] = (int)ceil(u1) + kTapsL / 2 + 1 - N.l_first[w] + 1;
         if (N.l_first[w] < 1) return LMMEW_OK;
         N.l_off[w] = N.nl;               // (lines start at multiples of 8 nodes)
         N.nl += (N.l_count[w] + 7) & ~7;
-        // 18 nodes per sigma where E'(x) is steepest (7 taps: 1e-8 of a term), and
+        // 17 nodes per sigma where E'(x) is steepest (9 taps: 1e-7 of a term at 6
+        // sigma, 3e-6 at 8), and
         // enough that the attenuation changes by 4 % per node at most over the
         // longest way through the map
         auto slope = [&](double e) {     // |dE'/dx|
@@ -1587,7 +1671,8 @@ int build_nodes(lm_handle* h) {
         };
         double want = 32.0;
         auto sample = [&](double e) {
-            want = std::max(want, 2.0 * pi * slope(e) * std::max(18.0 / (kappa * sqrt(e)), mu_slope(e) * way / 0.04));
+            want = std::max(want, 2.0 * pi * slope(e) * std::max(kPerSigmaN * denser(eb) / (kappa * sqrt(e)),
+                                                               mu_slope(e) * way / 0.04));
         };
         for (int i = 1; i < 512; ++i) sample(e0 / (1.0 + k0 * (1.0 - cos(pi * i / 512))));
         // knots inside E', by offset; the segment of mu on either side
@@ -1607,7 +1692,8 @@ int build_nodes(lm_handle* h) {
             segs.push_back(seg - 1);
         }
         if (!(want < 16384.0) || m.A > 16384) return LMMEW_OK;
-        N.n_dir[w] = ((int)ceil(want) + m.A - 1) / m.A * m.A;
+        N.angle_step[w] = ((int)ceil(want) + m.A - 1) / m.A;
+        N.n_dir[w] = N.angle_step[w] * m.A;
         N.n_off[w] = N.nn;
         N.nn += N.n_dir[w];
         N.m_count[w] = N.n_dir[w] / 2 + 1;
@@ -1625,43 +1711,40 @@ int build_nodes(lm_handle* h) {
         };
         auto fold = [&](double u) { return fabs(u) > 0.5 * n ? n - fabs(u) : fabs(u); };
         slot_start.resize(N.m_off[w] + count + 1, (int)slots.size());
+        N.slot_off[w] = (int)slots.size();
         for (int i = 0; i < count; ++i) {
             slot_start[N.m_off[w] + i] = (int)slots.size();
             const int own = branch_of(i);
             for (int b = 0; b <= N.kinks[w]; ++b) {
                 if (b == own) continue;
                 const float lo = b == 0 ? -1.f : N.kink[w][b - 1], hi = b == N.kinks[w] ? 1e9f : N.kink[w][b];
-                int d0 = half + 1, d1 = -half - 1;
+                bool reached = false;
                 for (int d = -half; d <= half; ++d) {
                     // paths centred there: i + d - 1/2 .. i + d + 1/2, folded
-                    const double u0 = fold(i + d - 0.5), u1 = fold(i + d + 0.5);
-                    const double a = std::min({u0, u1, fold(i + d)}), z = std::max({u0, u1, fold(i + d)});
-                    if (z < lo || a > hi) continue;
-                    d0 = std::min(d0, d);
-                    d1 = std::max(d1, d);
+                    const double u0 = fold(i + d - 0.5), u1 = fold(i + d + 0.5), u2 = fold(i + d);
+                    reached |= std::max({u0, u1, u2}) + 1e-3 >= lo && std::min({u0, u1, u2}) - 1e-3 <= hi;
                 }
-                if (d0 > d1) continue;
+                if (!reached) continue;
                 const double e = e0 / (1.0 + k0 * (1.0 - cos(2.0 * pi * i / n)));
                 const double mu_b = m.knot_mu[segs[b]] + (e - m.knot_e[segs[b]]) * m.knot_slope[segs[b]];
-                slots.push_back({N.m_off[w] + i, b, d0, d1, lo, hi, (float)(mu_b * log2e)});
+                slots.push_back({N.m_off[w] + i, b, (float)(mu_b * log2e)});
             }
         }
         slot_start.back() = (int)slots.size();
-        slot_start.resize(N.nm_pad + 1, (int)slots.size());
         constexpr int kTile = kOffThreads * kOffPer;
         for (int i = 0; i < count; i += kTile)
             N.tile_slots = std::max(N.tile_slots, slot_start[N.m_off[w] + std::min(i + kTile, count)] -
                                                       slot_start[N.m_off[w] + i]);
-        // windows of centres (from the detector direction) with a knot among their taps
+        // windows of c - s with a knot among the taps, both turns of the circle
         N.win_off[w] = (int)wins.size();
         std::vector<int2> around;
-        for (double x : at) {
-            const double u = x * n / (2.0 * pi);
-            const int lo = (int)floor(u) - half - 1, hi = (int)ceil(u) + half + 1;
-            around.push_back(make_int2(lo, hi));
-            around.push_back(make_int2(-hi, -lo));
-        }
-        // a window past half a turn goes on at the other end: unrolled, merged
+        for (double x : at)
+            for (int turn = -1; turn <= 1; ++turn)
+                for (int sign = -1; sign <= 1; sign += 2) {
+                    const double u = sign * x * n / (2.0 * pi) + turn * n;
+                    const int lo = std::max((int)floor(u) - half - 1, -n), hi = std::min((int)ceil(u) + half + 1, n);
+                    if (lo <= hi) around.push_back(make_int2(lo, hi));
+                }
         std::sort(around.begin(), around.end(), [](int2 a, int2 b) { return a.x < b.x; });
         for (const int2& r : around) {
             if ((int)wins.size() > N.win_off[w] && r.x <= wins.back().y + 1)
@@ -1669,23 +1752,19 @@ int build_nodes(lm_handle* h) {
             else
                 wins.push_back(r);
         }
-        if ((int)wins.size() > N.win_off[w]) {
-            int2& first = wins[N.win_off[w]];
-            if ((int)wins.size() > N.win_off[w] + 1 && wins.back().y >= first.x + n) {   // they meet
-                first.x = wins.back().x - n;
-                wins.pop_back();
-            }
-            if (first.y - first.x >= n) first.y = first.x + n - 1;
-        }
+        if ((int)wins.size() - N.win_off[w] > kMostWindows) return LMMEW_OK;
         N.reach_lo[w] = h->reach_lo[w];
         N.reach_hi[w] = h->reach_hi[w];
     }
     N.win_off[m.W] = (int)wins.size();
-    for (int w = m.W; w < 4; ++w) N.win_off[w + 1] = N.win_off[w];
-    N.slots = (int)slots.size();
+    N.slots = N.slot_off[m.W] = (int)slots.size();
+    slot_start.resize(N.nm_pad + 1, N.slots);
+    const int sides = 1 + *std::max_element(N.kinks, N.kinks + 4);
+    std::vector<short> slot_at((size_t)sides * N.nm_pad, -1);
     N.nl_pad = (N.nl + 31) & ~31;
-    if (N.tile_slots > 256) return LMMEW_OK;   // (k_ang_bins stages them)
-    if (N.nl > 6000 || N.nk > 1024 || N.nn > 32768 || (int64_t)m.np * N.nn >= (int64_t(1) << 31))
+    if (N.tile_slots > 256 || N.slots > 32767) return LMMEW_OK;   // (staged by k_ang_bins, named by short)
+    for (int z = 0; z < N.slots; ++z) slot_at[(size_t)slots[z].side * N.nm_pad + slots[z].offset] = (short)z;
+    if (N.nl > 6000 || N.nk > 1152 || N.nn > 32768 || (int64_t)m.np * N.nn >= (int64_t(1) << 31))
         return LMMEW_OK;
     const size_t pair_bytes = (12 + 4 * (size_t)m.W) * (size_t)pairs;
     if (pair_bytes > (size_t(64) << 20)) {
@@ -1703,7 +1782,7 @@ int build_nodes(lm_handle* h) {
         const double e0 = m.line_e[w], k0 = e0 / me, step = cos(2.0 * pi / N.n_dir[w]);
         double c = 1.0, before = step;
         for (int i = 0; i < N.m_count[w]; ++i) {
-            const double u = t_of(e0 / (1.0 + k0 * (1.0 - c))) * kPerUnitL - N.l_first[w];
+            const double u = t_of(e0 / (1.0 + k0 * (1.0 - c))) * N.per_l - N.l_first[w];
             const int o = N.m_off[w] + i, first = N.l_off[w] + (int)floor(u + 0.5) - kTapsL / 2;
             psi_l[o] = first;
             for (int l = first; l < first + kTapsL; ++l) {
@@ -1728,13 +1807,13 @@ int build_nodes(lm_handle* h) {
     int2* l_of_k = k_of_l + lt;
     for (int w = 0; w < m.W; ++w)
         for (int i = 0; i < N.l_count[w]; ++i) {
-            // |E_k - E_l| <= 9 sigma_l between the nodes just outside the band
+            // |E_k - E_l| <= 10.2 sigma_l between the nodes just outside the band
             const int l = N.l_off[w] + i;
-            const double x = 0.5 * kappa * (N.l_first[w] + i) / kPerUnitL, e = x * x;
+            const double x = 0.5 * kappa * (N.l_first[w] + i) / N.per_l, e = x * x;
             const double s = kBandSigmas * kappa * x;
-            const double v0 = e > s ? t_of(e - s) * kPerUnitK : -1e9;
+            const double v0 = e > s ? t_of(e - s) * N.per_k : -1e9;
             const int k0 = std::max(0, (int)floor(v0) - N.k_first);
-            const int k1 = std::min(N.nk, (int)ceil(t_of(e + s) * kPerUnitK) - N.k_first + 1);
+            const int k1 = std::min(N.nk, (int)ceil(t_of(e + s) * N.per_k) - N.k_first + 1);
             if (k0 >= k1) continue;
             k_of_l[l / 32].x = std::min(k_of_l[l / 32].x, k0);
             k_of_l[l / 32].y = std::max(k_of_l[l / 32].y, k1);
@@ -1775,6 +1854,7 @@ int build_nodes(lm_handle* h) {
         T.l_of_k = T.k_of_l + lt;
         T.slot = bump<NodeSlot>(p, slots.size());
         T.slot_start = bump<int>(p, slot_start.size());
+        T.slot_at = bump<short>(p, slot_at.size());
         T.win = bump<int2>(p, wins.size());
         d_run = bump<int2>(p, run.size());
         d_most = bump<int>(p, 2);
@@ -1820,6 +1900,7 @@ int build_nodes(lm_handle* h) {
     put(T.k_of_l, bands.data(), 8 * bands.size());
     put(T.slot, slots.data(), sizeof(NodeSlot) * slots.size());
     put(T.slot_start, slot_start.data(), 4 * slot_start.size());
+    put(T.slot_at, slot_at.data(), sizeof(short) * slot_at.size());
     put(T.win, wins.data(), 8 * wins.size());
     put(d_run, run.data(), 8 * run.size());
     LMMEW_CUDA(cudaMemcpy(h->d_node_tables, blob.data(), host_bytes, cudaMemcpyHostToDevice));
@@ -1908,11 +1989,13 @@ int node_spread(lm_handle* h, const float* lam_v, float* H, int a0, int a_step, 
     int rc = prof_start(h, st);
     if (rc != LMMEW_OK) return rc;
     const int units = H ? h->mc.np * tiles : 0;
-    const int64_t sides = (int64_t)angles * h->mc.np * P.N.slots;
-    const int64_t blocks = (units + kSpreadWarps - 1) / kSpreadWarps +
-                           (sides + 32 * kSpreadWarps - 1) / (32 * kSpreadWarps);
+    int64_t sides = 0;
+    for (int w = 0; w < P.N.W; ++w)
+        if (P.N.kinks[w] > 0) sides += (int64_t)angles * h->mc.np;
+    const int side_blocks = (int)((sides + kSpreadWarps - 1) / kSpreadWarps);
+    const int blocks = side_blocks + (units + kSpreadWarps - 1) / kSpreadWarps;
     if (blocks == 0) return LMMEW_OK;
-    k_ang_spread<<<(unsigned)blocks, 32 * kSpreadWarps, 0, st>>>(P, tiles, units);
+    k_ang_spread<<<(unsigned)blocks, 32 * kSpreadWarps, 0, st>>>(P, tiles, units, side_blocks);
     ++h->launches;
     LMMEW_CUDA(cudaGetLastError());
     return prof_stop(h, H ? (double)h->mc.W * h->mc.nq * h->mc.np : 0.0, st);

@@ -12,10 +12,13 @@ import pytest
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
+import oracle  # noqa: E402
 import paper_2305_17111_gb300 as lm  # noqa: E402
 from synthetic import preset  # noqa: E402
+from synthetic.mc import EventList  # noqa: E402
 
 ROUTE_RTOL = 2e-6   # node route vs row route: FP32 sums in another order
+PARITY_RTOL = 1e-5  # parity with the FP64 oracle
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -57,6 +60,36 @@ def test_projections_for_every_sort_size(n, scatter_n, voxels):
     on = bp_rows != 0
     assert bool((bp[~on] == 0).all())
     assert float(((bp - bp_rows)[on] / bp_rows[on]).abs().max()) < ROUTE_RTOL
+    gpu.close()
+
+
+@pytest.mark.parametrize("voxels", [16385, 16641])
+def test_global_sort_matches_the_oracle(voxels):
+    """Past the largest sort in shared memory.  Nine scatter points: the rows'
+    rounding of a single path (5e-6) is too coarse a reference there."""
+    sc = preset("tiny_8").with_(n=129, pixel_cm=25.6 / 129, n_bins=9, scatter_n=3)
+    rho = np.ones((129, 129), np.float32)
+    support = (np.arange(129 * 129) < voxels).astype(np.uint8)
+    gpu = lm.Model.from_scenario(sc, rho, support=support)
+    orc = oracle.Model.from_scenario(sc, rho, support=support)
+    assert gpu.nq == voxels
+    dev = _events(sc, 5, 129)
+    z = np.zeros(len(dev), np.int32)
+    ev = EventList(dev.angle.cpu().numpy().astype(np.uint16), dev.bin.cpu().numpy().astype(np.uint16),
+                   dev.energy.cpu().numpy(), z, z.astype(np.uint8), z.astype(bool))
+    rng = np.random.default_rng(voxels)
+    lam = (rng.uniform(0.2, 3.0, 129 * 129) * support).astype(np.float32)
+    w = rng.uniform(0.1, 1.0, len(dev)).astype(np.float32)
+    gpu.profile_enable(True)
+    y = gpu.forward(dev, torch.from_numpy(lam).cuda()).double().cpu().numpy()
+    assert gpu.profile_read()["terms"] == gpu.n_lines * gpu.nq * gpu.np_scatter    # the node route
+    ref = orc.forward(ev, lam.astype(np.float64))
+    assert float((np.abs(y - ref) / ref).max()) < PARITY_RTOL
+    bp = gpu.backproject(dev, torch.from_numpy(w).cuda()).double().cpu().numpy()
+    ref = orc.backproject(ev, w)
+    on = ref > 0
+    assert np.all(bp[~on] == 0)
+    assert float((np.abs(bp - ref)[on] / ref[on]).max()) < PARITY_RTOL
     gpu.close()
 
 
