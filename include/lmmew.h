@@ -50,12 +50,18 @@
  *   - dense event lists are projected through nodes: the exact model's forward
  *     and back projections and LM-OSEM take, instead of one row per event, sums
  *     on direction and energy nodes whose cost hardly grows with the events
- *     (the same model to FP32 rounding; lm_forward and lm_backproject from 2
- *     events per angle (8 for back projections of small models), lm_osem and lm_osem_batch, per realisation, from 120
- *     per angle where a sub-iteration's rows are estimated to take twice the
- *     nodes' time).  The route needs up to 4 lines, the square-root energy
- *     resolution (exponent -1/2), the FP32 form and energy pruning on;
- *     everything else goes through the rows;
+ *     (the same model; interpolation adds 1e-7 of a path's value up to 6 sigma
+ *     from its energy and 3e-6 at the 8 sigma where the reach ends, no more than
+ *     the rows' rounding there; a path further than 10 sigma from an event adds
+ *     nothing, and an infinite image value or weight may give NaN).
+ *     lm_forward and lm_backproject take them from 2 events per angle (8 for
+ *     back projections of small models), lm_osem and lm_osem_batch, per
+ *     realisation, from 120 per angle where a sub-iteration's rows are estimated
+ *     to take twice the nodes' time.  The route needs up to 4 lines, the
+ *     square-root energy resolution (exponent -1/2), the FP32 form and energy
+ *     pruning on; everything else goes through the rows.  Where the node sums of
+ *     one angle exceed the 16 MiB of lm_forward_noalloc, lm_forward keeps the
+ *     rows too for the lists whose rows fit there;
  *   - reconstructions of two iterations or more that go through the rows keep
  *     their scatter rows from the first iteration for the later ones, in the
  *     handle's scratch, when the rows of the whole call take at most 16 GiB

@@ -309,10 +309,9 @@ int launch_row_ranks(lm_handle* h, const RowLaunch& L, const SortedEvents& se, i
     return LMMEW_OK;
 }
 
-ForwardPlan forward_plan(const lm_handle* h, int64_t n, int64_t cap_max) {
+ForwardPlan forward_plan(const lm_handle* h, int64_t n, int64_t cap_max, int te) {
     ForwardPlan p;
     p.G = sort_groups(h, h->mc.A);
-    const int te = h->tile_ev;
     p.n = n;
     // at most ceil(n / te) + G tiles: one row block of that many whole tiles
     // when it fits cap_max, else blocks of as many tiles as fit
@@ -394,11 +393,18 @@ size_t forward_nodes_bytes(const lm_handle* h, int block) {
     return forward_nodes_fixed(h) + (size_t)block * node_angle_bytes(h);
 }
 
-// Scratch of lm_forward_noalloc's rows for n events.
-size_t noalloc_rows_bytes(const lm_handle* h, int64_t n) {
-    const ForwardPlan fp = forward_plan(h, n, int64_t(1) << 40);
+// Scratch of lm_forward_noalloc's rows for n events in tiles of te.
+size_t noalloc_rows_bytes(const lm_handle* h, int64_t n, int te) {
+    const ForwardPlan fp = forward_plan(h, n, int64_t(1) << 40, te);
     return bump_bytes(sizeof(int) * h->mc.A) + 2 * bump_bytes(sizeof(int) * fp.G) +
            forward_region_bytes(h, fp);
+}
+
+// The routes follow the model, the forms set on the handle and the list's length
+// alone: not the tile size, which the autotuner changes between calls of one
+// reconstruction.
+static bool node_model(const lm_handle* h) {
+    return h->node_route && h->n_classes > 1 && h->prec == 0 && h->scatter_model == LMMEW_SCATTER_EXACT;
 }
 
 // Projections of 2 events or more per detector angle go through the nodes, at a
@@ -406,12 +412,12 @@ size_t noalloc_rows_bytes(const lm_handle* h, int64_t n) {
 // 378 us at 864 voxels and 60; the rows take 177 and 1025 us for 2 events per
 // angle, and 150 and 631 us for 1, where little is gained.
 bool node_use(const lm_handle* h, int64_t n) {
-    return h->node_route && h->n_classes > 1 && h->prec == 0 &&
-           h->scatter_model == LMMEW_SCATTER_EXACT && n >= (int64_t)2 * h->mc.A &&
+    return node_model(h) && n >= (int64_t)2 * h->mc.A &&
            // lm_forward_noalloc takes the same route as lm_forward for every
            // list it accepts: where its array does not hold the node sums of
-           // one angle, both keep the rows for those lists
-           (forward_nodes_block(h, kNoAllocBytes) > 0 || noalloc_rows_bytes(h, n) > kNoAllocBytes);
+           // one angle, both keep the rows for the lists whose rows it holds
+           // (in the smallest tiles, which take least)
+           (forward_nodes_block(h, kNoAllocBytes) > 0 || noalloc_rows_bytes(h, n, kETMin) > kNoAllocBytes);
 }
 
 // Back projections of small models (fewer than 100 000 voxel-point pairs) from 8
@@ -419,7 +425,8 @@ bool node_use(const lm_handle* h, int64_t n) {
 // for 2, 4 and 8 events per angle, nodes 220 to 247.  From 827 voxels x 207 points
 // on the nodes are ahead at 2 (347 for 376 us).
 bool node_use_back(const lm_handle* h, int64_t n) {
-    return node_use(h, n) && ((int64_t)h->mc.nq * h->mc.np >= 100000 || n >= (int64_t)8 * h->mc.A);
+    const int64_t pairs = (int64_t)h->mc.nq * h->mc.np;
+    return node_model(h) && n >= (pairs >= 100000 ? 2 : 8) * (int64_t)h->mc.A;
 }
 
 // Reconstructions: the estimated time of a sub-iteration's rows has to be twice
@@ -434,7 +441,7 @@ bool node_use_back(const lm_handle* h, int64_t n) {
 // events, 8 subsets: rows 2150, nodes 190.  Below 120 events per angle the rows
 // cost less than the nodes once kept at any size.
 bool node_use_osem(const lm_handle* h, int64_t n, int n_subsets) {
-    if (!node_use(h, n) || n < (int64_t)120 * h->mc.A) return false;
+    if (!node_model(h) || n < (int64_t)120 * h->mc.A) return false;
     const double angles = (double)h->mc.A / std::max(1, n_subsets);
     const double paths = (double)h->mc.nq * h->mc.np;
     const double rows = 70.0 + 2e-8 * paths * h->mc.W * ((double)n / std::max(1, n_subsets) + 700.0 * angles);
@@ -880,7 +887,7 @@ int lm_forward(lm_handle* h, const lm_events* ev, const float* image, float* out
     GroupArrays ga;
     rc = group_arrays(h, 1, &ga);
     if (rc != LMMEW_OK) return rc;
-    const ForwardPlan fp = forward_plan(h, ev->n, (int64_t)(kRowBudgetFloats / h->mc.nqt));
+    const ForwardPlan fp = forward_plan(h, ev->n, (int64_t)(kRowBudgetFloats / h->mc.nqt), h->tile_ev);
     rc = ensure(h, h->scratch_sort, forward_region_bytes(h, fp), st);
     if (rc != LMMEW_OK) return rc;
     return forward_async(h, ev, image, out_y, ga, fp, (char*)h->scratch_sort.ptr, st);
@@ -1023,7 +1030,7 @@ int lm_backproject(lm_handle* h, const lm_events* ev, const float* weight, float
     if (rc != LMMEW_OK) return rc;
     const int64_t n = ev->n;
     const int G = sort_groups(h, m.A), rs = row_stride_of(h);
-    const ForwardPlan fp = forward_plan(h, n, (int64_t)(kRowBudgetFloats / rs));
+    const ForwardPlan fp = forward_plan(h, n, (int64_t)(kRowBudgetFloats / rs), h->tile_ev);
     const int64_t ppc = bp_parts(fp.cap);
     rc = ensure(h, h->scratch_sort, sort_scratch_bytes(n, G), st);
     if (rc == LMMEW_OK)

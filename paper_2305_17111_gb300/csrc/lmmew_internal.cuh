@@ -385,7 +385,7 @@ struct ForwardPlan {
     int64_t n, cap;
     int tpc, blocks;
 };
-ForwardPlan forward_plan(const lm_handle* h, int64_t n, int64_t cap_max);
+ForwardPlan forward_plan(const lm_handle* h, int64_t n, int64_t cap_max, int te);   // te: tile size
 size_t forward_region_bytes(const lm_handle* h, const ForwardPlan& p);
 int forward_async(lm_handle* h, const lm_events* ev, const float* image, float* out_y,
                   const GroupArrays& ga, const ForwardPlan& p, char* arena, cudaStream_t st);
@@ -396,7 +396,7 @@ int forward_nodes(lm_handle* h, const lm_events* ev, const float* image, float* 
                   char* arena, cudaStream_t st);
 int forward_nodes_block(const lm_handle* h, size_t bytes);
 size_t forward_nodes_bytes(const lm_handle* h, int block);
-size_t noalloc_rows_bytes(const lm_handle* h, int64_t n);
+size_t noalloc_rows_bytes(const lm_handle* h, int64_t n, int te);
 constexpr size_t kNoAllocBytes = size_t(16) << 20;   // lm_forward_noalloc's static array: 16 MiB
 bool node_use(const lm_handle* h, int64_t n);
 bool node_use_back(const lm_handle* h, int64_t n);   // the same for lm_backproject

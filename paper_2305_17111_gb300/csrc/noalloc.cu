@@ -64,8 +64,8 @@ extern "C" int lm_forward_noalloc(lm_handle* h, const lm_events* ev, const float
         return set_error(LMMEW_ERR_INVALID_ARG, "at most 2^31 - 1 events per call");
     // one row block of every event; every word of the region is written
     // before it is read within a call, so nothing has to start at zero
-    const ForwardPlan fp = forward_plan(h, n, int64_t(1) << 40);
-    const size_t need = noalloc_rows_bytes(h, n);
+    const ForwardPlan fp = forward_plan(h, n, int64_t(1) << 40, h->tile_ev);
+    const size_t need = noalloc_rows_bytes(h, n, h->tile_ev);
     if (need > kNoAllocBytes)
         return set_error(LMMEW_ERR_INVALID_ARG,
                          "lm_forward_noalloc: " + std::to_string(n) + " events need " +
