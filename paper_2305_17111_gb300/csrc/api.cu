@@ -1425,12 +1425,15 @@ int lm_osem_batch(lm_handle* h, int n_real, const lm_events* events, int n_subse
     // the number of events, so there is nothing to share); the others share
     // row launches
     std::vector<lm_events> rest;
-    std::vector<int> rest_of;
-    for (int r = 0; r < n_real; ++r)
-        if (!node_use_osem(h, events[r].n, n_subsets)) {
+    std::vector<int> rest_of, dense;
+    for (int r = 0; r < n_real; ++r) {
+        if (node_use_osem(h, events[r].n, n_subsets)) {
+            dense.push_back(r);
+        } else {
             rest.push_back(events[r]);
             rest_of.push_back(r);
         }
+    }
     if ((int)rest.size() == n_real)
         return osem_batch_rows(h, n_real, events, nullptr, n_subsets, n_iters, images, loglik, stream);
     cudaStream_t st = (cudaStream_t)stream;
@@ -1438,10 +1441,11 @@ int lm_osem_batch(lm_handle* h, int n_real, const lm_events* events, int n_subse
     for (int r = 0; r < n_real && rc == LMMEW_OK; ++r) rc = launch_validate(h, &events[r], st);
     if (rc == LMMEW_OK) rc = take_status(h, st);
     if (rc == LMMEW_OK) rc = subset_sensitivity(h, n_subsets, st);
-    for (int r = 0; r < n_real && rc == LMMEW_OK; ++r)
-        if (node_use_osem(h, events[r].n, n_subsets))
-            rc = lm_osem(h, &events[r], n_subsets, n_iters, 0, 0, images + (size_t)r * m.n * m.n,
-                         loglik ? loglik + (size_t)r * n_iters * n_subsets : nullptr, stream);
+    for (size_t i = 0; i < dense.size() && rc == LMMEW_OK; ++i) {
+        const int r = dense[i];
+        rc = lm_osem(h, &events[r], n_subsets, n_iters, 0, 0, images + (size_t)r * m.n * m.n,
+                     loglik ? loglik + (size_t)r * n_iters * n_subsets : nullptr, stream);
+    }
     if (rc != LMMEW_OK || rest.empty()) return rc;
     return osem_batch_rows(h, (int)rest.size(), rest.data(), rest_of.data(), n_subsets, n_iters,
                            images, loglik, stream);

@@ -79,6 +79,23 @@ def test_tile_size_has_no_say(big):
         gpu.forward_noalloc(_events(sc, 120_000, 2), lam, torch.empty(120_000, device="cuda"))
 
 
+def test_batch_reconstructs_every_realisation_after_a_retune(big):
+    sc, gpu, lam = big
+    lists = [_events(sc, n, 10 + n) for n in (40_000, 3_000, 60_000)]
+    gpu.set_tile_events(128)
+    want = []
+    for d in lists:
+        img = lam.clone()
+        gpu.osem(d, img, 10, 1)
+        want.append(img)
+    for tile in (128, 32):
+        gpu.set_tile_events(tile)
+        imgs = lam.repeat(3, 1).contiguous()
+        gpu.osem_batch(lists, imgs, 10, 1)
+        for i in range(3):
+            assert torch.equal(imgs[i], want[i]), f"realisation {i}, {tile}-event tiles"
+
+
 def test_noalloc_goes_through_blocks_of_angles():
     """The 64 x 64 scanner: a few angles' node sums at a time in the array."""
     sc = preset("lmmew_64")
