@@ -247,8 +247,11 @@ int lm_backproject(lm_handle* h, const lm_events* events, const float* weight,
  * by an earlier call and the next (start_iter, start_subset) reproduces an
  * uninterrupted run bit for bit.  The row kernel's launch shape (event lists
  * below the nodes' density) is chosen by the autotuner described at
- * lm_batch_tuning before the first sub-iteration.
- * Errors: as lm_forward. */
+ * lm_batch_tuning before the first sub-iteration.  Dense lists stay on their
+ * nodes however little memory is free (the angles' sums in smaller blocks; OOM
+ * where those of one angle find no room), where lm_forward and lm_backproject
+ * take the rows instead.
+ * Errors: as lm_forward, OOM. */
 int lm_osem(lm_handle* h, const lm_events* events, int n_subsets, int n_iters,
             int start_iter, int start_subset, float* image, double* loglik,
             lm_stream stream);

@@ -894,7 +894,7 @@ int lm_forward(lm_handle* h, const lm_events* ev, const float* image, float* out
 }
 
 // Scratch of the node route's sorted forms for sets of at most `angles` angles;
-// the forward sums go `block` angles at a time.
+// the forward sums go s->block angles at a time (the bits do not depend on it).
 namespace {
 struct NodeScratch {
     int block;
@@ -905,7 +905,6 @@ size_t node_scratch(const lm_handle* h, int angles, char* base, NodeScratch* s) 
     const ModelConst& m = h->mc;
     const NodeConst& N = h->nodes;
     const size_t cells = (size_t)angles * m.B, nq_pad = (size_t)m.nqt * kQT;
-    s->block = std::min(angles, std::max(1, forward_nodes_block(h, kNodeBudgetBytes)));
     char* p = base;
     s->lam = bump<float>(p, m.nq);
     s->HT = bump<float>(p, (size_t)node_back_parts(h, angles) * m.np * N.nn);
@@ -923,6 +922,18 @@ size_t node_scratch(const lm_handle* h, int angles, char* base, NodeScratch* s) 
     s->ll = bump<double>(p, cells);
     s->num = bump<double>(p, m.nq);
     return (size_t)(p - base) + 256;
+}
+
+// The same, allocated: in smaller blocks where all angles at once do not fit.
+int ensure_node_scratch(lm_handle* h, int angles, NodeScratch* s, cudaStream_t st) {
+    s->block = std::min(angles, std::max(1, forward_nodes_block(h, kNodeBudgetBytes)));
+    int rc = ensure(h, h->scratch_work, node_scratch(h, angles, nullptr, s), st);
+    while (rc == LMMEW_ERR_OOM && s->block > 1) {
+        s->block /= 2;
+        rc = ensure(h, h->scratch_work, node_scratch(h, angles, nullptr, s), st);
+    }
+    if (rc == LMMEW_OK) node_scratch(h, angles, (char*)h->scratch_work.ptr, s);
+    return rc;
 }
 
 int node_forward_blocks(lm_handle* h, const NodeScratch& s, int a0, int a_step, int angles,
@@ -947,9 +958,8 @@ int backproject_nodes(lm_handle* h, const lm_events* ev, const float* weight, fl
     if (rc != LMMEW_OK) return rc;
     NodeScratch s;
     rc = ensure(h, h->scratch_sort, cell_scratch_bytes(h, ev->n), st);
-    if (rc == LMMEW_OK) rc = ensure(h, h->scratch_work, node_scratch(h, m.A, nullptr, &s), st);
+    if (rc == LMMEW_OK) rc = ensure_node_scratch(h, m.A, &s, st);
     if (rc != LMMEW_OK) return rc;
-    node_scratch(h, m.A, (char*)h->scratch_work.ptr, &s);
     char* arena = (char*)h->scratch_sort.ptr;
     CellEvents ce;
     rc = sort_cells(h, ev, ga.rank_of_angle, &ce, arena, st);
@@ -975,9 +985,8 @@ int osem_nodes(lm_handle* h, const lm_events* ev, int n_subsets, int n_iters, in
     const int most = (m.A + n_subsets - 1) / n_subsets;
     NodeScratch s;
     rc = ensure(h, h->scratch_sort, cell_scratch_bytes(h, ev->n), st);
-    if (rc == LMMEW_OK) rc = ensure(h, h->scratch_work, node_scratch(h, most, nullptr, &s), st);
+    if (rc == LMMEW_OK) rc = ensure_node_scratch(h, most, &s, st);
     if (rc != LMMEW_OK) return rc;
-    node_scratch(h, most, (char*)h->scratch_work.ptr, &s);
     char* arena = (char*)h->scratch_sort.ptr;
     CellEvents ce;
     rc = sort_cells(h, ev, ga.rank_of_angle, &ce, arena, st);
@@ -1083,10 +1092,10 @@ int lm_osem(lm_handle* h, const lm_events* ev, int n_subsets, int n_iters, int s
     cudaStream_t st = (cudaStream_t)stream;
     rc = subset_sensitivity(h, n_subsets, st);
     if (rc != LMMEW_OK) return rc;
-    if (node_use_osem(h, ev->n, n_subsets)) {
-        rc = osem_nodes(h, ev, n_subsets, n_iters, start_iter, start_subset, image, loglik, st);
-        if (rc != LMMEW_ERR_OOM) return rc;   // no room for the node sums: the rows
-    }
+    // (no rows where the node sums find no room: a reconstruction resumed in
+    // another state of the memory would take another route than its first part)
+    if (node_use_osem(h, ev->n, n_subsets))
+        return osem_nodes(h, ev, n_subsets, n_iters, start_iter, start_subset, image, loglik, st);
     GroupArrays ga;
     rc = group_arrays(h, n_subsets, &ga);
     if (rc != LMMEW_OK) return rc;

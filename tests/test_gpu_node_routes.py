@@ -109,3 +109,28 @@ def test_noalloc_goes_through_blocks_of_angles():
     gpu.forward_noalloc(dev, lam, out)
     assert torch.equal(out, y)
     gpu.close()
+
+
+def test_a_reconstruction_keeps_its_route_when_memory_is_short():
+    """80 MiB free, where the node sums of all 24 angles at once take 120: the
+    same bits as with all of the memory (in smaller blocks), not the rows."""
+    sc = preset("lmmew_64").with_(n_angles=24, n_subsets=1)
+    rho = sc.make_phantom().rho
+    dev = _events(sc, 6_000, 3)
+    lam = torch.from_numpy((rho.reshape(-1) > 0).astype(np.float32)).cuda()
+    want, got = lam.clone(), lam.clone()
+    gpu = lm.Model.from_scenario(sc, rho)
+    gpu.osem(dev, want, 1, 2)
+    gpu.close()
+    gpu = lm.Model.from_scenario(sc, rho)
+    gpu.set_tile_events(32)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    rest = torch.empty(torch.cuda.mem_get_info()[0] - (80 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        gpu.osem(dev, got, 1, 2)
+    finally:
+        del rest
+        torch.cuda.empty_cache()
+    assert torch.equal(got, want)
+    gpu.close()
