@@ -63,9 +63,11 @@
  *     one angle exceed the 16 MiB of lm_forward_noalloc, lm_forward keeps the
  *     rows too for the lists whose rows fit there;
  *   - reconstructions of two iterations or more that go through the rows keep
- *     their scatter rows from the first iteration for the later ones, in the
- *     handle's scratch, when the rows of the whole call take at most 16 GiB
- *     and half of the free memory (the results are the same bits);
+ *     their scatter rows from the first iteration for the later ones when the
+ *     rows of the whole call take at most 16 GiB and half of the free memory
+ *     (the results are the same bits): in the handle's scratch up to 4 GiB, the
+ *     most a row block takes without them, and more in an allocation that is
+ *     given back in stream order at the end of the call;
  *   - there is no CPU fallback: every step runs in this library's kernels.
  *
  * Images are n*n arrays in raster order [iy*n + ix]; pixel (ix, iy) has its

@@ -248,6 +248,28 @@ bool keep_rows_fit(const lm_handle* h, int64_t n, int iterations) {
     return bytes <= (free_b + h->scratch_work.bytes) / 2;
 }
 
+// Kept rows beyond what a handle's row block may take anyway are not left in its
+// scratch: they are allocated for the call, in stream order, and given back at
+// its end.
+struct CallRows {
+    cudaStream_t st;
+    float* p = nullptr;
+    ~CallRows() { release(); }
+    void release() {
+        if (p) cudaFreeAsync(p, st);
+        p = nullptr;
+    }
+    // keep: whether rows of `floats` are kept at all
+    void take(size_t floats, bool* keep) {
+        if (!*keep || floats <= kRowBudgetFloats) return;
+        if (cudaMallocAsync((void**)&p, sizeof(float) * floats, st) != cudaSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+            *keep = false;
+        }
+    }
+};
+
 }  // namespace
 
 int prof_start(lm_handle* h, cudaStream_t st) {
@@ -801,9 +823,11 @@ static int osem_planned(lm_handle* h, const lm_events* ev, int n_subsets, int n_
         }
     }
     bool keep = keep_rows_fit(h, se.n_valid, n_iters - start_iter);
-    auto need = [&](bool all) {
-        return bump_bytes(sizeof(float) * m.nq) +
-               bump_bytes(sizeof(float) * rs * std::max<int64_t>(all ? se.n_valid : biggest, 1)) +
+    CallRows kept{st};
+    kept.take((size_t)rs * se.n_valid, &keep);
+    auto scratch_rows = [&] { return kept.p ? 0 : (size_t)rs * std::max<int64_t>(keep ? se.n_valid : biggest, 1); };
+    auto need = [&] {
+        return bump_bytes(sizeof(float) * m.nq) + bump_bytes(sizeof(float) * scratch_rows()) +
                bump_bytes(sizeof(float) * m.nqt * std::max<int64_t>(biggest, 1)) +
                bump_bytes(sizeof(float) * std::max<int64_t>(parts_max, 1) * m.nq) +
                bump_bytes(sizeof(double) * std::max<int64_t>(parts_max, 1)) +
@@ -811,15 +835,17 @@ static int osem_planned(lm_handle* h, const lm_events* ev, int n_subsets, int n_
     };
     rc = surrogate_prepare(h, biggest, st);
     if (rc != LMMEW_OK) return rc;
-    rc = ensure(h, h->scratch_work, need(keep), st);
+    rc = ensure(h, h->scratch_work, need(), st);
     if (rc == LMMEW_ERR_OOM && keep) {
         keep = false;
-        rc = ensure(h, h->scratch_work, need(false), st);
+        kept.release();
+        rc = ensure(h, h->scratch_work, need(), st);
     }
     if (rc != LMMEW_OK) return rc;
     char* w = (char*)h->scratch_work.ptr;
     float* lam_v = bump<float>(w, m.nq);
-    float* rows = bump<float>(w, (size_t)rs * std::max<int64_t>(keep ? se.n_valid : biggest, 1));
+    float* rows = bump<float>(w, scratch_rows());
+    if (kept.p) rows = kept.p;
     float* ypart = bump<float>(w, (size_t)m.nqt * std::max<int64_t>(biggest, 1));
     float* bpart = bump<float>(w, (size_t)std::max<int64_t>(parts_max, 1) * m.nq);
     double* llpart = bump<double>(w, std::max<int64_t>(parts_max, 1));
@@ -1135,23 +1161,27 @@ int lm_osem(lm_handle* h, const lm_events* ev, int n_subsets, int n_iters, int s
     // rows of one row block, or of every event (kept after a subset's first
     // sub-iteration)
     bool keep = keep_rows_fit(h, n, n_iters - start_iter);
-    auto need = [&](bool all) {
-        return bump_bytes(sizeof(float) * m.nq) +
-               bump_bytes(sizeof(float) * (size_t)rs * (all ? (size_t)n : (size_t)cap)) +
+    CallRows kept{st};
+    kept.take((size_t)rs * (size_t)n, &keep);
+    auto scratch_rows = [&] { return kept.p ? 0 : (size_t)rs * (keep ? (size_t)n : (size_t)cap); };
+    auto need = [&] {
+        return bump_bytes(sizeof(float) * m.nq) + bump_bytes(sizeof(float) * scratch_rows()) +
                bump_bytes(sizeof(float) * (size_t)m.nqt * cap) +
                bump_bytes(sizeof(float) * (size_t)blocks * ppc * m.nq) +
                bump_bytes(sizeof(double) * (size_t)blocks * ppc) + bump_bytes(sizeof(double) * m.nq) +
                bump_bytes(sizeof(ChunkRange) * (size_t)n_subsets * blocks);
     };
-    rc = ensure(h, h->scratch_work, need(keep), st);
+    rc = ensure(h, h->scratch_work, need(), st);
     if (rc == LMMEW_ERR_OOM && keep) {
         keep = false;
-        rc = ensure(h, h->scratch_work, need(false), st);
+        kept.release();
+        rc = ensure(h, h->scratch_work, need(), st);
     }
     if (rc != LMMEW_OK) return rc;
     char* w = (char*)h->scratch_work.ptr;
     float* lam_v = bump<float>(w, m.nq);
-    float* rows = bump<float>(w, (size_t)rs * (keep ? (size_t)n : (size_t)cap));
+    float* rows = bump<float>(w, scratch_rows());
+    if (kept.p) rows = kept.p;
     float* ypart = bump<float>(w, (size_t)m.nqt * cap);
     float* bpart = bump<float>(w, (size_t)blocks * ppc * m.nq);
     double* llpart = bump<double>(w, (size_t)blocks * ppc);
@@ -1281,9 +1311,11 @@ static int osem_batch_rows(lm_handle* h, int n_real, const lm_events* events, co
         parts_max = std::max(parts_max, c);
     }
     bool keep = keep_rows_fit(h, se.n_total, n_iters);
-    auto need = [&](bool all) {
-        return bump_bytes(sizeof(float) * (size_t)R * m.nq) +
-               bump_bytes(sizeof(float) * (size_t)rs * (all ? std::max<int64_t>(se.n_total, 1) : biggest)) +
+    CallRows kept{st};
+    kept.take((size_t)rs * se.n_total, &keep);
+    auto scratch_rows = [&] { return kept.p ? 0 : (size_t)rs * (keep ? std::max<int64_t>(se.n_total, 1) : biggest); };
+    auto need = [&] {
+        return bump_bytes(sizeof(float) * (size_t)R * m.nq) + bump_bytes(sizeof(float) * scratch_rows()) +
                bump_bytes(sizeof(float) * (size_t)m.nqt * biggest) +
                bump_bytes(sizeof(float) * parts_max * m.nq) + bump_bytes(sizeof(double) * parts_max) +
                bump_bytes(sizeof(double) * (size_t)R * m.nq) + bump_bytes(sizeof(BpChunk) * max_chunks) +
@@ -1291,15 +1323,17 @@ static int osem_batch_rows(lm_handle* h, int n_real, const lm_events* events, co
                bump_bytes(sizeof(int64_t) * (size_t)(n_blk + 1)) +
                bump_bytes(sizeof(int) * (size_t)(G + 1)) + bump_bytes(sizeof(int) * (size_t)R);
     };
-    rc = ensure(h, h->scratch_work, need(keep), st);
+    rc = ensure(h, h->scratch_work, need(), st);
     if (rc == LMMEW_ERR_OOM && keep) {
         keep = false;
-        rc = ensure(h, h->scratch_work, need(false), st);
+        kept.release();
+        rc = ensure(h, h->scratch_work, need(), st);
     }
     if (rc != LMMEW_OK) return rc;
     char* w = (char*)h->scratch_work.ptr;
     float* lam_v = bump<float>(w, (size_t)R * m.nq);
-    float* rows = bump<float>(w, (size_t)rs * (keep ? std::max<int64_t>(se.n_total, 1) : biggest));
+    float* rows = bump<float>(w, scratch_rows());
+    if (kept.p) rows = kept.p;
     float* ypart = bump<float>(w, (size_t)m.nqt * biggest);
     float* bpart = bump<float>(w, parts_max * m.nq);
     double* llpart = bump<double>(w, parts_max);

@@ -56,3 +56,29 @@ def test_iterations_on_kept_rows_match_recomputed_ones(name, n, scatter):
     for i in range(2):
         assert torch.equal(imgs[i], want[i][0]), f"realisation {i}"
     gpu.close()
+
+
+def test_rows_beyond_a_row_block_are_given_back():
+    """10 GB of kept rows (energy pruning off: the rows' route for a dense list):
+    the same bits as one iteration per call, and the handle keeps no more than
+    the 4 GiB a row block may take (with its eighth to spare and the sort)."""
+    sc = preset("lmmew_64").with_(n_subsets=1)
+    ph = sc.make_phantom()
+    gpu = lm.Model.from_scenario(sc, ph.rho)
+    gpu.set_energy_pruning(False)
+    n = 3_000_000
+    rng = np.random.default_rng(1)
+    dev = lm.DeviceEvents(rng.integers(0, sc.n_angles, n), rng.integers(16, 48, n),
+                          rng.uniform(60.0, 290.0, n).astype(np.float32))
+    assert 4 * n * gpu.nq > 10e9
+    lam0 = torch.from_numpy((ph.rho.reshape(-1) > 0).astype(np.float32)).cuda()
+    both, one = lam0.clone(), lam0.clone()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    gpu.osem(dev, both, 1, 2)
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] < 5.5 * 2**30
+    gpu.osem(dev, one, 1, 1)
+    gpu.osem(dev, one, 1, 2, 1, 0)
+    assert torch.equal(both, one)
+    gpu.close()
