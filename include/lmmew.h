@@ -501,7 +501,8 @@ int lm_profile_read(lm_handle* h, double* out5);
 /* Model sizes, for work accounting: out8[0] = voxels in the support,
  * out8[1] = scatter points with rho > 0, out8[2] = emission lines,
  * out8[3] = angles, out8[4] = bins, out8[5] = exponentials per event row,
- * out8[6] = bytes of device tables, out8[7] = set-up time in microseconds. */
+ * out8[6] = bytes of the device's path and node tables, out8[7] = set-up time in
+ * microseconds (of all tables, on the host's clock). */
 int lm_model_info(const lm_handle* h, int64_t* out8);
 
 /* Exponential throughput of the current GPU (an instrument of this library,

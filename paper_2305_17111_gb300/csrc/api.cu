@@ -3,6 +3,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <chrono>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -561,12 +562,15 @@ int lm_create(const lm_geometry* g, const lm_attenuation* at, const lm_lines* ln
                               ? (m.knot_mu[i + 1] - m.knot_mu[i]) / (m.knot_e[i + 1] - m.knot_e[i])
                               : 0.0;
     h->n_subsets_default = n_subsets;
+    const auto t0 = std::chrono::steady_clock::now();
     int rc = build_tables(h, at->rho, support);
     if (rc == LMMEW_OK) {
         line_reaches(h);
         build_energy_classes(h);
         rc = build_nodes(h);
     }
+    // (both return with the device idle)
+    h->setup_ms = std::chrono::duration<float, std::milli>(std::chrono::steady_clock::now() - t0).count();
     if (rc == LMMEW_OK &&
         (cudaMalloc(&h->d_term_counter, sizeof(unsigned long long)) != cudaSuccess ||
          cudaMemset(h->d_term_counter, 0, sizeof(unsigned long long)) != cudaSuccess ||
@@ -656,7 +660,7 @@ int lm_model_info(const lm_handle* h, int64_t* out8) {
     out8[3] = h->mc.A;
     out8[4] = h->mc.B;
     out8[5] = h->terms_per_event;
-    out8[6] = (int64_t)h->tab_bytes;
+    out8[6] = (int64_t)(h->tab_bytes + h->node_bytes);
     out8[7] = (int64_t)(h->setup_ms * 1000.0f);
     return LMMEW_OK;
 }

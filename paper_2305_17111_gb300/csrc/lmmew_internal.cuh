@@ -195,6 +195,7 @@ struct lm_handle {
     lmmew::NodeTables node_tables{};
     int node_route = 0;            // 1: the model has the node route
     void* d_node_tables = nullptr;
+    size_t node_bytes = 0;         // of the node tables and the grouped collimator values
     float* d_node_groups = nullptr;   // collimator values of 8 scatter points at a time
     lmmew::ChunkRange* d_clip = nullptr;   // a row launch's tiles clipped to one angle block
     // cached subset sensitivities for the last partition asked for

@@ -1889,6 +1889,7 @@ int build_nodes(lm_handle* h) {
         cudaGetLastError();
         return LMMEW_OK;                 // no room: the rows
     }
+    h->node_bytes = bytes;
     layout((char*)h->d_node_tables);
     std::vector<char> blob(host_bytes, 0);
     auto put = [&](const void* dst, const void* src, size_t n) {
@@ -1958,6 +1959,7 @@ int build_nodes(lm_handle* h) {
         cudaGetLastError();
         return LMMEW_OK;
     }
+    h->node_bytes += sizeof(float) * per_angle * m.A;
     k_group_values<<<dim3((unsigned)((per_angle + 255) / 256), m.A), 256>>>(
         h->d_cs, T.rank, T.grp_pt, T.grp_bins, m.B, m.np, m.npc, groups, N.nbg_max, h->d_node_groups);
     h->launches += 8;

@@ -582,11 +582,6 @@ int subset_sensitivity(lm_handle* h, int parts, cudaStream_t st) {
 int build_tables(lm_handle* h, const float* rho_host, const uint8_t* support_host) {
     ModelConst& m = h->mc;
     const int n = m.n;
-    cudaEvent_t e0, e1;
-    cudaEventCreate(&e0);
-    cudaEventCreate(&e1);
-    cudaEventRecord(e0, 0);
-
     // support voxel list (raster order)
     std::vector<int> q_pix;
     for (int i = 0; i < n * n; ++i)
@@ -856,11 +851,7 @@ int build_tables(lm_handle* h, const float* rho_host, const uint8_t* support_hos
     d_mu_line.p = nullptr;
     LMMEW_CUDA(cudaMalloc(&h->d_status, sizeof(int)));
     LMMEW_CUDA(cudaMemset(h->d_status, 0, sizeof(int)));
-    cudaEventRecord(e1, 0);
     LMMEW_CUDA(cudaDeviceSynchronize());
-    cudaEventElapsedTime(&h->setup_ms, e0, e1);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
     return subset_sensitivity(h, h->n_subsets_default, 0) == LMMEW_OK
                ? (cudaDeviceSynchronize() == cudaSuccess ? LMMEW_OK
                                                          : set_error(LMMEW_ERR_CUDA, "set-up"))

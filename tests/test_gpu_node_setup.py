@@ -104,3 +104,22 @@ def test_tables_of_a_small_model_take_few_launches():
         count[frac] = gpu.profile_read()["kernels"]
         gpu.close()
     assert 1 <= count[0.10] - count[0.02] <= 9
+
+
+def test_node_tables_are_part_of_the_accounts():
+    """lm_model_info's table bytes and set-up time cover the node tables: 12 + 4
+    bytes a line for every pair of voxel and scatter point at least."""
+    sc = preset("small_24").with_(n_angles=24, scatter_n=12)
+    rho = sc.make_phantom().rho
+    ms = {}
+    for frac in (0.10, 0.02):
+        for _ in range(12):
+            gpu = lm.Model.from_scenario(sc.with_(fwhm_frac=frac), rho)
+            ms[frac] = min(ms.get(frac, 1e9), gpu.setup_ms)
+            nodes = gpu.table_bytes - gpu.table_streaming()[1]
+            if frac == 0.10:
+                assert nodes > (12 + 4 * gpu.n_lines) * gpu.nq * gpu.np_scatter
+            else:
+                assert nodes == 0
+            gpu.close()
+    assert ms[0.10] > ms[0.02] + 0.05
