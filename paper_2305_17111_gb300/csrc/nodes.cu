@@ -1601,7 +1601,7 @@ size_t band_smem(int band) {
 // launches, one allocation more for the grouped collimator values, a copy up and
 // one down; a model of 24 x 24 voxels, 12 x 12 cells and 24 angles takes 1.5 ms
 // with them (2.2 ms with host tables and global sorts, 1.75 ms without any).
-int build_nodes(lm_handle* h) {
+static int build_node_tables(lm_handle* h) {
     const ModelConst& m = h->mc;
     NodeConst& N = h->nodes;
     NodeTables& T = h->node_tables;
@@ -1967,6 +1967,19 @@ int build_nodes(lm_handle* h) {
     LMMEW_CUDA(cudaDeviceSynchronize());   // (the tables are used on any stream)
     h->node_route = 1;
     return LMMEW_OK;
+}
+
+int build_nodes(lm_handle* h) {
+    const int rc = build_node_tables(h);
+    if (h->node_route == 0) {            // given up, or an error: nothing reads the tables
+        cudaFree(h->d_node_tables);
+        cudaFree(h->d_node_groups);
+        h->d_node_tables = nullptr;
+        h->d_node_groups = nullptr;
+        h->node_tables = NodeTables{};
+        h->node_bytes = 0;
+    }
+    return rc;
 }
 
 size_t node_angle_bytes(const lm_handle* h) {
