@@ -82,3 +82,35 @@ def test_rows_beyond_a_row_block_are_given_back():
     gpu.osem(dev, one, 1, 2, 1, 0)
     assert torch.equal(both, one)
     gpu.close()
+
+
+@pytest.mark.parametrize("n", [31, 300])
+@pytest.mark.parametrize("form", ["surrogate", "fp16", "bf16"])
+def test_other_forms_keep_the_same_rows(n, form):
+    """The full surrogate and the reduced-precision forms, one call and batched."""
+    sc = preset("small_24")
+    ph = sc.make_phantom()
+    gpu = lm.Model.from_scenario(sc, ph.rho)
+    net = lm.Surrogate(3)
+    if form == "surrogate":
+        gpu.set_scatter_model(form, net)
+    else:
+        gpu.set_scatter_precision(form)
+    devs = [lm.DeviceEvents.from_list(simulate(sc, n_events=k, seed=90 + k)) for k in (n, 2 * n + 5)]
+    lam0 = torch.from_numpy((ph.rho.reshape(-1) > 0).astype(np.float32)).cuda()
+    n_sub, n_it = sc.n_subsets, 3
+    want = []
+    for d in devs:
+        one, l1 = lam0.clone(), torch.zeros(n_it * n_sub, dtype=torch.float64, device="cuda")
+        for it in range(n_it):
+            gpu.osem(d, one, n_sub, it + 1, start_iter=it, loglik=l1)
+        want.append(one)
+        all3, l3 = lam0.clone(), torch.zeros_like(l1)
+        gpu.osem(d, all3, n_sub, n_it, loglik=l3)
+        assert torch.equal(all3, one)
+        assert torch.equal(l3, l1)
+    imgs = lam0.repeat(2, 1).contiguous()
+    gpu.osem_batch(devs, imgs, n_sub, n_it)
+    for i in range(2):
+        assert torch.equal(imgs[i], want[i]), f"realisation {i}"
+    gpu.close()

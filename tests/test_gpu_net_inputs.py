@@ -41,3 +41,25 @@ def test_forward_rounds_rows_of_any_alignment(n):
     # outputs over the first inputs
     _forward(net, x.data_ptr(), n, x.data_ptr())
     assert torch.equal(x[:n], a)
+
+
+@pytest.mark.parametrize("n", [1, 127, 129, 1000])
+@pytest.mark.parametrize("weighted", [False, True])
+def test_gradient_rounds_its_inputs(n, weighted):
+    """FP32 inputs give what inputs already in BF16 give, with the loss, also where
+    the scratch has grown since a smaller call and is larger than the call needs."""
+    net = lm.Surrogate(seed=4)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    x = torch.randn(n, 32, generator=g, device="cuda")
+    t = torch.randn(n, generator=g, device="cuda")
+    w = torch.rand(n, generator=g, device="cuda") + 0.5 if weighted else None
+    rounded = x.bfloat16().float()
+    first = net.gradient(x, t, w)
+    again = net.gradient(rounded, t, w)
+    big = torch.randn(3001, 32, generator=g, device="cuda")
+    net.gradient(big, torch.randn(3001, generator=g, device="cuda"))     # the scratch grows
+    later = net.gradient(x, t, w)
+    assert torch.isfinite(first[0]).all() and first[1] > 0.0
+    for other in (again, later):
+        assert torch.equal(first[0], other[0]) and first[1] == other[1]
+    net.close()
