@@ -263,7 +263,7 @@ __device__ __forceinline__ int offset_of(const NodeConst& N, int w, int r) {
 // that walks its paths takes 28 us more for 60 angles, a thread for all slots
 // 290 us instead of 10 at 3464 voxels: both wait for one path after the other.)
 constexpr int kMostWindows = 64;   // of a line: 4 per knot
-constexpr int kSlotWords = (kTapsN + 2) * 32 + 2 * kMostWindows;   // a warp's: taps, positions, sides, runs
+constexpr int kSlotWords = (kTapsN + 1) * 32 + 2 * kMostWindows;   // a warp's: taps, positions, runs
 __device__ __forceinline__ void slot_taps(const NodeParams& P, int ai, int p, int w, float* sh) {
     constexpr int kHalf = kTapsN / 2;
     const int lane = threadIdx.x & 31;
@@ -273,19 +273,27 @@ __device__ __forceinline__ void slot_taps(const NodeParams& P, int ai, int p, in
     const int* pq = P.path_q + (size_t)p * P.nq;
     const float* pb = P.path_b + ((size_t)w * P.np + p) * P.nq;
     int* pos = reinterpret_cast<int*>(sh + kTapsN * 32);
-    int* on = pos + 32;
-    // the windows' runs of directions, a lane each
-    const int windows = P.N.win_off[w + 1] - P.N.win_off[w];
-    int2* run = reinterpret_cast<int2*>(on + 32);
-    for (int k = lane; k < windows; k += 32) {
-        const int2 win = P.win[P.N.win_off[w] + k];
-        const int c0 = max(s + win.x, 0), c1 = min(s + win.y, n);
-        run[k] = c0 <= c1 ? make_int2(st[c0], st[c1 + 1]) : make_int2(0, 0);
+    // the windows' runs of directions, a lane each, empty ones left out
+    int windows = 0;
+    int2* run = reinterpret_cast<int2*>(pos + 32);
+    for (int k0 = P.N.win_off[w]; k0 < P.N.win_off[w + 1]; k0 += 32) {
+        int2 mine = make_int2(0, 0);
+        if (k0 + lane < P.N.win_off[w + 1]) {
+            const int2 win = P.win[k0 + lane];
+            const int c0 = max(s + win.x, 0), c1 = min(s + win.y, n);
+            if (c0 <= c1) mine = make_int2(st[c0], st[c1 + 1]);
+        }
+        const unsigned some = __ballot_sync(0xffffffffu, mine.x < mine.y);
+        if (mine.x < mine.y) run[windows + __popc(some & ((1u << lane) - 1))] = mine;
+        windows += __popc(some);
     }
     __syncwarp();
     for (int z0 = P.N.slot_off[w]; z0 < P.N.slot_off[w + 1]; z0 += 32) {
-        const int count = min(32, P.N.slot_off[w + 1] - z0), shares = 32 / count;
-        const int z = z0 + lane % count, share = lane / count;
+        const int count = min(32, P.N.slot_off[w + 1] - z0);
+        // lanes per slot, each with every so many paths of the 32
+        const int shares = count > 16 ? 1 : count > 8 ? 2 : 4, slots = 32 / shares;
+        const int z = z0 + min(lane & (slots - 1), count - 1), share = lane / slots;
+        const unsigned paths = (shares == 1 ? ~0u : shares == 2 ? 0x55555555u : 0x11111111u) << share;
         const int m = P.slot[z].offset - P.N.m_off[w], side = P.slot[z].side;
         float sum = 0.f;
         int k = 0, r = 0, r1 = 0;
@@ -306,6 +314,7 @@ __device__ __forceinline__ void slot_taps(const NodeParams& P, int ai, int p, in
             }
             if (fill == 0) break;
             __syncwarp();
+            int own = -1;
             if (mine >= 0) {
                 int c;
                 const float f = direction_pos(fix[mine], n, &c);
@@ -317,23 +326,27 @@ __device__ __forceinline__ void slot_taps(const NodeParams& P, int ai, int p, in
                 if (2 * d > n) d -= n;
                 if (2 * d <= -n) d += n;
                 pos[lane] = d;
-                on[lane] = side_of_knots(P.N, w, d, f);
+                own = side_of_knots(P.N, w, d, f);
+            }
+            unsigned todo = 0;          // paths of the slot's side
+            for (int b = 0; b <= P.N.kinks[w]; ++b) {
+                const unsigned there = __ballot_sync(0xffffffffu, own == b);
+                if (b == side) todo = there & paths;
             }
             __syncwarp();
-            if (share < shares)
-                for (int i = share; i < fill; i += shares) {
-                    if (on[i] != side) continue;
-                    // the path's tap on node s + m, and on s - m where that is another
-                    int t = m - pos[i] + kHalf;
-                    if (t >= n) t -= n;
-                    if ((unsigned)t < kTapsN) sum += sh[t * 32 + i];
-                    t = -m - pos[i] + kHalf;
-                    if (t < 0) t += n;
-                    if ((unsigned)t < kTapsN && m > 0 && 2 * m != n) sum += sh[t * 32 + i];
-                }
+            for (; todo; todo &= todo - 1) {
+                const int i = __ffs(todo) - 1;
+                // the path's tap on node s + m, and on s - m where that is another
+                int t = m - pos[i] + kHalf;
+                if (t >= n) t -= n;
+                if ((unsigned)t < kTapsN) sum += sh[t * 32 + i];
+                t = -m - pos[i] + kHalf;
+                if (t < 0) t += n;
+                if ((unsigned)t < kTapsN && m > 0 && 2 * m != n) sum += sh[t * 32 + i];
+            }
         }
         float all = sum;
-        for (int j = 1; j < shares; ++j) all += __shfl_down_sync(0xffffffffu, sum, j * count);
+        for (int j = 1; j < shares; ++j) all += __shfl_down_sync(0xffffffffu, sum, j * slots);
         if (lane < count) P.side[((size_t)ai * P.np + p) * P.N.slots + z] = all;
     }
 }
