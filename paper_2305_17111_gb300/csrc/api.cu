@@ -431,8 +431,8 @@ static bool node_model(const lm_handle* h) {
 }
 
 // Projections of 2 events or more per detector angle go through the nodes, at a
-// cost that does not depend on the events: 138 us at 484 voxels and 32 angles,
-// 378 us at 864 voxels and 60; the rows take 177 and 1025 us for 2 events per
+// cost that does not depend on the events: 135 us at 484 voxels and 32 angles,
+// 395 us at 864 voxels and 60; the rows take 177 and 1025 us for 2 events per
 // angle, and 150 and 631 us for 1, where little is gained.
 bool node_use(const lm_handle* h, int64_t n) {
     return node_model(h) && n >= (int64_t)2 * h->mc.A &&

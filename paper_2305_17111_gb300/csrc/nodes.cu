@@ -54,9 +54,9 @@
 //
 // Measured (864 voxels and 864 points, 3 lines, 60 angles of 64 bins; times
 // below that name no size are this model's): a forward projection of 100 000
-// events 0.33 ms of kernels, 19.5 ms through the rows and 0.79 ms with the
+// events 0.34 ms of kernels, 19.5 ms through the rows and 0.79 ms with the
 // image spread at every angle anew through the path tables; a back projection
-// 0.62 ms (12.0 ms, 0.70 ms); a sub-iteration of 8 angles 0.19 ms (2.15 ms,
+// 0.51 ms (12.0 ms, 0.70 ms); a sub-iteration of 8 angles 0.19 ms (2.15 ms,
 // 0.32 ms).  At 3464 voxels and 120 angles of 128 bins a sub-iteration of 15
 // angles takes 0.61 ms (26 ms, 1.29 ms).
 #include <math.h>
@@ -358,10 +358,11 @@ __device__ __forceinline__ void slot_taps(const NodeParams& P, int ai, int p, in
 // and the last of each adds them to the centre's sums.  At the end each node
 // collects its taps from the 9 centres around it.  No two lanes add to one
 // place, and every sum has its order.  Bound by instruction issue (66 %) once
-// the loads are a group ahead: 37 us; 47 us with a lane per centre, which
-// waits on three dependent loads per path, 42 us with a block per 122 nodes.
+// the loads are a group ahead: 41 us (with 7 taps 37 us, and then 47 us with a lane
+// per centre, which waits on three dependent loads per path, 42 us with a block
+// per tile).
 // Where a centre has more than kSpreadDense paths the scan's steps cost more
-// than those waits, and a lane takes a centre's paths: 80 us instead of 118 us
+// than those waits, and a lane takes a centre's paths: with 7 taps 80 instead of 118 us
 // at 3464 voxels (11, 6 and 3 paths a centre; limits of 2 and 4 are equal
 // there, 1 costs 83 us).  The first blocks form the slots' taps, a warp per
 // (angle, point, line with a knot).
@@ -497,8 +498,10 @@ __global__ void __launch_bounds__(32 * kSpreadWarps) k_ang_spread(const NodePara
 
 // S's part of one (angle, 32 scatter points, line): two direction offsets m a
 // thread, the points one after the other, 16 bins at a time (a collimator value
-// read from shared memory serves both offsets).  Bound by FP32 issue: 115 us for
-// 60 angles, 20 us for 8.
+// read from shared memory serves both offsets).  Bound by FP32 issue: 106 us for
+// 60 angles, 20 us for 8.  (The slots' shares go in after the points, in the warps
+// that hold one: 367 us for a forward projection, 444 us with the taps formed here
+// and added point by point.)
 constexpr int kOffThreads = 128, kOffPer = 2;
 
 __global__ void __launch_bounds__(kOffThreads, 6) k_ang_bins(const NodeParams P, int tiles) {
@@ -624,8 +627,8 @@ __global__ void __launch_bounds__(kOffThreads, 6) k_ang_bins(const NodeParams P,
 // A row's (angle, bin) sums over the chunks of its run of scatter points, then
 // from the direction offsets onto the scattered-energy nodes: a block per row;
 // the blocks past those form the unscattered sums, a warp per (row, line).
-// Bound by load latency: 8 loads in flight per thread, whatever the run.  91 us
-// for 60 angles, 16 us for 8.
+// Bound by load latency: 8 loads in flight per thread, whatever the run.  75 us
+// for 60 angles, 14 us for 8.
 constexpr int kRowThreadsN = 512, kRowChunks = 512;
 __global__ void __launch_bounds__(kRowThreadsN) k_node_bins(const NodeParams P) {
     extern __shared__ float srow[];   // [nm_pad]
@@ -698,8 +701,8 @@ __global__ void __launch_bounds__(kRowThreadsN) k_node_bins(const NodeParams P) 
 
 // out[row][x] = sum_y m[y][x] in[row][y] over the band of y each x reaches,
 // for 8 rows and 32 x per block: the warps share the band's y (a run each, the
-// loads of a run in flight together), their sums are added in warp order.  63 us
-// forward and 78 us back for 60 angles, 13 and 14 us for 8.
+// loads of a run in flight together), their sums are added in warp order.  69 us
+// forward and 76 us back for 60 angles, 13 and 14 us for 8.
 __device__ __forceinline__ void band_product(const float* in, int in_stride, const float* m,
                                              int m_stride, float* out, int out_stride, int rows,
                                              int r0, int x0, int lo, int hi, float* sh) {
@@ -841,8 +844,9 @@ __global__ void __launch_bounds__(256) k_ang_psi(const NodeParams P) {
 // the points' collimator values, bins and line integrals of a batch of angles
 // are staged in shared memory together, which leaves one load latency (PSI's, 8
 // bins in flight) per angle.  Bound by issue (54 %) and that latency; eight
-// blocks an SM put every warp of the grid on the chip at once: 412 us for 60
-// angles and 54 us for 8 (503 and 66 us with the collimator values read bin by
+// blocks an SM put every warp of the grid on the chip at once: 293 us for 60
+// angles and 40 us for 8 (at 2792 direction nodes, where it took 412 and 54 us:
+// 503 and 66 us with the collimator values read bin by
 // bin; 16 or 4 bins in flight: 426, 468 us; one warp a block: 410 us, but 264
 // instead of 210 us for 15 angles at 3464 voxels).  A grid that leaves most of
 // the chip idle is split over the angles, up to 8 parts that k_ang_paths adds
@@ -1002,8 +1006,9 @@ __device__ __forceinline__ float beyond_knots(const NodeParams& P, int w, int p,
 }
 
 // The paths' values in direction order, a thread per (point, path): the taps
-// of consecutive paths are consecutive nodes.  15 us; kSplit adds the parts of
-// a split k_ang_back (a loop over one part cost 17 us, and 79 instead of 52 us
+// of consecutive paths are consecutive nodes.  24 us for 8 angles, 14 of them without the
+// knots; kSplit adds the parts of a split k_ang_back (with 7 taps and no knots a
+// loop over one part cost 17 instead of 15 us, and 79 instead of 52 us
 // at 3464 voxels).
 template <bool kSplit>
 __global__ void __launch_bounds__(256) k_ang_paths(const NodeParams P) {
@@ -1625,12 +1630,6 @@ static int build_node_tables(lm_handle* h) {
     const double pi = 3.14159265358979323846, log2e = 1.4426950408889634, me = 510.99895;
     const double kappa = m.fwhm_frac * sqrt(m.e_ref) / (2.0 * sqrt(2.0 * log(2.0)));   // sigma = kappa sqrt(E)
     auto t_of = [&](double e) { return 2.0 * sqrt(e) / kappa; };
-    auto mu_of = [&](double e) {
-        if (m.n_knots == 1) return m.knot_mu[0];
-        int s = 0;
-        while (s < m.n_knots - 2 && e >= m.knot_e[s + 1]) ++s;
-        return m.knot_mu[s] + (e - m.knot_e[s]) * m.knot_slope[s];
-    };
     N.W = m.W;
     std::vector<NodeSlot> slots;
     std::vector<int> slot_start;
@@ -2014,8 +2013,6 @@ int node_spread(lm_handle* h, const float* lam_v, float* H, int a0, int a_step, 
     P.side = side;
     int tiles = 0;
     for (int w = 0; w < P.N.W; ++w) tiles += (P.N.n_dir[w] + kSpreadOut - 1) / kSpreadOut;
-    int rc = prof_start(h, st);
-    if (rc != LMMEW_OK) return rc;
     const int units = H ? h->mc.np * tiles : 0;
     int64_t sides = 0;
     for (int w = 0; w < P.N.W; ++w)
@@ -2023,6 +2020,8 @@ int node_spread(lm_handle* h, const float* lam_v, float* H, int a0, int a_step, 
     const int side_blocks = (int)((sides + kSpreadWarps - 1) / kSpreadWarps);
     const int blocks = side_blocks + (units + kSpreadWarps - 1) / kSpreadWarps;
     if (blocks == 0) return LMMEW_OK;
+    int rc = prof_start(h, st);
+    if (rc != LMMEW_OK) return rc;
     k_ang_spread<<<(unsigned)blocks, 32 * kSpreadWarps, 0, st>>>(P, tiles, units, side_blocks);
     ++h->launches;
     LMMEW_CUDA(cudaGetLastError());
