@@ -53,7 +53,8 @@
  *     (the same model; interpolation adds 1e-7 of a path's value up to 6 sigma
  *     from its energy and 3e-6 at the 8 sigma where the reach ends, no more than
  *     the rows' rounding there; a path further than 10 sigma from an event adds
- *     nothing, and an infinite image value or weight may give NaN).
+ *     nothing, values 1e-22 of a bin's largest may round to either side of 0, and
+ *     an infinite image value or weight may give NaN).
  *     lm_forward and lm_backproject take them from 2 events per angle (8 for
  *     back projections of small models), lm_osem and lm_osem_batch, per
  *     realisation, from 120 per angle where a sub-iteration's rows are estimated
